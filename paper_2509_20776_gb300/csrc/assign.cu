@@ -771,7 +771,7 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
     SP_TRY((assign_stage<RP, CI, VT, IX>(ctx, pl, tcol, tval, cv.at<unsigned>(o_tk), s)));
     const RowsWs w1 = rows_bind(cv, nI, nt, r1);
     const int kb = ceil_log2_u64(uint64_t(A.ncols));
-    SP_TRY((run_rows<CI, VT, NoGather<CI, VT>>(ctx, s, pl->vp, nI, nt, kb, w1, nullptr, true, tcol, tval)));
+    SP_TRY((sort_rows_in_place<CI, VT>(ctx, s, pl->vp, nI, nt, kb, w1, tcol, tval)));
   }
   // assembly: runs of untouched rows from A, rows of I from the staging buffer (or left
   // to the merge)
@@ -884,26 +884,15 @@ struct FusedGs {
   const IX* qinv;  // null: identity
   const long long* sstart;
   long long nnzA, ntemp, n;
-  __device__ long long src(long long i) const { return sstart[i]; }
-  __device__ CI col(long long pos) const {
-    if (pos & kStaged) {
-      const long long q = pos & ~kStaged;
-      return q < ntemp ? ld_stream(tcol + q) : CI(0);
-    }
-    return (pos >= 0 && pos < nnzA) ? ld_stream(colA + pos) : CI(0);
+  __device__ const long long* srcs() const { return sstart; }
+  __device__ GsView<CI, VT> view(long long src, long long L) const {
+    const long long q = src & ~kStaged;
+    if (src & kStaged) return q + L <= ntemp ? GsView<CI, VT>{tcol + q, tval + q, 0u} : GsView<CI, VT>{};
+    return q + L <= nnzA ? GsView<CI, VT>{colA + q, valA + q, 0u} : GsView<CI, VT>{};
   }
-  __device__ VT val(long long pos) const {
-    if (pos & kStaged) {
-      const long long q = pos & ~kStaged;
-      return q < ntemp ? ld_stream(tval + q) : VT(0);
-    }
-    return (pos >= 0 && pos < nnzA) ? ld_stream(valA + pos) : VT(0);
-  }
-  __device__ CI map(long long, CI c) const {
+  __device__ uint32_t map(unsigned, uint32_t c) const {  // a column outside: SP_ERR_INDEX_RANGE by the sort
     if (!qinv) return c;
-    const long long cl = (long long)c;
-    if (cl < 0 || cl >= n) return CI(-1);  // reported as SP_ERR_INDEX_RANGE by the sort
-    return CI(ld_map(qinv + cl));
+    return c > uint32_t(n - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
   }
 };
 
@@ -971,8 +960,8 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
                               qinv, sstart, A.nnz, nt, n};
   const RowsWs w = rows_bind(cv, m, nnz_out, ro);
   const int kb = ceil_log2_u64(uint64_t(n));
-  return run_rows(ctx, s, vp, m, nnz_out, kb, w, &g, true, static_cast<CI*>(out->colidx),
-                  static_cast<VT*>(out->values));
+  return sort_rows_from(ctx, s, vp, m, nnz_out, kb, w, g, static_cast<CI*>(out->colidx),
+                        static_cast<VT*>(out->values));
 }
 
 }  // namespace sp

@@ -445,8 +445,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
     SP_TRY(ctx_workspace(ctx, cw.total(), s, &base));
     cw.bind(base);
     const RowsWs w = rows_bind(cw, nreq, jtot, ro);
-    SP_TRY((run_rows<IX, uint32_t, NoGather<IX, uint32_t>>(ctx, s, b->djoff, nreq, jtot, b->key_bits, w,
-                                                           nullptr, true, jkey, b->jpos)));
+    SP_TRY((sort_rows_in_place<IX, uint32_t>(ctx, s, b->djoff, nreq, jtot, b->key_bits, w, jkey, b->jpos)));
     {
       SP_PHASE(SP_PHASE_MAP);
       k_batch_jdup<IX><<<grid_for(jtot, 256, nsm * 8), 256, 0, s>>>(b->djoff, nreq, jkey, jtot, ctx->dstatus);
@@ -518,11 +517,11 @@ sp_status batch_fill_body(sp_ctx* ctx, sp_batch* b, sp_csr* out, cudaStream_t s,
       SP_PHASE(SP_PHASE_GATHER);
       const XBatchSrc<CI, VT> src{b->rreq, b->rv, b->jrp};
       k_xfill<XBatchSrc<CI, VT>, false><<<grid_for((rows + 31) / 32 * 32, XB, ctx->num_sms * 8), XB, 0, s>>>(
-          src, rows, b->rs0, b->rsn, b->vp, oc, ov, w.fin, w.counters + 0, w.fin_cap, w.huge, w.huge_n(),
+          src, rows, b->rs0, b->rsn, b->vp, oc, ov, w.runs(), w.huge, w.huge_n(),
           w.huge_cap, kb, b->max_nj <= 0xFFFFFFFFll ? XF_LANE : 0, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
-    return sort_queued<CI, VT>(ctx, s, w, kb, oc, ov);
+    return sort_queued<CI, VT>(ctx, s, w, nnz, kb, oc, ov);
   }
   {
     SP_PHASE(SP_PHASE_GATHER);
@@ -537,7 +536,7 @@ sp_status batch_fill_body(sp_ctx* ctx, sp_batch* b, sp_csr* out, cudaStream_t s,
   SP_TRY(ctx_workspace(ctx, cf.total(), s, &base));
   cf.bind(base);
   const RowsWs w = rows_bind(cf, rows, nnz, rf, true, n_slow);
-  return run_rows<CI, VT, NoGather<CI, VT>>(ctx, s, b->vp, rows, nnz, kb, w, nullptr, true, oc, ov);
+  return sort_rows_in_place<CI, VT>(ctx, s, b->vp, rows, nnz, kb, w, oc, ov);
 }
 
 template <class RP, class CI, class VT, class IX>

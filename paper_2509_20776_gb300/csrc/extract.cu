@@ -51,10 +51,9 @@ struct ExtractRangeGs {
   const VT* v_;
   const long long* sstart;
   long long j0;
-  __device__ long long src(long long i) const { return sstart[i]; }
-  __device__ CI col(long long pos) const { return ld_stream(c_ + pos); }
-  __device__ VT val(long long pos) const { return ld_stream(v_ + pos); }
-  __device__ CI map(long long, CI c) const { return CI((long long)c - j0); }
+  __device__ const long long* srcs() const { return sstart; }
+  __device__ GsView<CI, VT> view(long long src, long long) const { return {c_ + src, v_ + src, 0u}; }
+  __device__ CI map_ci(unsigned, CI c) const { return CI((long long)c - j0); }
 };
 
 // Repeated J (Sec. 2.2 allows repeats): column c of A feeds every position b with
@@ -329,8 +328,8 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
     SP_TRY(ctx_workspace(ctx, cw.total(), s, &base));
     cw.bind(base);
     const RowsWs w = rows_bind(cw, 1, nJ, ro);
-    SP_TRY((run_rows<uint32_t, uint32_t, NoGather<uint32_t, uint32_t>>(ctx, s, vp2, 1, nJ, ceil_log2_u64(uint64_t(n)),
-                                                                       w, nullptr, true, pl->jsk, pl->jsp)));
+    SP_TRY((sort_rows_in_place<uint32_t, uint32_t>(ctx, s, vp2, 1, nJ, ceil_log2_u64(uint64_t(n)), w, pl->jsk,
+                                                   pl->jsp)));
   }
   if (nI > 0) {
     const RP* rp = static_cast<const RP*>(A.rowptr);
@@ -388,7 +387,7 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     const ExtractRangeGs<CI, VT> g{static_cast<const CI*>(A.colidx), static_cast<const VT*>(A.values),
                                    pl->sstart, pl->j0};
     const RowsWs w = rows_bind(cv, nI, nnz_out, ro, false);
-    return run_rows(ctx, s, pl->vp, nI, nnz_out, 0, w, &g, false, oc, ov);
+    return gather_rows(ctx, s, pl->vp, nI, nnz_out, w, g, oc, ov);
   }
   if (pl->j_shape == 3) {
     // repeated J: every kept entry once per position of its column, then the row sort
@@ -406,7 +405,7 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     SP_CUDA(cudaGetLastError());
     const RowsWs w = rows_bind(cv, nI, nnz_out, ro);
     const int kb = ceil_log2_u64(uint64_t(pl->nJ));
-    return run_rows<CI, VT, NoGather<CI, VT>>(ctx, s, pl->vp, nI, nnz_out, kb, w, nullptr, true, oc, ov);
+    return sort_rows_in_place<CI, VT>(ctx, s, pl->vp, nI, nnz_out, kb, w, oc, ov);
   }
   const bool sorted = pl->j_shape == 1;  // ascending J: the relabelling keeps rows in order
   rows_reserve(cv, nI, nnz_out, sizeof(VT), ro, !sorted, pl->n_slow);
@@ -431,12 +430,12 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
       SP_PHASE(SP_PHASE_GATHER);
       const XOne<CI, VT, Rel> src{ci, vv, rel};
       if (sorted)
-        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.fin,
-                                                          w.counters + 0, w.fin_cap, w.huge, w.huge_n(),
+        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.runs(),
+                                                          w.huge, w.huge_n(),
                                                           w.huge_cap, kb, lane_rows, ctx->dstatus);
       else
-        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.fin,
-                                                           w.counters + 0, w.fin_cap, w.huge, w.huge_n(),
+        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.runs(),
+                                                           w.huge, w.huge_n(),
                                                            w.huge_cap, kb, lane_rows, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
@@ -456,7 +455,7 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     SP_TRY(fill(JSorted{pl->jsk, pl->jsp, pl->nJ}));
   if (sorted) return SP_OK;
   // the rows the warp path did not sort (more than XFAST source entries)
-  return sort_queued<CI, VT>(ctx, s, w, kb, oc, ov);
+  return sort_queued<CI, VT>(ctx, s, w, nnz_out, kb, oc, ov);
 }
 
 sp_status plan_release(sp_ctx* ctx, sp_plan* pl) {

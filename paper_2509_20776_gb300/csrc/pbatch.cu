@@ -147,17 +147,21 @@ struct PermBatchGs {
   using VT = VTt;
   const PermView* pv;
   const long long* rsrc;
-  __device__ long long src(long long r) const { return rsrc[r]; }
-  __device__ CI col(long long pos) const {
-    const CI* c = reinterpret_cast<const CI*>(__ldg(&pv[pos >> kReqShift].col));
-    return ld_stream(c + (pos & kEntryMask));
+  __device__ const long long* srcs() const { return rsrc; }
+  __device__ GsView<CI, VT> view(long long src, long long) const {
+    const PermView* v = pv + (src >> kReqShift);
+    const long long e = src & kEntryMask;
+    return {reinterpret_cast<const CI*>(__ldg(&v->col)) + e, reinterpret_cast<const VT*>(__ldg(&v->val)) + e,
+            unsigned(src >> kReqShift)};
   }
-  __device__ VT val(long long pos) const {
-    const VT* v = reinterpret_cast<const VT*>(__ldg(&pv[pos >> kReqShift].val));
-    return ld_stream(v + (pos & kEntryMask));
+  __device__ uint32_t map(unsigned mid, uint32_t c) const {
+    const PermView* v = pv + mid;
+    const IX* qinv = reinterpret_cast<const IX*>(__ldg(&v->qinv));
+    if (!qinv) return c;
+    return c > uint32_t(__ldg(&v->ncol) - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
   }
-  __device__ CI map(long long pos, CI c) const {
-    const PermView* v = pv + (pos >> kReqShift);
+  __device__ CI map_ci(unsigned mid, CI c) const {
+    const PermView* v = pv + mid;
     const IX* qinv = reinterpret_cast<const IX*>(__ldg(&v->qinv));
     if (!qinv) return c;
     const long long cl = (long long)c;
@@ -247,11 +251,12 @@ sp_status pbatch_fill_impl(sp_ctx* ctx, sp_pbatch* b, sp_csr* out, cudaStream_t 
   if (nnz == 0 || rows == 0) return SP_OK;
   CI* oc = static_cast<CI*>(out->colidx);
   VT* ov = static_cast<VT*>(out->values);
-  // phase 1: gather + relabel over the whole batch; phase 2 (any column map): row sort
-  const RowsWs w = rows_bind(cv, rows, nnz, b->ro);
+  // gather + relabel over the whole batch; with any column map also the row sort
+  const RowsWs w = rows_bind(cv, rows, nnz, b->ro, b->qtot > 0);
   const int kb = ceil_log2_u64(uint64_t(b->max_cols > 1 ? b->max_cols : 1));
   const PermBatchGs<CI, VT, IX> g{views, rsrc};
-  return run_rows(ctx, s, vp, rows, nnz, kb, w, &g, b->qtot > 0, oc, ov);
+  if (b->qtot == 0) return gather_rows(ctx, s, vp, rows, nnz, w, g, oc, ov);
+  return sort_rows_from(ctx, s, vp, rows, nnz, kb, w, g, oc, ov);
 }
 
 }  // namespace sp
@@ -315,7 +320,7 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
   b->o_rsn = cv.reserve(size_t(b->rows) * 8);
   b->o_vp = cv.reserve(size_t(b->rows + 1) * 8);
   b->o_scan = cv.reserve(scan_ws_bytes(b->rows));
-  rows_reserve(cv, b->rows, b->nnz, vs, b->ro);
+  rows_reserve(cv, b->rows, b->nnz, vs, b->ro, b->qtot > 0);
   cudaStream_t s = (cudaStream_t)stream;
   b->stream = s;
   if (cudaSetDevice(ctx->device) != cudaSuccess) {

@@ -46,10 +46,12 @@ struct PermGs {
   const IX* qinv;           // old column -> new column (null: identity)
   const long long* sstart;  // source start of output row r
   long long n;
-  __device__ long long src(long long r) const { return sstart[r]; }
-  __device__ CI col(long long pos) const { return ld_stream(c_ + pos); }
-  __device__ VT val(long long pos) const { return ld_stream(v_ + pos); }
-  __device__ CI map(long long, CI c) const {
+  __device__ const long long* srcs() const { return sstart; }
+  __device__ GsView<CI, VT> view(long long src, long long) const { return {c_ + src, v_ + src, 0u}; }
+  __device__ uint32_t map(unsigned, uint32_t c) const {  // (a sort follows only a column permutation: n > 0)
+    return c > uint32_t(n - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
+  }
+  __device__ CI map_ci(unsigned, CI c) const {
     if (!qinv) return c;
     const long long cl = (long long)c;
     if (cl < 0 || cl >= n) return CI(-1);
@@ -71,7 +73,7 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   const size_t o_scan = cv.reserve(scan_ws_bytes(m));
   const size_t o_ss = cv.reserve(size_t(m) * 8);
   size_t ro[kRowsSlots];
-  rows_reserve(cv, m, nnz, sizeof(VT), ro);
+  rows_reserve(cv, m, nnz, sizeof(VT), ro, q != nullptr);
   char* base;
   SP_TRY(ctx_workspace(ctx, cv.total(), s, &base));
   cv.bind(base);
@@ -114,12 +116,12 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   if (nnz == 0 || m == 0) return SP_OK;
   CI* out_col = static_cast<CI*>(B->colidx);
   VT* out_val = static_cast<VT*>(B->values);
-  // phase 1: gather + relabel; phase 2 (a column permutation only): sort every row
+  // gather and relabel; with a column permutation also sort every row
   const PermGs<CI, VT, IX> g{static_cast<const CI*>(A->colidx), static_cast<const VT*>(A->values), qinv,
                              sstart, n};
-  const RowsWs w = rows_bind(cv, m, nnz, ro);
-  const int kb = ceil_log2_u64(uint64_t(n));
-  return run_rows(ctx, s, vp, m, nnz, kb, w, &g, q != nullptr, out_col, out_val);
+  const RowsWs w = rows_bind(cv, m, nnz, ro, q != nullptr);
+  if (!q) return gather_rows(ctx, s, vp, m, nnz, w, g, out_col, out_val);
+  return sort_rows_from(ctx, s, vp, m, nnz, ceil_log2_u64(uint64_t(n)), w, g, out_col, out_val);
 }
 
 sp_status alloc_csr(sp_ctx* ctx, sp_csr* B, cudaStream_t s) {

@@ -1,18 +1,17 @@
-// Two-phase Build step (Sec. 3.1, Algorithm 2's fill pass and the per-row sort):
-//   phase 1, k_gather_chunks: every output row gets its source entries, relabelled,
-//     at its final row position but in source order (a load-balanced gather over
-//     fixed chunks of output positions: no shared-memory sort, all loads independent);
-//   phase 2, the rows of the output are sorted in place:
-//     * rows of at most CP entries (512, or 1024 with the run-time tile shape 1) in
-//       tiles of consecutive rows, at most 2 * CP entries each, k_seg_sort<SsTile> or
-//       k_seg_sort<SsTileL>;
-//     * rows of CP < L <= SS_RUN_MAX entries alone, k_seg_sort<SsRunT<VT>>;
-//     * longer rows are first cut by key range (k_split: a coarse, then a fine split) into runs of at
-//       most SS_RUN_MAX entries, which k_seg_sort<SsRunT<VT>> then sorts.
-//   Buckets of more keys than the (run-time) heavy threshold are queued as runs for up
-//   to SS_PASSES later passes.
-// One scan over the output rows (RowsPartition) cuts the tiles and the gather chunks
-// and lists the rows that do not fit a tile.
+// The Build step (Sec. 3.1, Algorithm 2's fill pass and the per-row sort): every output row
+// takes its source entries, relabelled, and is sorted by column.
+//   * Rows of at most TMAX entries (512, or 1024 with the run-time tile shape 1) go in tiles
+//     of consecutive rows, k_seg_sort<SsTile / SsTileL>: the tile reads its rows' source
+//     entries itself (column, relabel lookup, value), sorts them in shared memory and
+//     writes them once.
+//   * Rows of TMAX < L <= SS_RUN_MAX entries go alone, k_seg_sort<SsRun> (of at most
+//     SS_SMALL_RUN entries: k_seg_sort<SsRunS>), read and written the same way.
+//   * Longer rows are gathered in chunks to their place in the output (k_gather_long), cut
+//     by key range (k_split: a coarse, then a fine split) into runs of at most SS_RUN_MAX
+//     entries, and the runs sorted by k_seg_sort<SsRun / SsRunS>.
+// Rows that lie in the output already (a sort alone) take the same kernels with the output
+// as their source; a gather without a sort is k_gather_chunks.  One pass over the row
+// pointer (RowsPartition) finds the tiles' first rows and lists the rows that fit none.
 #pragma once
 
 #include <type_traits>
@@ -21,58 +20,65 @@
 
 namespace sp {
 
-constexpr int SS_ROW_W = 4;                    // partition weight of a row
 constexpr int SS_HEAVY = 128;                  // default (and smallest) heavy-bucket threshold
-constexpr int SS_PASSES = 3;                   // passes over queued heavy buckets
+constexpr int SS_LEVELS = 3;                   // levels a heavy bucket is bucketed again
 
-// A sort configuration: BLOCK threads sort items of at most CAP entries, MINB CTAs per
-// SM; a tile holds the rows whose partition coordinate starts in a window of
-// CP = CAP / 2, so at most ROWS = CP / SS_ROW_W rows (one thread each) of at most CP
-// entries.  A single run of L entries uses at most ss_nb(L) <= CAP / 2 bucket counters.
-template <int BLOCK_, int CAP_, bool TILES_, int MINB_, bool BACK_ = false>
+// A sort configuration: B threads hold ITEMS entries each of an item of at most CAP = B *
+// ITEMS entries, MINB CTAs per SM.  A tile holds the rows whose partition coordinate (the
+// row's output position + W for every earlier row) lies in a window of WIN, so at most
+// ROWS = WIN / W rows; of those it sorts the rows of at most TMAX entries, as many whole
+// rows at a time as fit in CAP (a second round takes what a window's last rows add).
+template <int BLOCK_, int ITEMS_, int MINB_, bool TILES_ = false>
 struct SsCfg {
-  static constexpr int B = BLOCK_, CAP = CAP_, CP = CAP_ / 2, ROWS = CP / SS_ROW_W, MINB = MINB_;
-  static constexpr int WORDS = CAP_ / 32;  // row-start bitmap words
+  static constexpr int B = BLOCK_, ITEMS = ITEMS_, CAP = B * ITEMS, MINB = MINB_;
+  static constexpr int TMAX = CAP / 2, WIN = CAP - CAP / 16, W = 4, ROWS = WIN / W;
+  static constexpr int RPT = (ROWS + B - 1) / B;  // rows a thread sets up
+  static constexpr int WORDS = CAP / 32;   // row-start bitmap words
   static constexpr bool kTiles = TILES_;   // items are tiles (else: single runs)
-  static constexpr bool kBack = BACK_;     // runs: taken from the back of the run list
-  static constexpr int CNT = TILES_ ? CAP_ : CAP_ / 2;  // bucket counters
-  static_assert(!TILES_ || ROWS <= B, "one thread per row of a tile");
-  static_assert(WORDS % 32 == 0, "one warp scans the bitmap");
   static_assert(B % 32 == 0 && B * MINB <= 2048, "whole warps, resident CTAs");
+  static_assert(CAP <= 4096 && ROWS < 65536 / 2, "packed positions and counts");
 };
-using SsTile = SsCfg<128, 1024, true, 9>;   // tiles of rows of at most 512 entries
-using SsTileL = SsCfg<256, 2048, true, 4>;  // tile shape 1: rows of at most 1024 entries
-// single runs of at most 4096 entries: with 4-byte values three CTAs of 384 threads fit
-// an SM (72 KB of shared memory each), with 8-byte values two of 512 (88 KB)
-template <class VT>
-using SsRunT = std::conditional_t<sizeof(VT) == 4, SsCfg<384, 4096, false, 3>, SsCfg<512, 4096, false, 2>>;
-// runs of at most 1024 entries (the back of the run list): 128 threads, 8 CTAs per SM
-using SsRunS = SsCfg<128, 1024, false, 8, true>;
-constexpr int SS_SMALL_RUN = SsRunS::CAP;
-constexpr int SS_TILE_MAX = SsTile::CP;  // longest row a tile accepts (the smaller tile shape)
-constexpr int SS_RUN_MAX = 4096;         // longest row sorted alone
-static_assert(SsRunT<uint32_t>::CAP == SS_RUN_MAX && SsRunT<unsigned long long>::CAP == SS_RUN_MAX,
-              "one run capacity");
+// Shapes by measurement (R-MAT scale 25, 1.05 G entries, whole permutation; start 21.0 ms):
+// few entries per thread and many threads -- 256 x 4 at 5 CTAs per SM 17.6 ms, 6 CTAs 18.4,
+// 4 CTAs 18.4, 128 x 8 at 8 CTAs 24.0, 64 x 16 31 (longer unrolled code, and the lookups of a
+// thread in flight at once evict one another's lines from the L1 that shared memory leaves).
+using SsTile = SsCfg<256, 4, 5, true>;   // tiles of rows of at most 512 entries
+using SsTileL = SsCfg<256, 8, 4, true>;  // tile shape 1: rows of at most 1024 entries
+using SsRun = SsCfg<512, 8, 2>;          // single runs of at most 4096 entries
+using SsRunM = SsCfg<256, 8, 4>;         // of at most 2048
+using SsRunS = SsCfg<256, 4, 5>;         // of at most 1024
+constexpr int SS_SMALL_RUN = SsRunS::CAP, SS_MID_RUN = SsRunM::CAP;
+constexpr int SS_TILE_MAX = SsTile::TMAX;  // longest row a tile accepts (the smaller tile shape)
+constexpr int SS_RUN_MAX = 4096;           // longest row sorted alone
+static_assert(SsRun::CAP == SS_RUN_MAX, "run capacity");
+static_assert(SsTile::W == SsTileL::W && SsTile::WIN <= SsTileL::WIN, "one bound on the number of tiles");
 
-// Runs handed from one kernel to the next: in the output arrays or in the temporary
-// arrays (keys as uint32, values) at the same offsets.
-enum BufId : int { BUF_TEMP = 0, BUF_OUT = 1 };
+// Where a run's entries are: in the output arrays or in the temporary arrays (keys as
+// uint32, values) at the run's output offset, or still at the row's source.
+enum BufId : int { BUF_TEMP = 0, BUF_OUT = 1, BUF_SRC = 2 };
 
-struct FinalEntry {  // a run of at most SS_RUN_MAX entries left to sort in place
-  long long off;
-  long long len;
+struct FinalEntry {  // a run of at most SS_RUN_MAX entries left to sort
+  long long off;     // output offset
+  int len;
   int buf;
-  int pad;
+  long long row;     // BUF_SRC: the output row
 };
-// The run list is filled from both ends: n[0] counts the runs at its front, n[1] the runs
-// of at most SS_SMALL_RUN entries at its back (k_seg_sort<SsRunS>, small CTAs, sorts those;
-// k_seg_sort<SsRunT> the front).  cap bounds all the runs a pass queues, so the two ends
-// never meet.
-__device__ __forceinline__ void queue_run(FinalEntry* list, unsigned* n, long long cap, const FinalEntry& e,
-                                          DevStatus* st, long long err) {
-  const bool small = e.len <= SS_SMALL_RUN;
-  const unsigned q = atomicAdd(n + (small ? 1 : 0), 1u);
-  if (q < cap) list[small ? cap - 1 - q : q] = e;
+// The run lists: slices of one array, by what sorts them -- runs of at most SS_WARP_RUN
+// entries a warp (k_sort_warp_runs; only where a caller queues them: an empty slice passes
+// them on), of at most SS_SMALL_RUN, SS_MID_RUN, SS_RUN_MAX entries a CTA of SsRunS,
+// SsRunM, SsRun -- each with its own count and bound.
+constexpr int SS_WARP_RUN = 128;
+struct RunLists {
+  FinalEntry* list;
+  unsigned* n;               // 4 counts
+  long long c0, c1, c2, c3;  // capacity of each slice
+  __device__ __forceinline__ FinalEntry* slice(int k) const { return list + (k > 0 ? c0 : 0) + (k > 1 ? c1 : 0) + (k > 2 ? c2 : 0); }
+  __device__ __forceinline__ long long cap(int k) const { return k == 0 ? c0 : k == 1 ? c1 : k == 2 ? c2 : c3; }
+};
+__device__ __forceinline__ void queue_run(const RunLists& rl, const FinalEntry& e, DevStatus* st, long long err) {
+  const int k = e.len <= SS_WARP_RUN && rl.c0 > 0 ? 0 : e.len <= SS_SMALL_RUN ? 1 : e.len <= SS_MID_RUN ? 2 : 3;
+  const unsigned q = atomicAdd(rl.n + k, 1u);
+  if (q < rl.cap(k)) rl.slice(k)[q] = e;
   else dev_fail(st, SP_ERR_INTERNAL, err);
 }
 struct HugeEntry {  // a run longer than SS_RUN_MAX; coarse split: keys in [lo, lo + 2^wb)
@@ -82,7 +88,13 @@ struct HugeEntry {  // a run longer than SS_RUN_MAX; coarse split: keys in [lo, 
   int wb;
   int buf;
   int pad;
+  long long row;    // the output row (rows gathered by k_gather_long)
 };
+struct LongChunk {  // SL_CH output positions of a row longer than SS_RUN_MAX
+  unsigned huge;    // its slot of the huge list
+  unsigned chunk;
+};
+constexpr int SL_CH = 4096;
 
 // The rows queued for the key-range split.  n[0] counts the rows queued at the front of
 // the list, n[1] the rows of at least SPLIT_HUB entries queued from its back; the split
@@ -90,12 +102,13 @@ struct HugeEntry {  // a run longer than SS_RUN_MAX; coarse split: keys in [lo, 
 // once instead of wherever the queueing order put it.  cap >= nnz / SS_RUN_MAX + 1 bounds
 // the number of rows longer than SS_RUN_MAX, so the two ends never meet.
 constexpr long long SPLIT_HUB = 1ll << 16;
-__device__ __forceinline__ void queue_huge(HugeEntry* list, unsigned* n, long long cap, const HugeEntry& e,
+__device__ __forceinline__ long long queue_huge(HugeEntry* list, unsigned* n, long long cap, const HugeEntry& e,
                                            DevStatus* st, long long err) {
   const bool hub = e.len >= SPLIT_HUB;
   const unsigned q = atomicAdd(n + (hub ? 1 : 0), 1u);
   if (q < cap) list[hub ? cap - 1 - q : q] = e;
   else dev_fail(st, SP_ERR_INTERNAL, err);
+  return q < cap ? (hub ? cap - 1 - q : q) : -1;
 }
 
 constexpr int GC_BLOCK = 256;                  // gather: threads per CTA
@@ -105,69 +118,78 @@ constexpr int GC_MINB = 5;                     // gather: resident CTAs per SM (
 constexpr int GC_H = 4;                        // gather: positions a thread loads before it stores
 
 // ---- partition ----------------------------------------------------------------------
-// Row r weighs SS_ROW_W plus its length when a tile sorts it (length <= tmax, the tile
-// shape's CP).  With c(r) the exclusive prefix of the weights, tile t holds the rows with
-// c(r) in [t*tmax, (t+1)*tmax): at most tmax / SS_ROW_W rows and 2*tmax entries.  Gather
-// chunk k starts at the row holding output position k*GC_CH.
-__device__ __forceinline__ long long rows_weight(const long long* vp, long long r, long long tmax) {
-  const long long L = vp[r + 1] - vp[r];
-  return SS_ROW_W + (L <= tmax ? L : 0);
-}
-
-struct RowsWeight {
-  const long long* vp;
-  long long tmax;
-  __device__ long long operator()(long long r) const { return rows_weight(vp, r, tmax); }
-};
-
+// Row r has the coordinate c(r) = vp[r] + W * r; tile t holds the rows with c(r) in
+// [t * win, (t + 1) * win): a closed form of the row pointer, so no scan of weights is
+// needed and the number of tiles is known on the host (a window inside a longer row is an
+// empty tile).  Gather chunk k starts at the row holding output position k * GC_CH.
+// The row pointer is clamped to nnz (lengths that do not add up to it were reported), so
+// no tile, run or chunk reaches past the output arrays.
 struct RowsPartition {
-  const long long* vp;
-  long long nrows;
-  long long ntiles_cap;  // tile_first holds ntiles_cap + 1 entries
-  long long* tile_first;
-  long long* ntiles;
+  long long nrows, nnz;
+  long long ntiles;         // tile_first holds ntiles + 1 entries
+  long long* tile_first;    // null: no tiles (nothing is sorted)
   long long nchunks;
-  long long* chunk_first;
-  FinalEntry* fin;  // rows sorted alone
-  unsigned* fin_n;
-  long long fin_cap;
-  HugeEntry* huge;  // rows for k_split
-  unsigned* huge_n;  // two counts (queue_huge)
+  long long* chunk_first;   // null: no gather chunks
+  RunLists runs;            // rows sorted alone
+  HugeEntry* huge;          // rows for k_split
+  unsigned* huge_n;         // two counts (queue_huge)
   long long huge_cap;
+  LongChunk* lchunk;        // chunks of the rows for k_split
+  unsigned* lchunk_n;
+  long long lchunk_cap;
   int key_bits;
-  int classify;  // list the rows that do not fit a tile (only when the rows are sorted)
-  long long tmax;  // longest row a tile accepts
+  int buf;                  // where the rows' entries are: BUF_SRC or BUF_OUT
+  int win, tmax;            // the tile shape's window and longest row
   DevStatus* st;
-  __device__ void operator()(long long r, long long c) const {
-    if (r == nrows) {  // c = total weight
-      long long nt = c / tmax + 1;
-      if (nt > ntiles_cap) {
-        dev_fail(st, SP_ERR_INTERNAL, -14);
-        nt = ntiles_cap;
+  // row r at output positions [o0, o1)
+  __device__ void operator()(long long r, long long o0, long long o1) const {
+    o0 = o0 < nnz ? o0 : nnz;
+    o1 = o1 < nnz ? o1 : nnz;
+    const long long L = o1 - o0;
+    if (tile_first) {
+      constexpr int W = SsTile::W;
+      if (r == 0) tile_first[0] = 0;
+      const long long c0 = o0 + W * r;
+      long long t = c0 / win + 1;
+      const long long c1 = o1 + W * (r + 1);
+      if (c1 >= t * win)
+        for (const long long t_hi = r + 1 == nrows ? ntiles : c1 / win; t <= t_hi && t <= ntiles; ++t)
+          tile_first[t] = r + 1;
+      else if (r + 1 == nrows)
+        for (; t <= ntiles; ++t) tile_first[t] = nrows;
+      if (L > tmax) {
+        if (L <= SS_RUN_MAX) {
+          queue_run(runs, FinalEntry{o0, int(L), buf, r}, st, -15);
+        } else {
+          const long long h =
+              queue_huge(huge, huge_n, huge_cap, HugeEntry{o0, L, 0u, key_bits, BUF_OUT, 0, r}, st, -16);
+          if (buf == BUF_SRC && h >= 0) {
+            const unsigned nc = unsigned((L + SL_CH - 1) / SL_CH), c = atomicAdd(lchunk_n, nc);
+            if (c + (unsigned long long)nc > (unsigned long long)lchunk_cap) {
+              dev_fail(st, SP_ERR_INTERNAL, -14);
+            } else {
+              for (unsigned k = 0; k < nc; ++k) lchunk[c + k] = LongChunk{unsigned(h), k};
+            }
+          }
+        }
       }
-      *ntiles = nt;
-      tile_first[nt] = nrows;
-      return;
     }
-    if (r == 0) tile_first[0] = 0;
-    const long long o0 = vp[r], o1 = vp[r + 1], L = o1 - o0;
-    const long long e = c + SS_ROW_W + (L <= tmax ? L : 0);
-    long long t_lo = c / tmax + 1, t_hi = e / tmax;
-    if (t_hi > ntiles_cap - 1) t_hi = ntiles_cap - 1;
-    for (long long t = t_lo; t <= t_hi; ++t) tile_first[t] = r + 1;
-    if (L <= 0) return;
-    long long k_hi = (o1 - 1) / GC_CH;
-    if (k_hi > nchunks - 1) k_hi = nchunks - 1;
-    for (long long k = (o0 + GC_CH - 1) / GC_CH; k <= k_hi; ++k) chunk_first[k] = r;
-    if (classify && L > tmax) {
-      if (L <= SS_RUN_MAX) {
-        queue_run(fin, fin_n, fin_cap, FinalEntry{o0, L, BUF_OUT, 0}, st, -15);
-      } else {
-        queue_huge(huge, huge_n, huge_cap, HugeEntry{o0, L, 0u, key_bits, BUF_OUT, 0}, st, -16);
-      }
+    if (chunk_first && L > 0) {
+      long long k_hi = (o1 - 1) / GC_CH;
+      if (k_hi > nchunks - 1) k_hi = nchunks - 1;
+      for (long long k = (o0 + GC_CH - 1) / GC_CH; k <= k_hi; ++k) chunk_first[k] = r;
     }
+    if (chunk_first && r + 1 == nrows)  // none, unless the lengths do not add up to nnz
+      for (long long k = (o1 + GC_CH - 1) / GC_CH; k < nchunks; ++k) chunk_first[k] = nrows;
   }
 };
+
+template <int kDummy = 0>
+__global__ void k_partition(RowsPartition part, const long long* __restrict__ vp) {
+  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < part.nrows;
+       r += (long long)gridDim.x * blockDim.x)
+    part(r, vp[r], vp[r + 1]);
+}
 
 // ---- conflict-free block scans over shared arrays ------------------------------------------
 // Each warp owns a contiguous segment of n / (B / 32) entries and walks it 32 entries at a
@@ -230,25 +252,63 @@ __device__ void smem_incl_max_w(uint32_t* a, int n, uint32_t* tmp) {
   __syncthreads();
 }
 
-// ---- phase 1: gather ----------------------------------------------------------------
+// ---- sources -------------------------------------------------------------------------
+// Where an output row's entries are and how their columns are relabelled:
+//   struct Gs {
+//     using CI, VT;                            // column / value words
+//     const long long* srcs() const;           // source start of every output row (packed
+//                                              // with whatever view() needs)
+//     GsView<CI, VT> view(long long src, long long L) const;  // the row's first entry
+//     uint32_t map(unsigned mid, uint32_t c) const;  // new column (0xFFFFFFFF: c lies
+//                                              // outside the matrix)
+//     CI map_ci(unsigned mid, CI c) const;     // the same in the column's own width
+//   };
+template <class CI, class VT>
+struct GsView {
+  const CI* c;   // null: the row's source is inconsistent (a library bug)
+  const VT* v;
+  unsigned mid;  // which relabelling
+};
+// A stored column as a 32-bit key; a 64-bit one outside [0, 2^32) becomes the key
+// 0xFFFFFFFF, which is outside every matrix that the sort takes.
+__device__ __forceinline__ uint32_t ss_key(int32_t c) { return uint32_t(c); }
+__device__ __forceinline__ uint32_t ss_key(uint32_t c) { return c; }
+__device__ __forceinline__ uint32_t ss_key(int64_t c) {
+  return (uint64_t(c) >> 32) ? 0xFFFFFFFFu : uint32_t(c);
+}
+
+// Rows that lie in the output already, as the source of the sort.
+template <class CIt, class VTt>
+struct RowsInPlace {
+  using CI = CIt;
+  using VT = VTt;
+  static constexpr bool kInPlace = true;
+  const long long* vp;
+  const CI* c_;
+  const VT* v_;
+  __device__ const long long* srcs() const { return vp; }
+  __device__ GsView<CI, VT> view(long long src, long long) const { return {c_ + src, v_ + src, 0u}; }
+  __device__ uint32_t map(unsigned, uint32_t c) const { return c; }
+};
+template <class Gs, class = void>
+struct in_place : std::false_type {};
+template <class Gs>
+struct in_place<Gs, std::void_t<decltype(Gs::kInPlace)>> : std::bool_constant<Gs::kInPlace> {};
+
+// ---- gather without a sort ----------------------------------------------------------------
 // Chunk k is GC_CH consecutive output positions, starting inside row chunk_first[k].
-// Gs: using CI, VT;
-//     __device__ long long src(long long r) const;     // source start of output row r
-//     __device__ typename Gs::CI col(long long pos) const;  // source column
-//     __device__ typename Gs::CI map(long long pos, typename Gs::CI c) const;  // new column
-//     __device__ typename Gs::VT val(long long pos) const;
 template <class Gs>
 __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, const long long* __restrict__ vp,
                                                             long long nrows, long long total,
                                                             const long long* __restrict__ chunk_first,
                                                             long long nchunks,
                                                             typename Gs::CI* __restrict__ out_col,
-                                                            typename Gs::VT* __restrict__ out_val) {
+                                                            typename Gs::VT* __restrict__ out_val, DevStatus* st) {
   using CI = typename Gs::CI;
   using VT = typename Gs::VT;
   constexpr int B = GC_BLOCK, ITEMS = GC_ITEMS;
   __shared__ uint32_t owner[GC_CH];
-  __shared__ long long r_off[B];
+  __shared__ GsView<CI, VT> r_v[B];  // the row's source
   __shared__ long long r_o0[B];
   __shared__ long long r_o1[B];
   __shared__ uint32_t tmp32[B / 32 + 1];
@@ -263,7 +323,7 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
     if (r < nrows) {
       a = vp[r];
       b = vp[r + 1];
-      s = gs.src(r);
+      s = gs.srcs()[r];
     }
   };
   // persistent: chunks blockIdx.x, + gridDim.x, ...; a batch is B consecutive rows.  The
@@ -277,9 +337,13 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
     const long long c0 = c * (long long)GC_CH, c1 = c0 + GC_CH < total ? c0 + GC_CH : total;
     const long long cn = c + gridDim.x;
     const long long rb_next_chunk = cn < nchunks ? chunk_first[cn] : 0;
-    const bool active = rb + t < nrows && o1 > o0 && o1 > c0 && o0 < c1;
+    bool active = rb + t < nrows && o1 > o0 && o1 > c0 && o0 < c1;
     if (active) {
-      r_off[t] = so;
+      r_v[t] = gs.view(so, o1 - o0);
+      if (!r_v[t].c) {
+        dev_fail(st, SP_ERR_INTERNAL, -13);
+        active = false;
+      }
       r_o0[t] = o0;
       r_o1[t] = o1;
     }
@@ -307,7 +371,8 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
     for (int h = 0; h < ITEMS; h += H) {
       CI cv[H];
       VT v[H];
-      long long pos[H];
+      int kk[H];
+      long long off[H];
       bool ok[H];
 #pragma unroll
       for (int u = 0; u < H; ++u) {
@@ -315,25 +380,27 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
         const long long g = c0 + x;
         const int ow = single ? 1 : int(owner[x]);
         ok[u] = false;
-        pos[u] = 0;
+        off[u] = 0;
+        kk[u] = 0;
         if (g < c1 && ow > 0) {
           const int k = ow - 1;
           const long long o = r_o0[k];
           // positions past this batch of rows belong to the next batch
           if (g >= o && g < r_o1[k]) {
             ok[u] = true;
-            pos[u] = r_off[k] + (g - o);
+            kk[u] = k;
+            off[u] = g - o;
           }
         }
       }
 #pragma unroll
-      for (int u = 0; u < H; ++u) cv[u] = ok[u] ? gs.col(pos[u]) : CI(0);
+      for (int u = 0; u < H; ++u) cv[u] = ok[u] ? ld_stream(r_v[kk[u]].c + off[u]) : CI(0);
 #pragma unroll
       for (int u = 0; u < H; ++u)
-        if (ok[u]) v[u] = gs.val(pos[u]);
+        if (ok[u]) v[u] = ld_stream(r_v[kk[u]].v + off[u]);
 #pragma unroll
       for (int u = 0; u < H; ++u)
-        if (ok[u]) cv[u] = gs.map(pos[u], cv[u]);
+        if (ok[u]) cv[u] = gs.map_ci(r_v[kk[u]].mid, cv[u]);
 #pragma unroll
       for (int u = 0; u < H; ++u) {
         if (!ok[u]) continue;
@@ -352,6 +419,56 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
   }
 }
 
+// The rows longer than SS_RUN_MAX: chunk by chunk of SL_CH entries, relabelled, to their
+// place in the output (k_split cuts them there).
+template <class Gs>
+__global__ void __launch_bounds__(GC_BLOCK, GC_MINB)
+    k_gather_long(Gs gs, const HugeEntry* __restrict__ huge, const LongChunk* __restrict__ chunks,
+                  const unsigned* __restrict__ n_p, long long cap, typename Gs::CI* __restrict__ out_col,
+                  typename Gs::VT* __restrict__ out_val, DevStatus* st) {
+  using CI = typename Gs::CI;
+  using VT = typename Gs::VT;
+  constexpr int H = GC_H, ITEMS = SL_CH / GC_BLOCK;
+  long long n = *n_p;
+  if (n > cap) n = cap;
+  for (long long k = blockIdx.x; k < n; k += gridDim.x) {
+    const LongChunk lc = chunks[k];
+    const HugeEntry he = huge[lc.huge];
+    const long long e0 = (long long)lc.chunk * SL_CH, o = he.off + e0;
+    const int len = he.len - e0 < SL_CH ? int(he.len - e0) : SL_CH;
+    const GsView<CI, VT> gv = gs.view(gs.srcs()[he.row], he.len);
+    if (!gv.c) {
+      if (threadIdx.x == 0) dev_fail(st, SP_ERR_INTERNAL, -13);
+      continue;
+    }
+#pragma unroll
+    for (int h = 0; h < ITEMS; h += H) {
+      CI cv[H];
+      VT v[H];
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const int x = threadIdx.x + (h + u) * GC_BLOCK;
+        cv[u] = x < len ? ld_stream(gv.c + e0 + x) : CI(0);
+      }
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const int x = threadIdx.x + (h + u) * GC_BLOCK;
+        v[u] = x < len ? ld_stream(gv.v + e0 + x) : VT(0);
+      }
+      uint32_t key[H];
+#pragma unroll
+      for (int u = 0; u < H; ++u) key[u] = gs.map(gv.mid, ss_key(cv[u]));
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const int x = threadIdx.x + (h + u) * GC_BLOCK;
+        if (x >= len) continue;
+        st_stream(out_col + o + x, CI(key[u]));
+        st_stream(out_val + o + x, v[u]);
+      }
+    }
+  }
+}
+
 // ---- approximate square-root bucketing of the row sort -----------------------------------
 // Bucket of key k in a row of L entries: nb = 2^(ceil(log2 L) - 1) buckets spaced evenly
 // in an approximate square root of k over the row's key range [0, kmax].  The root is
@@ -360,7 +477,6 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
 // scale nb / root(kmax) maps [0, kmax] onto the nb buckets.  The square root keeps
 // buckets balanced both for uniformly relabelled columns and for labels crowded at the
 // low end (degree-descending orderings).
-__device__ __forceinline__ uint32_t ss_nb(uint32_t L) { return L <= 2 ? 1u : 1u << (31 - __clz(L - 1)); }
 __device__ __forceinline__ float ss_root(uint32_t k) {
   return __uint_as_float((__float_as_uint(__uint2float_rn(k)) >> 1) + 0x1FC00000u);
 }
@@ -401,7 +517,7 @@ struct SplitFine {
 };
 constexpr int SS_RUN_LOG = 12;             // SS_RUN_MAX = 2^SS_RUN_LOG
 static_assert((1 << SS_RUN_LOG) == SS_RUN_MAX, "run capacity is a power of two");
-constexpr int GROUP_CAP = SS_RUN_MAX / 2;  // small buckets grouped up to this start window
+constexpr int GROUP_CAP = SS_SMALL_RUN;    // small buckets grouped up to this start window: runs of at most SS_MID_RUN
 template <class S, class VT>
 constexpr size_t split_smem_bytes() {
   // counts / starts / cursors, previous non-empty bucket, next group boundary; staged:
@@ -415,7 +531,7 @@ template <class S, class CI, class VT>
 __global__ void __launch_bounds__(S::B, S::MINB)
     k_split(const HugeEntry* __restrict__ runs, const unsigned* __restrict__ nruns_p, long long runs_cap,
             unsigned* ticket, uint32_t* __restrict__ tkey, VT* __restrict__ tval, CI* __restrict__ out_col,
-            VT* __restrict__ out_val, FinalEntry* __restrict__ fin, unsigned* fin_n, long long fin_cap,
+            VT* __restrict__ out_val, RunLists rl,
             HugeEntry* __restrict__ nxt, unsigned* nxt_n, long long nxt_cap, DevStatus* st) {
   constexpr int B = S::B, U = S::U, NBM = 1 << S::NBL;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -564,17 +680,17 @@ __global__ void __launch_bounds__(S::B, S::MINB)
       const uint32_t sb = hist[x], cc = bend(x) - sb;
       if (big) {
         if (cc <= uint32_t(SS_RUN_MAX)) {
-          queue_run(fin, fin_n, fin_cap, FinalEntry{g0 + sb, cc, dbuf, 0}, st, -6);
+          queue_run(rl, FinalEntry{g0 + sb, int(cc), dbuf, 0}, st, -6);
         } else {
           const unsigned q = atomicAdd(nxt_n, 1u);  // the fine split finds its key range itself
-          if (q < nxt_cap) nxt[q] = HugeEntry{g0 + sb, cc, 0u, 0, dbuf, 0};
+          if (q < nxt_cap) nxt[q] = HugeEntry{g0 + sb, cc, 0u, 0, dbuf, 0, 0};
           else dev_fail(st, SP_ERR_INTERNAL, -7);
         }
       } else if (head) {
         // reversed index of x+1 holds max over buckets >= x+1 of (L - start) -> min start
         const uint32_t nx = (x + 1 < NBM) ? nxb[NBM - 1 - (x + 1)] : 0u;
         const uint32_t end = nx ? uint32_t(L) - nx : uint32_t(L);
-        queue_run(fin, fin_n, fin_cap, FinalEntry{g0 + sb, (long long)(end - sb), dbuf, 0}, st, -6);
+        queue_run(rl, FinalEntry{g0 + sb, int(end - sb), dbuf, 0}, st, -6);
       }
     }
     __syncthreads();
@@ -675,83 +791,142 @@ __global__ void __launch_bounds__(S::B, S::MINB)
   }
 }
 
-// ---- phase 2: in-place sort of output rows ---------------------------------------------
+// ---- the sort of tiles and runs ----------------------------------------------------------
 
 template <class Cfg, class VT>
 __host__ __device__ constexpr size_t ss_smem_bytes() {
-  // values, keys in packed and bucket order, counters, bucket and source of each entry;
-  // tiles add the per-row tables and the row-start bitmap (an entry's row is its rank
-  // among the row starts, recomputed where needed: no per-entry row array, which keeps
-  // a tile CTA small enough for 9 per SM)
-  return size_t(Cfg::CAP) * (sizeof(VT) + 4 * 2 + 2 * 2) + size_t(Cfg::CNT) * 4 +
-         (Cfg::kTiles ? size_t(Cfg::ROWS) * (4 * 2 + 2 * 2) + size_t(Cfg::WORDS) * 4 * 2 : 0);
+  // values (sorted), keys (bucket order, then sorted), bucket counters; tiles add the row
+  // tables and the row-start bitmap with its word prefix
+  return size_t(Cfg::CAP) * (sizeof(VT) + 4 + 4) +
+         (Cfg::kTiles ? size_t(Cfg::ROWS) * 32 + size_t(Cfg::WORDS) * 8 : 0);
 }
 
-// In-place exclusive sum of a[0, n); thread t owns the ceil(n / B) consecutive entries
-// starting at t * ceil(n / B) (few per thread for the item sizes here, so the blocked
-// layout's bank conflicts cost less than a second pass would).
-template <int B>
-__device__ __forceinline__ void ss_excl_sum(uint32_t* a, int n, uint32_t* tmp) {
-  const int t = threadIdx.x;
-  const int per = (n + B - 1) / B;
-  const int x0 = t * per, x1 = x0 + per < n ? x0 + per : n;
+struct SsRow {     // a tile's row (one 16-byte word)
+  uint32_t rdel;   // output offset from base - packed start
+  uint32_t ps_L;   // packed start | length << 16
+  float scale;     // bucket scale
+  unsigned mid;    // which relabelling
+};
+
+// Exclusive scan of the bucket counters cnt[0, B * ITEMS) in place, thread t owning ITEMS
+// consecutive ones; each becomes start | count << 16 (both at most CAP <= 4096).
+template <int B, int ITEMS>
+__device__ __forceinline__ void ss_scan(uint32_t* cnt, uint32_t* tmp) {
+  static_assert(ITEMS % 4 == 0 && B * ITEMS <= 4096, "16-byte words; 16-bit halves");
+  constexpr int NW = B / 32, Q = ITEMS / 4;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  uint4* c4 = reinterpret_cast<uint4*>(cnt) + t * Q;
   uint32_t s = 0;
-  for (int x = x0; x < x1; ++x) s += a[x];
-  uint32_t total;
-  uint32_t run = block_excl_sum<B>(s, tmp, &total);
-  for (int x = x0; x < x1; ++x) {
-    const uint32_t v = a[x];
-    a[x] = run;
-    run += v;
+#pragma unroll
+  for (int j = 0; j < Q; ++j) {
+    const uint4 v = c4[j];
+    s += v.x + v.y + v.z + v.w;
+  }
+  const uint32_t inc = warp_incl_sum(s);
+  if (lane == 31) tmp[w] = inc;
+  __syncthreads();
+  uint32_t run = inc - s;
+#pragma unroll
+  for (int k = 0; k < NW - 1; ++k) run += k < w ? tmp[k] : 0u;
+#pragma unroll
+  for (int j = 0; j < Q; ++j) {
+    uint4 v = c4[j];
+    uint32_t c;
+    c = v.x, v.x = run | (c << 16), run += c;
+    c = v.y, v.y = run | (c << 16), run += c;
+    c = v.z, v.z = run | (c << 16), run += c;
+    c = v.w, v.w = run | (c << 16), run += c;
+    c4[j] = v;
   }
   __syncthreads();
 }
 
-// Work items: tiles [0, *ntiles) of the partition, or runs fin[0, *fin_n) (from the
-// back of the list, fin[cap - 1 - k], with Cfg::kBack): rows of SS_TILE_MAX < L <=
-// SS_RUN_MAX entries, in the output arrays, and k_split's runs, in the output or in the
-// temporary arrays.  Every item's entries are loaded into shared memory
-// before any of them is written back, so a run is sorted in place.  A bucket of more
-// than SS_HEAVY keys (skewed keys) is written in bucket order and queued in hv[] as a
-// run for a later pass, which buckets it over its own key range; without hv (the last
-// pass) every bucket is ranked directly.
-template <class Cfg, class CI, class VT>
+template <int B, int ITEMS>
+__device__ __forceinline__ void ss_clear(uint32_t* cnt) {
+  uint4* c4 = reinterpret_cast<uint4*>(cnt) + threadIdx.x * (ITEMS / 4);
+#pragma unroll
+  for (int j = 0; j < ITEMS / 4; ++j) c4[j] = make_uint4(0, 0, 0, 0);
+}
+
+// Rank of `key` among its bucket's keys sk[s, s + c): the first four without a loop (most
+// buckets hold one or two keys, and a warp would loop to its largest), the rest in one.
+__device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint32_t c, uint32_t key) {
+  const uint32_t* b = sk + s;
+  uint32_t p = s;
+  if (c > 1u) {
+    const uint32_t k0 = b[0], k1 = b[1];
+    p += (k0 < key) + (k1 < key);
+  }
+  if (c > 2u) p += b[2] < key;
+  if (c > 3u) {
+    p += b[3] < key;
+#pragma unroll 1
+    for (uint32_t q = 4; q < c; ++q) p += b[q] < key;
+  }
+  return p;
+}
+
+// Work items: tiles [0, ntiles) of the partition, or the runs of one slice of the run
+// lists: whole rows at their source, rows in the output arrays, and k_split's runs in the
+// output or in the temporary arrays.  Every
+// item's entries are loaded before any of them is written, so a run is sorted in place.
+//
+// The bucket sort: an entry's bucket counter (shared memory) returns its arrival number,
+// one block scan turns the counters into bucket starts, the entry's key is put at start +
+// arrival, and its owner (the thread that loaded it, which keeps key and bucket in
+// registers) ranks it among its bucket's keys, two on average.  Keys then go to their
+// sorted position with the index of their value, and both are written coalesced.
+// A bucket of more than `heavy` keys (skewed keys): a tile writes it in bucket order and
+// queues it as a run; a run buckets it again over its own key range, in the counters of
+// its own positions, for up to SS_LEVELS levels (the last ranks whatever is left).
+//
+// A position past the item's end carries a padding entry: its bucket is the counter of its
+// own position, which no bucket uses, so it passes through the sort in place and every pass
+// runs without a bounds check; only loads and stores look at the length.
+//
+// What bounds it: shared-memory wavefronts and issue slots (a profile of a tile sort of
+// 512-entry rows: 80 % of the LSU data pipe, 53 % of issue, 15 % of DRAM), and for a matrix
+// whose column map exceeds L2 the random lookups.  So the gather is part of the sort (one
+// pass over the entries instead of two), an entry stays with its thread from load to
+// staging, and buckets hold one key on average.  Uniform rows of 32 over 2^25 columns: 25.8
+// -> 16.4 ms per permutation, of which the lookups alone take 12.9 in a plain gather; rows
+// of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms.
+template <class Cfg, class Gs>
 __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
-    k_seg_sort(const long long* __restrict__ vp, const long long* __restrict__ tile_first,
-               const long long* __restrict__ ntiles_p, const FinalEntry* __restrict__ fin,
-               const unsigned* __restrict__ fin_n, long long fin_cap, const uint32_t* __restrict__ tkey_g,
-               const VT* __restrict__ tval_g, CI* __restrict__ out_col, VT* __restrict__ out_val,
-               FinalEntry* __restrict__ hv, unsigned* hv_n, long long hv_cap, int key_bits, int heavy,
-               DevStatus* st) {
-  constexpr int B = Cfg::B, CAP = Cfg::CAP, ROWS = Cfg::ROWS, WORDS = Cfg::WORDS;
+    k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nnz, const long long* __restrict__ tile_first,
+               long long ntiles,
+               RunLists rl, int slice, const uint32_t* __restrict__ tkey_g,
+               const typename Gs::VT* __restrict__ tval_g, typename Gs::CI* __restrict__ out_col,
+               typename Gs::VT* __restrict__ out_val, int key_bits, int heavy, DevStatus* st) {
+  using CI = typename Gs::CI;
+  using VT = typename Gs::VT;
+  constexpr int B = Cfg::B, ITEMS = Cfg::ITEMS, CAP = Cfg::CAP, ROWS = Cfg::ROWS, WORDS = Cfg::WORDS, RPT = Cfg::RPT;
   extern __shared__ __align__(16) unsigned char smem[];
   VT* sval = reinterpret_cast<VT*>(smem);
-  uint32_t* skey = reinterpret_cast<uint32_t*>(smem + size_t(CAP) * sizeof(VT));  // packed order
-  uint32_t* tkey = skey + CAP;        // bucket order
-  uint32_t* cnt = tkey + CAP;         // bucket counters
-  uint16_t* slot = reinterpret_cast<uint16_t*>(cnt + Cfg::CNT);  // bucket of packed entry
-  uint16_t* tidx = slot + CAP;        // packed entry of each bucket-order position
+  uint32_t* skey = reinterpret_cast<uint32_t*>(smem + size_t(CAP) * sizeof(VT));
+  uint32_t* cnt = skey + CAP;
   // tiles only (runs allocate none of these)
-  uint32_t* rdel = reinterpret_cast<uint32_t*>(tidx + CAP);  // per row: output offset from base - packed start
-  float* rsc = reinterpret_cast<float*>(rdel + ROWS);        // per row: bucket scale
-  uint32_t* bits = rdel + 2 * ROWS;   // row starts
-  uint32_t* wpre = bits + WORDS;      // row starts in earlier words
-  uint16_t* rps = reinterpret_cast<uint16_t*>(wpre + WORDS);  // per row: packed start
-  uint16_t* rnm = rps + ROWS;         // per row: last bucket
+  SsRow* rows = reinterpret_cast<SsRow*>(cnt + CAP);
+  ulonglong2* rptr = reinterpret_cast<ulonglong2*>(rows + ROWS);  // the row's column / value pointers - packed start
+  uint32_t* bits = reinterpret_cast<uint32_t*>(rptr + ROWS);      // row starts
+  uint32_t* wpre = bits + WORDS;                                  // row starts in earlier words
   __shared__ uint32_t tmp32[B / 32 + 1];
-  __shared__ uint32_t s_min, s_max;
-  // tiles: row pointers vp[r0 .. r1] of the next tile, copied in while this one is sorted
-  __shared__ long long pre_o[Cfg::kTiles ? ROWS + 1 : 1];
-  const int t = threadIdx.x;
+  __shared__ uint32_t s_min[2], s_max[2];
+  __shared__ int s_cut, s_cutE;
+  // tiles: row pointers vp[r0 .. r1] and source starts of the next tile, copied in while
+  // this one is sorted
+  __shared__ long long pre_o[Cfg::kTiles ? ROWS + 1 : 1], pre_s[Cfg::kTiles ? ROWS + 1 : 1];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const uint32_t kmax = key_bits >= 32 ? 0xFFFFFFFFu : (1u << key_bits) - 1u;
   const float isr = ss_inv_root(kmax);
   long long nitems;
   if constexpr (Cfg::kTiles) {
-    nitems = *ntiles_p;
+    nitems = ntiles;
   } else {
-    nitems = *fin_n;
-    if (nitems > fin_cap) nitems = fin_cap;  // overflow was reported by the producer
+    nitems = rl.n[slice];
+    if (nitems > rl.cap(slice)) nitems = rl.cap(slice);  // overflow was reported by the producer
   }
+  if (blockIdx.x >= nitems) return;
 
   // the next item's descriptor is loaded one item ahead, so its latency hides behind
   // the current item's sort
@@ -760,477 +935,611 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
   // tiles: start copying the row pointers of the tile whose range is in (pf0, pf1)
   auto prefetch_rows = [&](bool any) {
     if (any) {
-      long long n = pf1 - pf0;
-      n = n < 0 ? 0 : (n < ROWS ? n : ROWS);
-      for (int x = t; x <= n; x += B) cp_async8(pre_o + x, vp + pf0 + x);
+      int n = int(pf1 - pf0);
+      n = n < ROWS ? n : ROWS;
+      for (int x = t; n > 0 && x <= n; x += B) {  // (an empty tile waits for no copy)
+        cp_async8(pre_o + x, vp + pf0 + x);
+        if (x < n) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
+      }
     }
     cp_async_commit();
   };
-  if (blockIdx.x < nitems) {
-    if constexpr (Cfg::kTiles) {
-      pf0 = tile_first[blockIdx.x];
-      pf1 = tile_first[blockIdx.x + 1];
-      prefetch_rows(true);
-    } else {
-      pfe = fin[Cfg::kBack ? fin_cap - 1 - (long long)blockIdx.x : (long long)blockIdx.x];
+  if constexpr (Cfg::kTiles) {
+    pf0 = tile_first[blockIdx.x];
+    pf1 = tile_first[blockIdx.x + 1];
+    prefetch_rows(true);
+  } else {
+    pfe = rl.slice(slice)[blockIdx.x];
+    if (t < 2) {
+      s_min[t] = 0xFFFFFFFFu;
+      s_max[t] = 0u;
     }
   }
-  for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
+  int par = 0;
+  int ra = 0;  // tiles: the round's first row
+  for (long long item = blockIdx.x; item < nitems;) {
     const long long nx = item + gridDim.x;
-    if constexpr (Cfg::kTiles) {
-      for (int w = t; w < WORDS; w += B) bits[w] = 0;
-    } else if (t == 0) {
-      s_min = 0xFFFFFFFFu;
-      s_max = 0u;
-    }
     long long base;
-    int buf = BUF_OUT;
-    int E;
+    int E, nrow = 0, rnext = 0;
+    uint32_t key[ITEMS], seg[ITEMS];  // seg: bucket | arrival << 16, then start | count << 16
+    VT val[ITEMS];
+    uint32_t out[Cfg::kTiles ? ITEMS : 1];  // tiles: the position's output offset from base
+    // the row of packed entry x of a tile: the row starts at or before x
+    auto row_of = [&](int x) -> uint32_t {
+      const int w = x >> 5;
+      return wpre[w] + __popc(bits[w] & (0xFFFFFFFFu >> (31 - (x & 31)))) - 1u;
+    };
     if constexpr (Cfg::kTiles) {
-      uint32_t myL = 0;
-      long long o0 = 0;
-      const long long r0 = pf0;
-      long long r1 = pf1;
-      if (nx < nitems) {
-        pf0 = tile_first[nx];
-        pf1 = tile_first[nx + 1];
-      }
-      cp_async_wait_all();  // this tile's row pointers
-      __syncthreads();
-      base = pre_o[0];
-      if (r1 - r0 > ROWS) {  // cannot happen: see RowsPartition
+      nrow = int(pf1 - pf0);
+      if (nrow > ROWS) {  // cannot happen: see RowsPartition
         if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -17);
-        r1 = r0;
+        nrow = ROWS;
       }
-      if (t < r1 - r0) {
-        o0 = pre_o[t];
-        const long long L = pre_o[t + 1] - o0;
-        if (L > 0 && L <= Cfg::CP) {
-          if (o0 - base > 0xFFFFFFFFll - CAP) dev_fail(st, SP_ERR_OVERFLOW, r0 + t);
-          else myL = uint32_t(L);
+      if (nrow == 0) {  // a window inside a longer row
+        item = nx;
+        if (nx < nitems) {
+          pf0 = tile_first[nx];
+          pf1 = tile_first[nx + 1];
         }
-      }
-      // packed start (high half) and rank among the item's rows (low half)
-      uint32_t tot;
-      const uint32_t pre = block_excl_sum<B>(myL ? ((myL << 16) | 1u) : 0u, tmp32, &tot);
-      E = int(tot >> 16);  // <= 2 * Cfg::CP by the partition
-      if (E > CAP) {       // cannot happen: see RowsPartition
-        if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -19);
-        prefetch_rows(nx < nitems);  // every thread has read pre_o (barriers above)
-        __syncthreads();
+        prefetch_rows(nx < nitems);
         continue;
       }
-      if (myL) {
-        const uint32_t k = pre & 0xFFFFu, ps = pre >> 16;
-        const uint32_t nb = ss_nb(myL);
-        rps[k] = uint16_t(ps);
-        rnm[k] = uint16_t(nb - 1);
-        rsc[k] = float(nb) * isr;
-        rdel[k] = uint32_t(o0 - base) - ps;
+      cp_async_wait_all();  // this tile's row pointers
+      __syncthreads();      // and the previous round's last reads of the tables
+      ss_clear<B, ITEMS>(cnt);
+      for (int w = t; w < WORDS; w += B) bits[w] = 0;
+      base = pre_o[0];
+      uint32_t L[RPT], off[RPT], mine = 0;
+      long long src[RPT];
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) {
+        const int r = ra + t * RPT + k;
+        L[k] = off[k] = 0;
+        if (r < nrow) {
+          const long long o0 = pre_o[r], l = pre_o[r + 1] - o0;
+          off[k] = uint32_t(o0 - base);  // < WIN
+          src[k] = pre_s[r];
+          if (l > 0 && l <= Cfg::TMAX && o0 + l <= nnz) L[k] = uint32_t(l);
+        }
+        mine += L[k] ? ((L[k] << 16) | 1u) : 0u;
+      }
+      // packed start (high half) and rank among the item's rows (low half)
+      const uint32_t inc = warp_incl_sum(mine);
+      if (lane == 31) tmp32[wid] = inc;
+      __syncthreads();
+      uint32_t pre = inc - mine, tot = 0;
+#pragma unroll
+      for (int k = 0; k < B / 32; ++k) {
+        const uint32_t x = tmp32[k];
+        pre += k < wid ? x : 0u;
+        tot += x;
+      }
+      E = int(tot >> 16);
+      rnext = nrow;
+      if (E == 0) {  // only longer (or empty) rows: the next tile
+        item = nx;
+        ra = 0;
+        __syncthreads();  // pre_o has been read
+        if (nx < nitems) {
+          pf0 = tile_first[nx];
+          pf1 = tile_first[nx + 1];
+        }
+        prefetch_rows(nx < nitems);
+        continue;
+      }
+      if (E > CAP) {  // the rows that fit now, the others in another round
+        uint32_t q = pre >> 16;
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+          if (q <= uint32_t(CAP) && q + L[k] > uint32_t(CAP)) {
+            s_cut = ra + t * RPT + k;
+            s_cutE = int(q);
+          }
+          q += L[k];
+        }
+        __syncthreads();
+        rnext = s_cut;
+        E = s_cutE;
+      }
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) {
+        const uint32_t ps = pre >> 16, pe = ps + L[k], i = pre & 0xFFFFu;
+        if (L[k] == 0 || pe > uint32_t(E)) continue;
+        GsView<CI, VT> gv = gs.view(src[k], L[k]);
+        if (!gv.c) {
+          dev_fail(st, SP_ERR_INTERNAL, -13);
+          gv = GsView<CI, VT>{out_col, out_val, 0u};  // readable: at most nnz entries in
+        }
+        rows[i] = SsRow{off[k] - ps, ps | (L[k] << 16), float(L[k]) * isr, gv.mid};
+        rptr[i] = make_ulonglong2((unsigned long long)(gv.c - ps), (unsigned long long)(gv.v - ps));
         atomicOr(&bits[ps >> 5], 1u << (ps & 31));
-      }
-      for (int x = t; x < E; x += B) cnt[x] = 0;
-      __syncthreads();
-      if (t < 32) {
-        constexpr int WL = WORDS / 32;  // words per lane
-        uint32_t c[WL], s = 0;
-#pragma unroll
-        for (int j = 0; j < WL; ++j) {
-          c[j] = __popc(bits[t * WL + j]);
-          s += c[j];
-        }
-        uint32_t run = warp_incl_sum(s) - s;
-#pragma unroll
-        for (int j = 0; j < WL; ++j) {
-          wpre[t * WL + j] = run;
-          run += c[j];
-        }
+        // the words whose first entry comes after this row's first: i + 1 starts before them
+        for (uint32_t w = (ps >> 5) + 1; (w << 5) <= pe && w < WORDS; ++w) wpre[w] = i + 1;
+        if (i == 0) wpre[0] = 0;
+        pre += (L[k] << 16) | 1u;
       }
       __syncthreads();
-      prefetch_rows(nx < nitems);  // the next tile's row pointers arrive during this sort
+      if (rnext == nrow) {  // the last round: the next tile's row pointers arrive during this sort
+        if (nx < nitems) {
+          pf0 = tile_first[nx];
+          pf1 = tile_first[nx + 1];
+        }
+        prefetch_rows(nx < nitems);
+      }
+      // load: key, value and bucket of every entry
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const int x = t + j * B;
+        seg[j] = x < E ? row_of(x) : 0u;
+        const ulonglong2 rp = rptr[seg[j]];
+        key[j] = x < E ? ss_key(ld_stream(reinterpret_cast<const CI*>(rp.x) + x)) : 0u;
+        val[j] = x < E ? ld_stream(reinterpret_cast<const VT*>(rp.y) + x) : VT(0);
+      }
+      if constexpr (!in_place<Gs>::value) {
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) key[j] = gs.map(rows[seg[j]].mid, key[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const int x = t + j * B;
+        const SsRow r = rows[seg[j]];
+        out[j] = r.rdel + x;
+        if (key[j] > kmax) {  // a column outside [0, ncols)
+          if (x < E) dev_fail(st, SP_ERR_INDEX_RANGE, base + out[j]);
+          key[j] = kmax;
+        }
+        const uint32_t sl =
+            x < E ? (r.ps_L & 0xFFFFu) + ss_bucket(key[j], r.scale, (r.ps_L >> 16) - 1u) : uint32_t(x);
+        seg[j] = sl | (atomicAdd(&cnt[sl], 1u) << 16);
+      }
     } else {
       const FinalEntry fe = pfe;
-      if (nx < nitems) pfe = fin[Cfg::kBack ? fin_cap - 1 - nx : nx];
+      if (nx < nitems) pfe = rl.slice(slice)[nx];
       base = fe.off;
-      buf = fe.buf;
-      E = int(fe.len);
+      E = fe.len;
       if (fe.len < 0 || fe.len > CAP) {
         if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -18);
         E = 0;
       }
-      for (int x = t; x < int(ss_nb(uint32_t(E))); x += B) cnt[x] = 0;
-      __syncthreads();
-    }
-    // load: key and value of every packed entry, bucket histogram
-    constexpr int LU = 4;
-    if constexpr (Cfg::kTiles) {
-      for (int x0 = t; x0 < E; x0 += B * LU) {
-        uint32_t kk[LU], kr[LU], oo[LU];  // key, row, offset from base
-        VT vv[LU];
-#pragma unroll
-        for (int u = 0; u < LU; ++u) {
-          const int x = x0 + u * B;
-          kr[u] = 0;
-          oo[u] = 0;
-          if (x < E) {
-            const int w = x >> 5;
-            kr[u] = wpre[w] + __popc(bits[w] & (0xFFFFFFFFu >> (31 - (x & 31)))) - 1u;
-            oo[u] = rdel[kr[u]] + uint32_t(x);
-          }
-        }
-        {  // tiles live in the output arrays
-          const CI* kp = out_col + base;
-          const VT* vq = out_val + base;
-#pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) kk[u] = uint32_t(ld_stream(kp + oo[u]));
-#pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) vv[u] = ld_stream(vq + oo[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < LU; ++u) {
-          const int x = x0 + u * B;
-          if (x >= E) continue;
-          uint32_t key = kk[u];
-          if (key > kmax) {  // a column outside [0, ncols)
-            dev_fail(st, SP_ERR_INDEX_RANGE, base + oo[u]);
-            key = kmax;
-          }
-          const uint32_t sl = rps[kr[u]] + ss_bucket(key, rsc[kr[u]], rnm[kr[u]]);
-          skey[x] = key;
-          sval[x] = vv[u];
-          slot[x] = uint16_t(sl);
-          atomicAdd(&cnt[sl], 1u);
-        }
-      }
-    } else {
+      __syncthreads();  // the previous run's last reads of the staging arrays
+      ss_clear<B, ITEMS>(cnt);
       // a single run (a row sorted alone or a key-range group of a long row): its
       // buckets span the run's own key range [min, max], found while loading
       uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-      const CI* kp = out_col + base;
-      const VT* vq = out_val + base;
-      for (int x0 = t; x0 < E; x0 += B * LU) {
-        uint32_t kk[LU];
-        VT vv[LU];
-        if (buf == BUF_TEMP) {
+      auto load = [&](const auto* cp, const VT* vq) {
 #pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) kk[u] = ld_stream(tkey_g + base + x0 + u * B);
-#pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) vv[u] = ld_stream(tval_g + base + x0 + u * B);
-        } else {
-#pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) kk[u] = uint32_t(ld_stream(kp + x0 + u * B));
-#pragma unroll
-          for (int u = 0; u < LU; ++u)
-            if (x0 + u * B < E) vv[u] = ld_stream(vq + x0 + u * B);
+        for (int j = 0; j < ITEMS; ++j) {
+          const int x = t + j * B;
+          key[j] = x < E ? ss_key(ld_stream(cp + x)) : 0u;
+          val[j] = x < E ? ld_stream(vq + x) : VT(0);
         }
-#pragma unroll
-        for (int u = 0; u < LU; ++u) {
-          const int x = x0 + u * B;
-          if (x >= E) continue;
-          uint32_t key = kk[u];
-          if (key > kmax) {
-            dev_fail(st, SP_ERR_INDEX_RANGE, base + x);
-            key = kmax;
-          }
-          skey[x] = key;
-          sval[x] = vv[u];
-          mn = key < mn ? key : mn;
-          mx = key > mx ? key : mx;
+      };
+      if (!in_place<Gs>::value && fe.buf == BUF_SRC) {
+        GsView<CI, VT> gv = gs.view(gs.srcs()[fe.row], E);
+        if (!gv.c) {
+          if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -13);
+          gv = GsView<CI, VT>{out_col + base, out_val + base, 0u};
         }
+        load(gv.c, gv.v);
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) key[j] = gs.map(gv.mid, key[j]);
+      } else if (fe.buf == BUF_TEMP) {
+        load(tkey_g + base, tval_g + base);
+      } else {
+        load(out_col + base, out_val + base);
+      }
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const bool ok = t + j * B < E;
+        if (key[j] > kmax) {
+          if (ok) dev_fail(st, SP_ERR_INDEX_RANGE, base + t + j * B);
+          key[j] = kmax;
+        }
+        mn = ok && key[j] < mn ? key[j] : mn;
+        mx = ok && key[j] > mx ? key[j] : mx;
       }
       mn = __reduce_min_sync(0xFFFFFFFFu, mn);
       mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-      if ((t & 31) == 0) {
-        atomicMin(&s_min, mn);
-        atomicMax(&s_max, mx);
+      if (lane == 0) {
+        atomicMin(&s_min[par], mn);
+        atomicMax(&s_max[par], mx);
       }
       __syncthreads();
-      const uint32_t lo = s_min, w = s_max > s_min ? s_max - s_min : 0u;
-      const uint32_t nb = ss_nb(uint32_t(E)), last = nb - 1;
-      const float sc = float(nb) * ss_inv_root(w);
-      for (int x = t; x < E; x += B) {
-        const uint32_t sl = ss_bucket(skey[x] - lo, sc, last);
-        slot[x] = uint16_t(sl);
-        atomicAdd(&cnt[sl], 1u);
+      const uint32_t lo = s_min[par], w = s_max[par] > lo ? s_max[par] - lo : 0u;
+      if (t == 0) {  // for the next run (its own pair was read a barrier ago)
+        s_min[par ^ 1] = 0xFFFFFFFFu;
+        s_max[par ^ 1] = 0u;
+      }
+      par ^= 1;
+      const float sc = float(E) * ss_inv_root(w);
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const int x = t + j * B;
+        const uint32_t sl = x < E ? ss_bucket(key[j] - lo, sc, uint32_t(E) - 1u) : uint32_t(x);
+        seg[j] = sl | (atomicAdd(&cnt[sl], 1u) << 16);
       }
     }
     __syncthreads();
-    // counters in use: a tile's rows' buckets lie in [0, E), a run's in [0, ss_nb(E))
-    ss_excl_sum<B>(cnt, Cfg::kTiles ? E : int(ss_nb(uint32_t(E))), tmp32);
-    // scatter to bucket order; afterwards cnt[s] = end of bucket s, cnt[s-1] its start
-    for (int x = t; x < E; x += B) {
-      const uint32_t p = atomicAdd(&cnt[slot[x]], 1u);
-      tkey[p] = skey[x];
-      tidx[p] = uint16_t(x);
+    ss_scan<B, ITEMS>(cnt, tmp32);
+    bool hv = false;
+    uint32_t open = 0;  // entries in a heavy bucket
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const uint32_t sc = cnt[seg[j] & 0xFFFFu], p = (sc & 0xFFFFu) + (seg[j] >> 16);
+      skey[p] = key[j];
+      if ((sc >> 16) > uint32_t(heavy)) {
+        open |= 1u << j;
+        hv = true;
+        if constexpr (Cfg::kTiles) {  // left in bucket order, queued as a run
+          if ((seg[j] >> 16) == 0u)
+            queue_run(rl, FinalEntry{base + out[j] - uint32_t(t + j * B) + p, int(sc >> 16), BUF_OUT, 0}, st, -22);
+          seg[j] = p;
+          continue;
+        }
+      }
+      seg[j] = sc;
+    }
+    if constexpr (Cfg::kTiles) {
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j)
+        if (!((open >> j) & 1u)) seg[j] = ss_rank(skey, seg[j] & 0xFFFFu, seg[j] >> 16, key[j]);
+    } else {
+      hv = __syncthreads_or(hv);
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j)
+        if (!((open >> j) & 1u)) seg[j] = ss_rank(skey, seg[j] & 0xFFFFu, seg[j] >> 16, key[j]);
+      for (int level = 1; hv; ++level) {
+        // skewed keys: the entries of heavy buckets are bucketed again over their bucket's
+        // own key range (found at the bucket's first two words); the others keep their
+        // place through the scan
+        __syncthreads();  // the bucket order has been read
+        ss_clear<B, ITEMS>(cnt);
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j)
+          if ((open >> j) & 1u) {
+            skey[seg[j] & 0xFFFFu] = 0xFFFFFFFFu;
+            skey[(seg[j] & 0xFFFFu) + 1] = 0u;
+          }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j)
+          if ((open >> j) & 1u) {
+            atomicMin(&skey[seg[j] & 0xFFFFu], key[j]);
+            atomicMax(&skey[(seg[j] & 0xFFFFu) + 1], key[j]);
+          }
+        __syncthreads();
+        uint32_t arr[ITEMS];
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+          uint32_t sl = seg[j] & 0xFFFFu;
+          if ((open >> j) & 1u) {
+            const uint32_t lo = skey[sl], w = skey[sl + 1] - lo, nb = seg[j] >> 16;
+            sl += ss_bucket(key[j] - lo, float(nb) * ss_inv_root(w), nb - 1);
+          }
+          arr[j] = sl | (atomicAdd(&cnt[sl], 1u) << 16);
+        }
+        __syncthreads();
+        ss_scan<B, ITEMS>(cnt, tmp32);
+        bool more = false;
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+          if (!((open >> j) & 1u)) continue;
+          seg[j] = cnt[arr[j] & 0xFFFFu];
+          skey[(seg[j] & 0xFFFFu) + (arr[j] >> 16)] = key[j];
+          more |= (seg[j] >> 16) > uint32_t(heavy);
+        }
+        hv = __syncthreads_or(more) && level < SS_LEVELS;
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+          if (!((open >> j) & 1u) || (hv && (seg[j] >> 16) > uint32_t(heavy))) continue;
+          seg[j] = ss_rank(skey, seg[j] & 0xFFFFu, seg[j] >> 16, key[j]);
+          open &= ~(1u << j);
+        }
+      }
+    }
+    __syncthreads();  // the bucket order and the counters have been read
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      skey[seg[j]] = key[j];
+      sval[seg[j]] = val[j];
     }
     __syncthreads();
-    // rank inside the bucket and write (heavy buckets: in bucket order, queued)
     CI* const oc = out_col + base;
     VT* const ov = out_val + base;
-    for (int p = t; p < E; p += B) {
-      const uint32_t x = tidx[p], k = tkey[p];
-      const uint32_t s = slot[x];
-      const uint32_t end = cnt[s], start = s ? cnt[s - 1] : 0u;
-      uint32_t rd = 0u;
-      if constexpr (Cfg::kTiles) {  // the entry's row: the row starts at or before x
-        const int w = int(x >> 5);
-        rd = rdel[wpre[w] + __popc(bits[w] & (0xFFFFFFFFu >> (31 - (x & 31)))) - 1u];
-      }
-      if (hv && end - start > uint32_t(heavy)) {
-        st_stream(oc + rd + p, CI(k));
-        st_stream(ov + rd + p, sval[x]);
-        if (uint32_t(p) == start) {
-          const unsigned q = atomicAdd(hv_n, 1u);
-          if (q < hv_cap) hv[q] = FinalEntry{base + rd + start, (long long)(end - start), BUF_OUT, 0};
-          else dev_fail(st, SP_ERR_INTERNAL, -22);
-        }
-        continue;
-      }
-      uint32_t rank = 0;
-      for (uint32_t q = start; q < end; ++q) rank += tkey[q] < k;
-      const uint32_t g = rd + start + rank;
-      st_stream(oc + g, CI(k));
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const int x = t + j * B;
+      if (x >= E) continue;
+      const uint32_t g = Cfg::kTiles ? out[Cfg::kTiles ? j : 0] : uint32_t(x);
+      st_stream(oc + g, CI(skey[x]));
       st_stream(ov + g, sval[x]);
     }
-    __syncthreads();
+    if constexpr (Cfg::kTiles) {
+      if (rnext < nrow) {
+        ra = rnext;
+      } else {
+        ra = 0;
+        item = nx;
+      }
+    } else {
+      item = nx;
+    }
+  }
+}
+
+// Runs of at most SS_WARP_RUN entries (the first slice of the run lists: rows in the output
+// arrays, k_split's groups in either buffer), a warp each: every lane keeps four entries and counts the run's smaller keys,
+// four at a time from shared memory (broadcast).
+constexpr int WR_BLOCK = 256, WR_MINB = 4;
+template <class CI, class VT>
+__global__ void __launch_bounds__(WR_BLOCK, WR_MINB)
+    k_sort_warp_runs(RunLists rl, const uint32_t* __restrict__ tkey, const VT* __restrict__ tval,
+                     CI* __restrict__ out_col, VT* __restrict__ out_val, uint32_t kmax, DevStatus* st) {
+  constexpr int NW = WR_BLOCK / 32, PER = SS_WARP_RUN / 32;
+  __shared__ __align__(16) uint32_t s_key[NW][SS_WARP_RUN];
+  const int lane = threadIdx.x & 31;
+  uint32_t* wk = s_key[threadIdx.x >> 5];
+  long long n = rl.n[0];
+  if (n > rl.c0) n = rl.c0;
+  const long long nw = (long long)gridDim.x * NW;
+  for (long long i = (long long)blockIdx.x * NW + (threadIdx.x >> 5); i < n; i += nw) {
+    const FinalEntry fe = rl.list[i];
+    const int E = fe.len;
+    if (E <= 0 || E > SS_WARP_RUN) {
+      if (lane == 0) dev_fail(st, SP_ERR_INTERNAL, -20);
+      continue;
+    }
+    CI* const oc = out_col + fe.off;
+    VT* const ov = out_val + fe.off;
+    uint32_t key[PER];
+    VT val[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int x = lane + 32 * j;
+      const bool tmp = fe.buf == BUF_TEMP;
+      key[j] = x < E ? (tmp ? ld_stream(tkey + fe.off + x) : ss_key(ld_stream(oc + x))) : 0xFFFFFFFFu;
+      val[j] = x < E ? ld_stream(tmp ? tval + fe.off + x : ov + x) : VT(0);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (lane + 32 * j < E && key[j] > kmax) {
+        dev_fail(st, SP_ERR_INDEX_RANGE, fe.off + lane + 32 * j);
+        key[j] = kmax;
+      }
+      wk[lane + 32 * j] = key[j];  // (padding is below no key)
+    }
+    __syncwarp();
+    int rank[PER] = {};
+    const uint4* w4 = reinterpret_cast<const uint4*>(wk);
+    const int nq = (E + 3) >> 2;
+    auto count = [&](auto per) {
+      constexpr int P = decltype(per)::value;
+      for (int q = 0; q < nq; ++q) {
+        const uint4 k = w4[q];
+#pragma unroll
+        for (int j = 0; j < P; ++j)
+          rank[j] += int(k.x < key[j]) + int(k.y < key[j]) + int(k.z < key[j]) + int(k.w < key[j]);
+      }
+    };
+    if (E <= 32) count(std::integral_constant<int, 1>{});
+    else if (E <= 64) count(std::integral_constant<int, 2>{});
+    else count(std::integral_constant<int, PER>{});
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (lane + 32 * j >= E) continue;
+      st_stream(oc + rank[j], CI(key[j]));
+      st_stream(ov + rank[j], val[j]);
+    }
   }
 }
 
 // ---- host side --------------------------------------------------------------------------
 struct RowsWs {
-  long long ntiles_cap = 0, nchunks = 0, fin_cap = 0, huge_cap = 0, nxt_cap = 0, hv_cap = 0;
+  long long ntiles_cap = 0, nchunks = 0, huge_cap = 0, nxt_cap = 0, lchunk_cap = 0;
+  long long run_cap[4] = {0, 0, 0, 0};
   long long* tile_first = nullptr;
   long long* chunk_first = nullptr;
-  long long* ntiles = nullptr;
-  unsigned* counters = nullptr;  // [0..1] run list counts (front, back) [2] spare [3..4] tickets [5] spare
-                                 // [6..7] heavy-run counts [8..9] zero (no tiles)
-                                 // [10..11] huge list counts [12..13] nxt list counts
+  unsigned* counters = nullptr;  // [0..3] run list counts [4..5] split tickets [7] spare
+                                 // [6] long chunks [10..11] huge list counts [12..13] nxt list counts
   FinalEntry* fin = nullptr;
   HugeEntry* huge = nullptr;
   HugeEntry* nxt = nullptr;
-  FinalEntry* hv[2] = {nullptr, nullptr};  // heavy buckets queued for the next pass
+  LongChunk* lchunk = nullptr;
   uint32_t* tkey = nullptr;
   void* tval = nullptr;
-  char* scan_ws = nullptr;
+  long long runs_total() const { return run_cap[0] + run_cap[1] + run_cap[2] + run_cap[3]; }
+  RunLists runs() const { return RunLists{fin, counters, run_cap[0], run_cap[1], run_cap[2], run_cap[3]}; }
+  unsigned* lchunk_n() const { return counters + 6; }
   unsigned* huge_n() const { return counters + 10; }
   unsigned* nxt_n() const { return counters + 12; }
 };
 
-constexpr int kRowsSlots = 12;
+constexpr int kRowsSlots = 9;
 
-// extra_fin: runs a caller queues itself (beyond the partition's and the split's)
-inline void rows_caps(long long nrows, long long nnz, RowsWs* w, long long extra_fin = 0) {
-  w->ntiles_cap = (nnz + SS_ROW_W * nrows) / SS_TILE_MAX + 1;
-  w->nchunks = (nnz + GC_CH - 1) / GC_CH;
-  w->fin_cap = 2 * (3 * (nnz / GROUP_CAP) + nnz / SS_RUN_MAX + 16) + nnz / SS_TILE_MAX + 1 + extra_fin;
-  w->huge_cap = nnz / SS_RUN_MAX + 1;
-  w->nxt_cap = nnz / SS_RUN_MAX + 1;
-  w->hv_cap = nnz / (SS_HEAVY + 1) + 1;  // heavy buckets are disjoint runs of > SS_HEAVY
-}
-
-// Workspace of run_rows; `sort` = false reserves only what the gather needs.
-inline void rows_reserve(Carver& cv, long long nrows, long long nnz, size_t vbytes, size_t* off,
-                         bool sort = true, long long extra_fin = 0) {
+// Workspace layout of run_rows.  sort = false: only what the gather needs.  extra_runs: runs
+// a caller queues itself (beyond the partition's and the split's).
+inline RowsWs rows_caps(long long nrows, long long nnz, bool sort, long long extra_runs) {
   RowsWs w;
-  rows_caps(nrows, nnz, &w, extra_fin);
-  if (!sort) w.fin_cap = w.huge_cap = w.nxt_cap = w.hv_cap = 0;
-  const bool need_temp = sort && nnz > SS_RUN_MAX;
-  off[0] = cv.reserve(size_t(w.ntiles_cap + 1) * 8);
-  off[1] = cv.reserve(size_t(w.nchunks + 1) * 8);
-  off[2] = cv.reserve(8);
-  off[3] = cv.reserve(16 * 4);
-  off[4] = cv.reserve(size_t(w.fin_cap) * sizeof(FinalEntry));
-  off[5] = cv.reserve(size_t(w.huge_cap) * sizeof(HugeEntry));
-  off[6] = cv.reserve(size_t(w.nxt_cap) * sizeof(HugeEntry));
-  off[7] = cv.reserve(need_temp ? size_t(nnz) * 4 : 0);
-  off[8] = cv.reserve(need_temp ? size_t(nnz) * vbytes : 0);
-  off[9] = cv.reserve(scan_ws_bytes(nrows));
-  off[10] = cv.reserve(size_t(w.hv_cap) * sizeof(FinalEntry));
-  off[11] = cv.reserve(size_t(w.hv_cap) * sizeof(FinalEntry));
-}
-
-inline RowsWs rows_bind(const Carver& cv, long long nrows, long long nnz, const size_t* off,
-                        bool sort = true, long long extra_fin = 0) {
-  RowsWs w;
-  rows_caps(nrows, nnz, &w, extra_fin);
-  if (!sort) w.fin_cap = w.huge_cap = w.nxt_cap = w.hv_cap = 0;
-  w.tile_first = cv.at<long long>(off[0]);
-  w.chunk_first = cv.at<long long>(off[1]);
-  w.ntiles = cv.at<long long>(off[2]);
-  w.counters = cv.at<unsigned>(off[3]);
-  w.fin = cv.at<FinalEntry>(off[4]);
-  w.huge = cv.at<HugeEntry>(off[5]);
-  w.nxt = cv.at<HugeEntry>(off[6]);
-  w.tkey = cv.at<uint32_t>(off[7]);
-  w.tval = cv.at<void>(off[8]);
-  w.scan_ws = cv.at<char>(off[9]);
-  w.hv[0] = cv.at<FinalEntry>(off[10]);
-  w.hv[1] = cv.at<FinalEntry>(off[11]);
+  w.nchunks = sort ? 0 : (nnz + GC_CH - 1) / GC_CH;
+  if (!sort) return w;
+  w.ntiles_cap = (nnz + SsTile::W * nrows) / SsTile::WIN + 1;
+  // the split's groups (at most three per GROUP_CAP entries of both splits), the rows
+  // sorted alone, the tiles' heavy buckets (more than SS_HEAVY entries each)
+  const long long groups = 2 * (3 * (nnz / GROUP_CAP) + nnz / SS_RUN_MAX + 16);
+  w.run_cap[0] = extra_runs > 0 ? groups + extra_runs : 0;
+  w.run_cap[1] = groups + nnz / SS_HEAVY + 1;
+  w.run_cap[2] = groups + nnz / SS_SMALL_RUN + 1;
+  w.run_cap[3] = groups + nnz / SS_MID_RUN + 1;
+  w.huge_cap = nnz / SS_RUN_MAX + 1;
+  w.nxt_cap = nnz / SS_RUN_MAX + 1;
+  w.lchunk_cap = nnz / SL_CH + w.huge_cap;
   return w;
 }
 
-// Phase-1 functor for callers that only sort (the rows are in place already).
-template <class CIt, class VTt>
-struct NoGather {
-  using CI = CIt;
-  using VT = VTt;
-  __device__ long long src(long long) const { return 0; }
-  __device__ CI col(long long) const { return CI(0); }
-  __device__ CI map(long long, CI c) const { return c; }
-  __device__ VT val(long long) const { return VT(0); }
-};
-
-// Key-range split of the rows queued in w.huge (counts w.huge_n()) into runs queued in w.fin.
-template <class CI, class VT>
-sp_status split_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, CI* out_col, VT* out_val) {
-  const int nsm = ctx->num_sms;
-  VT* tval = static_cast<VT*>(w.tval);
-  constexpr size_t csm = split_smem_bytes<SplitCoarse, VT>(), fsm = split_smem_bytes<SplitFine, VT>();
-  SP_CUDA(set_smem(k_split<SplitCoarse, CI, VT>, csm));
-  SP_CUDA(set_smem(k_split<SplitFine, CI, VT>, fsm));
-  {
-    SP_PHASE(SP_PHASE_HUGE);
-    k_split<SplitCoarse, CI, VT><<<SplitCoarse::MINB * nsm, SplitCoarse::B, csm, s>>>(
-        w.huge, w.huge_n(), w.huge_cap, w.counters + 3, w.tkey, tval, out_col, out_val, w.fin, w.counters + 0,
-        w.fin_cap, w.nxt, w.nxt_n(), w.nxt_cap, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  // the fine split: the coarse buckets that hold more than SS_RUN_MAX entries (skewed keys
-  // or very long rows); an empty list costs one short launch
-  {
-    SP_PHASE(SP_PHASE_HUGE);
-    k_split<SplitFine, CI, VT><<<SplitFine::MINB * nsm, SplitFine::B, fsm, s>>>(
-        w.nxt, w.nxt_n(), w.nxt_cap, w.counters + 4, w.tkey, tval, out_col, out_val, w.fin, w.counters + 0,
-        w.fin_cap, w.nxt, w.counters + 5, 0, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  return SP_OK;
+inline void rows_reserve(Carver& cv, long long nrows, long long nnz, size_t vbytes, size_t* off,
+                         bool sort = true, long long extra_runs = 0) {
+  const RowsWs w = rows_caps(nrows, nnz, sort, extra_runs);
+  const bool need_temp = sort && nnz > SS_RUN_MAX;
+  off[0] = cv.reserve(size_t(w.ntiles_cap + 1) * 8);
+  off[1] = cv.reserve(size_t(w.nchunks) * 8);
+  off[2] = cv.reserve(16 * 4);
+  off[3] = cv.reserve(size_t(w.runs_total()) * sizeof(FinalEntry));
+  off[4] = cv.reserve(size_t(w.huge_cap) * sizeof(HugeEntry));
+  off[5] = cv.reserve(size_t(w.nxt_cap) * sizeof(HugeEntry));
+  off[6] = cv.reserve(need_temp ? size_t(nnz) * 4 : 0);
+  off[7] = cv.reserve(need_temp ? size_t(nnz) * vbytes : 0);
+  off[8] = cv.reserve(size_t(w.lchunk_cap) * sizeof(LongChunk));
 }
 
-// Sorts the runs queued in w.fin (counters 0 and 1: its two ends), then the heavy buckets
-// queued by any sort pass (counters 6, 7), in place.
+inline RowsWs rows_bind(const Carver& cv, long long nrows, long long nnz, const size_t* off,
+                        bool sort = true, long long extra_runs = 0) {
+  RowsWs w = rows_caps(nrows, nnz, sort, extra_runs);
+  w.tile_first = cv.at<long long>(off[0]);
+  w.chunk_first = cv.at<long long>(off[1]);
+  w.counters = cv.at<unsigned>(off[2]);
+  w.fin = cv.at<FinalEntry>(off[3]);
+  w.huge = cv.at<HugeEntry>(off[4]);
+  w.nxt = cv.at<HugeEntry>(off[5]);
+  w.tkey = cv.at<uint32_t>(off[6]);
+  w.tval = cv.at<void>(off[7]);
+  w.lchunk = cv.at<LongChunk>(off[8]);
+  return w;
+}
+
+// Key-range split of the rows queued in w.huge (counts w.huge_n()) into runs queued in w.fin
+// (defined and instantiated in rowsort.cu for the column and value words of the library).
 template <class CI, class VT>
-sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits, CI* out_col, VT* out_val) {
-  const int nsm = ctx->num_sms;
-  const int heavy = ctx->cur.heavy;
-  VT* tval = static_cast<VT*>(w.tval);
-  const long long* no_tiles = reinterpret_cast<const long long*>(w.counters + 8);
-  using SsRun = SsRunT<VT>;
-  constexpr size_t rsm = ss_smem_bytes<SsRun, VT>(), ssm = ss_smem_bytes<SsRunS, VT>();
-  // the runs of at most SS_SMALL_RUN entries (the back of the list), then the others
-  SP_CUDA(set_smem(k_seg_sort<SsRunS, CI, VT>, ssm));
-  {
+sp_status split_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, CI* out_col, VT* out_val);
+// Sorts in place the rows a caller queued itself in w.runs() / w.huge (of nnz entries in
+// all; w.counters zeroed before the caller queued them).
+template <class CI, class VT>
+sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz, int key_bits, CI* out_col, VT* out_val);
+// Sorts in place every row of the output arrays (row pointer vp).
+template <class CI, class VT>
+sp_status sort_rows_in_place(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
+                             int key_bits, const RowsWs& w, CI* out_col, VT* out_val);
+
+// Sorts the queued runs; nnz bounds their length.
+template <class Gs>
+sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz, int key_bits, const Gs& gs,
+                    typename Gs::CI* out_col, typename Gs::VT* out_val) {
+  using VT = typename Gs::VT;
+  auto run = [&](auto cfg, int slice) -> sp_status {
+    using Cfg = decltype(cfg);
+    constexpr size_t sm = ss_smem_bytes<Cfg, VT>();
+    SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_LONG);
-    k_seg_sort<SsRunS, CI, VT><<<SsRunS::MINB * nsm, SsRunS::B, ssm, s>>>(
-        nullptr, nullptr, no_tiles, w.fin, w.counters + 1, w.fin_cap, w.tkey, tval, out_col, out_val, w.hv[0],
-        w.counters + 6, w.hv_cap, key_bits, heavy, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  SP_CUDA(set_smem(k_seg_sort<SsRun, CI, VT>, rsm));
-  {
-    SP_PHASE(SP_PHASE_LONG);
-    k_seg_sort<SsRun, CI, VT><<<SsRun::MINB * nsm, SsRun::B, rsm, s>>>(
-        nullptr, nullptr, no_tiles, w.fin, w.counters + 0, w.fin_cap, w.tkey, tval, out_col, out_val, w.hv[0],
-        w.counters + 6, w.hv_cap, key_bits, heavy, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  // heavy buckets: runs over their own key range; the last pass ranks every bucket
-  for (int pass = 0; pass < SS_PASSES; ++pass) {
-    const int a = pass & 1, b = a ^ 1;
-    const bool last = pass == SS_PASSES - 1;
-    SP_CUDA(cudaMemsetAsync(w.counters + 6 + b, 0, 4, s));
-    {
-      SP_PHASE(SP_PHASE_LONG);
-      k_seg_sort<SsRun, CI, VT><<<SsRun::MINB * nsm, SsRun::B, rsm, s>>>(
-          nullptr, nullptr, no_tiles, w.hv[a], w.counters + 6 + a, w.hv_cap, w.tkey, tval, out_col, out_val,
-          last ? nullptr : w.hv[b], w.counters + 6 + b, w.hv_cap, key_bits, heavy, ctx->dstatus);
-    }
+    const long long cap = (long long)Cfg::MINB * ctx->num_sms, g = w.run_cap[slice] < cap ? w.run_cap[slice] : cap;
+    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, nullptr, 0, nullptr, 0, w.runs(), slice, w.tkey,
+                                                        static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
+                                                        ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
-  }
+    return SP_OK;
+  };
+  SP_TRY(run(SsRunS{}, 1));
+  if (nnz > SS_SMALL_RUN) SP_TRY(run(SsRunM{}, 2));
+  if (nnz > SS_MID_RUN) SP_TRY(run(SsRun{}, 3));
   return SP_OK;
 }
 
-// Sorts in place the rows a caller queued itself in w.fin / w.huge (counters 0, 1 and
-// w.huge_n(), zeroed with the rest of w.counters before the caller queued them).
-template <class CI, class VT>
-sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits, CI* out_col, VT* out_val) {
-  SP_TRY((split_queued<CI, VT>(ctx, s, w, out_col, out_val)));
-  return sort_runs<CI, VT>(ctx, s, w, key_bits, out_col, out_val);
-}
-
-// Partition the output rows (row pointer vp, nnz entries), gather them with `gs`
-// (when given) and sort every row in place (when `sort`).
-template <class CI, class VT, class Gs>
-sp_status run_rows(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
-                   int key_bits, const RowsWs& w, const Gs* gs, bool sort, CI* out_col, VT* out_val) {
+// The output rows (row pointer vp, nnz entries) from their source `gs`, sorted.
+template <class Gs>
+sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
+                         int key_bits, const RowsWs& w, const Gs& gs, typename Gs::CI* out_col,
+                         typename Gs::VT* out_val) {
+  using VT = typename Gs::VT;
+  constexpr bool here = in_place<Gs>::value;
   if (nrows == 0 || nnz == 0) return SP_OK;
   SP_CUDA(cudaMemsetAsync(w.counters, 0, 16 * 4, s));
   const int nsm = ctx->num_sms;
-  unsigned* fin_n = w.counters + 0;
-  unsigned* huge_n = w.huge_n();
   // kernel shapes of this call (context options or the tuning table)
   const bool large_tiles = ctx->cur.tile_shape == 1;
-  const long long tmax = large_tiles ? SsTileL::CP : SsTile::CP;
-  const int heavy = ctx->cur.heavy;
-  SP_TRY(launch_scan(ctx, s, RowsWeight{vp, tmax},
-                     RowsPartition{vp, nrows, w.ntiles_cap, w.tile_first, w.ntiles, w.nchunks, w.chunk_first,
-                                   w.fin, fin_n, w.fin_cap, w.huge, huge_n, w.huge_cap, key_bits,
-                                   sort ? 1 : 0, tmax, ctx->dstatus},
-                     nrows, w.scan_ws, SP_PHASE_PARTITION));
-  if (gs) {
-    if (w.nchunks > 0x7fffffffll) return SP_ERR_OVERFLOW;
-    {
-      SP_PHASE(SP_PHASE_GATHER);
-      const long long g = w.nchunks < (long long)GC_MINB * nsm ? w.nchunks : (long long)GC_MINB * nsm;  // persistent
-      k_gather_chunks<Gs><<<unsigned(g), GC_BLOCK, 0, s>>>(*gs, vp, nrows, nnz, w.chunk_first, w.nchunks,
-                                                           out_col, out_val);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  if (!sort) return SP_OK;
-  // The key-range split (rows longer than SS_RUN_MAX, queued by the partition) and the
-  // tile sort (rows of at most tmax) touch disjoint rows.  With the context's overlap on,
-  // the split runs on the context's side stream, whose higher priority dispatches its CTAs
-  // (a hub row's first) ahead of the tiles', while the tiles run on `s`: the SMs that the
-  // split's tail leaves idle take tiles.  The runs, which the split queues, wait for both.
-  constexpr size_t tsm = ss_smem_bytes<SsTile, VT>(), lsm = ss_smem_bytes<SsTileL, VT>();
-  SP_CUDA(set_smem(large_tiles ? k_seg_sort<SsTileL, CI, VT> : k_seg_sort<SsTile, CI, VT>, large_tiles ? lsm : tsm));
-  const bool fork = nnz > SS_RUN_MAX && ctx->overlap && ctx->side;
-  if (fork) {
-    SP_CUDA(cudaEventRecord(ctx->fork_ev, s));
-    SP_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0));
-    const sp_status st = split_queued<CI, VT>(ctx, ctx->side, w, out_col, out_val);
-    SP_CUDA(cudaEventRecord(ctx->join_ev, ctx->side));
-    if (st != SP_OK) {
-      SP_CUDA(cudaStreamWaitEvent(s, ctx->join_ev, 0));
-      return st;
-    }
-  } else if (nnz > SS_RUN_MAX) {
-    SP_TRY((split_queued<CI, VT>(ctx, s, w, out_col, out_val)));
-  }
-  // tiles, then the runs, then the heavy buckets queued by either
-  const unsigned* no_runs = w.counters + 8;
-  VT* tval = static_cast<VT*>(w.tval);
+  const int win = large_tiles ? SsTileL::WIN : SsTile::WIN, tmax = large_tiles ? SsTileL::TMAX : SsTile::TMAX;
+  const long long ntiles = (nnz + SsTile::W * nrows) / win + 1;
   {
-    SP_PHASE(SP_PHASE_TILE);
-    if (large_tiles)
-      k_seg_sort<SsTileL, CI, VT><<<SsTileL::MINB * nsm, SsTileL::B, lsm, s>>>(
-          vp, w.tile_first, w.ntiles, w.fin, no_runs, 0, w.tkey, tval, out_col, out_val, w.hv[0],
-          w.counters + 6, w.hv_cap, key_bits, heavy, ctx->dstatus);
-    else
-      k_seg_sort<SsTile, CI, VT><<<SsTile::MINB * nsm, SsTile::B, tsm, s>>>(
-          vp, w.tile_first, w.ntiles, w.fin, no_runs, 0, w.tkey, tval, out_col, out_val, w.hv[0],
-          w.counters + 6, w.hv_cap, key_bits, heavy, ctx->dstatus);
+    SP_PHASE(SP_PHASE_PARTITION);
+    const RowsPartition part{nrows, nnz, ntiles, w.tile_first, 0, nullptr, w.runs(), w.huge, w.huge_n(),
+                             w.huge_cap, w.lchunk, w.lchunk_n(), w.lchunk_cap, key_bits,
+                             here ? BUF_OUT : BUF_SRC, win, tmax, ctx->dstatus};
+    k_partition<0><<<grid_for(nrows, 256, nsm * 16), 256, 0, s>>>(part, vp);
   }
-  const cudaError_t launched = cudaGetLastError();
+  SP_CUDA(cudaGetLastError());
+  // The rows longer than SS_RUN_MAX (gathered to their place, cut by key range) and the
+  // tiles (rows of at most tmax) are disjoint.  With the context's overlap on, the long
+  // rows run on the context's side stream, whose higher priority dispatches their CTAs (a
+  // hub row's first) ahead of the tiles', while the tiles run on `s`: the SMs that the
+  // split's tail leaves idle take tiles.  The runs, which the split queues, wait for both.
+  const bool any_long = nnz > SS_RUN_MAX, fork = any_long && ctx->overlap && ctx->side;
+  sp_status lst = SP_OK;
+  if (any_long) {
+    cudaStream_t ls = fork ? ctx->side : s;
+    if (fork) {
+      SP_CUDA(cudaEventRecord(ctx->fork_ev, s));
+      SP_CUDA(cudaStreamWaitEvent(ls, ctx->fork_ev, 0));
+    }
+    if constexpr (!here) {
+      {
+        ::sp::PhaseScope ph(ctx, ls, SP_PHASE_GATHER);
+        const long long cap = (long long)GC_MINB * nsm, g = w.lchunk_cap < cap ? w.lchunk_cap : cap;
+        k_gather_long<Gs><<<unsigned(g), GC_BLOCK, 0, ls>>>(gs, w.huge, w.lchunk, w.lchunk_n(), w.lchunk_cap, out_col,
+                                                            out_val, ctx->dstatus);
+      }
+      const cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) {
+        note_cuda_error(e, __FILE__, __LINE__);
+        lst = SP_ERR_CUDA;
+      }
+    }
+    if (lst == SP_OK) lst = split_queued(ctx, ls, w, out_col, out_val);
+    if (fork) SP_CUDA(cudaEventRecord(ctx->join_ev, ls));
+  }
+  auto tiles = [&](auto cfg) -> sp_status {
+    using Cfg = decltype(cfg);
+    constexpr size_t sm = ss_smem_bytes<Cfg, VT>();
+    SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
+    SP_PHASE(SP_PHASE_TILE);
+    const long long cap = (long long)Cfg::MINB * nsm, g = ntiles < cap ? ntiles : cap;
+    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
+                                                        static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
+                                                        ctx->cur.heavy, ctx->dstatus);
+    SP_CUDA(cudaGetLastError());
+    return SP_OK;
+  };
+  sp_status tst = SP_OK;
+  if (lst == SP_OK) tst = large_tiles ? tiles(SsTileL{}) : tiles(SsTile{});
   if (fork) SP_CUDA(cudaStreamWaitEvent(s, ctx->join_ev, 0));
-  SP_CUDA(launched);
-  return sort_runs<CI, VT>(ctx, s, w, key_bits, out_col, out_val);
+  SP_TRY(lst);
+  SP_TRY(tst);
+  return sort_runs(ctx, s, w, nnz, key_bits, gs, out_col, out_val);
+}
+
+// The output rows gathered from `gs` and relabelled, in source order.
+template <class Gs>
+sp_status gather_rows(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
+                      const RowsWs& w, const Gs& gs, typename Gs::CI* out_col, typename Gs::VT* out_val) {
+  if (nrows == 0 || nnz == 0) return SP_OK;
+  if (w.nchunks > 0x7fffffffll) return SP_ERR_OVERFLOW;
+  const int nsm = ctx->num_sms;
+  {
+    SP_PHASE(SP_PHASE_PARTITION);
+    RowsPartition part{};
+    part.nrows = nrows;
+    part.nnz = nnz;
+    part.nchunks = w.nchunks;
+    part.chunk_first = w.chunk_first;
+    k_partition<0><<<grid_for(nrows, 256, nsm * 16), 256, 0, s>>>(part, vp);
+  }
+  SP_CUDA(cudaGetLastError());
+  {
+    SP_PHASE(SP_PHASE_GATHER);
+    const long long g = w.nchunks < (long long)GC_MINB * nsm ? w.nchunks : (long long)GC_MINB * nsm;  // persistent
+    k_gather_chunks<Gs><<<unsigned(g), GC_BLOCK, 0, s>>>(gs, vp, nrows, nnz, w.chunk_first, w.nchunks, out_col, out_val,
+                                                         ctx->dstatus);
+  }
+  SP_CUDA(cudaGetLastError());
+  return SP_OK;
 }
 
 }  // namespace sp

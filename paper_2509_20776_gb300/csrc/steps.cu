@@ -37,8 +37,8 @@ sp_status sort_rows_impl(sp_ctx* ctx, sp_csr* M, cudaStream_t s) {
   }
   const RowsWs w = rows_bind(cv, m, nnz, ro);
   const int kb = ceil_log2_u64(uint64_t(M->ncols));
-  return run_rows<CI, VT, NoGather<CI, VT>>(ctx, s, vp, m, nnz, kb, w, nullptr, true,
-                                            static_cast<CI*>(M->colidx), static_cast<VT*>(M->values));
+  return sort_rows_in_place<CI, VT>(ctx, s, vp, m, nnz, kb, w, static_cast<CI*>(M->colidx),
+                                    static_cast<VT*>(M->values));
 }
 
 // canonical-form check: one warp per row
