@@ -430,13 +430,11 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
       SP_PHASE(SP_PHASE_GATHER);
       const XOne<CI, VT, Rel> src{ci, vv, rel};
       if (sorted)
-        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.runs(),
-                                                          w.huge, w.huge_n(),
-                                                          w.huge_cap, kb, lane_rows, ctx->dstatus);
+        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov,
+                                                          w.lists(), lane_rows, ctx->dstatus);
       else
-        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov, w.runs(),
-                                                           w.huge, w.huge_n(),
-                                                           w.huge_cap, kb, lane_rows, ctx->dstatus);
+        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov,
+                                                           w.lists(), lane_rows, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
     // rows of more than SRC_LONG source entries: one CTA each, kept entries in source order

@@ -341,26 +341,14 @@ __device__ __forceinline__ void x_put(CI* out_col, VT* out_val, long long pos, l
   }
 }
 
-// Sort job of a row the warp path did not sort (k kept entries at output offset o).
-__device__ __forceinline__ void x_queue(long long o, long long k, int key_bits, const RunLists& rl, HugeEntry* huge, unsigned* huge_n, long long huge_cap,
-                                        DevStatus* st) {
-  if (k <= 1) return;
-  if (k <= SS_RUN_MAX) {
-    queue_run(rl, FinalEntry{o, int(k), BUF_OUT, 0}, st, -27);
-  } else {
-    queue_huge(huge, huge_n, huge_cap, HugeEntry{o, k, 0u, key_bits, BUF_OUT, 0, 0}, st, -28);
-  }
-}
-
 // kSorted: the relabelling keeps the source order (ascending J), so slots are ranks and
 // no row is queued.
 template <class Src, bool kSorted>
 __global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const long long* __restrict__ rs0,
                                                 const long long* __restrict__ rsn, const long long* __restrict__ vp,
                                                 typename Src::CI* __restrict__ out_col,
-                                                typename Src::VT* __restrict__ out_val, RunLists rl,
-                                                HugeEntry* huge, unsigned* huge_n,
-                                                long long huge_cap, int key_bits, int lane_rows, DevStatus* st) {
+                                                typename Src::VT* __restrict__ out_val, SortLists sl, int lane_rows,
+                                                DevStatus* st) {
   // lane_rows: XF_LANE when every key is below kDropped (the lane path pads with it), else
   // 0; the lane path is compiled for 4-byte columns and values (its registers)
   using CI = typename Src::CI;
@@ -389,7 +377,8 @@ __global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const lo
       oe = vp[i + 1];
       h = src.handle(i);
     }
-    if (!kSorted && L > XFAST) x_queue(o, oe - o, key_bits, rl, huge, huge_n, huge_cap, st);
+    // a row the warp path does not sort
+    if (!kSorted && L > XFAST && oe - o > 1) queue_row(sl, o, oe - o, BUF_OUT, i, st, -27);
     // rows of at most lane_rows entries: the lane's own row, all its loads and relabels in
     // flight together, the kept entries sorted in registers and written once
     const bool by_lane = L <= (kLane ? lane_rows : 0);

@@ -5,37 +5,10 @@
 namespace sp {
 
 template <class CI, class VT>
-sp_status split_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, CI* out_col, VT* out_val) {
-  const int nsm = ctx->num_sms;
-  VT* tval = static_cast<VT*>(w.tval);
-  constexpr size_t csm = split_smem_bytes<SplitCoarse, VT>(), fsm = split_smem_bytes<SplitFine, VT>();
-  SP_CUDA(set_smem(k_split<SplitCoarse, CI, VT>, csm));
-  SP_CUDA(set_smem(k_split<SplitFine, CI, VT>, fsm));
-  // at most one CTA per row that the lists can hold
-  auto grid = [&](long long minb, long long cap) { return unsigned(cap < minb * nsm ? cap : minb * nsm); };
-  {
-    SP_PHASE(SP_PHASE_HUGE);
-    k_split<SplitCoarse, CI, VT><<<grid(SplitCoarse::MINB, w.huge_cap), SplitCoarse::B, csm, s>>>(
-        w.huge, w.huge_n(), w.huge_cap, w.counters + 4, w.tkey, tval, out_col, out_val, w.runs(),
-        w.nxt, w.nxt_n(), w.nxt_cap, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  // the fine split: the coarse buckets that hold more than SS_RUN_MAX entries (skewed keys
-  // or very long rows); an empty list costs one short launch
-  {
-    SP_PHASE(SP_PHASE_HUGE);
-    k_split<SplitFine, CI, VT><<<grid(SplitFine::MINB, w.nxt_cap), SplitFine::B, fsm, s>>>(
-        w.nxt, w.nxt_n(), w.nxt_cap, w.counters + 5, w.tkey, tval, out_col, out_val, w.runs(),
-        w.nxt, w.counters + 7, 0, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
-  return SP_OK;
-}
-
-template <class CI, class VT>
 sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz, int key_bits, CI* out_col,
                       VT* out_val) {
-  if (nnz > SS_RUN_MAX) SP_TRY((split_queued<CI, VT>(ctx, s, w, out_col, out_val)));
+  const RowsInPlace<CI, VT> gs{nullptr, out_col, out_val};
+  if (nnz > SS_RUN_MAX) SP_TRY(split_long(ctx, s, w, key_bits, gs, out_col, out_val));
   if (w.run_cap[0] > 0) {
     SP_PHASE(SP_PHASE_LONG);
     const long long need = (w.run_cap[0] + 7) / 8, cap = (long long)WR_MINB * ctx->num_sms;
@@ -43,7 +16,7 @@ sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nn
         w.runs(), w.tkey, static_cast<const VT*>(w.tval), out_col, out_val, key_bits >= 32 ? 0xFFFFFFFFu : (1u << key_bits) - 1u, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
   }
-  return sort_runs(ctx, s, w, nnz, key_bits, RowsInPlace<CI, VT>{nullptr, out_col, out_val}, out_col, out_val);
+  return sort_runs(ctx, s, w, nnz, key_bits, gs, out_col, out_val);
 }
 
 template <class CI, class VT>
@@ -54,7 +27,6 @@ sp_status sort_rows_in_place(sp_ctx* ctx, cudaStream_t s, const long long* vp, l
 }
 
 #define SP_ROWSORT(CI, VT)                                                                                            \
-  template sp_status split_queued<CI, VT>(sp_ctx*, cudaStream_t, const RowsWs&, CI*, VT*);                            \
   template sp_status sort_queued<CI, VT>(sp_ctx*, cudaStream_t, const RowsWs&, long long, int, CI*, VT*);             \
   template sp_status sort_rows_in_place<CI, VT>(sp_ctx*, cudaStream_t, const long long*, long long, long long, int,   \
                                                 const RowsWs&, CI*, VT*);

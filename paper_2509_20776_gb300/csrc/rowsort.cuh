@@ -81,34 +81,47 @@ __device__ __forceinline__ void queue_run(const RunLists& rl, const FinalEntry& 
   if (q < rl.cap(k)) rl.slice(k)[q] = e;
   else dev_fail(st, SP_ERR_INTERNAL, err);
 }
-struct HugeEntry {  // a run longer than SS_RUN_MAX; coarse split: keys in [lo, lo + 2^wb)
-  long long off;
+struct HugeEntry {     // a run longer than SS_RUN_MAX
+  long long off;       // output offset
   long long len;
-  unsigned lo;
-  int wb;
-  int buf;
+  long long row;       // BUF_SRC: the output row
+  int buf;             // where its entries are
+  unsigned arrived;    // chunks whose histogram is written (k_long_hist)
+  int bad;             // a key outside the matrix (reported): not cut
   int pad;
-  long long row;    // the output row (rows gathered by k_gather_long)
 };
-struct LongChunk {  // SL_CH output positions of a row longer than SS_RUN_MAX
-  unsigned huge;    // its slot of the huge list
+struct LongChunk {     // SL_CH entries of a row longer than SS_RUN_MAX
+  unsigned huge;       // its slot of the huge list
   unsigned chunk;
 };
 constexpr int SL_CH = 4096;
 
-// The rows queued for the key-range split.  n[0] counts the rows queued at the front of
-// the list, n[1] the rows of at least SPLIT_HUB entries queued from its back; the split
-// hands out the back first, so that a hub row (one CTA for up to milliseconds) starts at
-// once instead of wherever the queueing order put it.  cap >= nnz / SS_RUN_MAX + 1 bounds
-// the number of rows longer than SS_RUN_MAX, so the two ends never meet.
-constexpr long long SPLIT_HUB = 1ll << 16;
-__device__ __forceinline__ long long queue_huge(HugeEntry* list, unsigned* n, long long cap, const HugeEntry& e,
-                                           DevStatus* st, long long err) {
-  const bool hub = e.len >= SPLIT_HUB;
-  const unsigned q = atomicAdd(n + (hub ? 1 : 0), 1u);
-  if (q < cap) list[hub ? cap - 1 - q : q] = e;
-  else dev_fail(st, SP_ERR_INTERNAL, err);
-  return q < cap ? (hub ? cap - 1 - q : q) : -1;
+// What a pass over the output rows queues for the sort: rows of at most SS_RUN_MAX entries
+// as runs, longer ones for the key-range split, chunk by chunk.  The capacities bound what
+// nnz entries can hold (huge_cap rows longer than SS_RUN_MAX, lchunk_cap chunks of them).
+struct SortLists {
+  RunLists runs;
+  HugeEntry* huge;
+  unsigned* huge_n;
+  long long huge_cap;
+  LongChunk* lchunk;
+  unsigned* lchunk_n;
+  long long lchunk_cap;
+};
+__device__ __forceinline__ void queue_row(const SortLists& sl, long long off, long long L, int buf, long long row,
+                                          DevStatus* st, long long err) {
+  if (L <= SS_RUN_MAX) {
+    queue_run(sl.runs, FinalEntry{off, int(L), buf, row}, st, err);
+    return;
+  }
+  const unsigned h = atomicAdd(sl.huge_n, 1u), nc = unsigned((L + SL_CH - 1) / SL_CH);
+  const unsigned c = atomicAdd(sl.lchunk_n, nc);
+  if (h >= sl.huge_cap || (long long)c + nc > sl.lchunk_cap) {
+    dev_fail(st, SP_ERR_INTERNAL, err);
+    return;
+  }
+  sl.huge[h] = HugeEntry{off, L, row, buf, 0u, 0, 0};
+  for (unsigned k = 0; k < nc; ++k) sl.lchunk[c + k] = LongChunk{h, k};
 }
 
 constexpr int GC_BLOCK = 256;                  // gather: threads per CTA
@@ -130,14 +143,7 @@ struct RowsPartition {
   long long* tile_first;    // null: no tiles (nothing is sorted)
   long long nchunks;
   long long* chunk_first;   // null: no gather chunks
-  RunLists runs;            // rows sorted alone
-  HugeEntry* huge;          // rows for k_split
-  unsigned* huge_n;         // two counts (queue_huge)
-  long long huge_cap;
-  LongChunk* lchunk;        // chunks of the rows for k_split
-  unsigned* lchunk_n;
-  long long lchunk_cap;
-  int key_bits;
+  SortLists lists;          // rows that fit no tile
   int buf;                  // where the rows' entries are: BUF_SRC or BUF_OUT
   int win, tmax;            // the tile shape's window and longest row
   DevStatus* st;
@@ -157,22 +163,7 @@ struct RowsPartition {
           tile_first[t] = r + 1;
       else if (r + 1 == nrows)
         for (; t <= ntiles; ++t) tile_first[t] = nrows;
-      if (L > tmax) {
-        if (L <= SS_RUN_MAX) {
-          queue_run(runs, FinalEntry{o0, int(L), buf, r}, st, -15);
-        } else {
-          const long long h =
-              queue_huge(huge, huge_n, huge_cap, HugeEntry{o0, L, 0u, key_bits, BUF_OUT, 0, r}, st, -16);
-          if (buf == BUF_SRC && h >= 0) {
-            const unsigned nc = unsigned((L + SL_CH - 1) / SL_CH), c = atomicAdd(lchunk_n, nc);
-            if (c + (unsigned long long)nc > (unsigned long long)lchunk_cap) {
-              dev_fail(st, SP_ERR_INTERNAL, -14);
-            } else {
-              for (unsigned k = 0; k < nc; ++k) lchunk[c + k] = LongChunk{unsigned(h), k};
-            }
-          }
-        }
-      }
+      if (L > tmax) queue_row(lists, o0, L, buf, r, st, -15);
     }
     if (chunk_first && L > 0) {
       long long k_hi = (o1 - 1) / GC_CH;
@@ -419,56 +410,6 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
   }
 }
 
-// The rows longer than SS_RUN_MAX: chunk by chunk of SL_CH entries, relabelled, to their
-// place in the output (k_split cuts them there).
-template <class Gs>
-__global__ void __launch_bounds__(GC_BLOCK, GC_MINB)
-    k_gather_long(Gs gs, const HugeEntry* __restrict__ huge, const LongChunk* __restrict__ chunks,
-                  const unsigned* __restrict__ n_p, long long cap, typename Gs::CI* __restrict__ out_col,
-                  typename Gs::VT* __restrict__ out_val, DevStatus* st) {
-  using CI = typename Gs::CI;
-  using VT = typename Gs::VT;
-  constexpr int H = GC_H, ITEMS = SL_CH / GC_BLOCK;
-  long long n = *n_p;
-  if (n > cap) n = cap;
-  for (long long k = blockIdx.x; k < n; k += gridDim.x) {
-    const LongChunk lc = chunks[k];
-    const HugeEntry he = huge[lc.huge];
-    const long long e0 = (long long)lc.chunk * SL_CH, o = he.off + e0;
-    const int len = he.len - e0 < SL_CH ? int(he.len - e0) : SL_CH;
-    const GsView<CI, VT> gv = gs.view(gs.srcs()[he.row], he.len);
-    if (!gv.c) {
-      if (threadIdx.x == 0) dev_fail(st, SP_ERR_INTERNAL, -13);
-      continue;
-    }
-#pragma unroll
-    for (int h = 0; h < ITEMS; h += H) {
-      CI cv[H];
-      VT v[H];
-#pragma unroll
-      for (int u = 0; u < H; ++u) {
-        const int x = threadIdx.x + (h + u) * GC_BLOCK;
-        cv[u] = x < len ? ld_stream(gv.c + e0 + x) : CI(0);
-      }
-#pragma unroll
-      for (int u = 0; u < H; ++u) {
-        const int x = threadIdx.x + (h + u) * GC_BLOCK;
-        v[u] = x < len ? ld_stream(gv.v + e0 + x) : VT(0);
-      }
-      uint32_t key[H];
-#pragma unroll
-      for (int u = 0; u < H; ++u) key[u] = gs.map(gv.mid, ss_key(cv[u]));
-#pragma unroll
-      for (int u = 0; u < H; ++u) {
-        const int x = threadIdx.x + (h + u) * GC_BLOCK;
-        if (x >= len) continue;
-        st_stream(out_col + o + x, CI(key[u]));
-        st_stream(out_val + o + x, v[u]);
-      }
-    }
-  }
-}
-
 // ---- approximate square-root bucketing of the row sort -----------------------------------
 // Bucket of key k in a row of L entries: nb = 2^(ceil(log2 L) - 1) buckets spaced evenly
 // in an approximate square root of k over the row's key range [0, kmax].  The root is
@@ -488,306 +429,381 @@ __device__ __forceinline__ uint32_t ss_bucket(uint32_t key, float scale, uint32_
   return b < last ? b : last;
 }
 
-// ---- key-range split of long runs ------------------------------------------------------
-// A run of more than SS_RUN_MAX entries with keys in [lo, lo + 2^wb) is cut into nb = 2^nbl
-// buckets of 2^(wb - nbl) consecutive keys: pass 1 counts the bucket sizes, one scan gives
-// their offsets, pass 2 moves the run bucket by bucket into the other buffer (output <->
-// temporary) at the same offsets.  Consecutive small buckets whose starts fall in one
-// GROUP_CAP window form one run for k_seg_sort; a bucket of more than GROUP_CAP entries is
-// a run of its own, or (more than SS_RUN_MAX entries) a run for the fine split.
-//   Coarse split (SplitCoarse): nb = 2^10 buckets evenly spaced over [lo, lo + 2^wb).  A run
-//     is sorted as a whole afterwards, so pass 2 only has to bring every entry into its
-//     group's range, not its bucket's: it stages each chunk of B * U entries in shared
-//     memory by group and writes every group's share of the chunk as one contiguous piece
-//     (groups hold hundreds to thousands of entries, so the writes are coalesced whatever
-//     the key distribution).
-//   Fine split (SplitFine, the buckets of the coarse split that hold more than SS_RUN_MAX entries,
-//     e.g. hub rows under a degree-descending relabelling): 2^13 buckets evenly spaced over
-//     the bucket's own [min, max] keys (found by a first pass), scattered directly.  A
-//     coarse bucket spans 2^(wb - 10) <= 2^22 keys, so a fine bucket spans at most
-//     2^9 < SS_RUN_MAX keys: with keys unique within a row it holds fewer than SS_RUN_MAX
-//     entries and no third split is needed.
-struct SplitCoarse {
-  static constexpr int NBL = 10, B = 256, MINB = 4, U = 8;
-  static constexpr bool kStaged = true;
-};
-struct SplitFine {
-  static constexpr int NBL = 13, B = 512, MINB = 2, U = 4;
-  static constexpr bool kStaged = false;
-};
+// ---- key-range split of long rows ------------------------------------------------------
+// A row of more than SS_RUN_MAX entries is cut by key into runs of at most SS_RUN_MAX
+// entries, chunk by chunk of SL_CH entries so that a hub row is spread over the chip (one
+// CTA per row took up to 2.4 ms for a row of 640 K entries, and set the time of this phase
+// on every power-law matrix of a few M entries):
+//   k_long_hist    reads a chunk (at the row's source, relabelled, its keys written to the
+//                  row's place in the output; or in the output already) and counts its keys
+//                  in 2^10 buckets evenly spaced over [0, 2^key_bits).  The CTA that
+//                  finishes a row's last chunk adds up the counts and forms groups:
+//                  consecutive small buckets whose starts fall in one GROUP_CAP window are
+//                  one run; a bucket of more than GROUP_CAP entries is a run of its own,
+//                  or (more than SS_RUN_MAX entries) goes to the fine split.
+//   k_long_scatter moves a chunk's entries to their groups in the temporary arrays: staged
+//                  in shared memory by group, then each group's share written as one piece
+//                  at a place taken from the group's cursor.
+//   k_split_fine   one CTA per oversized bucket (skewed keys): 2^13 buckets over the
+//                  bucket's own [min, max] keys, from the temporary to the output arrays.
+//                  A coarse bucket spans 2^(key_bits - 10) <= 2^22 keys, so a fine bucket
+//                  spans at most 2^9 < SS_RUN_MAX keys: with keys unique within a row it
+//                  holds fewer than SS_RUN_MAX entries and no third split is needed; with
+//                  key_bits <= 22 no coarse bucket can be oversized and it is not launched.
+// The runs are then sorted by k_seg_sort.
+constexpr int SL_NBL = 10, SL_NB = 1 << SL_NBL;
+constexpr int SL_HB = 256, SL_HMINB = 5;  // k_long_hist
+constexpr int SL_SB = 512;                // k_long_scatter
+template <class VT>
+constexpr int sl_sminb() { return sizeof(VT) == 4 ? 3 : 2; }
+constexpr int SF_NBL = 13, SF_B = 512, SF_MINB = 2, SF_U = 4;  // k_split_fine
 constexpr int SS_RUN_LOG = 12;             // SS_RUN_MAX = 2^SS_RUN_LOG
 static_assert((1 << SS_RUN_LOG) == SS_RUN_MAX, "run capacity is a power of two");
+static_assert(32 - SL_NBL - SF_NBL <= SS_RUN_LOG, "fine-split buckets fit a run");
 constexpr int GROUP_CAP = SS_SMALL_RUN;    // small buckets grouped up to this start window: runs of at most SS_MID_RUN
-template <class S, class VT>
-constexpr size_t split_smem_bytes() {
-  // counts / starts / cursors, previous non-empty bucket, next group boundary; staged:
-  // the group of each bucket, the chunk's counts / starts per group, the chunk's base in
-  // each group, the chunk's keys and values
-  return size_t(1 << S::NBL) * 4 * 3 +
-         (S::kStaged ? size_t(1 << S::NBL) * 4 * 3 + size_t(S::B * S::U) * (4 + sizeof(VT)) : 0);
+// A row's groups: at most one per GROUP_CAP window of starts, one per bucket of more than
+// GROUP_CAP entries and one after each such bucket: 3 L / GROUP_CAP + 1 < L / SL_GSLOT - 1
+// for L > SS_RUN_MAX, so a row's cursors fit the slots [off / SL_GSLOT, (off + L) / SL_GSLOT).
+constexpr int SL_GSLOT = 256;
+static_assert(GROUP_CAP == 4 * SL_GSLOT && SS_RUN_MAX > 3 * GROUP_CAP, "cursor slots");
+// A chunk's histogram (SL_NB 16-bit counts) goes to its row's part of the temporary keys,
+// which nothing else uses before the scatter: ceil(L / SL_CH) * SL_NB / 2 <= L words.
+static_assert(SL_CH / (SL_NB / 2) >= 2, "chunk histograms fit the temporary keys");
+
+// Groups of a split: hist (exclusive starts of nb buckets, SIZE of them scanned, the rest
+// empty; total L) -> a bucket is big, or the head of a group.  All threads of the CTA call
+// it; prv and nxb hold SIZE words.  Afterwards emit(x, big, start, end) is called for every
+// big bucket and every group (end: the next group's or big bucket's start).
+template <int B, int SIZE, class Emit>
+__device__ void split_groups(const uint32_t* hist, uint32_t* prv, uint32_t* nxb, uint32_t* tmp32, int nb, uint32_t L,
+                             Emit&& emit) {
+  const int t = threadIdx.x;
+  // bucket x holds [hist[x], end(x)); bucket order is key order
+  auto bend = [&](int x) { return x + 1 < nb ? hist[x + 1] : L; };
+  // previous non-empty bucket (inclusive max-scan of x+1 over non-empty buckets)
+  for (int x = t; x < SIZE; x += B) prv[x] = (x < nb && bend(x) > hist[x]) ? uint32_t(x + 1) : 0u;
+  __syncthreads();
+  smem_incl_max_w<B>(prv, SIZE, tmp32);
+  // A bucket of more than GROUP_CAP entries ("big") stands alone; a small non-empty bucket
+  // starts a new group ("head") unless the previous non-empty bucket is small and starts in
+  // the same GROUP_CAP window.
+  auto kind = [&](int x, bool& big, bool& head) {
+    const uint32_t sb = hist[x], cc = x < nb ? bend(x) - sb : 0u;
+    big = cc > uint32_t(GROUP_CAP);
+    head = false;
+    if (cc > 0 && !big) {
+      const uint32_t pv = x > 0 ? prv[x - 1] : 0u;
+      if (pv == 0) {
+        head = true;
+      } else {
+        const int y = int(pv) - 1;
+        head = bend(y) - hist[y] > uint32_t(GROUP_CAP) || (hist[y] / GROUP_CAP) != (sb / GROUP_CAP);
+      }
+    }
+  };
+  // next group boundary after each bucket: suffix min of boundary starts, as a prefix
+  // max over the reversed array of (L - start)
+  for (int x = t; x < SIZE; x += B) {
+    bool big, head;
+    kind(x, big, head);
+    nxb[SIZE - 1 - x] = (big || head) ? L - hist[x] : 0u;
+  }
+  __syncthreads();
+  smem_incl_max_w<B>(nxb, SIZE, tmp32);
+  for (int x = t; x < SIZE; x += B) {
+    bool big, head;
+    kind(x, big, head);
+    if (!big && !head) continue;
+    const uint32_t nx = (x + 1 < SIZE) ? nxb[SIZE - 1 - (x + 1)] : 0u;
+    emit(x, big, hist[x], big ? bend(x) : (nx ? L - nx : L));
+  }
 }
 
-template <class S, class CI, class VT>
-__global__ void __launch_bounds__(S::B, S::MINB)
-    k_split(const HugeEntry* __restrict__ runs, const unsigned* __restrict__ nruns_p, long long runs_cap,
-            unsigned* ticket, uint32_t* __restrict__ tkey, VT* __restrict__ tval, CI* __restrict__ out_col,
-            VT* __restrict__ out_val, RunLists rl,
-            HugeEntry* __restrict__ nxt, unsigned* nxt_n, long long nxt_cap, DevStatus* st) {
-  constexpr int B = S::B, U = S::U, NBM = 1 << S::NBL;
+template <class Gs>
+__global__ void __launch_bounds__(SL_HB, SL_HMINB)
+    k_long_hist(Gs gs, SortLists sl, uint32_t* __restrict__ tkey, typename Gs::CI* __restrict__ out_col,
+                uint16_t* __restrict__ gmap, uint32_t* __restrict__ cursor, HugeEntry* __restrict__ nxt,
+                unsigned* nxt_n, long long nxt_cap, int key_bits, DevStatus* st) {
+  using CI = typename Gs::CI;
+  constexpr int B = SL_HB, NB = SL_NB, ITEMS = SL_CH / B, H = 4;
+  __shared__ uint32_t hist[NB], prv[NB], nxb[NB];
+  __shared__ uint32_t tmp32[B / 32 + 1];
+  __shared__ int s_last;
+  const int t = threadIdx.x;
+  const uint32_t kmax = key_bits >= 32 ? 0xFFFFFFFFu : (1u << key_bits) - 1u;
+  const int nbl = key_bits < SL_NBL ? key_bits : SL_NBL, sh = key_bits - nbl, nb = 1 << nbl;
+  long long n = *sl.lchunk_n;
+  if (n > sl.lchunk_cap) n = sl.lchunk_cap;
+  for (long long k = blockIdx.x; k < n; k += gridDim.x) {
+    const LongChunk lc = sl.lchunk[k];
+    HugeEntry* const hp = sl.huge + lc.huge;
+    const long long off = hp->off, L = hp->len, e0 = (long long)lc.chunk * SL_CH;
+    const int len = L - e0 < SL_CH ? int(L - e0) : SL_CH;
+    const unsigned nc = unsigned((L + SL_CH - 1) / SL_CH);
+    for (int x = t; x < NB; x += B) hist[x] = 0;
+    __syncthreads();
+    const bool here = in_place<Gs>::value || hp->buf != BUF_SRC;
+    GsView<CI, typename Gs::VT> gv{out_col + off, nullptr, 0u};
+    if (!here) gv = gs.view(gs.srcs()[hp->row], L);
+    bool bad = false;
+    if (!gv.c) {
+      if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -13);
+      bad = true;
+    } else {
+      CI* const oc = out_col + off + e0;
+      const CI* const cp = gv.c + e0;
+#pragma unroll
+      for (int h = 0; h < ITEMS; h += H) {
+        uint32_t key[H];
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+          const int x = t + (h + u) * B;
+          key[u] = x < len ? ss_key(ld_stream(cp + x)) : 0u;
+        }
+        if (!here) {
+#pragma unroll
+          for (int u = 0; u < H; ++u) key[u] = gs.map(gv.mid, key[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+          const int x = t + (h + u) * B;
+          if (x >= len) continue;
+          if (!here) st_stream(oc + x, CI(key[u]));
+          if (key[u] <= kmax) {
+            atomicAdd(&hist[key[u] >> sh], 1u);
+          } else {  // a column outside [0, ncols)
+            dev_fail(st, SP_ERR_INDEX_RANGE, off + e0 + x);
+            bad = true;
+          }
+        }
+      }
+    }
+    if (bad) hp->bad = 1;
+    __syncthreads();
+    uint32_t* const ch = tkey + off;  // chunk c's histogram at c * NB / 2
+    for (int w = t; w < NB / 2; w += B)
+      __stcg(ch + (long long)lc.chunk * (NB / 2) + w, hist[2 * w] | (hist[2 * w + 1] << 16));
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(&hp->arrived, 1u) == nc - 1;
+    __syncthreads();
+    if (!s_last) continue;
+    // the row's last chunk: add up the counts and form the groups
+    __threadfence();
+    if (__ldcg(&hp->bad)) continue;  // uniform: written before the last arrival
+    for (int w = t; w < NB / 2; w += B) {
+      uint32_t lo = 0, hi = 0;
+#pragma unroll 4
+      for (unsigned c = 0; c < nc; ++c) {
+        const uint32_t v = __ldcg(ch + (long long)c * (NB / 2) + w);
+        lo += v & 0xFFFFu;
+        hi += v >> 16;
+      }
+      hist[2 * w] = lo;
+      hist[2 * w + 1] = hi;
+    }
+    __syncthreads();
+    smem_excl_sum_w<B>(hist, NB, tmp32);
+    uint32_t* const cur = cursor + off / SL_GSLOT;
+    split_groups<B, NB>(hist, prv, nxb, tmp32, nb, uint32_t(L), [&](int, bool big, uint32_t s, uint32_t e) {
+      if (e - s <= uint32_t(SS_RUN_MAX)) {
+        queue_run(sl.runs, FinalEntry{off + s, int(e - s), BUF_TEMP, 0}, st, -6);
+      } else {
+        const unsigned q = atomicAdd(nxt_n, 1u);  // the fine split finds its key range itself
+        if (q < nxt_cap) nxt[q] = HugeEntry{off + s, (long long)(e - s), 0, BUF_TEMP, 0u, 0, 0};
+        else dev_fail(st, SP_ERR_INTERNAL, -7);
+      }
+    });
+    __syncthreads();  // prv has been read
+    // number the groups: group of bucket x = starts at or before x, minus 1
+    for (int x = t; x < NB; x += B) {
+      const uint32_t a = nxb[NB - 1 - x], b = x + 1 < NB ? nxb[NB - 1 - (x + 1)] : 0u;
+      prv[x] = a != b ? 1u : 0u;  // the suffix minimum changes exactly at a start
+    }
+    __syncthreads();
+    smem_excl_sum_w<B>(prv, NB, tmp32);
+    for (int x = t; x < NB; x += B) {
+      const uint32_t a = nxb[NB - 1 - x], b = x + 1 < NB ? nxb[NB - 1 - (x + 1)] : 0u;
+      const bool start = a != b;
+      const uint32_t g = prv[x] - (start ? 0u : 1u);
+      gmap[(long long)lc.huge * NB + x] = uint16_t(g);
+      if (start) cur[g] = hist[x];
+    }
+    __syncthreads();
+  }
+}
+
+template <class VT>
+constexpr size_t long_scatter_smem() {
+  return size_t(SL_NB) * (4 + 4 + 2) + size_t(SL_CH) * (4 + sizeof(VT));
+}
+template <class Gs>
+__global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
+    k_long_scatter(Gs gs, SortLists sl, uint32_t* __restrict__ tkey, typename Gs::VT* __restrict__ tval,
+                   const typename Gs::CI* __restrict__ out_col, const typename Gs::VT* __restrict__ out_val,
+                   const uint16_t* __restrict__ gmap, uint32_t* __restrict__ cursor, int key_bits) {
+  using VT = typename Gs::VT;
+  constexpr int B = SL_SB, NB = SL_NB, U = SL_CH / B;
+  extern __shared__ __align__(16) unsigned char smem[];
+  VT* sv = reinterpret_cast<VT*>(smem);                        // the chunk's values by group
+  uint32_t* sk = reinterpret_cast<uint32_t*>(sv + SL_CH);      // and keys
+  uint32_t* lh = sk + SL_CH;                                   // its count, then start, in each group
+  uint32_t* gb = lh + NB;                                      // where its share of the group goes
+  uint16_t* gm = reinterpret_cast<uint16_t*>(gb + NB);         // group of each bucket
+  __shared__ uint32_t tmp32[B / 32 + 1];
+  const int t = threadIdx.x;
+  const int sh = key_bits - (key_bits < SL_NBL ? key_bits : SL_NBL);
+  long long n = *sl.lchunk_n;
+  if (n > sl.lchunk_cap) n = sl.lchunk_cap;
+  for (long long k = blockIdx.x; k < n; k += gridDim.x) {
+    const LongChunk lc = sl.lchunk[k];
+    const HugeEntry he = sl.huge[lc.huge];
+    if (he.bad) continue;
+    const long long e0 = (long long)lc.chunk * SL_CH;
+    const int len = he.len - e0 < SL_CH ? int(he.len - e0) : SL_CH;
+    const VT* vp = out_val + he.off;
+    if (!in_place<Gs>::value && he.buf == BUF_SRC) vp = gs.view(gs.srcs()[he.row], he.len).v;
+    for (int x = t; x < NB; x += B) {
+      lh[x] = 0;
+      gm[x] = gmap[(long long)lc.huge * NB + x];
+    }
+    uint32_t key[U], pk[U];  // group << 16 | rank in the group's share of the chunk
+    VT val[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = t + u * B;
+      key[u] = x < len ? ss_key(ld_stream(out_col + he.off + e0 + x)) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int x = t + u * B;
+      val[u] = x < len ? ld_stream(vp + e0 + x) : VT(0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      pk[u] = 0xFFFFFFFFu;
+      if (t + u * B >= len) continue;
+      const uint32_t g = gm[key[u] >> sh];
+      pk[u] = (g << 16) | atomicAdd(&lh[g], 1u);
+    }
+    __syncthreads();
+    uint32_t* const cur = cursor + he.off / SL_GSLOT;
+    for (int g = t; g < NB; g += B) gb[g] = lh[g] ? atomicAdd(cur + g, lh[g]) : 0u;
+    smem_excl_sum_w<B>(lh, NB, tmp32);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (pk[u] == 0xFFFFFFFFu) continue;
+      const uint32_t q = lh[pk[u] >> 16] + (pk[u] & 0xFFFFu);
+      sk[q] = key[u];
+      sv[q] = val[u];
+    }
+    __syncthreads();
+    for (int i = t; i < len; i += B) {
+      const uint32_t kk = sk[i], g = gm[kk >> sh];
+      const uint32_t q = gb[g] + (uint32_t(i) - lh[g]);
+      if (q >= uint32_t(he.len)) continue;
+      st_stream(tkey + he.off + q, kk);
+      st_stream(tval + he.off + q, sv[i]);
+    }
+    __syncthreads();
+  }
+}
+
+constexpr size_t split_fine_smem() { return size_t(1 << SF_NBL) * 4 * 3; }
+template <class CI, class VT>
+__global__ void __launch_bounds__(SF_B, SF_MINB)
+    k_split_fine(const HugeEntry* __restrict__ runs, const unsigned* __restrict__ nruns_p, long long runs_cap,
+                 unsigned* ticket, const uint32_t* __restrict__ tkey, const VT* __restrict__ tval,
+                 CI* __restrict__ out_col, VT* __restrict__ out_val, RunLists rl, DevStatus* st) {
+  constexpr int B = SF_B, U = SF_U, NBM = 1 << SF_NBL;
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* hist = reinterpret_cast<uint32_t*>(smem);  // bucket sizes, then starts, then cursors
-  uint32_t* prv = hist + NBM;   // 1 + last non-empty bucket at or before x (0: none)
-  uint32_t* nxb = prv + NBM;    // reversed: L - start of the first group boundary >= x
-  uint32_t* hd = nxb + NBM;     // staged: 1 + first bucket of each bucket's group
-  uint32_t* lh = hd + NBM;      // staged: the chunk's count, then start, in each group
-  uint32_t* gb = lh + NBM;      // staged: the chunk's offset in each group
-  uint32_t* sk = gb + NBM;      // staged: the chunk's keys by group
-  VT* sv = reinterpret_cast<VT*>(sk + B * U);  // and values
+  uint32_t* prv = hist + NBM;
+  uint32_t* nxb = prv + NBM;
   __shared__ uint32_t tmp32[B / 32 + 1];
   __shared__ unsigned s_item;
   const int t = threadIdx.x;
-  // the list's back (rows of >= SPLIT_HUB entries) first, then its front
-  long long nb_ = nruns_p[1], nf_ = nruns_p[0];
-  if (nb_ > runs_cap) nb_ = runs_cap;
-  if (nf_ > runs_cap - nb_) nf_ = runs_cap - nb_;
-  const long long count = nb_ + nf_;
+  long long count = *nruns_p;
+  if (count > runs_cap) count = runs_cap;
   for (;;) {
     if (t == 0) s_item = atomicAdd(ticket, 1u);
     __syncthreads();
     const long long item = s_item;
     if (item >= count) break;
-    const HugeEntry he = runs[item < nb_ ? runs_cap - 1 - item : item - nb_];
-    const long long g0 = he.off, L = he.len;
-    const int sbuf = he.buf;
-    const int dbuf = sbuf == BUF_TEMP ? BUF_OUT : BUF_TEMP;
+    const long long g0 = runs[item].off, L = runs[item].len;
     const uint32_t* skp = tkey + g0;
-    const CI* sop = out_col + g0;
-    auto key_at = [&](long long e) -> uint32_t {
-      return sbuf == BUF_TEMP ? ld_stream(skp + e) : uint32_t(ld_stream(sop + e));
-    };
-    uint32_t lo;
-    int wb, nbl;
-    if constexpr (S::kStaged) {
-      lo = he.lo;
-      wb = he.wb;
-      nbl = wb < S::NBL ? wb : S::NBL;
-      static_assert(32 - S::NBL - SplitFine::NBL <= SS_RUN_LOG, "fine-split buckets fit a run");
-    } else {
-      // the bucket's own key range
-      uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-      for (long long e0 = t; e0 < L; e0 += (long long)B * U) {
-        uint32_t k[U];
+    const VT* svp = tval + g0;
+    // the bucket's own key range
+    uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+    for (long long e0 = t; e0 < L; e0 += (long long)B * U) {
+      uint32_t k[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (e0 + (long long)u * B < L) k[u] = key_at(e0 + (long long)u * B);
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) k[u] = ld_stream(skp + e0 + (long long)u * B);
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (e0 + (long long)u * B < L) {
-            mn = k[u] < mn ? k[u] : mn;
-            mx = k[u] > mx ? k[u] : mx;
-          }
-      }
-      mn = __reduce_min_sync(0xFFFFFFFFu, mn);
-      mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-      if ((t & 31) == 0) {
-        tmp32[t >> 5] = mn;
-        hist[t >> 5] = mx;  // hist is cleared below
-      }
-      __syncthreads();
-      mn = 0xFFFFFFFFu;
-      mx = 0u;
-      for (int w = 0; w < B / 32; ++w) {
-        mn = tmp32[w] < mn ? tmp32[w] : mn;
-        mx = hist[w] > mx ? hist[w] : mx;
-      }
-      __syncthreads();
-      lo = mn;
-      const uint32_t span = mx >= mn ? mx - mn : 0u;  // keys in [lo, lo + span]
-      wb = span ? 32 - __clz(span) : 0;                // 2^wb > span
-      nbl = wb < S::NBL ? wb : S::NBL;
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) {
+          mn = k[u] < mn ? k[u] : mn;
+          mx = k[u] > mx ? k[u] : mx;
+        }
     }
-    const int nb = 1 << nbl;
-    const int sh = wb - nbl;
-    const uint32_t rmax = wb >= 32 ? 0xFFFFFFFFu : (1u << wb) - 1u;  // largest offset from lo
-    // bucket of key k, or 0xFFFFFFFF for a key outside the run's range (a column outside
-    // [0, ncols): reported by pass 1)
-    auto bucket = [&](uint32_t k) -> uint32_t {
-      if (k < lo || k - lo > rmax) return 0xFFFFFFFFu;
-      return (k - lo) >> sh;
-    };
+    mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if ((t & 31) == 0) {
+      tmp32[t >> 5] = mn;
+      hist[t >> 5] = mx;  // hist is cleared below
+    }
+    __syncthreads();
+    mn = 0xFFFFFFFFu;
+    mx = 0u;
+    for (int w = 0; w < B / 32; ++w) {
+      mn = tmp32[w] < mn ? tmp32[w] : mn;
+      mx = hist[w] > mx ? hist[w] : mx;
+    }
+    __syncthreads();
+    const uint32_t lo = mn, span = mx >= mn ? mx - mn : 0u;  // keys in [lo, lo + span]
+    const int wb = span ? 32 - __clz(span) : 0;               // 2^wb > span
+    const int nbl = wb < SF_NBL ? wb : SF_NBL, nb = 1 << nbl, sh = wb - nbl;
     for (int x = t; x < NBM; x += B) hist[x] = 0;
     __syncthreads();
     // pass 1: bucket sizes
     for (long long e0 = t; e0 < L; e0 += (long long)B * U) {
       uint32_t k[U];
 #pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) k[u] = ld_stream(skp + e0 + (long long)u * B);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) atomicAdd(&hist[(k[u] - lo) >> sh], 1u);
+    }
+    __syncthreads();
+    smem_excl_sum_w<B>(hist, NBM, tmp32);
+    split_groups<B, NBM>(hist, prv, nxb, tmp32, nb, uint32_t(L), [&](int, bool, uint32_t s, uint32_t e) {
+      if (e - s <= uint32_t(SS_RUN_MAX)) queue_run(rl, FinalEntry{g0 + s, int(e - s), BUF_OUT, 0}, st, -6);
+      else dev_fail(st, SP_ERR_INTERNAL, -7);  // repeated keys (reported where the map was built)
+    });
+    __syncthreads();
+    // pass 2 (hist now serves as the bucket cursors): scatter entry by entry
+    for (long long e0 = t; e0 < L; e0 += (long long)B * U) {
+      uint32_t k[U];
+      VT v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) k[u] = ld_stream(skp + e0 + (long long)u * B);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (e0 + (long long)u * B < L) v[u] = ld_stream(svp + e0 + (long long)u * B);
+#pragma unroll
       for (int u = 0; u < U; ++u) {
-        const long long e = e0 + (long long)u * B;
-        if (e < L) k[u] = key_at(e);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const long long e = e0 + (long long)u * B;
-        if (e >= L) continue;
-        const uint32_t bk = bucket(k[u]);
-        if (bk != 0xFFFFFFFFu) atomicAdd(&hist[bk], 1u);
-        else dev_fail(st, SP_ERR_INDEX_RANGE, g0 + e);  // a column outside [0, ncols)
+        if (e0 + (long long)u * B >= L) continue;
+        const uint32_t q = atomicAdd(&hist[(k[u] - lo) >> sh], 1u);
+        if (q >= uint32_t(L)) continue;
+        st_stream(out_col + g0 + q, CI(k[u]));
+        st_stream(out_val + g0 + q, v[u]);
       }
     }
     __syncthreads();
-    const uint32_t total = smem_excl_sum_w<B>(hist, NBM, tmp32);
-    if (total != uint32_t(L)) {
-      if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -5);
-      continue;
-    }
-    // bucket x holds [hist[x], end(x)); bucket order is key order
-    auto bend = [&](int x) { return x + 1 < nb ? hist[x + 1] : uint32_t(L); };
-    // previous non-empty bucket (inclusive max-scan of x+1 over non-empty buckets)
-    for (int x = t; x < NBM; x += B) prv[x] = (x < nb && bend(x) > hist[x]) ? uint32_t(x + 1) : 0u;
-    __syncthreads();
-    smem_incl_max_w<B>(prv, NBM, tmp32);
-    // Groups: a bucket of more than GROUP_CAP entries ("big") stands alone; a small
-    // non-empty bucket starts a new group ("head") unless the previous non-empty
-    // bucket is small and starts in the same GROUP_CAP window.
-    auto kind = [&](int x, bool& big, bool& head) {
-      const uint32_t sb = hist[x], cc = x < nb ? bend(x) - sb : 0u;
-      big = cc > uint32_t(GROUP_CAP);
-      head = false;
-      if (cc > 0 && !big) {
-        const uint32_t pv = x > 0 ? prv[x - 1] : 0u;
-        if (pv == 0) {
-          head = true;
-        } else {
-          const int y = int(pv) - 1;
-          head = bend(y) - hist[y] > uint32_t(GROUP_CAP) || (hist[y] / GROUP_CAP) != (sb / GROUP_CAP);
-        }
-      }
-    };
-    // next group boundary after each bucket: suffix min of boundary starts, as a prefix
-    // max over the reversed array of (L - start)
-    for (int x = t; x < NBM; x += B) {
-      bool big, head;
-      kind(x, big, head);
-      nxb[NBM - 1 - x] = (big || head) ? uint32_t(L) - hist[x] : 0u;
-      if constexpr (S::kStaged) hd[x] = (big || head) ? uint32_t(x + 1) : 0u;
-    }
-    __syncthreads();
-    smem_incl_max_w<B>(nxb, NBM, tmp32);
-    if constexpr (S::kStaged) smem_incl_max_w<B>(hd, NBM, tmp32);  // group of each bucket
-    for (int x = t; x < nb; x += B) {
-      bool big, head;
-      kind(x, big, head);
-      const uint32_t sb = hist[x], cc = bend(x) - sb;
-      if (big) {
-        if (cc <= uint32_t(SS_RUN_MAX)) {
-          queue_run(rl, FinalEntry{g0 + sb, int(cc), dbuf, 0}, st, -6);
-        } else {
-          const unsigned q = atomicAdd(nxt_n, 1u);  // the fine split finds its key range itself
-          if (q < nxt_cap) nxt[q] = HugeEntry{g0 + sb, cc, 0u, 0, dbuf, 0, 0};
-          else dev_fail(st, SP_ERR_INTERNAL, -7);
-        }
-      } else if (head) {
-        // reversed index of x+1 holds max over buckets >= x+1 of (L - start) -> min start
-        const uint32_t nx = (x + 1 < NBM) ? nxb[NBM - 1 - (x + 1)] : 0u;
-        const uint32_t end = nx ? uint32_t(L) - nx : uint32_t(L);
-        queue_run(rl, FinalEntry{g0 + sb, int(end - sb), dbuf, 0}, st, -6);
-      }
-    }
-    __syncthreads();
-    // pass 2 (hist now serves as the bucket cursors)
-    const VT* svp = sbuf == BUF_TEMP ? tval + g0 : out_val + g0;
-    if constexpr (S::kStaged) {
-      // chunk by chunk: rank every entry within its group's share of the chunk, stage the
-      // chunk by group, then write each share to the group's next free range
-      constexpr int CH = B * U;
-      for (long long c0 = 0; c0 < L; c0 += CH) {
-        const int n = L - c0 < CH ? int(L - c0) : CH;
-        for (int x = t; x < NBM; x += B) lh[x] = 0;
-        __syncthreads();
-        uint32_t k[U], pk[U];  // key; group << 16 | rank in the group's share (CH <= 2^16)
-        VT v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = t + u * B;
-          if (e < n) k[u] = key_at(c0 + e);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = t + u * B;
-          if (e < n) v[u] = ld_stream(svp + c0 + e);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = t + u * B;
-          pk[u] = 0xFFFFFFFFu;
-          if (e >= n) continue;
-          const uint32_t bk = bucket(k[u]);
-          if (bk == 0xFFFFFFFFu) continue;
-          const uint32_t g = hd[bk] - 1u;  // every non-empty bucket lies in a group
-          pk[u] = (g << 16) | atomicAdd(&lh[g], 1u);
-        }
-        __syncthreads();
-        for (int x = t; x < nb; x += B) {
-          gb[x] = hist[x];
-          hist[x] += lh[x];
-        }
-        const uint32_t nst = smem_excl_sum_w<B>(lh, NBM, tmp32);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          if (pk[u] == 0xFFFFFFFFu) continue;
-          const uint32_t q = lh[pk[u] >> 16] + (pk[u] & 0xFFFFu);
-          sk[q] = k[u];
-          sv[q] = v[u];
-        }
-        __syncthreads();
-        for (int i = t; i < int(nst); i += B) {
-          const uint32_t key = sk[i], g = hd[bucket(key)] - 1u;
-          const uint32_t q = gb[g] + (uint32_t(i) - lh[g]);
-          if (q >= uint32_t(L)) continue;
-          if (dbuf == BUF_TEMP) {
-            st_stream(tkey + g0 + q, key);
-            st_stream(tval + g0 + q, sv[i]);
-          } else {
-            st_stream(out_col + g0 + q, CI(key));
-            st_stream(out_val + g0 + q, sv[i]);
-          }
-        }
-        __syncthreads();
-      }
-    } else {
-      // scatter entry by entry
-      for (long long e0 = t; e0 < L; e0 += (long long)B * U) {
-        uint32_t k[U];
-        VT v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const long long e = e0 + (long long)u * B;
-          if (e < L) k[u] = key_at(e);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const long long e = e0 + (long long)u * B;
-          if (e < L) v[u] = ld_stream(svp + e);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const long long e = e0 + (long long)u * B;
-          if (e >= L) continue;
-          const uint32_t bk = bucket(k[u]);
-          if (bk == 0xFFFFFFFFu) continue;
-          const uint32_t q = atomicAdd(&hist[bk], 1u);
-          if (q >= uint32_t(L)) continue;
-          if (dbuf == BUF_TEMP) {
-            st_stream(tkey + g0 + q, k[u]);
-            st_stream(tval + g0 + q, v[u]);
-          } else {
-            st_stream(out_col + g0 + q, CI(k[u]));
-            st_stream(out_val + g0 + q, v[u]);
-          }
-        }
-      }
-      __syncthreads();
-    }
   }
 }
 
@@ -1337,44 +1353,49 @@ __global__ void __launch_bounds__(WR_BLOCK, WR_MINB)
 
 // ---- host side --------------------------------------------------------------------------
 struct RowsWs {
-  long long ntiles_cap = 0, nchunks = 0, huge_cap = 0, nxt_cap = 0, lchunk_cap = 0;
+  long long ntiles_cap = 0, nchunks = 0, huge_cap = 0, lchunk_cap = 0, cur_cap = 0;
   long long run_cap[4] = {0, 0, 0, 0};
   long long* tile_first = nullptr;
   long long* chunk_first = nullptr;
-  unsigned* counters = nullptr;  // [0..3] run list counts [4..5] split tickets [7] spare
-                                 // [6] long chunks [10..11] huge list counts [12..13] nxt list counts
+  unsigned* counters = nullptr;  // [0..3] run list counts [4] fine split ticket [5] fine split list
+                                 // [6] long chunks [7] long rows
   FinalEntry* fin = nullptr;
   HugeEntry* huge = nullptr;
-  HugeEntry* nxt = nullptr;
+  HugeEntry* nxt = nullptr;      // oversized buckets (fine split); as many as long rows
   LongChunk* lchunk = nullptr;
+  uint16_t* gmap = nullptr;      // long rows: group of each bucket
+  uint32_t* cursor = nullptr;    // long rows: next free place of each group
   uint32_t* tkey = nullptr;
   void* tval = nullptr;
   long long runs_total() const { return run_cap[0] + run_cap[1] + run_cap[2] + run_cap[3]; }
   RunLists runs() const { return RunLists{fin, counters, run_cap[0], run_cap[1], run_cap[2], run_cap[3]}; }
-  unsigned* lchunk_n() const { return counters + 6; }
-  unsigned* huge_n() const { return counters + 10; }
-  unsigned* nxt_n() const { return counters + 12; }
+  SortLists lists() const {
+    return SortLists{runs(), huge, counters + 7, huge_cap, lchunk, counters + 6, lchunk_cap};
+  }
 };
 
-constexpr int kRowsSlots = 9;
+constexpr int kRowsSlots = 11;
 
-// Workspace layout of run_rows.  sort = false: only what the gather needs.  extra_runs: runs
-// a caller queues itself (beyond the partition's and the split's).
+// Workspace layout of the sort (sort = false: of the gather alone).  extra_runs: runs a
+// caller queues itself (beyond the partition's and the split's).
 inline RowsWs rows_caps(long long nrows, long long nnz, bool sort, long long extra_runs) {
   RowsWs w;
   w.nchunks = sort ? 0 : (nnz + GC_CH - 1) / GC_CH;
   if (!sort) return w;
   w.ntiles_cap = (nnz + SsTile::W * nrows) / SsTile::WIN + 1;
-  // the split's groups (at most three per GROUP_CAP entries of both splits), the rows
-  // sorted alone, the tiles' heavy buckets (more than SS_HEAVY entries each)
-  const long long groups = 2 * (3 * (nnz / GROUP_CAP) + nnz / SS_RUN_MAX + 16);
+  // the split's groups (at most 3 L / GROUP_CAP + 1 of a row, and as many of the fine
+  // split's buckets), the rows sorted alone, the tiles' heavy buckets (more than SS_HEAVY
+  // entries each)
+  const long long groups = nnz > SS_RUN_MAX ? 2 * (3 * (nnz / GROUP_CAP) + nnz / SS_RUN_MAX + 16) : 0;
   w.run_cap[0] = extra_runs > 0 ? groups + extra_runs : 0;
   w.run_cap[1] = groups + nnz / SS_HEAVY + 1;
   w.run_cap[2] = groups + nnz / SS_SMALL_RUN + 1;
   w.run_cap[3] = groups + nnz / SS_MID_RUN + 1;
-  w.huge_cap = nnz / SS_RUN_MAX + 1;
-  w.nxt_cap = nnz / SS_RUN_MAX + 1;
-  w.lchunk_cap = nnz / SL_CH + w.huge_cap;
+  if (nnz > SS_RUN_MAX) {
+    w.huge_cap = nnz / SS_RUN_MAX + 1;
+    w.lchunk_cap = nnz / SL_CH + w.huge_cap;
+    w.cur_cap = nnz / SL_GSLOT + 1;
+  }
   return w;
 }
 
@@ -1387,10 +1408,12 @@ inline void rows_reserve(Carver& cv, long long nrows, long long nnz, size_t vbyt
   off[2] = cv.reserve(16 * 4);
   off[3] = cv.reserve(size_t(w.runs_total()) * sizeof(FinalEntry));
   off[4] = cv.reserve(size_t(w.huge_cap) * sizeof(HugeEntry));
-  off[5] = cv.reserve(size_t(w.nxt_cap) * sizeof(HugeEntry));
+  off[5] = cv.reserve(size_t(w.huge_cap) * sizeof(HugeEntry));
   off[6] = cv.reserve(need_temp ? size_t(nnz) * 4 : 0);
   off[7] = cv.reserve(need_temp ? size_t(nnz) * vbytes : 0);
   off[8] = cv.reserve(size_t(w.lchunk_cap) * sizeof(LongChunk));
+  off[9] = cv.reserve(size_t(w.huge_cap) * SL_NB * 2);
+  off[10] = cv.reserve(size_t(w.cur_cap) * 4);
 }
 
 inline RowsWs rows_bind(const Carver& cv, long long nrows, long long nnz, const size_t* off,
@@ -1405,21 +1428,57 @@ inline RowsWs rows_bind(const Carver& cv, long long nrows, long long nnz, const 
   w.tkey = cv.at<uint32_t>(off[6]);
   w.tval = cv.at<void>(off[7]);
   w.lchunk = cv.at<LongChunk>(off[8]);
+  w.gmap = cv.at<uint16_t>(off[9]);
+  w.cursor = cv.at<uint32_t>(off[10]);
   return w;
 }
 
-// Key-range split of the rows queued in w.huge (counts w.huge_n()) into runs queued in w.fin
-// (defined and instantiated in rowsort.cu for the column and value words of the library).
-template <class CI, class VT>
-sp_status split_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, CI* out_col, VT* out_val);
-// Sorts in place the rows a caller queued itself in w.runs() / w.huge (of nnz entries in
-// all; w.counters zeroed before the caller queued them).
+// Sorts in place the rows a caller queued itself in w.lists() (of nnz entries in all;
+// w.counters zeroed before the caller queued them).  Defined and instantiated in rowsort.cu
+// for the column and value words of the library, as sort_rows_in_place.
 template <class CI, class VT>
 sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz, int key_bits, CI* out_col, VT* out_val);
 // Sorts in place every row of the output arrays (row pointer vp).
 template <class CI, class VT>
 sp_status sort_rows_in_place(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
                              int key_bits, const RowsWs& w, CI* out_col, VT* out_val);
+
+// Cuts the queued long rows (nnz > SS_RUN_MAX) into runs.
+template <class Gs>
+sp_status split_long(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits, const Gs& gs,
+                     typename Gs::CI* out_col, typename Gs::VT* out_val) {
+  using CI = typename Gs::CI;
+  using VT = typename Gs::VT;
+  const int nsm = ctx->num_sms;
+  VT* tval = static_cast<VT*>(w.tval);
+  const SortLists sl = w.lists();
+  auto grid = [&](long long minb, long long cap) { return unsigned(cap < minb * nsm ? cap : minb * nsm); };
+  {
+    ::sp::PhaseScope ph(ctx, s, in_place<Gs>::value ? SP_PHASE_HUGE : SP_PHASE_GATHER);
+    k_long_hist<Gs><<<grid(SL_HMINB, w.lchunk_cap), SL_HB, 0, s>>>(gs, sl, w.tkey, out_col, w.gmap, w.cursor, w.nxt,
+                                                                  w.counters + 5, w.huge_cap, key_bits, ctx->dstatus);
+  }
+  SP_CUDA(cudaGetLastError());
+  constexpr size_t ssm = long_scatter_smem<VT>();
+  SP_CUDA(set_smem(k_long_scatter<Gs>, ssm));
+  {
+    SP_PHASE(SP_PHASE_HUGE);
+    k_long_scatter<Gs><<<grid(sl_sminb<VT>(), w.lchunk_cap), SL_SB, ssm, s>>>(gs, sl, w.tkey, tval, out_col, out_val,
+                                                                       w.gmap, w.cursor, key_bits);
+  }
+  SP_CUDA(cudaGetLastError());
+  if (key_bits <= SL_NBL + SS_RUN_LOG) return SP_OK;  // a bucket spans at most SS_RUN_MAX keys
+  constexpr size_t fsm = split_fine_smem();
+  SP_CUDA(set_smem(k_split_fine<CI, VT>, fsm));
+  {
+    SP_PHASE(SP_PHASE_HUGE);
+    k_split_fine<CI, VT><<<grid(SF_MINB, w.huge_cap), SF_B, fsm, s>>>(w.nxt, w.counters + 5, w.huge_cap, w.counters + 4,
+                                                                     w.tkey, tval, out_col, out_val, w.runs(),
+                                                                     ctx->dstatus);
+  }
+  SP_CUDA(cudaGetLastError());
+  return SP_OK;
+}
 
 // Sorts the queued runs; nnz bounds their length.
 template <class Gs>
@@ -1460,17 +1519,15 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
   const long long ntiles = (nnz + SsTile::W * nrows) / win + 1;
   {
     SP_PHASE(SP_PHASE_PARTITION);
-    const RowsPartition part{nrows, nnz, ntiles, w.tile_first, 0, nullptr, w.runs(), w.huge, w.huge_n(),
-                             w.huge_cap, w.lchunk, w.lchunk_n(), w.lchunk_cap, key_bits,
+    const RowsPartition part{nrows, nnz, ntiles, w.tile_first, 0, nullptr, w.lists(),
                              here ? BUF_OUT : BUF_SRC, win, tmax, ctx->dstatus};
     k_partition<0><<<grid_for(nrows, 256, nsm * 16), 256, 0, s>>>(part, vp);
   }
   SP_CUDA(cudaGetLastError());
-  // The rows longer than SS_RUN_MAX (gathered to their place, cut by key range) and the
-  // tiles (rows of at most tmax) are disjoint.  With the context's overlap on, the long
-  // rows run on the context's side stream, whose higher priority dispatches their CTAs (a
-  // hub row's first) ahead of the tiles', while the tiles run on `s`: the SMs that the
-  // split's tail leaves idle take tiles.  The runs, which the split queues, wait for both.
+  // The rows longer than SS_RUN_MAX (cut by key range) and the tiles (rows of at most tmax)
+  // are disjoint.  With the context's overlap on, the long rows run on the context's side
+  // stream, whose higher priority dispatches their CTAs ahead of the tiles', while the
+  // tiles run on `s`.  The runs, which the split queues, wait for both.
   const bool any_long = nnz > SS_RUN_MAX, fork = any_long && ctx->overlap && ctx->side;
   sp_status lst = SP_OK;
   if (any_long) {
@@ -1479,20 +1536,7 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
       SP_CUDA(cudaEventRecord(ctx->fork_ev, s));
       SP_CUDA(cudaStreamWaitEvent(ls, ctx->fork_ev, 0));
     }
-    if constexpr (!here) {
-      {
-        ::sp::PhaseScope ph(ctx, ls, SP_PHASE_GATHER);
-        const long long cap = (long long)GC_MINB * nsm, g = w.lchunk_cap < cap ? w.lchunk_cap : cap;
-        k_gather_long<Gs><<<unsigned(g), GC_BLOCK, 0, ls>>>(gs, w.huge, w.lchunk, w.lchunk_n(), w.lchunk_cap, out_col,
-                                                            out_val, ctx->dstatus);
-      }
-      const cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) {
-        note_cuda_error(e, __FILE__, __LINE__);
-        lst = SP_ERR_CUDA;
-      }
-    }
-    if (lst == SP_OK) lst = split_queued(ctx, ls, w, out_col, out_val);
+    lst = split_long(ctx, ls, w, key_bits, gs, out_col, out_val);
     if (fork) SP_CUDA(cudaEventRecord(ctx->join_ev, ls));
   }
   auto tiles = [&](auto cfg) -> sp_status {
