@@ -234,7 +234,7 @@ struct SegWordStore {
   long long m, nw, cap;
   long long* nseg;
   DevStatus* dst;
-  __device__ void operator()(long long w, long long j) const {
+  __device__ void operator()(long long w, long long j, long long) const {
     if (w == nw) {  // j = number of segments; the sentinel closes the last one
       if (j > cap) {
         dev_fail(dst, SP_ERR_INTERNAL, -33);
@@ -699,14 +699,13 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
 }
 
 // The rebuilt rows of I (kept entries of both parts, relabelled) into the staging buffer
-// at the rebuilt-row pointer pl->vp, in source order.  `ticket` holds 16 bytes.
+// at the rebuilt-row pointer pl->vp, in source order.  `ticket` holds 16 bytes, cleared.
 template <class RP, class CI, class VT, class IX>
 sp_status assign_stage(sp_ctx* ctx, sp_plan* pl, CI* tcol, VT* tval, unsigned* ticket, cudaStream_t s) {
   const sp_csr& A = pl->A;
   const sp_csr& B = pl->B;
   const long long nI = pl->nI;
   const int nsm = ctx->num_sms;
-  SP_CUDA(cudaMemsetAsync(ticket, 0, 16, s));
   auto fill = [&](const auto& ld) -> sp_status {
     {
       SP_PHASE(SP_PHASE_GATHER);
@@ -768,6 +767,7 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
   const int nsm = ctx->num_sms;
   if (staged) {
     // rebuilt rows: A's surviving entries and B's relabelled ones, staged, then sorted
+    SP_CUDA(cudaMemsetAsync(cv.at<char>(o_tk), 0, 16, s));
     SP_TRY((assign_stage<RP, CI, VT, IX>(ctx, pl, tcol, tval, cv.at<unsigned>(o_tk), s)));
     const RowsWs w1 = rows_bind(cv, nI, nt, r1);
     const int kb = ceil_log2_u64(uint64_t(A.ncols));
@@ -906,13 +906,17 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
   Carver cv;
   const size_t o_tc = cv.reserve(size_t(nt) * sizeof(CI));
   const size_t o_tv = cv.reserve(size_t(nt) * sizeof(VT));
+  // cleared by one memset: tickets, the sort's counters, the scan's status words, the bitmaps
+  const size_t o_zero = cv.total();
   const size_t o_tk = cv.reserve(16);
-  const size_t o_qinv = cv.reserve(q ? size_t(n) * sizeof(IX) : 0);
+  const size_t o_cnt = cv.reserve(16 * 4);
+  const size_t o_scan = cv.reserve(scan_ws_bytes(m));
   const size_t o_qbits = cv.reserve(q ? size_t((n + 31) / 32) * 4 : 0);
   const size_t o_pbits = cv.reserve((p && !sym) ? size_t((m + 31) / 32) * 4 : 0);
+  const size_t zero_bytes = cv.total() - o_zero;
+  const size_t o_qinv = cv.reserve(q ? size_t(n) * sizeof(IX) : 0);
   const size_t o_vp = cv.reserve(out64 ? 0 : size_t(m + 1) * 8);
   const size_t o_ss = cv.reserve(size_t(m) * 8);
-  const size_t o_scan = cv.reserve(scan_ws_bytes(m));
   size_t ro[kRowsSlots];
   rows_reserve(cv, m, nnz_out, sizeof(VT), ro);
   char* base;
@@ -920,24 +924,13 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
   cv.bind(base);
   const int nsm = ctx->num_sms;
   IX* qinv = q ? cv.at<IX>(o_qinv) : nullptr;
-  if (q) {
-    uint32_t* qbits = cv.at<uint32_t>(o_qbits);
-    SP_CUDA(cudaMemsetAsync(qinv, 0xFF, size_t(n) * sizeof(IX), s));
-    SP_CUDA(cudaMemsetAsync(qbits, 0, size_t((n + 31) / 32) * 4, s));
+  SP_CUDA(cudaMemsetAsync(cv.at<char>(o_zero), 0, zero_bytes, s));
+  const IX* pcheck = sym ? nullptr : p;
+  if ((q && n > 0) || (pcheck && m > 0)) {
     {
       SP_PHASE(SP_PHASE_MAP);
-      k_inverse_map_bits<IX><<<grid_for(n, 256, nsm * 8), 256, 0, s>>>(q, n, n, qinv, qbits, ctx->dstatus,
-                                                                        SP_ERR_NOT_PERMUTATION);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  if (p && !sym) {
-    uint32_t* bits = cv.at<uint32_t>(o_pbits);
-    SP_CUDA(cudaMemsetAsync(bits, 0, size_t((m + 31) / 32) * 4, s));
-    {
-      SP_PHASE(SP_PHASE_MAP);
-      k_mark_bits<IX><<<grid_for(m, 256, nsm * 8), 256, 0, s>>>(p, m, m, bits, ctx->dstatus,
-                                                                SP_ERR_NOT_PERMUTATION);
+      k_perm_maps<IX><<<grid_for(n > m ? n : m, 256, nsm * 8), 256, 0, s>>>(
+          q, n, qinv, cv.at<uint32_t>(o_qbits), pcheck, m, cv.at<uint32_t>(o_pbits), ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
   }
@@ -949,16 +942,19 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
   long long* sstart = cv.at<long long>(o_ss);
   const FusedLen<RP, IX> len{p, pl->vp_out, static_cast<const IX*>(pl->rowmap), pl->vp,
                              static_cast<const RP*>(A.rowptr), m, sstart};
+  RowsWs w = rows_bind(cv, m, nnz_out, ro);
+  w.counters = cv.at<unsigned>(o_cnt);
+  const RowsPartition part = sort_partition(ctx, w, m, nnz_out, BUF_SRC);
   if (out64) {
-    SP_TRY(launch_scan(ctx, s, len, StoreDual<long long>{vp, nullptr, ctx->dstatus}, m, cv.at<char>(o_scan)));
+    SP_TRY(launch_scan(ctx, s, len, StorePartition<long long>{vp, nullptr, part, ctx->dstatus}, m, cv.at<char>(o_scan),
+                       SP_PHASE_SCAN, true));
   } else {
-    SP_TRY(launch_scan(ctx, s, len, StoreDual<int32_t>{vp, static_cast<int32_t*>(out->rowptr), ctx->dstatus}, m,
-                       cv.at<char>(o_scan)));
+    SP_TRY(launch_scan(ctx, s, len, StorePartition<int32_t>{vp, static_cast<int32_t*>(out->rowptr), part, ctx->dstatus},
+                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
   }
   if (nnz_out == 0) return SP_OK;
   const FusedGs<CI, VT, IX> g{static_cast<const CI*>(A.colidx), static_cast<const VT*>(A.values), tcol, tval,
                               qinv, sstart, A.nnz, nt, n};
-  const RowsWs w = rows_bind(cv, m, nnz_out, ro);
   const int kb = ceil_log2_u64(uint64_t(n));
   return sort_rows_from(ctx, s, vp, m, nnz_out, kb, w, g, static_cast<CI*>(out->colidx),
                         static_cast<VT*>(out->values));

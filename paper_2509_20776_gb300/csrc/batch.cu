@@ -54,7 +54,7 @@ struct ReqView {
 }  // namespace sp
 
 struct sp_batch {
-  long long nreq = 0, nmats = 0, rows = 0, jtot = 0, nnz = 0, max_nj = 0;
+  long long nreq = 0, nmats = 0, rows = 0, jtot = 0, nnz = 0, max_nj = 0, max_ni = 0;
   sp_itype idx_type = SP_I32, rowptr_type = SP_I64, colidx_type = SP_I32;
   sp_vtype value_type = SP_F32;
   int key_bits = 0;
@@ -98,6 +98,16 @@ __device__ __forceinline__ long long batch_req_of(const long long* __restrict__ 
   return lo;
 }
 
+// Grid of a pass over every request's indices: blockIdx.x strides the requests, blockIdx.y
+// the slices of one, so a large request is spread over many CTAs (one CTA per request: the
+// largest of 3000 requests, 64 K indices, set the time of each pass).
+constexpr int XB_SLICE = 2048;  // indices of a request per CTA and step
+inline dim3 batch_grid(long long nreq, long long longest) {
+  long long y = (longest + XB_SLICE - 1) / XB_SLICE;
+  y = y < 1 ? 1 : y > 64 ? 64 : y;
+  return dim3(unsigned(nreq < 65535 ? nreq : 65535), unsigned(y));
+}
+
 // every request's J into one array (positions as values); range-checked
 template <class IX>
 __global__ void k_batch_gather_j(const BatchReq* __restrict__ reqs, const BatchMat* __restrict__ mats,
@@ -107,7 +117,7 @@ __global__ void k_batch_gather_j(const BatchReq* __restrict__ reqs, const BatchM
     const BatchReq q = reqs[k];
     const long long n = mats[q.mat].ncols;
     const IX* J = static_cast<const IX*>(q.J);
-    for (long long b = threadIdx.x; b < q.nJ; b += blockDim.x) {
+    for (long long b = blockIdx.y * (long long)blockDim.x + threadIdx.x; b < q.nJ; b += (long long)gridDim.y * blockDim.x) {
       const long long c = (long long)J[b];
       if (c < 0 || c >= n) dev_fail(st, SP_ERR_INDEX_RANGE, q.joff + b);
       jkey[q.joff + b] = IX(c < 0 || c >= n ? 0 : c);
@@ -124,7 +134,7 @@ __global__ void k_batch_mark(const BatchReq* __restrict__ reqs, const BatchMat* 
     const BatchReq q = reqs[k];
     const long long n = mats[q.mat].ncols;
     const IX* J = static_cast<const IX*>(q.J);
-    for (long long b = threadIdx.x; b < q.nJ; b += blockDim.x) {
+    for (long long b = blockIdx.y * (long long)blockDim.x + threadIdx.x; b < q.nJ; b += (long long)gridDim.y * blockDim.x) {
       const long long c = (long long)J[b];
       if (c < 0 || c >= n) {
         dev_fail(st, SP_ERR_INDEX_RANGE, q.joff + b);
@@ -144,7 +154,7 @@ __global__ void k_batch_jrank(const BatchReq* __restrict__ reqs, const BatchMat*
     const BatchReq q = reqs[k];
     const long long n = mats[q.mat].ncols;
     const IX* J = static_cast<const IX*>(q.J);
-    for (long long b = threadIdx.x; b < q.nJ; b += blockDim.x) {
+    for (long long b = blockIdx.y * (long long)blockDim.x + threadIdx.x; b < q.nJ; b += (long long)gridDim.y * blockDim.x) {
       const long long c = (long long)J[b];
       if (c < 0 || c >= n) continue;  // reported by k_batch_mark
       const unsigned long long w = meta[q.moff + (c >> 5)];
@@ -165,7 +175,7 @@ __global__ void k_batch_rowinfo(const BatchReq* __restrict__ reqs, const BatchMa
     const BatchMat a = mats[q.mat];
     const IX* I = static_cast<const IX*>(q.I);
     const RP* rp = static_cast<const RP*>(a.rowptr);
-    for (long long t = threadIdx.x; t < q.nI; t += blockDim.x) {
+    for (long long t = blockIdx.y * (long long)blockDim.x + threadIdx.x; t < q.nI; t += (long long)gridDim.y * blockDim.x) {
       const long long r = q.roff + t, src = (long long)I[t];
       long long s = 0, L = 0;
       if (src < 0 || src >= a.nrows) {
@@ -309,7 +319,7 @@ struct StoreCappedRp {
   T* out;
   long long cap;
   DevStatus* st;
-  __device__ void operator()(long long i, long long v) const {
+  __device__ void operator()(long long i, long long v, long long) const {
     if (v > cap) {
       dev_fail(st, SP_ERR_OVERFLOW, i);
       v = cap;
@@ -415,7 +425,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
     if (jtot > 0) {
       {
         SP_PHASE(SP_PHASE_MAP);
-        k_batch_mark<IX><<<unsigned(nreq < 65535 ? nreq : 65535), 256, 0, s>>>(b->reqs, b->mats, nreq, b->jbits,
+        k_batch_mark<IX><<<batch_grid(nreq, b->max_nj), 256, 0, s>>>(b->reqs, b->mats, nreq, b->jbits,
                                                                             ctx->dstatus);
       }
       SP_CUDA(cudaGetLastError());
@@ -425,7 +435,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
     if (jtot > 0) {
       {
         SP_PHASE(SP_PHASE_MAP);
-        k_batch_jrank<IX><<<unsigned(nreq < 65535 ? nreq : 65535), 256, 0, s>>>(b->reqs, b->mats, nreq, b->jmeta,
+        k_batch_jrank<IX><<<batch_grid(nreq, b->max_nj), 256, 0, s>>>(b->reqs, b->mats, nreq, b->jmeta,
                                                                              b->jrp);
       }
       SP_CUDA(cudaGetLastError());
@@ -433,7 +443,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
   } else if (jtot > 0) {
     {
       SP_PHASE(SP_PHASE_MAP);
-      k_batch_gather_j<IX><<<unsigned(nreq < 65535 ? nreq : 65535), 256, 0, s>>>(b->reqs, b->mats, nreq, jkey,
+      k_batch_gather_j<IX><<<batch_grid(nreq, b->max_nj), 256, 0, s>>>(b->reqs, b->mats, nreq, jkey,
                                                                                  b->jpos, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
@@ -457,7 +467,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
     // every output row's source, then the count of k_xcount (lane-per-row, grouped loads)
     {
       SP_PHASE(SP_PHASE_COUNT);
-      k_batch_rowinfo<RP, IX><<<unsigned(nreq < 65535 ? nreq : 65535), 256, 0, s>>>(
+      k_batch_rowinfo<RP, IX><<<batch_grid(nreq, b->max_ni), 256, 0, s>>>(
           b->reqs, b->mats, nreq, b->rs0, b->rsn, b->rreq, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
@@ -620,6 +630,7 @@ extern "C" sp_status sp_extract_batch_count(sp_ctx* ctx, const sp_csr* mats, int
     b->rows += q.nI;
     b->jtot += q.nJ;
     if (q.nJ > b->max_nj) b->max_nj = q.nJ;
+    if (q.nI > b->max_ni) b->max_ni = q.nI;
   }
   b->roff[nreq] = b->rows;
   b->key_bits = ceil_log2_u64(uint64_t(max_cols));

@@ -132,7 +132,7 @@ struct StoreRank {
   const uint32_t* bits;
   unsigned long long* meta;
   long long nw;
-  __device__ void operator()(long long w, long long v) const {
+  __device__ void operator()(long long w, long long v, long long) const {
     if (w < nw) meta[w] = (unsigned long long)bits[w] | ((unsigned long long)v << 32);
   }
 };

@@ -56,6 +56,37 @@ __global__ void k_inverse_map_bits(const IX* __restrict__ idx, long long len, lo
   }
 }
 
+// A permutation's two vectors in one pass: the inverse column map qinv[q[j]] = j with q's
+// bitmap, and p's bitmap (either vector may be null).  The bitmaps (cleared before the
+// launch) find repeats; qinv is not cleared: for a permutation every entry is written, and
+// for any other q the call has failed (an entry left as it was is at most a wrong column,
+// which the sort checks against the matrix like any other).
+template <class IX>
+__global__ void k_perm_maps(const IX* __restrict__ q, long long n, IX* __restrict__ qinv, uint32_t* __restrict__ qbits,
+                            const IX* __restrict__ p, long long m, uint32_t* __restrict__ pbits, DevStatus* st) {
+  const long long len = q && n > (p ? m : 0) ? n : (p ? m : 0);
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
+       k += (long long)gridDim.x * blockDim.x) {
+    auto mark = [&](const IX* x, long long size, uint32_t* bits) -> long long {  // the index, or -1
+      if (!x || k >= size) return -1;
+      const long long v = (long long)x[k];
+      if (v < 0 || v >= size) {
+        dev_fail(st, SP_ERR_INDEX_RANGE, k);
+        return -1;
+      }
+      const uint32_t b = 1u << (v & 31);
+      if (atomicOr(bits + (v >> 5), b) & b) {
+        dev_fail(st, SP_ERR_NOT_PERMUTATION, k);
+        return -1;
+      }
+      return v;
+    };
+    const long long c = mark(q, n, qbits);
+    if (c >= 0) qinv[c] = IX(k);
+    mark(p, m, pbits);
+  }
+}
+
 // membership bitmap (1 bit per index); repeated indices are reported as dup_code, or
 // only flagged in *dup_flag when one is given
 template <class IX>

@@ -12,6 +12,7 @@
 //   two-phase path of the single permutation over the whole batch: partition of the
 //   output rows, load-balanced chunk gather with the relabelling through each row's
 //   request, in-place row sort.
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -28,6 +29,7 @@ struct PermReq {  // a request with its offsets in the batch's rows, map words a
   long long roff;  // first output row
   long long qoff;  // first entry of the request's qinv
   long long boff;  // first word of the request's row bitmap
+  long long qboff; // first word of its column bitmap
 };
 
 // what an output row needs from its request (read through the read-only cache)
@@ -73,42 +75,41 @@ inline sp_status upload(char* dst, const void* src, size_t bytes, cudaStream_t s
   return SP_OK;
 }
 
-// per request: qinv[q[j]] = j (a repeat or an index out of range is not a permutation)
-// and the bitmap of p
+// Grid of a pass over every request's indices: blockIdx.x strides the requests, blockIdx.y
+// the slices of one, so a large request is spread over many CTAs (one CTA per request took
+// 0.34 ms for the maps of 400 requests of up to 64 K rows).
+constexpr int PB_SLICE = 2048;  // indices of a request per CTA and step
+inline dim3 pbatch_grid(long long nreq, long long longest) {
+  long long y = (longest + PB_SLICE - 1) / PB_SLICE;
+  y = y < 1 ? 1 : y > 64 ? 64 : y;
+  return dim3(unsigned(nreq < 65535 ? nreq : 65535), unsigned(y));
+}
+
+// per request: qinv[q[j]] = j and the bitmaps of q and p, which find repeats (an index that
+// repeats or lies out of range: not a permutation)
 template <class IX>
 __global__ void k_pbatch_maps(const PermReq* __restrict__ reqs, long long nreq, IX* __restrict__ qinv,
-                              uint32_t* __restrict__ pbits, DevStatus* st) {
+                              uint32_t* __restrict__ bits, DevStatus* st) {
+  const long long first = blockIdx.y * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.y * blockDim.x;
   for (long long k = blockIdx.x; k < nreq; k += gridDim.x) {
     const PermReq r = reqs[k];
     const IX* q = static_cast<const IX*>(r.q);
     const IX* p = static_cast<const IX*>(r.p);
-    if (q) {
-      for (long long j = threadIdx.x; j < r.ncols; j += blockDim.x) {
-        const long long c = (long long)q[j];
-        if (c < 0 || c >= r.ncols) {
-          dev_fail(st, SP_ERR_NOT_PERMUTATION, j);
-          continue;
-        }
-        IX* slot = qinv + r.qoff + c;
-        if constexpr (sizeof(IX) == 4) {
-          if (atomicCAS(reinterpret_cast<int*>(slot), -1, int(j)) != -1) dev_fail(st, SP_ERR_NOT_PERMUTATION, j);
-        } else {
-          if (atomicCAS(reinterpret_cast<unsigned long long*>(slot), ~0ull, (unsigned long long)j) != ~0ull)
-            dev_fail(st, SP_ERR_NOT_PERMUTATION, j);
-        }
-      }
-    }
-    if (p) {
-      for (long long i = threadIdx.x; i < r.nrows; i += blockDim.x) {
-        const long long v = (long long)p[i];
-        if (v < 0 || v >= r.nrows) {
-          dev_fail(st, SP_ERR_NOT_PERMUTATION, i);
-          continue;
-        }
+    auto mark = [&](long long v, long long size, uint32_t* b, long long at) -> bool {
+      if (v >= 0 && v < size) {
         const uint32_t m = 1u << (v & 31);
-        if (atomicOr(pbits + r.boff + (v >> 5), m) & m) dev_fail(st, SP_ERR_NOT_PERMUTATION, i);
+        if (!(atomicOr(b + (v >> 5), m) & m)) return true;
       }
-    }
+      dev_fail(st, SP_ERR_NOT_PERMUTATION, at);
+      return false;
+    };
+    if (q)
+      for (long long j = first; j < r.ncols; j += step) {
+        const long long c = (long long)q[j];
+        if (mark(c, r.ncols, bits + r.qboff, j)) qinv[r.qoff + c] = IX(j);
+      }
+    if (p && !(p == q && r.nrows == r.ncols))
+      for (long long i = first; i < r.nrows; i += step) mark((long long)p[i], r.nrows, bits + r.boff, i);
   }
 }
 
@@ -121,7 +122,8 @@ __global__ void k_pbatch_rowinfo(const PermReq* __restrict__ reqs, const sp_csr*
     const sp_csr a = mats[r.mat];
     const IX* p = static_cast<const IX*>(r.p);
     const RP* rp = static_cast<const RP*>(a.rowptr);
-    for (long long i = threadIdx.x; i < r.nrows; i += blockDim.x) {
+    for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < r.nrows;
+         i += (long long)gridDim.y * blockDim.x) {
       const long long src = p ? (long long)p[i] : i;
       long long s = 0, L = 0;
       if (src >= 0 && src < r.nrows) {  // else reported by k_pbatch_maps
@@ -179,21 +181,23 @@ struct StoreCapped {
   long long* vp;
   T* out;  // may be null
   long long n, cap;
+  RowsPartition part;
   DevStatus* st;
-  __device__ void operator()(long long i, long long v) const {
+  __device__ void operator()(long long i, long long v, long long vn) const {
     if (v > cap || (i == n && v != cap)) {
       dev_fail(st, SP_ERR_NOT_CANONICAL, i);
       if (v > cap) v = cap;
     }
     vp[i] = v;
     if (out) out[i] = T(v);
+    if (i < n) part(i, v, vn);  // (clamped to nnz there)
   }
 };
 
 }  // namespace sp
 
 struct sp_pbatch {
-  long long nreq = 0, nmats = 0, rows = 0, nnz = 0, qtot = 0, btot = 0, max_cols = 0;
+  long long nreq = 0, nmats = 0, rows = 0, nnz = 0, qtot = 0, btot = 0, max_cols = 0, longest = 0;
   sp_itype idx_type = SP_I32, rowptr_type = SP_I64, colidx_type = SP_I32;
   sp_vtype value_type = SP_F32;
   std::vector<long long> roff;  // host: first output row of every request (+ total)
@@ -204,7 +208,7 @@ struct sp_pbatch {
   size_t buf_bytes = 0;
   cudaStream_t stream = nullptr;
   size_t o_req = 0, o_view = 0, o_mat = 0, o_qinv = 0, o_bits = 0, o_rsrc = 0, o_rsn = 0, o_vp = 0,
-         o_scan = 0;
+         o_scan = 0, o_cnt = 0, zero_bytes = 0;
   size_t ro[sp::kRowsSlots] = {};
 };
 
@@ -223,9 +227,9 @@ sp_status pbatch_fill_impl(sp_ctx* ctx, sp_pbatch* b, sp_csr* out, cudaStream_t 
   long long* rsrc = cv.at<long long>(b->o_rsrc);
   long long* rsn = cv.at<long long>(b->o_rsn);
   long long* vp = cv.at<long long>(b->o_vp);
-  const unsigned gq = unsigned(nreq < 65535 ? nreq : 65535);
-  if (b->qtot > 0) SP_CUDA(cudaMemsetAsync(qinv, 0xFF, size_t(b->qtot) * sizeof(IX), s));
-  if (b->btot > 0) SP_CUDA(cudaMemsetAsync(pbits, 0, size_t(b->btot) * 4, s));
+  const dim3 gq = pbatch_grid(nreq, b->longest);
+  // one memset: the bitmaps, the scan's status words, the sort's counters
+  SP_CUDA(cudaMemsetAsync(pbits, 0, b->zero_bytes, s));
   if (nreq > 0) {
     {
       SP_PHASE(SP_PHASE_MAP);
@@ -238,24 +242,27 @@ sp_status pbatch_fill_impl(sp_ctx* ctx, sp_pbatch* b, sp_csr* out, cudaStream_t 
     }
     SP_CUDA(cudaGetLastError());
   }
+  const bool sort = b->qtot > 0;
+  RowsWs w = rows_bind(cv, rows, nnz, b->ro, sort);
+  w.counters = cv.at<unsigned>(b->o_cnt);
+  const RowsPartition part = sort ? sort_partition(ctx, w, rows, nnz, BUF_SRC) : gather_partition(ctx, w, rows, nnz);
   // row pointer of the batch: scan of the row lengths, mirrored into the output's type
   if (out->rowptr_type == SP_I64) {
     SP_TRY(launch_scan(ctx, s, LoadArray<long long>{rsn},
-                       StoreCapped<long long>{vp, static_cast<long long*>(out->rowptr), rows, nnz, ctx->dstatus},
-                       rows, cv.at<char>(b->o_scan)));
+                       StoreCapped<long long>{vp, static_cast<long long*>(out->rowptr), rows, nnz, part, ctx->dstatus},
+                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true));
   } else {
     SP_TRY(launch_scan(ctx, s, LoadArray<long long>{rsn},
-                       StoreCapped<int32_t>{vp, static_cast<int32_t*>(out->rowptr), rows, nnz, ctx->dstatus},
-                       rows, cv.at<char>(b->o_scan)));
+                       StoreCapped<int32_t>{vp, static_cast<int32_t*>(out->rowptr), rows, nnz, part, ctx->dstatus},
+                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true));
   }
   if (nnz == 0 || rows == 0) return SP_OK;
   CI* oc = static_cast<CI*>(out->colidx);
   VT* ov = static_cast<VT*>(out->values);
   // gather + relabel over the whole batch; with any column map also the row sort
-  const RowsWs w = rows_bind(cv, rows, nnz, b->ro, b->qtot > 0);
   const int kb = ceil_log2_u64(uint64_t(b->max_cols > 1 ? b->max_cols : 1));
   const PermBatchGs<CI, VT, IX> g{views, rsrc};
-  if (b->qtot == 0) return gather_rows(ctx, s, vp, rows, nnz, w, g, oc, ov);
+  if (!sort) return gather_rows(ctx, s, vp, rows, nnz, w, g, oc, ov);
   return sort_rows_from(ctx, s, vp, rows, nnz, kb, w, g, oc, ov);
 }
 
@@ -300,12 +307,20 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
       return SP_ERR_INVALID_ARG;
     }
     const sp_csr& a = mats[q.mat];
-    b->hreq[size_t(k)] = PermReq{q.mat, a.nrows, a.ncols, q.p, q.q, b->rows, q.q ? b->qtot : 0, q.p ? b->btot : 0};
+    b->hreq[size_t(k)] = PermReq{q.mat, a.nrows, a.ncols, q.p, q.q, b->rows, q.q ? b->qtot : 0, 0, 0};
     b->roff[size_t(k)] = b->rows;
     b->rows += a.nrows;
     b->nnz += a.nnz;
     if (q.q) b->qtot += a.ncols;
-    if (q.p) b->btot += (a.nrows + 31) / 32;
+    if (q.p) {
+      b->hreq[size_t(k)].boff = b->btot;
+      b->btot += (a.nrows + 31) / 32;
+    }
+    if (q.q) {
+      b->hreq[size_t(k)].qboff = b->btot;
+      b->btot += (a.ncols + 31) / 32;
+    }
+    b->longest = std::max(b->longest, (long long)std::max(a.nrows, a.ncols));
     if (a.ncols > b->max_cols) b->max_cols = a.ncols;
   }
   b->roff[size_t(nreq)] = b->rows;
@@ -316,10 +331,12 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
   b->o_mat = cv.reserve(size_t(nmats) * sizeof(sp_csr));
   b->o_qinv = cv.reserve(size_t(b->qtot) * is);
   b->o_bits = cv.reserve(size_t(b->btot) * 4);
+  b->o_scan = cv.reserve(scan_ws_bytes(b->rows));
+  b->o_cnt = cv.reserve(16 * 4);
+  b->zero_bytes = cv.total() - b->o_bits;
   b->o_rsrc = cv.reserve(size_t(b->rows) * 8);
   b->o_rsn = cv.reserve(size_t(b->rows) * 8);
   b->o_vp = cv.reserve(size_t(b->rows + 1) * 8);
-  b->o_scan = cv.reserve(scan_ws_bytes(b->rows));
   rows_reserve(cv, b->rows, b->nnz, vs, b->ro, b->qtot > 0);
   cudaStream_t s = (cudaStream_t)stream;
   b->stream = s;

@@ -65,12 +65,17 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   const long long m = A->nrows, n = A->ncols, nnz = A->nnz;
   const bool sym = p && q && (const void*)p == (const void*)q && m == n;
   const bool out64 = B->rowptr_type == SP_I64;
+  const bool sort = q != nullptr && nnz > 0 && m > 0;
   Carver cv;
-  const size_t o_qinv = cv.reserve(q ? size_t(n) * sizeof(IX) : 0);
+  // cleared by one memset: the sort's counters, the scan's status words, the bitmaps
+  const size_t o_zero = cv.total();
+  const size_t o_cnt = cv.reserve(16 * 4);
+  const size_t o_scan = cv.reserve(scan_ws_bytes(m));
   const size_t o_qbits = cv.reserve(q ? size_t((n + 31) / 32) * 4 : 0);
   const size_t o_pbits = cv.reserve((p && !sym) ? size_t((m + 31) / 32) * 4 : 0);
+  const size_t zero_bytes = cv.total() - o_zero;
+  const size_t o_qinv = cv.reserve(q ? size_t(n) * sizeof(IX) : 0);
   const size_t o_vp = cv.reserve(out64 ? 0 : size_t(m + 1) * 8);
-  const size_t o_scan = cv.reserve(scan_ws_bytes(m));
   const size_t o_ss = cv.reserve(size_t(m) * 8);
   size_t ro[kRowsSlots];
   rows_reserve(cv, m, nnz, sizeof(VT), ro, q != nullptr);
@@ -80,38 +85,29 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   IX* qinv = q ? cv.at<IX>(o_qinv) : nullptr;
   long long* vp = out64 ? static_cast<long long*>(B->rowptr) : cv.at<long long>(o_vp);
   const int nsm = ctx->num_sms;
+  SP_CUDA(cudaMemsetAsync(cv.at<char>(o_zero), 0, zero_bytes, s));
   // Identify: inverse column map (validates q), row permutation check (validates p)
-  if (q) {
-    uint32_t* qbits = cv.at<uint32_t>(o_qbits);
-    SP_CUDA(cudaMemsetAsync(qinv, 0xFF, size_t(n) * sizeof(IX), s));
-    SP_CUDA(cudaMemsetAsync(qbits, 0, size_t((n + 31) / 32) * 4, s));
+  const IX* pcheck = sym ? nullptr : p;
+  if ((q && n > 0) || (pcheck && m > 0)) {
     {
       SP_PHASE(SP_PHASE_MAP);
-      k_inverse_map_bits<IX><<<grid_for(n, 256, nsm * 8), 256, 0, s>>>(q, n, n, qinv, qbits, ctx->dstatus,
-                                                                        SP_ERR_NOT_PERMUTATION);
+      k_perm_maps<IX><<<grid_for(n > m ? n : m, 256, nsm * 8), 256, 0, s>>>(
+          q, n, qinv, cv.at<uint32_t>(o_qbits), pcheck, m, cv.at<uint32_t>(o_pbits), ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
   }
-  if (p && !sym) {
-    uint32_t* bits = cv.at<uint32_t>(o_pbits);
-    SP_CUDA(cudaMemsetAsync(bits, 0, size_t((m + 31) / 32) * 4, s));
-    {
-      SP_PHASE(SP_PHASE_MAP);
-      k_mark_bits<IX><<<grid_for(m, 256, nsm * 8), 256, 0, s>>>(p, m, m, bits, ctx->dstatus,
-                                                                SP_ERR_NOT_PERMUTATION);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  // row pointer of B: exclusive scan of the permuted row lengths
+  // row pointer of B: exclusive scan of the permuted row lengths, which partitions the rows
+  RowsWs w = rows_bind(cv, m, nnz, ro, q != nullptr);
+  w.counters = cv.at<unsigned>(o_cnt);
   long long* sstart = cv.at<long long>(o_ss);
   PermLen<RP, IX> len{static_cast<const RP*>(A->rowptr), p, m, nnz, sstart};
+  RowsPartition part = sort ? sort_partition(ctx, w, m, nnz, BUF_SRC) : gather_partition(ctx, w, m, nnz);
   if (out64) {
-    SP_TRY(launch_scan(ctx, s, len, StoreDual<long long>{vp, nullptr, ctx->dstatus}, m,
-                       cv.at<char>(o_scan)));
+    SP_TRY(launch_scan(ctx, s, len, StorePartition<long long>{vp, nullptr, part, ctx->dstatus}, m,
+                       cv.at<char>(o_scan), SP_PHASE_SCAN, true));
   } else {
-    SP_TRY(launch_scan(ctx, s, len,
-                       StoreDual<int32_t>{vp, static_cast<int32_t*>(B->rowptr), ctx->dstatus}, m,
-                       cv.at<char>(o_scan)));
+    SP_TRY(launch_scan(ctx, s, len, StorePartition<int32_t>{vp, static_cast<int32_t*>(B->rowptr), part, ctx->dstatus},
+                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
   }
   if (nnz == 0 || m == 0) return SP_OK;
   CI* out_col = static_cast<CI*>(B->colidx);
@@ -119,8 +115,7 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   // gather and relabel; with a column permutation also sort every row
   const PermGs<CI, VT, IX> g{static_cast<const CI*>(A->colidx), static_cast<const VT*>(A->values), qinv,
                              sstart, n};
-  const RowsWs w = rows_bind(cv, m, nnz, ro, q != nullptr);
-  if (!q) return gather_rows(ctx, s, vp, m, nnz, w, g, out_col, out_val);
+  if (!sort) return gather_rows(ctx, s, vp, m, nnz, w, g, out_col, out_val);
   return sort_rows_from(ctx, s, vp, m, nnz, ceil_log2_u64(uint64_t(n)), w, g, out_col, out_val);
 }
 

@@ -22,6 +22,9 @@ sp_status sort_queued(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nn
 template <class CI, class VT>
 sp_status sort_rows_in_place(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
                              int key_bits, const RowsWs& w, CI* out_col, VT* out_val) {
+  if (nrows == 0 || nnz == 0) return SP_OK;
+  SP_CUDA(cudaMemsetAsync(w.counters, 0, 16 * 4, s));
+  SP_TRY(launch_partition(ctx, s, sort_partition(ctx, w, nrows, nnz, BUF_OUT), vp));
   return sort_rows_from(ctx, s, vp, nrows, nnz, key_bits, w, RowsInPlace<CI, VT>{vp, out_col, out_val}, out_col,
                         out_val);
 }

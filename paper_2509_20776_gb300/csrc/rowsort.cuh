@@ -31,10 +31,11 @@ constexpr int SS_LEVELS = 3;                   // levels a heavy bucket is bucke
 template <int BLOCK_, int ITEMS_, int MINB_, bool TILES_ = false>
 struct SsCfg {
   static constexpr int B = BLOCK_, ITEMS = ITEMS_, CAP = B * ITEMS, MINB = MINB_;
-  static constexpr int TMAX = CAP / 2, WIN = CAP - CAP / 16, W = 4, ROWS = WIN / W;
+  static constexpr int TMAX = CAP / 2, WIN = CAP, W = 4, ROWS = WIN / W;
   static constexpr int RPT = (ROWS + B - 1) / B;  // rows a thread sets up
   static constexpr int WORDS = CAP / 32;   // row-start bitmap words
   static constexpr bool kTiles = TILES_;   // items are tiles (else: single runs)
+  static_assert((CAP & (CAP - 1)) == 0, "a row's window by a shift");
   static_assert(B % 32 == 0 && B * MINB <= 2048, "whole warps, resident CTAs");
   static_assert(CAP <= 4096 && ROWS < 65536 / 2, "packed positions and counts");
 };
@@ -50,6 +51,7 @@ using SsRunS = SsCfg<256, 4, 5>;         // of at most 1024
 constexpr int SS_SMALL_RUN = SsRunS::CAP, SS_MID_RUN = SsRunM::CAP;
 constexpr int SS_TILE_MAX = SsTile::TMAX;  // longest row a tile accepts (the smaller tile shape)
 constexpr int SS_RUN_MAX = 4096;           // longest row sorted alone
+constexpr long long SS_ONE_LAUNCH = 1 << 17;  // sorts of at most this many entries take one launch for all runs
 static_assert(SsRun::CAP == SS_RUN_MAX, "run capacity");
 static_assert(SsTile::W == SsTileL::W && SsTile::WIN <= SsTileL::WIN, "one bound on the number of tiles");
 
@@ -132,7 +134,7 @@ constexpr int GC_H = 4;                        // gather: positions a thread loa
 
 // ---- partition ----------------------------------------------------------------------
 // Row r has the coordinate c(r) = vp[r] + W * r; tile t holds the rows with c(r) in
-// [t * win, (t + 1) * win): a closed form of the row pointer, so no scan of weights is
+// [t * 2^wlog, (t + 1) * 2^wlog): a closed form of the row pointer, so no scan of weights is
 // needed and the number of tiles is known on the host (a window inside a longer row is an
 // empty tile).  Gather chunk k starts at the row holding output position k * GC_CH.
 // The row pointer is clamped to nnz (lengths that do not add up to it were reported), so
@@ -145,7 +147,7 @@ struct RowsPartition {
   long long* chunk_first;   // null: no gather chunks
   SortLists lists;          // rows that fit no tile
   int buf;                  // where the rows' entries are: BUF_SRC or BUF_OUT
-  int win, tmax;            // the tile shape's window and longest row
+  int wlog, tmax;           // the tile shape's window (its logarithm) and longest row
   DevStatus* st;
   // row r at output positions [o0, o1)
   __device__ void operator()(long long r, long long o0, long long o1) const {
@@ -155,23 +157,19 @@ struct RowsPartition {
     if (tile_first) {
       constexpr int W = SsTile::W;
       if (r == 0) tile_first[0] = 0;
-      const long long c0 = o0 + W * r;
-      long long t = c0 / win + 1;
-      const long long c1 = o1 + W * (r + 1);
-      if (c1 >= t * win)
-        for (const long long t_hi = r + 1 == nrows ? ntiles : c1 / win; t <= t_hi && t <= ntiles; ++t)
-          tile_first[t] = r + 1;
-      else if (r + 1 == nrows)
-        for (; t <= ntiles; ++t) tile_first[t] = nrows;
+      // the tiles that start after this row: their first row is r + 1
+      long long t = ((o0 + W * r) >> wlog) + 1, t_hi = (o1 + W * (r + 1)) >> wlog;
+      if (r + 1 == nrows || t_hi > ntiles) t_hi = ntiles;
+      for (; t <= t_hi; ++t) tile_first[t] = r + 1;
       if (L > tmax) queue_row(lists, o0, L, buf, r, st, -15);
     }
     if (chunk_first && L > 0) {
-      long long k_hi = (o1 - 1) / GC_CH;
+      long long k_hi = (unsigned long long)(o1 - 1) / GC_CH;
       if (k_hi > nchunks - 1) k_hi = nchunks - 1;
-      for (long long k = (o0 + GC_CH - 1) / GC_CH; k <= k_hi; ++k) chunk_first[k] = r;
+      for (long long k = (unsigned long long)(o0 + GC_CH - 1) / GC_CH; k <= k_hi; ++k) chunk_first[k] = r;
     }
     if (chunk_first && r + 1 == nrows)  // none, unless the lengths do not add up to nnz
-      for (long long k = (o1 + GC_CH - 1) / GC_CH; k < nchunks; ++k) chunk_first[k] = nrows;
+      for (long long k = (unsigned long long)(o1 + GC_CH - 1) / GC_CH; k < nchunks; ++k) chunk_first[k] = nrows;
   }
 };
 
@@ -181,6 +179,24 @@ __global__ void k_partition(RowsPartition part, const long long* __restrict__ vp
        r += (long long)gridDim.x * blockDim.x)
     part(r, vp[r], vp[r + 1]);
 }
+
+// Scan output of a row pointer (vp, mirrored into a typed array) that partitions its rows
+// on the way.
+template <class T>
+struct StorePartition {
+  long long* vp;
+  T* out;  // may be null
+  RowsPartition part;
+  DevStatus* st;
+  __device__ void operator()(long long i, long long v, long long vn) const {
+    vp[i] = v;
+    if (out) {
+      if (sizeof(T) == 4 && v > 0x7fffffffll) dev_fail(st, SP_ERR_OVERFLOW, i);
+      out[i] = T(v);
+    }
+    if (i < part.nrows) part(i, v, vn);
+  }
+};
 
 // ---- conflict-free block scans over shared arrays ------------------------------------------
 // Each warp owns a contiguous segment of n / (B / 32) entries and walks it 32 entries at a
@@ -935,37 +951,75 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const uint32_t kmax = key_bits >= 32 ? 0xFFFFFFFFu : (1u << key_bits) - 1u;
   const float isr = ss_inv_root(kmax);
-  long long nitems;
+  long long nitems, n1 = 0, n2 = 0;
   if constexpr (Cfg::kTiles) {
     nitems = ntiles;
   } else {
-    nitems = rl.n[slice];
-    if (nitems > rl.cap(slice)) nitems = rl.cap(slice);  // overflow was reported by the producer
+    // (an overflow was reported by the producer)
+    auto count = [&](int k) -> long long { return rl.n[k] < rl.cap(k) ? rl.n[k] : rl.cap(k); };
+    if (slice >= 0) {
+      nitems = count(slice);
+    } else {
+      n1 = count(1);
+      n2 = n1 + count(2);
+      nitems = n2 + count(3);
+    }
   }
+  // run i of the slice (slice < 0: of slices 1, 2 and 3 together)
+  auto run_at = [&](long long i) -> FinalEntry {
+    if (slice >= 0) return rl.slice(slice)[i];
+    return i < n1 ? rl.slice(1)[i] : i < n2 ? rl.slice(2)[i - n1] : rl.slice(3)[i - n2];
+  };
   if (blockIdx.x >= nitems) return;
 
   // the next item's descriptor is loaded one item ahead, so its latency hides behind
   // the current item's sort
-  long long pf0 = 0, pf1 = 0;  // tiles: row range
+  long long pf0 = 0;           // tiles: first row
+  int pfn = 0;                 // and number of rows
   FinalEntry pfe{0, 0, 0, 0};  // runs
-  // tiles: start copying the row pointers of the tile whose range is in (pf0, pf1)
+  // tiles: the ranges of this CTA's next 32 tiles, one per lane, and which hold rows (a
+  // window inside a longer row is empty; on a power-law matrix half of them are, and one
+  // dependent load per empty tile took 1 ms of a scale-25 permutation)
+  long long lf0 = 0;
+  int ln = 0, lbase = 0;  // (ntiles < 2^31: checked by the launch)
+  unsigned lmask = 0;
+  // tiles: the next tile's first row and number of rows in (pf0, pfn), or false
+  auto next_tile = [&]() -> bool {
+    while (lmask == 0) {
+      if (lbase >= nitems) return false;
+      const int i = lbase + lane * int(gridDim.x);
+      ln = 0;
+      if (i >= 0 && i < nitems) {
+        lf0 = tile_first[i];
+        ln = int(tile_first[i + 1] - lf0);
+      }
+      lmask = __ballot_sync(0xffffffffu, ln > 0);
+      lbase = lbase > 0x7fffffff - 32 * int(gridDim.x) ? 0x7fffffff : lbase + 32 * int(gridDim.x);
+    }
+    const int k = __ffs(lmask) - 1;
+    lmask &= lmask - 1;
+    pf0 = __shfl_sync(0xffffffffu, lf0, k);
+    pfn = __shfl_sync(0xffffffffu, ln, k);
+    return true;
+  };
+  // tiles: start copying the row pointers of the tile in (pf0, pfn)
   auto prefetch_rows = [&](bool any) {
     if (any) {
-      int n = int(pf1 - pf0);
-      n = n < ROWS ? n : ROWS;
-      for (int x = t; n > 0 && x <= n; x += B) {  // (an empty tile waits for no copy)
+      const int n = pfn < ROWS ? pfn : ROWS;
+      for (int x = t; x <= n; x += B) {
         cp_async8(pre_o + x, vp + pf0 + x);
         if (x < n) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
       }
     }
     cp_async_commit();
   };
+  bool more_tiles = false;
   if constexpr (Cfg::kTiles) {
-    pf0 = tile_first[blockIdx.x];
-    pf1 = tile_first[blockIdx.x + 1];
-    prefetch_rows(true);
+    lbase = blockIdx.x;
+    more_tiles = next_tile();
+    prefetch_rows(more_tiles);
   } else {
-    pfe = rl.slice(slice)[blockIdx.x];
+    pfe = run_at(blockIdx.x);
     if (t < 2) {
       s_min[t] = 0xFFFFFFFFu;
       s_max[t] = 0u;
@@ -973,7 +1027,7 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
   }
   int par = 0;
   int ra = 0;  // tiles: the round's first row
-  for (long long item = blockIdx.x; item < nitems;) {
+  for (long long item = blockIdx.x; Cfg::kTiles ? more_tiles : item < nitems;) {
     const long long nx = item + gridDim.x;
     long long base;
     int E, nrow = 0, rnext = 0;
@@ -986,19 +1040,10 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       return wpre[w] + __popc(bits[w] & (0xFFFFFFFFu >> (31 - (x & 31)))) - 1u;
     };
     if constexpr (Cfg::kTiles) {
-      nrow = int(pf1 - pf0);
+      nrow = pfn;
       if (nrow > ROWS) {  // cannot happen: see RowsPartition
         if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -17);
         nrow = ROWS;
-      }
-      if (nrow == 0) {  // a window inside a longer row
-        item = nx;
-        if (nx < nitems) {
-          pf0 = tile_first[nx];
-          pf1 = tile_first[nx + 1];
-        }
-        prefetch_rows(nx < nitems);
-        continue;
       }
       cp_async_wait_all();  // this tile's row pointers
       __syncthreads();      // and the previous round's last reads of the tables
@@ -1033,14 +1078,10 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       E = int(tot >> 16);
       rnext = nrow;
       if (E == 0) {  // only longer (or empty) rows: the next tile
-        item = nx;
         ra = 0;
         __syncthreads();  // pre_o has been read
-        if (nx < nitems) {
-          pf0 = tile_first[nx];
-          pf1 = tile_first[nx + 1];
-        }
-        prefetch_rows(nx < nitems);
+        more_tiles = next_tile();
+        prefetch_rows(more_tiles);
         continue;
       }
       if (E > CAP) {  // the rows that fit now, the others in another round
@@ -1076,11 +1117,8 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       }
       __syncthreads();
       if (rnext == nrow) {  // the last round: the next tile's row pointers arrive during this sort
-        if (nx < nitems) {
-          pf0 = tile_first[nx];
-          pf1 = tile_first[nx + 1];
-        }
-        prefetch_rows(nx < nitems);
+        more_tiles = next_tile();
+        prefetch_rows(more_tiles);
       }
       // load: key, value and bucket of every entry
 #pragma unroll
@@ -1110,7 +1148,7 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       }
     } else {
       const FinalEntry fe = pfe;
-      if (nx < nitems) pfe = rl.slice(slice)[nx];
+      if (nx < nitems) pfe = run_at(nx);
       base = fe.off;
       E = fe.len;
       if (fe.len < 0 || fe.len > CAP) {
@@ -1272,12 +1310,7 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       st_stream(ov + g, sval[x]);
     }
     if constexpr (Cfg::kTiles) {
-      if (rnext < nrow) {
-        ra = rnext;
-      } else {
-        ra = 0;
-        item = nx;
-      }
+      ra = rnext < nrow ? rnext : 0;
     } else {
       item = nx;
     }
@@ -1490,40 +1523,61 @@ sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz,
     constexpr size_t sm = ss_smem_bytes<Cfg, VT>();
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_LONG);
-    const long long cap = (long long)Cfg::MINB * ctx->num_sms, g = w.run_cap[slice] < cap ? w.run_cap[slice] : cap;
-    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, nullptr, 0, nullptr, 0, w.runs(), slice, w.tkey,
+    const long long cap = (long long)Cfg::MINB * ctx->num_sms, n = slice >= 0 ? w.run_cap[slice] : w.runs_total();
+    k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, nullptr, 0, w.runs(), slice, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
     return SP_OK;
   };
+  // few runs in all: one launch whose CTAs take any of them (three launches, two of them
+  // empty or short, cost 6 us more than the small runs gain from small CTAs)
+  if (nnz > SS_SMALL_RUN && nnz <= SS_ONE_LAUNCH) return run(SsRun{}, -1);
   SP_TRY(run(SsRunS{}, 1));
   if (nnz > SS_SMALL_RUN) SP_TRY(run(SsRunM{}, 2));
   if (nnz > SS_MID_RUN) SP_TRY(run(SsRun{}, 3));
   return SP_OK;
 }
 
-// The output rows (row pointer vp, nnz entries) from their source `gs`, sorted.
+// The partition of a sort's rows (of nnz entries in all) with the kernel shapes of this call
+// (context options or the tuning table); buf: where the rows' entries are.  It runs as part
+// of the scan that makes the row pointer (StorePartition) or as a pass of its own; w.counters
+// are cleared before.
+inline RowsPartition sort_partition(sp_ctx* ctx, const RowsWs& w, long long nrows, long long nnz, int buf) {
+  const bool large = ctx->cur.tile_shape == 1;
+  const int wlog = large ? ceil_log2_u64(SsTileL::WIN) : ceil_log2_u64(SsTile::WIN);
+  return RowsPartition{nrows, nnz, ((nnz + SsTile::W * nrows) >> wlog) + 1, w.tile_first, 0, nullptr, w.lists(), buf,
+                       wlog, large ? SsTileL::TMAX : SsTile::TMAX, ctx->dstatus};
+}
+inline RowsPartition gather_partition(sp_ctx* ctx, const RowsWs& w, long long nrows, long long nnz) {
+  RowsPartition part{};
+  part.nrows = nrows;
+  part.nnz = nnz;
+  part.nchunks = w.nchunks;
+  part.chunk_first = w.chunk_first;
+  part.st = ctx->dstatus;
+  return part;
+}
+inline sp_status launch_partition(sp_ctx* ctx, cudaStream_t s, const RowsPartition& part, const long long* vp) {
+  {
+    SP_PHASE(SP_PHASE_PARTITION);
+    k_partition<0><<<grid_for(part.nrows, 256, ctx->num_sms * 16), 256, 0, s>>>(part, vp);
+  }
+  SP_CUDA(cudaGetLastError());
+  return SP_OK;
+}
+
+// The output rows (row pointer vp, nnz entries, partitioned by sort_partition) from their
+// source `gs`, sorted.
 template <class Gs>
 sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
                          int key_bits, const RowsWs& w, const Gs& gs, typename Gs::CI* out_col,
                          typename Gs::VT* out_val) {
   using VT = typename Gs::VT;
-  constexpr bool here = in_place<Gs>::value;
   if (nrows == 0 || nnz == 0) return SP_OK;
-  SP_CUDA(cudaMemsetAsync(w.counters, 0, 16 * 4, s));
   const int nsm = ctx->num_sms;
-  // kernel shapes of this call (context options or the tuning table)
   const bool large_tiles = ctx->cur.tile_shape == 1;
-  const int win = large_tiles ? SsTileL::WIN : SsTile::WIN, tmax = large_tiles ? SsTileL::TMAX : SsTile::TMAX;
-  const long long ntiles = (nnz + SsTile::W * nrows) / win + 1;
-  {
-    SP_PHASE(SP_PHASE_PARTITION);
-    const RowsPartition part{nrows, nnz, ntiles, w.tile_first, 0, nullptr, w.lists(),
-                             here ? BUF_OUT : BUF_SRC, win, tmax, ctx->dstatus};
-    k_partition<0><<<grid_for(nrows, 256, nsm * 16), 256, 0, s>>>(part, vp);
-  }
-  SP_CUDA(cudaGetLastError());
+  const long long ntiles = sort_partition(ctx, w, nrows, nnz, BUF_SRC).ntiles;
   // The rows longer than SS_RUN_MAX (cut by key range) and the tiles (rows of at most tmax)
   // are disjoint.  With the context's overlap on, the long rows run on the context's side
   // stream, whose higher priority dispatches their CTAs ahead of the tiles', while the
@@ -1551,31 +1605,22 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
     SP_CUDA(cudaGetLastError());
     return SP_OK;
   };
-  sp_status tst = SP_OK;
-  if (lst == SP_OK) tst = large_tiles ? tiles(SsTileL{}) : tiles(SsTile{});
+  sp_status tst = ntiles > 0x7fffffffll ? SP_ERR_OVERFLOW : SP_OK;
+  if (lst == SP_OK && tst == SP_OK) tst = large_tiles ? tiles(SsTileL{}) : tiles(SsTile{});
   if (fork) SP_CUDA(cudaStreamWaitEvent(s, ctx->join_ev, 0));
   SP_TRY(lst);
   SP_TRY(tst);
   return sort_runs(ctx, s, w, nnz, key_bits, gs, out_col, out_val);
 }
 
-// The output rows gathered from `gs` and relabelled, in source order.
+// The output rows (partitioned by gather_partition) gathered from `gs` and relabelled, in
+// source order.
 template <class Gs>
 sp_status gather_rows(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
                       const RowsWs& w, const Gs& gs, typename Gs::CI* out_col, typename Gs::VT* out_val) {
   if (nrows == 0 || nnz == 0) return SP_OK;
   if (w.nchunks > 0x7fffffffll) return SP_ERR_OVERFLOW;
   const int nsm = ctx->num_sms;
-  {
-    SP_PHASE(SP_PHASE_PARTITION);
-    RowsPartition part{};
-    part.nrows = nrows;
-    part.nnz = nnz;
-    part.nchunks = w.nchunks;
-    part.chunk_first = w.chunk_first;
-    k_partition<0><<<grid_for(nrows, 256, nsm * 16), 256, 0, s>>>(part, vp);
-  }
-  SP_CUDA(cudaGetLastError());
   {
     SP_PHASE(SP_PHASE_GATHER);
     const long long g = w.nchunks < (long long)GC_MINB * nsm ? w.nchunks : (long long)GC_MINB * nsm;  // persistent

@@ -16,6 +16,11 @@ namespace sp {
 constexpr unsigned long long kFlagAgg = 1ull << 62, kFlagInc = 2ull << 62,
                              kValMask = (1ull << 62) - 1;
 constexpr int SCAN_BLOCK = 256, SCAN_ITEMS = 16, SCAN_TILE = SCAN_BLOCK * SCAN_ITEMS;
+// Scans of at most SCAN_SMALL values take tiles of 4 values per thread: more CTAs, and a
+// short chain of loads and stores per thread (a permutation's scan of 4096 rows, which also
+// partitions them: 24 -> 13 us).
+constexpr int SCAN_ITEMS_S = 4;
+constexpr long long SCAN_SMALL = 1 << 17;
 
 struct ScanCtl {
   unsigned long long* status;  // one word per tile, zeroed before the launch
@@ -26,9 +31,9 @@ struct ScanCtl {
   long long n;
 };
 
-template <class Load, class Store>
+template <class Load, class Store, int IT = SCAN_ITEMS>
 __global__ void __launch_bounds__(SCAN_BLOCK, 5) k_scan(Load load, Store store, ScanCtl c) {
-  constexpr int B = SCAN_BLOCK, IT = SCAN_ITEMS, TILE = SCAN_TILE;
+  constexpr int B = SCAN_BLOCK, TILE = SCAN_BLOCK * IT;
   __shared__ long long buf[TILE + TILE / 16];
   __shared__ long long tmp[B / 32 + 1];
   __shared__ unsigned s_tile;
@@ -111,9 +116,10 @@ __global__ void __launch_bounds__(SCAN_BLOCK, 5) k_scan(Load load, Store store, 
   for (int j = 0; j < IT; ++j) {
     const int x = j * B + t;
     const long long i = base + x;
-    if (i < c.n) store(i, buf[x + (x >> 4)]);
+    const int y = x + 1;
+    if (i < c.n) store(i, buf[x + (x >> 4)], y < TILE ? buf[y + (y >> 4)] : s_excl + agg);
   }
-  if (base + TILE >= c.n && t == 0) store(c.n, s_excl + agg);
+  if (base + TILE >= c.n && t == 0) store(c.n, s_excl + agg, s_excl + agg);
 }
 
 // load functors
@@ -122,12 +128,13 @@ struct LoadArray {
   const T* a;
   __device__ long long operator()(long long i) const { return (long long)a[i]; }
 };
-// stores: the int64 row pointer, optionally mirrored into a typed output array
+// stores: (i, v, vn) with v the exclusive prefix of element i and vn that of i + 1 (i = n:
+// the total, twice).  The int64 row pointer, optionally mirrored into a typed output array
 template <class T>
 struct StoreTyped {
   T* out;
   DevStatus* st;
-  __device__ void operator()(long long i, long long v) const {
+  __device__ void operator()(long long i, long long v, long long) const {
     if (sizeof(T) == 4 && v > 0x7fffffffll) dev_fail(st, SP_ERR_OVERFLOW, i);
     out[i] = T(v);
   }
@@ -137,7 +144,7 @@ struct StoreDual {
   long long* vp;
   T* out;  // may be null
   DevStatus* st;
-  __device__ void operator()(long long i, long long v) const {
+  __device__ void operator()(long long i, long long v, long long) const {
     vp[i] = v;
     if (out) {
       if (sizeof(T) == 4 && v > 0x7fffffffll) dev_fail(st, SP_ERR_OVERFLOW, i);
@@ -146,17 +153,22 @@ struct StoreDual {
   }
 };
 
+inline long long scan_tiles(long long n) {
+  const long long tile = n <= SCAN_SMALL ? SCAN_BLOCK * SCAN_ITEMS_S : SCAN_TILE;
+  return n > 0 ? (n + tile - 1) / tile : 1;
+}
+// workspace of a scan of at most n values
 inline size_t scan_ws_bytes(long long n) {
-  long long tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+  const long long s = scan_tiles(n < SCAN_SMALL ? n : SCAN_SMALL), l = scan_tiles(n), tiles = s > l ? s : l;
   return align_up(size_t(tiles + 1) * 8) + kAlign;
 }
 
-// Exclusive scan of n values into n+1 outputs; `ws` must hold scan_ws_bytes(n).
+// Exclusive scan of n values into n+1 outputs; `ws` must hold scan_ws_bytes(n) (`zeroed`: it
+// is cleared already).
 template <class Load, class Store>
 sp_status launch_scan(sp_ctx* ctx, cudaStream_t s, Load load, Store store, long long n, char* ws,
-                      int phase = SP_PHASE_SCAN) {
-  long long tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  if (tiles == 0) tiles = 1;
+                      int phase = SP_PHASE_SCAN, bool zeroed = false) {
+  const long long tiles = scan_tiles(n);
   ScanCtl c;
   c.status = reinterpret_cast<unsigned long long*>(ws);
   c.ticket = reinterpret_cast<unsigned*>(ws + align_up(size_t(tiles + 1) * 8));
@@ -164,11 +176,12 @@ sp_status launch_scan(sp_ctx* ctx, cudaStream_t s, Load load, Store store, long 
   c.spin_limit = ctx->spin_limit;
   c.hold_tile = ctx->hold_tile;
   c.n = n;
-  SP_CUDA(cudaMemsetAsync(ws, 0, scan_ws_bytes(n), s));
+  if (!zeroed) SP_CUDA(cudaMemsetAsync(ws, 0, scan_ws_bytes(n), s));
   if (tiles > 0x7fffffffll) return SP_ERR_OVERFLOW;
   {
     SP_PHASE(phase);
-    k_scan<Load, Store><<<unsigned(tiles), SCAN_BLOCK, 0, s>>>(load, store, c);
+    if (n <= SCAN_SMALL) k_scan<Load, Store, SCAN_ITEMS_S><<<unsigned(tiles), SCAN_BLOCK, 0, s>>>(load, store, c);
+    else k_scan<Load, Store><<<unsigned(tiles), SCAN_BLOCK, 0, s>>>(load, store, c);
   }
   SP_CUDA(cudaGetLastError());
   return SP_OK;
@@ -177,7 +190,9 @@ sp_status launch_scan(sp_ctx* ctx, cudaStream_t s, Load load, Store store, long 
 template <class K>
 inline cudaError_t set_smem(K kernel, size_t bytes) {
   // set before every launch that needs it: a flag kept in an inline template is shared by
-  // every translation unit of the library, but each one launches its own copy of a kernel
+  // every translation unit of the library, but each one launches its own copy of a kernel.
+  // Up to 40 KB beside the kernel's static arrays need no attribute.
+  if (bytes <= 40 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
 }
 
