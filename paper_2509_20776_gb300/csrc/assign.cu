@@ -657,11 +657,11 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
       const CI* colA = static_cast<const CI*>(A.colidx);
       {
         SP_PHASE(SP_PHASE_COUNT);
-        const XOne<CI, uint32_t, AssignKeep> src{colA, nullptr, keep};
+        const XOne<CI, uint32_t, AssignKeep> src{colA, nullptr, keep, A.nnz};
         const XResolveI<RP, IX> res{static_cast<const RP*>(A.rowptr), I, m, A.nnz, pl->sstart, pl->slen,
                                     ctx->dstatus};
         k_xcount<<<grid_for((nI + 31) / 32 * 32, XB, nsm * 8), XB, 0, s>>>(
-            src, res, nI, pl->vp, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->counters + 4, ctx->dstatus);
+            src, res, nI, pl->vp, nullptr, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->counters + 4, ctx->dstatus);
       }
       SP_CUDA(cudaGetLastError());
       {

@@ -48,6 +48,7 @@ struct ReqView {
   const void* val;
   const unsigned long long* meta;  // the request's slice of the batch's rank words
   long long ncol;
+  long long nnz;
 };
 
 
@@ -75,6 +76,7 @@ struct sp_batch {
   long long* rs0 = nullptr;     // rank map: source start, length and request of every output row
   long long* rsn = nullptr;
   int* rreq = nullptr;
+  uint32_t* kmask = nullptr;    // kept entries of a row of at most 32 source entries
   sp::ReqView* rv = nullptr;    // rank map: every request's arrays and slice
   std::vector<sp::ReqView> hviews;  // host copy (kept: the copy to rv is asynchronous)
   long long n_slow = 0;         // rank map: output rows of more than XFAST source entries
@@ -208,6 +210,7 @@ struct XBatchSrc {
   const int* rreq;
   const ReqView* rv;
   const uint32_t* jrp;
+  __device__ __forceinline__ long long nnz(const H& h) const { return __ldg(&rv[h.k].nnz); }
   __device__ __forceinline__ H handle(long long r) const { return H{rreq[r]}; }
   __device__ static __forceinline__ H shfl(const H& h, int k) { return H{__shfl_sync(kFull, h.k, k)}; }
   __device__ __forceinline__ const CI* cols(const H& h) const { return static_cast<const CI*>(rv[h.k].col); }
@@ -353,6 +356,7 @@ sp_status batch_count_impl(sp_ctx* ctx, sp_batch* b, const std::vector<BatchMat>
   const size_t o_rs = cv.reserve(rank ? size_t(rows) * 8 : 0);
   const size_t o_rn = cv.reserve(rank ? size_t(rows) * 8 : 0);
   const size_t o_rq = cv.reserve(rank ? size_t(rows) * 4 : 0);
+  const size_t o_km = cv.reserve(rank ? size_t(rows) * 4 : 0);
   const size_t o_rv = cv.reserve(rank ? size_t(nreq) * sizeof(ReqView) : 0);
   const size_t o_ct = cv.reserve(64);
   b->buf = static_cast<char*>(ctx_alloc(ctx, cv.total(), s));
@@ -372,12 +376,13 @@ sp_status batch_count_impl(sp_ctx* ctx, sp_batch* b, const std::vector<BatchMat>
   b->rs0 = rank ? cv.at<long long>(o_rs) : nullptr;
   b->rsn = rank ? cv.at<long long>(o_rn) : nullptr;
   b->rreq = rank ? cv.at<int>(o_rq) : nullptr;
+  b->kmask = rank ? cv.at<uint32_t>(o_km) : nullptr;
   b->rv = rank ? cv.at<ReqView>(o_rv) : nullptr;
   if (rank && nreq > 0) {
     b->hviews.resize(size_t(nreq));
     for (long long k = 0; k < nreq; ++k) {
       const BatchMat& a = hm[size_t(hr[size_t(k)].mat)];
-      b->hviews[size_t(k)] = ReqView{a.colidx, a.values, b->jmeta + hr[size_t(k)].moff, a.ncols};
+      b->hviews[size_t(k)] = ReqView{a.colidx, a.values, b->jmeta + hr[size_t(k)].moff, a.ncols, a.nnz};
     }
     SP_CUDA(cudaMemcpyAsync(b->rv, b->hviews.data(), size_t(nreq) * sizeof(ReqView), cudaMemcpyHostToDevice, s));
   }
@@ -475,7 +480,7 @@ sp_status batch_device_count(sp_ctx* ctx, sp_batch* b, cudaStream_t s, sp_csr* o
       SP_PHASE(SP_PHASE_COUNT);
       const XBatchSrc<CI, uint32_t> src{b->rreq, b->rv, b->jrp};
       k_xcount<<<grid_for((rows + 31) / 32 * 32, XB, nsm * 8), XB, 0, s>>>(
-          src, XResolveRecorded{b->rs0, b->rsn}, rows, b->vp, nullptr, counters, 0, counters + 1, ctx->dstatus);
+          src, XResolveRecorded{b->rs0, b->rsn}, rows, b->vp, b->kmask, nullptr, counters, 0, counters + 1, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
   } else if (rows > 0) {
@@ -527,7 +532,7 @@ sp_status batch_fill_body(sp_ctx* ctx, sp_batch* b, sp_csr* out, cudaStream_t s,
       SP_PHASE(SP_PHASE_GATHER);
       const XBatchSrc<CI, VT> src{b->rreq, b->rv, b->jrp};
       k_xfill<XBatchSrc<CI, VT>, false><<<grid_for((rows + 31) / 32 * 32, XB, ctx->num_sms * 8), XB, 0, s>>>(
-          src, rows, b->rs0, b->rsn, b->vp, oc, ov, w.lists(),
+          src, rows, b->rs0, b->rsn, b->kmask, b->vp, oc, ov, w.lists(),
           b->max_nj <= 0xFFFFFFFFll ? XF_LANE : 0, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());

@@ -193,11 +193,13 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   const size_t o_scan = cv.reserve(scan_ws_bytes(nI > nw32 ? nI : nw32));
   const size_t o_ss = cv.reserve(size_t(nI) * 8);
   const size_t o_sn = cv.reserve(size_t(nI) * 8);
+  const size_t o_km = cv.reserve(size_t(nI) * 4);
   const size_t o_fl = cv.reserve(16);  // J strictly ascending / consecutive / repeats
   SP_TRY(plan_alloc(ctx, pl, cv.total(), s));
   cv.bind(pl->buf);
   pl->sstart = cv.at<long long>(o_ss);
   pl->slen = cv.at<long long>(o_sn);
+  pl->kmask = cv.at<uint32_t>(o_km);
   pl->jmeta = cv.at<unsigned long long>(o_meta);
   pl->jrpos = cv.at<void>(o_jrp);
   pl->jsk = cv.at<uint32_t>(o_jsk);
@@ -341,9 +343,9 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
       using Test = decltype(test);
       {
         SP_PHASE(SP_PHASE_COUNT);
-        const XOne<CI, uint32_t, Test> src{ci, nullptr, test};
+        const XOne<CI, uint32_t, Test> src{ci, nullptr, test, nnz};
         const XResolveI<RP, IX> res{rp, I, m, nnz, pl->sstart, pl->slen, ctx->dstatus};
-        k_xcount<<<g, XB, 0, s>>>(src, res, nI, pl->vp, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->counters + 4,
+        k_xcount<<<g, XB, 0, s>>>(src, res, nI, pl->vp, pl->kmask, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->counters + 4,
                                   ctx->dstatus);
       }
       SP_CUDA(cudaGetLastError());
@@ -429,12 +431,12 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     using Rel = decltype(rel);
     {
       SP_PHASE(SP_PHASE_GATHER);
-      const XOne<CI, VT, Rel> src{ci, vv, rel};
+      const XOne<CI, VT, Rel> src{ci, vv, rel, A.nnz};
       if (sorted)
-        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov,
+        k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->kmask, pl->vp, oc, ov,
                                                           w.lists(), lane_rows, ctx->dstatus);
       else
-        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->vp, oc, ov,
+        k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->kmask, pl->vp, oc, ov,
                                                            w.lists(), lane_rows, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());

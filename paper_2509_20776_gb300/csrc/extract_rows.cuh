@@ -13,18 +13,18 @@
 //   Count (k_xcount).  A warp takes 32 selected rows ("a block"): lane l resolves row
 //     i0 + l (I[i], range check, the row-pointer pair), so 32 index chains are in flight,
 //     and records the row's source start and length for the fill.  A row of at most
-//     XC_LANE entries is then counted by its own lane (all its columns loaded at once,
-//     every lane's row in flight together); the warp takes the longer rows XC_ROWS at a
-//     time (two columns per lane), tests each column against J's bitmap and counts the
-//     members (ballot + popc).
-//   Fill (k_xfill).  A warp again takes 32 rows.  A row of at most XF_LANE source
-//     entries is filled by its own lane: its columns and values loaded at once, the kept
-//     ones relabelled and sorted by a network in registers, written once.  For longer
-//     rows the warp loads XF_ROWS rows at once, relabels the kept entries (rank word +
-//     position), compacts them (ballot slots) into a per-warp shared buffer and ranks
-//     each among its row's new columns, so a row of at most XFAST source entries is
-//     written once, sorted, at its final place.  Longer rows are written in source order
-//     and queued for the row sort.
+//     xc_lane entries is then counted by its own lane (all its columns loaded at once as
+//     16-byte words, every lane's row in flight together); the warp takes the longer rows
+//     several at a time, tests each column against J's bitmap and counts the members
+//     (ballot + popc).  A row of at most 32 entries leaves the mask of its kept entries.
+//   Fill (k_xfill).  A warp again takes 32 rows.  A row of at most XF_LANE source entries is
+//     filled by its own lane: its columns loaded as 16-byte words, the kept ones relabelled
+//     and sorted by a network in registers with the index of their value.  For longer rows
+//     of at most 32 the warp loads several rows at once, only the entries of the mask (no
+//     second membership test), and ranks each new column among the row's, so the row is
+//     written once, sorted, at its final place; rows of at most XFAST entries the same way
+//     with two entries per lane and the test.  Longer rows are written in source order and
+//     queued for the row sort.
 //   Random lookups, not HBM bytes, bound both passes: one 4-byte lookup per SM cycle
 //   while its table is L2-resident (~300 G/s on GB300), fewer for tables above ~100 MB.
 #pragma once
@@ -38,13 +38,22 @@ namespace sp {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int XFAST = 64;     // rows of at most this many source entries: masks, warp sort
-constexpr int XC_ROWS = 6;    // rows whose columns a counting warp loads together
+constexpr int XC_ROWS1 = 8;   // rows of at most 32 entries whose columns a counting warp loads together
+constexpr int XC_ROWS = 4;    // the same for longer ones
 template <class CI>
 constexpr int xc_lane() { return sizeof(CI) == 4 ? 16 : 8; }  // rows a lane counts alone
-constexpr int XF_ROWS = 2;    // rows whose kept entries a filling warp loads together
-constexpr int XF_LANE = 8;    // rows of at most this many source entries: filled by their own lane
+// Rows of at most 32 entries whose kept entries a filling warp loads together.  Measured at 4
+// CTAs per SM (Erdos-Renyi 2^25 x 32, half of rows and columns / 3000 batched requests):
+// 3 rows 4.77 / 2.42 ms per fill, 4 rows 4.68 / 2.64, 2 rows 5.43 / 2.38; 5 CTAs with 4 or 2
+// rows 5.33 and 5.78, 3 CTAs 6.24 (the start's fill, which tested every entry: 5.65 / 2.75).
+template <class VT>
+constexpr int xf_rows1() { return sizeof(VT) == 4 ? 3 : 2; }
+constexpr int XF_MINB = 4;
+constexpr int XF_ROWS = 2;    // the same for longer ones
+constexpr int XF_LANE = 8;    // rows of at most this many source entries: filled by their own lane (a 5-point
+                              // mesh of 24 M rows, fp64: fill 0.80 -> 0.23 ms, count 0.34 -> 0.17 with whole-word loads)
 
-// Sorting network on XF_LANE (key, value) pairs held in registers: 19 comparators in 6
+// Sorting network on XF_LANE (key, payload) pairs held in registers: 19 comparators in 6
 // layers (a test checks the table on all 256 0/1 inputs, which by the 0-1 principle
 // proves it sorts every input).
 template <class VT>
@@ -61,6 +70,37 @@ __device__ __forceinline__ void sort8(uint32_t (&k)[8], VT (&v)[8]) {
     k[b] = sw ? ka : kb;
     v[a] = sw ? vb : va;
     v[b] = sw ? va : vb;
+  }
+}
+
+// The N entries of a lane's own row, p[0, L) with 0 < L <= N, in registers: whole 16-byte
+// words where they lie inside the array (`inside`: the row is at least three entries from
+// both of its ends), else one by one.  A lane reads its row alone, so 4-byte loads would
+// fetch a row's sector once per entry: the block's 32 rows do not stay in L1 between them
+// (hit rate 13 %).  Entries at L and beyond are unspecified.
+template <int N, class CI>
+__device__ __forceinline__ void load_row(const CI* p, int L, bool inside, CI (&c)[N]) {
+  constexpr int PER = 16 / int(sizeof(CI)), NV = (N + PER - 1 + PER - 1) / PER;
+  if (inside) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    const int k = int((a & 15) / sizeof(CI));
+    const uint4* w = reinterpret_cast<const uint4*>(a & ~uintptr_t(15));
+    CI t[NV * PER];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const uint4 x = v * PER < k + L ? __ldcs(w + v) : make_uint4(0, 0, 0, 0);
+      memcpy(&t[v * PER], &x, 16);
+    }
+    // shift down by k entries
+    if constexpr (PER == 4) {
+#pragma unroll
+      for (int i = 0; i + 2 < NV * PER; ++i) t[i] = (k & 2) ? t[i + 2] : t[i];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) c[i] = (k & 1) && i + 1 < NV * PER ? t[i + 1] : t[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) c[i] = i < L ? ld_stream(p + i) : CI(0);
   }
 }
 constexpr int XB = 256;       // threads per CTA of the count / fill
@@ -169,6 +209,7 @@ __global__ void k_jsorted_init(const IX* __restrict__ J, long long nJ, uint32_t*
 //   static H shfl(const H& h, int lane);     another lane's handle
 //   const CI* cols(const H&); const VT* vals(const H&);
 //   bool test(const H&, long long c);  bool map(const H&, long long c, uint32_t& key);
+//   long long nnz(const H&);                 entries of the row's matrix
 //   kLongCta: rows of more than SRC_LONG entries go to the CTA-per-row kernels
 // One matrix and one identify for every row:
 template <class CIt, class VTt, class Rel>
@@ -180,6 +221,8 @@ struct XOne {
   const CI* col;
   const VT* val;
   Rel rel;
+  long long nnzA;
+  __device__ __forceinline__ long long nnz(const H&) const { return nnzA; }
   __device__ __forceinline__ H handle(long long) const { return H{}; }
   __device__ static __forceinline__ H shfl(const H& h, int) { return h; }
   __device__ __forceinline__ const CI* cols(const H&) const { return col; }
@@ -225,14 +268,15 @@ struct XResolveRecorded {
 // ---- count ---------------------------------------------------------------------------
 // cnt[i] = kept entries of listed row i (with Src::kLongCta, rows of more than SRC_LONG
 // source entries are listed for k_count_long instead); *n_slow += rows of more than XFAST
-// source entries (the fill queues their sort).
+// source entries (the fill queues their sort); kmask (may be null): the kept entries of a
+// row of at most 32, one bit each.
 template <class Src, class Res>
 __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI, long long* __restrict__ cnt,
-                                                 long long* __restrict__ cl_rows, unsigned* n_cl, long long cl_cap,
-                                                 unsigned* n_slow, DevStatus* st) {
+                                                 uint32_t* __restrict__ kmask, long long* __restrict__ cl_rows,
+                                                 unsigned* n_cl, long long cl_cap, unsigned* n_slow, DevStatus* st) {
   using CI = typename Src::CI;
   using H = typename Src::H;
-  constexpr int R = XC_ROWS, XL = xc_lane<CI>();
+  constexpr int R1 = XC_ROWS1, R = XC_ROWS, XL = xc_lane<CI>();
   constexpr long long kLong = Src::kLongCta ? SRC_LONG : (1ll << 62);
   __shared__ unsigned char s_lane[XB / 32][32];  // the lanes of the warp's longer rows, in order
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -253,21 +297,50 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
     if (lane == 0 && slow) atomicAdd(n_slow, unsigned(__popc(slow)));
     if (L > kLong) push_row(cl_rows, n_cl, cl_cap, i, st);
     long long mine = 0;
+    uint32_t mask = 0;
     // short rows: the lane's own row, all its columns in flight at once
-    if (L <= XL) {
-      const CI* cp = src.cols(h);
+    if (L > 0 && L <= XL) {
       CI cc[XL];
+      load_row<XL>(src.cols(h) + s, int(L), s >= 3 && s + L + 3 <= src.nnz(h), cc);
 #pragma unroll
-      for (int e = 0; e < XL; ++e) cc[e] = e < L ? ld_stream(cp + s + e) : CI(0);
-#pragma unroll
-      for (int e = 0; e < XL; ++e) mine += (e < L && src.test(h, (long long)cc[e])) ? 1 : 0;
+      for (int e = 0; e < XL; ++e) mask |= (e < L && src.test(h, (long long)cc[e])) ? 1u << e : 0u;
+      mine = __popc(mask);
     }
-    // longer rows (up to kLong): the warp, XC_ROWS rows at a time
-    const unsigned lm = __ballot_sync(kFull, L > XL && L <= kLong);
-    if ((lm >> lane) & 1u) s_lane[wid][__popc(lm & lt)] = (unsigned char)lane;
+    // rows of at most 32 entries: the warp, one entry per lane, XC_ROWS1 rows at a time; then
+    // the longer ones (up to kLong), XC_ROWS at a time
+    const unsigned m1 = __ballot_sync(kFull, L > XL && L <= 32), m2 = __ballot_sync(kFull, L > 32 && L <= kLong);
+    const int nr1 = __popc(m1), nr = nr1 + __popc(m2);
+    if ((m1 >> lane) & 1u) s_lane[wid][__popc(m1 & lt)] = (unsigned char)lane;
+    if ((m2 >> lane) & 1u) s_lane[wid][nr1 + __popc(m2 & lt)] = (unsigned char)lane;
     __syncwarp();
-    const int nr = __popc(lm);
-    for (int g = 0; g < nr; g += R) {
+    for (int g = 0; g < nr1; g += R1) {
+      int LL[R1], ln[R1];
+      CI c0[R1];
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        ln[u] = g + u < nr1 ? int(s_lane[wid][g + u]) : 0;
+        const long long ss = __shfl_sync(kFull, s, ln[u]);
+        const int l = __shfl_sync(kFull, int(L), ln[u]);
+        LL[u] = g + u < nr1 ? l : 0;
+        const CI* cp = src.cols(Src::shfl(h, ln[u]));  // (shuffles: outside the condition)
+        c0[u] = lane < LL[u] ? ld_stream(cp + ss + lane) : CI(0);
+      }
+      bool k0[R1];
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        const H hu = Src::shfl(h, ln[u]);
+        k0[u] = lane < LL[u] && src.test(hu, (long long)c0[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        const unsigned m = __ballot_sync(kFull, k0[u]);
+        if (g + u < nr1 && lane == ln[u]) {
+          mask = m;
+          mine = __popc(m);
+        }
+      }
+    }
+    for (int g = nr1; g < nr; g += R) {
       long long ss[R];
       int LL[R];  // the row's length, capped (the loop over a longer row re-reads it)
       int ln[R];  // its lane
@@ -326,6 +399,7 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
     }
     __syncwarp();  // s_lane is rewritten by the next block of rows
     if (i < nI && L <= kLong) cnt[i] = mine;
+    if (kmask && i < nI) kmask[i] = mask;
   }
 }
 
@@ -344,22 +418,23 @@ __device__ __forceinline__ void x_put(CI* out_col, VT* out_val, long long pos, l
 // kSorted: the relabelling keeps the source order (ascending J), so slots are ranks and
 // no row is queued.
 template <class Src, bool kSorted>
-__global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const long long* __restrict__ rs0,
-                                                const long long* __restrict__ rsn, const long long* __restrict__ vp,
+__global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, const long long* __restrict__ rs0,
+                                                const long long* __restrict__ rsn, const uint32_t* __restrict__ kmask,
+                                                const long long* __restrict__ vp,
                                                 typename Src::CI* __restrict__ out_col,
                                                 typename Src::VT* __restrict__ out_val, SortLists sl, int lane_rows,
                                                 DevStatus* st) {
-  // lane_rows: XF_LANE when every key is below kDropped (the lane path pads with it), else
-  // 0; the lane path is compiled for 4-byte columns and values (its registers)
+  // lane_rows: XF_LANE when every key is below kDropped (the lane path pads with it), else 0
   using CI = typename Src::CI;
   using VT = typename Src::VT;
   using H = typename Src::H;
-  constexpr bool kLane = sizeof(CI) == 4 && sizeof(VT) == 4;
-  constexpr int R = XF_ROWS, NWB = XB / 32, KW = XFAST + 4;
+  constexpr int R1 = xf_rows1<VT>(), R = XF_ROWS, NWB = XB / 32, KW = XFAST + 4;
   constexpr long long kLong = Src::kLongCta ? SRC_LONG : (1ll << 62);
-  __shared__ __align__(16) uint32_t s_key[NWB][KW];  // a row's kept keys (+ padding for 4-wide loads)
+  // the kept keys of the warp's rows in flight (+ padding for 4-wide loads)
+  __shared__ __align__(16) uint32_t s_key[NWB][R1 * 36];
+  static_assert(R1 * 36 >= KW, "the two-entry path's buffer");
   __shared__ VT s_val[NWB][XFAST];
-  __shared__ unsigned char s_lane[NWB][32];  // the lanes of the warp's rows for the warp path, in order
+  __shared__ unsigned char s_lane[NWB][32];  // the lanes of the warp's rows for the warp paths, in order
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   uint32_t* wk = s_key[wid];
@@ -368,53 +443,110 @@ __global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const lo
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long i0 = w0 * 32; i0 < nI; i0 += nw * 32) {
     const long long i = i0 + lane;
-    long long s = 0, L = 0, o = 0, oe = 0;
+    long long s = 0, L = 0, o = 0;
+    uint32_t mask = 0;  // of a row of at most 32 entries
+    int nkeep = 0;
     H h{};
     if (i < nI) {
       s = rs0[i];
       L = rsn[i];
+      mask = kmask[i];
       o = vp[i];
-      oe = vp[i + 1];
+      const long long k = vp[i + 1] - o;
+      nkeep = k < (1 << 30) ? int(k) : (1 << 30);  // (only rows of at most XFAST entries use it)
       h = src.handle(i);
+      // a row the warp paths do not sort
+      if (!kSorted && L > XFAST && k > 1) queue_row(sl, o, k, BUF_OUT, i, st, -27);
+      if (L <= 32 && nkeep != __popc(mask)) {  // the count disagrees with the fill (a library bug)
+        dev_fail(st, SP_ERR_INTERNAL, -29);
+        mask = 0;
+      }
     }
-    // a row the warp path does not sort
-    if (!kSorted && L > XFAST && oe - o > 1) queue_row(sl, o, oe - o, BUF_OUT, i, st, -27);
     // rows of at most lane_rows entries: the lane's own row, all its loads and relabels in
     // flight together, the kept entries sorted in registers and written once
-    const bool by_lane = L <= (kLane ? lane_rows : 0);
-    if constexpr (kLane) if (by_lane && L > 0) {
-      const CI* cp = src.cols(h);
-      const VT* vq = src.vals(h);
+    const bool by_lane = L <= lane_rows;
+    if (by_lane && mask) {
       CI cc[XF_LANE];
-      VT vv[XF_LANE];
-      uint32_t kk[XF_LANE];
-#pragma unroll
-      for (int e = 0; e < XF_LANE; ++e) cc[e] = e < L ? ld_stream(cp + s + e) : CI(0);
-#pragma unroll
-      for (int e = 0; e < XF_LANE; ++e) vv[e] = e < L ? ld_stream(vq + s + e) : VT(0);
-      int nk = 0;
+      load_row<XF_LANE>(src.cols(h) + s, int(L), s >= 3 && s + L + 3 <= src.nnz(h), cc);
+      const VT* vq = src.vals(h) + s;
+      uint32_t kk[XF_LANE], id[XF_LANE];
 #pragma unroll
       for (int e = 0; e < XF_LANE; ++e) {
-        uint32_t key = kDropped;
-        const bool p = e < L && src.map(h, (long long)cc[e], key);
-        kk[e] = p ? key : kDropped;
-        nk += p ? 1 : 0;
+        kk[e] = kDropped;
+        id[e] = e;
+        uint32_t key;
+        if (((mask >> e) & 1u) && src.map(h, (long long)cc[e], key)) kk[e] = key;
       }
-      if (nk != oe - o) {  // the count disagrees with the fill (a library bug)
-        dev_fail(st, SP_ERR_INTERNAL, -29);
-      } else {
-        sort8(kk, vv);
+      sort8(kk, id);
 #pragma unroll
-        for (int e = 0; e < XF_LANE; ++e)
-          if (e < nk) x_put(out_col, out_val, o + e, oe, kk[e], vv[e], st);
+      for (int e = 0; e < XF_LANE; ++e) {
+        if (e >= nkeep) continue;
+        st_stream(out_col + o + e, CI(kk[e]));
+        st_stream(out_val + o + e, ld_stream(vq + id[e]));
       }
     }
-    // rows of lane_rows < L <= XFAST entries: the warp, XF_ROWS rows at a time
-    const unsigned lm = __ballot_sync(kFull, !by_lane && L <= XFAST);
-    if ((lm >> lane) & 1u) s_lane[wid][__popc(lm & lt)] = (unsigned char)lane;
+    const unsigned m1 = __ballot_sync(kFull, !by_lane && mask != 0u);
+    const unsigned lm = __ballot_sync(kFull, L > 32 && L <= XFAST);
+    const int nr1 = __popc(m1), nr = nr1 + __popc(lm);
+    if ((m1 >> lane) & 1u) s_lane[wid][__popc(m1 & lt)] = (unsigned char)lane;
+    if ((lm >> lane) & 1u) s_lane[wid][nr1 + __popc(lm & lt)] = (unsigned char)lane;
     __syncwarp();
-    const int nr = __popc(lm);
-    for (int g = 0; g < nr; g += R) {
+    // longer rows of at most 32 entries: the warp, one entry per lane and R1 rows at a
+    // time; a kept entry's place is its rank among the row's new columns (or its slot)
+    for (int g = 0; g < nr1; g += R1) {
+      uint32_t mk[R1], key[R1];
+      VT v[R1];
+      CI c[R1];
+      int ln[R1];
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        ln[u] = g + u < nr1 ? int(s_lane[wid][g + u]) : 0;
+        const uint32_t m = __shfl_sync(kFull, mask, ln[u]);
+        mk[u] = g + u < nr1 ? m : 0u;
+        const long long ss = __shfl_sync(kFull, s, ln[u]) + lane;
+        const H hu = Src::shfl(h, ln[u]);
+        const bool kept = (mk[u] >> lane) & 1u;
+        c[u] = kept ? ld_stream(src.cols(hu) + ss) : CI(0);
+        v[u] = kept ? ld_stream(src.vals(hu) + ss) : VT(0);
+      }
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        key[u] = kDropped;
+        const H hu = Src::shfl(h, ln[u]);
+        if ((mk[u] >> lane) & 1u) src.map(hu, (long long)c[u], key[u]);
+      }
+      if constexpr (!kSorted) {
+        __syncwarp();  // the previous group's ranks have been read
+#pragma unroll
+        for (int u = 0; u < R1; ++u) {
+          const int nk = __popc(mk[u]);
+          if ((mk[u] >> lane) & 1u) wk[u * 36 + __popc(mk[u] & lt)] = key[u];
+          if (lane < 4) wk[u * 36 + nk + lane] = kDropped;  // padding: never below a key
+        }
+        __syncwarp();
+      }
+#pragma unroll
+      for (int u = 0; u < R1; ++u) {
+        const long long ou = __shfl_sync(kFull, o, ln[u]);
+        int ra = 0;
+        if constexpr (kSorted) {
+          ra = __popc(mk[u] & lt);
+        } else {
+          const uint4* w4 = reinterpret_cast<const uint4*>(wk + u * 36);
+          const int nq = (__popc(mk[u]) + 3) >> 2;
+          for (int q = 0; q < nq; ++q) {
+            const uint4 x = w4[q];
+            ra += int(x.x < key[u]) + int(x.y < key[u]) + int(x.z < key[u]) + int(x.w < key[u]);
+          }
+        }
+        if ((mk[u] >> lane) & 1u) {
+          st_stream(out_col + ou + ra, CI(key[u]));
+          st_stream(out_val + ou + ra, v[u]);
+        }
+      }
+    }
+    // rows of 33 to XFAST entries: the warp, XF_ROWS rows at a time
+    for (int g = nr1; g < nr; g += R) {
       long long ss[R];
       int LL[R];
       int ln[R];
@@ -454,7 +586,7 @@ __global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const lo
       for (int u = 0; u < R; ++u) {
         if (LL[u] == 0) continue;  // warp-uniform: empty, long or beyond the block
         const long long ou = __shfl_sync(kFull, o, ln[u]);
-        const long long eu = __shfl_sync(kFull, oe, ln[u]);
+        const long long eu = ou + __shfl_sync(kFull, nkeep, ln[u]);
         const unsigned b0 = __ballot_sync(kFull, p0[u]), b1 = __ballot_sync(kFull, p1[u]);
         const int n0 = __popc(b0), nk = n0 + __popc(b1);
         if (nk != eu - ou) {  // the count disagrees with the fill (a library bug)
@@ -519,7 +651,7 @@ __global__ void __launch_bounds__(XB, 4) k_xfill(Src src, long long nI, const lo
       const CI* cp = src.cols(hk);
       const VT* vq = src.vals(hk);
       long long ok = __shfl_sync(kFull, o, k);
-      const long long ek = __shfl_sync(kFull, oe, k);
+      const long long ek = vp[i0 + k + 1];
       for (long long e0 = 0; e0 < Lk; e0 += 32 * LOAD_U) {
         CI cc[LOAD_U];
         VT vv[LOAD_U];

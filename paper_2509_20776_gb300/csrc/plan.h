@@ -32,6 +32,7 @@ struct sp_plan {
   long long j0 = 0;
   long long* sstart = nullptr;  // consecutive J: kept-segment start; else the source start
   long long* slen = nullptr;    // general J: source length of every listed row
+  uint32_t* kmask = nullptr;    // and the kept entries of a row of at most 32
   // repeated J: jcnt[c] = #{b : J[b] = c}, jptr = its exclusive scan, jpos the positions b
   // grouped by column (in the plan's second buffer)
   char* buf2 = nullptr;
