@@ -95,7 +95,7 @@ struct AssignMergeLoader {
   const VT* valB;
   const IX* I;
   const IX* J;
-  const IX* jinv;  // column of A -> position in J, -1 elsewhere
+  const IX* jinv;  // column of A in J -> position in J
   const uint32_t* jbits;
   long long m, n, nnzA, nJ, nnzB;
   int plus;  // 0: SELECT2ND, 1: PLUS
@@ -177,8 +177,8 @@ struct AssignMergeLoader {
 };
 
 // length of row r of A': len_A plus a correction that is non-zero only on rows of I
-// (rebuilt length - len_A, scattered by k_assign_delta), so the scan reads two dense
-// arrays and no map
+// (rebuilt length - len_A, scattered by the scan of the rebuilt lengths), so the scan reads
+// two dense arrays and no map
 template <class RP>
 __device__ __forceinline__ long long len_a(const RP* rpA, long long r, long long nnzA) {
   const long long s = (long long)rpA[r], e = (long long)rpA[r + 1];
@@ -191,18 +191,78 @@ struct AssignLen {
   long long nnzA;
   __device__ long long operator()(long long r) const { return len_a(rpA, r, nnzA) + (long long)delta[r]; }
 };
+// Scan output of the rebuilt rows' lengths: their row pointer, the corrections of A''s row
+// lengths, and with the last element the totals for the host.
 template <class RP, class IX>
-__global__ void k_assign_delta(const IX* __restrict__ I, long long nI, const RP* __restrict__ rpA, long long m,
-                               long long nnzA, const long long* __restrict__ vt, int* __restrict__ delta,
-                               DevStatus* st) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nI;
-       i += (long long)gridDim.x * blockDim.x) {
+struct StoreRebuilt {
+  StoreCounted counted;
+  const IX* I;
+  const RP* rpA;
+  long long m, nnzA;
+  int* delta;
+  const unsigned* max_lb;
+  DevStatus* st;
+  __device__ void operator()(long long i, long long v, long long vn) const {
+    counted(i, v, vn);
+    if (i == counted.n) {
+      counted.res[RES_MAXLB] = *max_lb;
+      return;
+    }
     const long long r = (long long)I[i];
-    if (r < 0 || r >= m) continue;  // reported by the row map
-    const long long d = (vt[i + 1] - vt[i]) - len_a(rpA, r, nnzA);
+    if (r < 0 || r >= m) return;  // reported by the row map
+    const long long d = (vn - v) - len_a(rpA, r, nnzA);
     if (d > 0x7fffffffll || d < -0x7fffffffll) dev_fail(st, SP_ERR_OVERFLOW, i);
     else delta[r] = int(d);
   }
+};
+
+// The index maps of an assignment in one pass: the row map (row of A -> position in I) with
+// I's bitmap, J's bitmap (with jinv, column of A -> position in J, for the union modes), B's
+// row pointer widened to int64, and the length of B's longest row (saturated at 2^32 - 1).
+// The bitmaps are cleared before the launch; they find repeats and say which entries of the
+// maps are set, so the maps are not cleared.
+template <class RPB, class IX>
+__global__ void k_assign_maps(const IX* __restrict__ I, long long nI, long long m, IX* __restrict__ rowmap,
+                              uint32_t* __restrict__ ibits, const IX* __restrict__ J, long long nJ, long long n,
+                              uint32_t* __restrict__ jbits, IX* __restrict__ jinv, const RPB* __restrict__ rpB,
+                              long long* __restrict__ rpB64, unsigned* max_lb, DevStatus* st) {
+  unsigned mx = 0;
+  const long long len = nI + 1 > nJ ? nI + 1 : nJ;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
+       k += (long long)gridDim.x * blockDim.x) {
+    auto mark = [&](const IX* x, long long size, uint32_t* bits) -> long long {  // the index, or -1
+      const long long v = (long long)x[k];
+      if (v < 0 || v >= size) {
+        dev_fail(st, SP_ERR_INDEX_RANGE, k);
+        return -1;
+      }
+      const uint32_t b = 1u << (v & 31);
+      if (atomicOr(bits + (v >> 5), b) & b) {
+        dev_fail(st, SP_ERR_DUPLICATE_INDEX, k);
+        return -1;
+      }
+      return v;
+    };
+    if (k < nI) {
+      const long long r = mark(I, m, ibits);
+      if (r >= 0) rowmap[r] = IX(k);
+    }
+    if (k < nJ) {
+      const long long c = mark(J, n, jbits);
+      if (jinv && c >= 0) jinv[c] = IX(k);
+    }
+    if (k <= nI) {
+      const long long a = (long long)rpB[k];
+      rpB64[k] = a;
+      if (k < nI) {
+        const long long l = (long long)rpB[k + 1] - a;
+        const unsigned u = l <= 0 ? 0u : (l > 0xFFFFFFFFll ? 0xFFFFFFFFu : unsigned(l));
+        mx = u > mx ? u : mx;
+      }
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(max_lb, mx);
 }
 
 // Assembly of A' as segments (segcopy.cuh): a segment starts at row 0, at every row of I
@@ -259,18 +319,6 @@ struct SegWordStore {
     }
   }
 };
-// Longest row of B (row pointer rpB, n rows), saturated at 2^32 - 1.
-__global__ void k_max_row_len(const long long* __restrict__ rp, long long n, unsigned* out) {
-  unsigned mx = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long L = rp[i + 1] - rp[i];
-    const unsigned l = L <= 0 ? 0u : (L > 0xFFFFFFFFll ? 0xFFFFFFFFu : unsigned(L));
-    mx = l > mx ? l : mx;
-  }
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  if ((threadIdx.x & 31) == 0 && mx) atomicMax(out, mx);
-}
-
 // REPLACE count (k_xcount over A's runs): an entry of A survives unless its column is
 // assigned; the rebuilt row adds all of B's row, so the row pointer's scan adds it.
 struct AssignKeep {
@@ -556,21 +604,25 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   const long long m = A.nrows, n = A.ncols, nI = pl->nI, nJ = pl->nJ;
   const IX* I = static_cast<const IX*>(pl->I);
   const IX* J = static_cast<const IX*>(pl->J);
+  const bool merge = pl->mode != SP_ASSIGN_REPLACE;
   Carver cv;
-  const size_t o_rm = cv.reserve(size_t(m) * sizeof(IX));
+  // cleared by one memset: the bitmaps, the counters, the row-length corrections (on rows of
+  // I), the status words of the two scans
+  const size_t o_zero = cv.total();
   const size_t o_jb = cv.reserve(size_t((n + 31) / 32) * 4);
+  const size_t o_ib = cv.reserve(size_t((m + 31) / 32) * 4);
+  const size_t o_cn = cv.reserve(64);
+  const size_t o_s1 = cv.reserve(scan_ws_bytes(nI));
+  const size_t o_s2 = cv.reserve(scan_ws_bytes(m));
+  const size_t o_dl = cv.reserve(size_t(m) * 4);
+  const size_t zero_bytes = cv.total() - o_zero;
+  const size_t o_rm = cv.reserve(size_t(m) * sizeof(IX));
   const size_t o_vt = cv.reserve(size_t(nI + 1) * 8);
   const size_t o_vo = cv.reserve(size_t(m + 1) * 8);
   const size_t o_rb = cv.reserve(size_t(nI + 1) * 8);
   pl->list_cap = nI + 1;
   const size_t o_cl = cv.reserve(size_t(pl->list_cap) * 8);
-  const size_t o_cn = cv.reserve(64);
-  const size_t o_s1 = cv.reserve(scan_ws_bytes(nI));
-  const size_t o_s2 = cv.reserve(scan_ws_bytes(m));
-  const bool merge = pl->mode != SP_ASSIGN_REPLACE;
   const size_t o_ji = cv.reserve(merge ? size_t(n) * sizeof(IX) : 0);
-  const size_t o_dl = cv.reserve(size_t(m) * 4);                 // row-length corrections on rows of I
-  const size_t o_ib = cv.reserve(size_t((m + 31) / 32) * 4);      // bitmap of I's rows
   const size_t o_r0 = cv.reserve(merge ? 0 : size_t(nI) * 8);  // REPLACE: A's run of every row of I
   const size_t o_rn = cv.reserve(merge ? 0 : size_t(nI) * 8);
   SP_TRY(plan_alloc(ctx, pl, cv.total(), s));
@@ -589,44 +641,20 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   pl->sstart = merge ? nullptr : cv.at<long long>(o_r0);
   pl->slen = merge ? nullptr : cv.at<long long>(o_rn);
   const int nsm = ctx->num_sms;
-  SP_CUDA(cudaMemsetAsync(pl->counters, 0, 64, s));
-  SP_CUDA(cudaMemsetAsync(rowmap, 0xFF, size_t(m) * sizeof(IX), s));
-  SP_CUDA(cudaMemsetAsync(jbits, 0, size_t((n + 31) / 32) * 4, s));
-  SP_CUDA(cudaMemsetAsync(pl->ibits, 0, size_t((m + 31) / 32) * 4, s));
-  SP_CUDA(cudaMemsetAsync(delta, 0, size_t(m) * 4, s));
-  if (nI > 0) {
-    {
-      SP_PHASE(SP_PHASE_MAP);
-      k_inverse_map_bits<IX><<<grid_for(nI, 256, nsm * 8), 256, 0, s>>>(I, nI, m, rowmap, pl->ibits,
-                                                                         ctx->dstatus, SP_ERR_DUPLICATE_INDEX);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  if (nJ > 0) {
-    {
-      SP_PHASE(SP_PHASE_MAP);
-      k_mark_bits<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, n, jbits, ctx->dstatus,
-                                                                  SP_ERR_DUPLICATE_INDEX);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
+  SP_CUDA(cudaMemsetAsync(cv.at<char>(o_zero), 0, zero_bytes, s));
   IX* jinv = merge ? cv.at<IX>(o_ji) : nullptr;
   pl->jinv = jinv;
-  if (merge && nJ > 0) {
-    SP_CUDA(cudaMemsetAsync(jinv, 0xFF, size_t(n) * sizeof(IX), s));
-    {
+  {
+    const long long len = nI + 1 > nJ ? nI + 1 : nJ;
+    const sp_status st = dispatch_i(B.rowptr_type, [&](auto rb) -> sp_status {
+      using RPB = decltype(rb);
       SP_PHASE(SP_PHASE_MAP);
-      k_inverse_map<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, n, jinv, ctx->dstatus,
-                                                                    SP_ERR_DUPLICATE_INDEX);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  SP_TRY(widen_rowptr(ctx, s, B.rowptr, B.rowptr_type, nI + 1, pl->rpB));
-  if (nI > 0) {
-    {
-      SP_PHASE(SP_PHASE_COUNT);
-      k_max_row_len<<<grid_for(nI, 256, nsm * 8), 256, 0, s>>>(pl->rpB, nI, pl->counters + 6);
-    }
+      k_assign_maps<RPB, IX><<<grid_for(len, 256, nsm * 8), 256, 0, s>>>(
+          I, nI, m, rowmap, pl->ibits, J, nJ, n, jbits, jinv, static_cast<const RPB*>(B.rowptr), pl->rpB,
+          pl->counters + 6, ctx->dstatus);
+      return SP_OK;
+    });
+    SP_TRY(st);
     SP_CUDA(cudaGetLastError());
   }
   if (nI > 0) {
@@ -672,29 +700,27 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
       SP_CUDA(cudaGetLastError());
     }
   }
+  const StoreRebuilt<RP, IX> rebuilt{StoreCounted{pl->vp, nI, ctx->dres, RES_TEMP, nullptr, pl->counters + 0},
+                                     I,
+                                     static_cast<const RP*>(A.rowptr),
+                                     m,
+                                     A.nnz,
+                                     delta,
+                                     pl->counters + 6,
+                                     ctx->dstatus};
   if (merge) {
-    SP_TRY(launch_scan(ctx, s, LoadArray<long long>{pl->vp},
-                       StoreDual<long long>{pl->vp, nullptr, ctx->dstatus}, nI, cv.at<char>(o_s1)));
+    SP_TRY(launch_scan(ctx, s, LoadArray<long long>{pl->vp}, rebuilt, nI, cv.at<char>(o_s1), SP_PHASE_SCAN, true));
   } else {
-    SP_TRY(launch_scan(ctx, s, RebuiltLen{pl->vp, pl->rpB}, StoreDual<long long>{pl->vp, nullptr, ctx->dstatus}, nI,
-                       cv.at<char>(o_s1)));
+    SP_TRY(launch_scan(ctx, s, RebuiltLen{pl->vp, pl->rpB}, rebuilt, nI, cv.at<char>(o_s1), SP_PHASE_SCAN, true));
   }
-  if (nI > 0) {
-    SP_PHASE(SP_PHASE_SCAN);
-    k_assign_delta<RP, IX><<<grid_for(nI, 256, nsm * 8), 256, 0, s>>>(I, nI, static_cast<const RP*>(A.rowptr), m,
-                                                                      A.nnz, pl->vp, delta, ctx->dstatus);
-  }
-  SP_CUDA(cudaGetLastError());
   AssignLen<RP> len{static_cast<const RP*>(A.rowptr), delta, A.nnz};
-  SP_TRY(launch_scan(ctx, s, len, StoreDual<long long>{pl->vp_out, nullptr, ctx->dstatus}, m,
-                     cv.at<char>(o_s2)));
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail, pl->vp_out + m, 8, cudaMemcpyDeviceToHost, s));
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail + 1, pl->vp + nI, 8, cudaMemcpyDeviceToHost, s));
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail + 2, pl->counters + 6, 4, cudaMemcpyDeviceToHost, s));
+  SP_TRY(launch_scan(ctx, s, len, StoreCounted{pl->vp_out, m, ctx->dres, RES_NNZ, nullptr, nullptr}, m,
+                     cv.at<char>(o_s2), SP_PHASE_SCAN, true));
   SP_TRY(ctx_collect(ctx, s));
-  pl->nnz_out = pl->h_tail[0];
-  pl->nnz_temp = pl->h_tail[1];
-  pl->max_lb = nI > 0 ? (long long)*reinterpret_cast<const unsigned*>(pl->h_tail + 2) : 0;
+  pl->nnz_out = ctx->hres[RES_NNZ];
+  pl->nnz_temp = ctx->hres[RES_TEMP];
+  pl->max_lb = ctx->hres[RES_MAXLB];
+  pl->n_long = ctx->hres[RES_LONG];
   return SP_OK;
 }
 
@@ -713,7 +739,7 @@ sp_status assign_stage(sp_ctx* ctx, sp_plan* pl, CI* tcol, VT* tval, unsigned* t
                                                                         ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
-    {
+    if (pl->n_long > 0) {
       SP_PHASE(SP_PHASE_GATHER);
       k_fill_long<<<nsm, 1024, 0, s>>>(ld, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->vp, ticket, tcol,
                                        tval, ctx->dstatus);
@@ -833,7 +859,7 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
                                                                             ctx->dstatus);
       launched = cudaGetLastError();
     }
-    if (launched == cudaSuccess) {
+    if (launched == cudaSuccess && pl->n_long > 0) {
       SP_PHASE(SP_PHASE_GATHER);
       k_assign_merge_long<<<nsm, 1024, 0, s>>>(ms, pl->cl_rows, pl->counters + 0, pl->list_cap, pl->vp,
                                                 pl->vp_out, ticket, oc, ov, ctx->dstatus);
@@ -855,7 +881,8 @@ template <class RP, class IX>
 struct FusedLen {
   const IX* p;
   const long long* vpa;  // row pointer of A'
-  const IX* rowmap;      // row of A -> position in I, -1 elsewhere
+  const IX* rowmap;      // row of A -> position in I
+  const uint32_t* ibits; // rows of I
   const long long* vt;   // row pointer of the staged rebuilt rows
   const RP* rpA;
   long long m;
@@ -866,8 +893,8 @@ struct FusedLen {
       sstart[i] = 0;
       return 0;  // reported by the permutation check
     }
-    const long long k = (long long)rowmap[r];
-    sstart[i] = k >= 0 ? (vt[k] | (1ll << 62)) : (long long)rpA[r];
+    const bool in_i = (ibits[r >> 5] >> (r & 31)) & 1u;
+    sstart[i] = in_i ? (vt[(long long)rowmap[r]] | (1ll << 62)) : (long long)rpA[r];
     return vpa[r + 1] - vpa[r];
   }
 };
@@ -940,7 +967,7 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
   // output row lengths (rows of A' moved by p) and their sources
   long long* vp = out64 ? static_cast<long long*>(out->rowptr) : cv.at<long long>(o_vp);
   long long* sstart = cv.at<long long>(o_ss);
-  const FusedLen<RP, IX> len{p, pl->vp_out, static_cast<const IX*>(pl->rowmap), pl->vp,
+  const FusedLen<RP, IX> len{p, pl->vp_out, static_cast<const IX*>(pl->rowmap), pl->ibits, pl->vp,
                              static_cast<const RP*>(A.rowptr), m, sstart};
   RowsWs w = rows_bind(cv, m, nnz_out, ro);
   w.counters = cv.at<unsigned>(o_cnt);

@@ -533,7 +533,7 @@ sp_status batch_fill_body(sp_ctx* ctx, sp_batch* b, sp_csr* out, cudaStream_t s,
       const XBatchSrc<CI, VT> src{b->rreq, b->rv, b->jrp};
       k_xfill<XBatchSrc<CI, VT>, false><<<grid_for((rows + 31) / 32 * 32, XB, ctx->num_sms * 8), XB, 0, s>>>(
           src, rows, b->rs0, b->rsn, b->kmask, b->vp, oc, ov, w.lists(),
-          b->max_nj <= 0xFFFFFFFFll ? XF_LANE : 0, ctx->dstatus);
+          b->max_nj <= 0xFFFFFFFFll ? XF_LANE : 0, nullptr, 0, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
     return sort_queued<CI, VT>(ctx, s, w, nnz, kb, oc, ov);

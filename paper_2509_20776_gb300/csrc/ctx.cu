@@ -50,7 +50,7 @@ sp_status ctx_workspace(sp_ctx* ctx, size_t bytes, cudaStream_t s, char** base) 
 }
 
 sp_status ctx_collect(sp_ctx* ctx, cudaStream_t s) {
-  SP_CUDA(cudaMemcpyAsync(ctx->hstatus, ctx->dstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
+  SP_CUDA(cudaMemcpyAsync(ctx->hstatus, ctx->dstatus, kStatusBytes, cudaMemcpyDeviceToHost, s));
   SP_CUDA(cudaStreamSynchronize(s));
   DevStatus h = *ctx->hstatus;
   if (h.code != 0) {
@@ -151,10 +151,10 @@ sp_status sp_ctx_create(sp_ctx** out, int device, const sp_allocator* allocator)
   }
   int prio_least = 0, prio_greatest = 0;
   if (cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-      cudaMalloc(&ctx->dstatus, sizeof(DevStatus)) != cudaSuccess ||
-      cudaMallocHost(&ctx->hstatus, sizeof(DevStatus)) != cudaSuccess ||
+      cudaMalloc(&ctx->dstatus, kStatusBytes) != cudaSuccess ||
+      cudaMallocHost(&ctx->hstatus, kStatusBytes) != cudaSuccess ||
       cudaMallocHost(&ctx->hbuf, 16 * sizeof(long long)) != cudaSuccess ||
-      cudaMemset(ctx->dstatus, 0, sizeof(DevStatus)) != cudaSuccess ||
+      cudaMemset(ctx->dstatus, 0, kStatusBytes) != cudaSuccess ||
       cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest) != cudaSuccess ||
       cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, prio_greatest) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
@@ -168,6 +168,8 @@ sp_status sp_ctx_create(sp_ctx** out, int device, const sp_allocator* allocator)
     delete ctx;
     return SP_ERR_CUDA;
   }
+  ctx->dres = reinterpret_cast<long long*>(ctx->dstatus + 1);
+  ctx->hres = reinterpret_cast<const long long*>(ctx->hstatus + 1);
   *out = ctx;
   return SP_OK;
 }

@@ -149,25 +149,10 @@ sp_status store_rowptr(sp_ctx* ctx, cudaStream_t s, const long long* vp, long lo
   return SP_OK;
 }
 
-sp_status widen_rowptr(sp_ctx* ctx, cudaStream_t s, const void* in, sp_itype t, long long n1,
-                       long long* out) {
-  if (t == SP_I64) {
-    SP_CUDA(cudaMemcpyAsync(out, in, size_t(n1) * 8, cudaMemcpyDeviceToDevice, s));
-    return SP_OK;
-  }
-  {
-    SP_PHASE(SP_PHASE_OTHER);
-    k_widen<int32_t><<<grid_for(n1, 256, ctx->num_sms * 8), 256, 0, s>>>(static_cast<const int32_t*>(in), n1, out);
-  }
-  SP_CUDA(cudaGetLastError());
-  return SP_OK;
-}
-
 sp_status plan_alloc(sp_ctx* ctx, sp_plan* pl, size_t bytes, cudaStream_t s) {
   pl->buf = static_cast<char*>(ctx_alloc(ctx, bytes, s));
   if (!pl->buf) return SP_ERR_OOM;
   pl->buf_bytes = bytes;
-  pl->h_tail = ctx->hbuf;  // every use is read back before the count call returns
   return SP_OK;
 }
 
@@ -180,21 +165,24 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   pl->identify = ctx->cur.identify;
   const long long nw32 = (n + 31) / 32;
   Carver cv;
+  // cleared by one memset: J's bitmap, the counters, the status words of the count's two scans
+  const size_t o_zero = cv.total();
+  const size_t o_jb = cv.reserve(size_t(nw32) * 4);
+  const size_t o_cn = cv.reserve(64);
+  const size_t o_scan = cv.reserve(scan_ws_bytes(nI));
+  const size_t o_scanj = cv.reserve(pl->identify == 0 ? scan_ws_bytes(nw32) : 0);
+  const size_t zero_bytes = cv.total() - o_zero;
   const size_t o_meta = cv.reserve(pl->identify == 0 ? size_t(nw32) * 8 : 0);
   const size_t o_jrp = cv.reserve(pl->identify == 0 ? size_t(nJ) * sizeof(IX) : 0);
   const size_t o_jsk = cv.reserve(pl->identify == 1 ? size_t(nJ) * 4 : 0);
   const size_t o_jsp = cv.reserve(pl->identify == 1 ? size_t(nJ) * 4 : 0);
   const size_t o_vp2 = cv.reserve(16);
-  const size_t o_jb = cv.reserve(size_t(nw32) * 4);
   const size_t o_vp = cv.reserve(size_t(nI + 1) * 8);
   pl->list_cap = nI + 1;
   const size_t o_cl = cv.reserve(size_t(pl->list_cap) * 8);
-  const size_t o_cn = cv.reserve(64);
-  const size_t o_scan = cv.reserve(scan_ws_bytes(nI > nw32 ? nI : nw32));
   const size_t o_ss = cv.reserve(size_t(nI) * 8);
   const size_t o_sn = cv.reserve(size_t(nI) * 8);
   const size_t o_km = cv.reserve(size_t(nI) * 4);
-  const size_t o_fl = cv.reserve(16);  // J strictly ascending / consecutive / repeats
   SP_TRY(plan_alloc(ctx, pl, cv.total(), s));
   cv.bind(pl->buf);
   pl->sstart = cv.at<long long>(o_ss);
@@ -210,32 +198,21 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   pl->cl_rows = cv.at<long long>(o_cl);
   pl->counters = cv.at<unsigned>(o_cn);
   const int nsm = ctx->num_sms;
-  // the shape of J picks the path: consecutive J needs neither maps nor membership tests
-  int* flags = cv.at<int>(o_fl);
-  SP_CUDA(cudaMemsetAsync(flags, 0, 16, s));
-  if (nJ > 1) {
-    {
-      SP_PHASE(SP_PHASE_MAP);
-      k_index_shape<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, flags);
-    }
-    SP_CUDA(cudaGetLastError());
-  }
-  // membership bitmap of J; repeats are flagged (flags[2]) and take the multi-map path
-  SP_CUDA(cudaMemsetAsync(jbits, 0, size_t((n + 31) / 32) * 4, s));
+  SP_CUDA(cudaMemsetAsync(cv.at<char>(o_zero), 0, zero_bytes, s));
+  // the shape of J picks the path: consecutive J needs neither maps nor membership tests,
+  // repeats take the multi-map path
+  const long long epoch = ++ctx->epoch;
   if (nJ > 0) {
     {
       SP_PHASE(SP_PHASE_MAP);
-      k_mark_bits<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, n, jbits, ctx->dstatus,
-                                                                  SP_ERR_DUPLICATE_INDEX, flags + 2);
+      k_j_shape_bits<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, n, jbits, ctx->dres, epoch, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
   }
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail + 1, flags, 16, cudaMemcpyDeviceToHost, s));
-  if (nJ > 0) SP_CUDA(cudaMemcpyAsync(pl->h_tail + 3, J, sizeof(IX), cudaMemcpyDeviceToHost, s));
   SP_TRY(ctx_collect(ctx, s));
-  int fl[3];
-  std::memcpy(fl, pl->h_tail + 1, 12);
-  pl->j_shape = nJ == 0 ? 0 : (fl[2] ? 3 : (fl[1] == 0 ? 2 : (fl[0] == 0 ? 1 : 0)));
+  const long long* fl = ctx->hres + RES_FLAG;
+  pl->j_shape = nJ == 0 ? 0 : (fl[2] == epoch ? 3 : (fl[1] != epoch ? 2 : (fl[0] != epoch ? 1 : 0)));
+  const StoreCounted counted{pl->vp, nI, ctx->dres, RES_NNZ, nullptr, nullptr};
   if (pl->j_shape == 3) {
     if (nI > 0) {
       SP_PHASE(SP_PHASE_MAP);
@@ -278,34 +255,27 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
           pl->jcnt, pl->jptr, jpos, pl->vp, nullptr, nullptr, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
-    SP_TRY(launch_scan(ctx, s, LoadArray<long long>{pl->vp},
-                       StoreDual<long long>{pl->vp, nullptr, ctx->dstatus}, nI, cv.at<char>(o_scan)));
-    SP_CUDA(cudaMemcpyAsync(pl->h_tail, pl->vp + nI, 8, cudaMemcpyDeviceToHost, s));
+    SP_TRY(launch_scan(ctx, s, LoadArray<long long>{pl->vp}, counted, nI, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
     SP_TRY(ctx_collect(ctx, s));
-    pl->nnz_out = pl->h_tail[0];
+    pl->nnz_out = ctx->hres[RES_NNZ];
     return SP_OK;
   }
   if (pl->j_shape == 2) {
-    IX first;
-    std::memcpy(&first, pl->h_tail + 3, sizeof(IX));
-    pl->j0 = (long long)first;
+    pl->j0 = ctx->hres[RES_FIRST];
     if (pl->j0 < 0 || pl->j0 + nJ > n) return SP_ERR_INDEX_RANGE;
     ExtractRangeLen<RP, CI, IX> len{static_cast<const RP*>(A.rowptr), static_cast<const CI*>(A.colidx), I,
                                     m, nnz, pl->j0, pl->j0 + nJ, pl->sstart, ctx->dstatus};
-    SP_TRY(launch_scan(ctx, s, len, StoreDual<long long>{pl->vp, nullptr, ctx->dstatus}, nI,
-                       cv.at<char>(o_scan)));
-    SP_CUDA(cudaMemcpyAsync(pl->h_tail, pl->vp + nI, 8, cudaMemcpyDeviceToHost, s));
+    SP_TRY(launch_scan(ctx, s, len, counted, nI, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
     SP_TRY(ctx_collect(ctx, s));
-    pl->nnz_out = pl->h_tail[0];
+    pl->nnz_out = ctx->hres[RES_NNZ];
     return SP_OK;
   }
   // general or ascending J: identify tables, then the count
-  SP_CUDA(cudaMemsetAsync(pl->counters, 0, 64, s));
   if (pl->identify == 0) {
     if (nJ > 0) {
       // rank words: bits | exclusive prefix of the words' popcounts; then the positions
-      SP_TRY(launch_scan(ctx, s, LoadPopc{jbits}, StoreRank{jbits, pl->jmeta, nw32}, nw32, cv.at<char>(o_scan),
-                         SP_PHASE_MAP));
+      SP_TRY(launch_scan(ctx, s, LoadPopc{jbits}, StoreRank{jbits, pl->jmeta, nw32}, nw32, cv.at<char>(o_scanj),
+                         SP_PHASE_MAP, true));
       {
         SP_PHASE(SP_PHASE_MAP);
         k_jrank_pos<IX><<<grid_for(nJ, 256, nsm * 8), 256, 0, s>>>(J, nJ, n, pl->jmeta, static_cast<IX*>(pl->jrpos));
@@ -320,9 +290,9 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
     }
     SP_CUDA(cudaGetLastError());
     long long* vp2 = cv.at<long long>(o_vp2);
-    pl->h_tail[4] = 0;
-    pl->h_tail[5] = nJ;
-    SP_CUDA(cudaMemcpyAsync(vp2, pl->h_tail + 4, 16, cudaMemcpyHostToDevice, s));
+    ctx->hbuf[0] = 0;
+    ctx->hbuf[1] = nJ;
+    SP_CUDA(cudaMemcpyAsync(vp2, ctx->hbuf, 16, cudaMemcpyHostToDevice, s));
     Carver cw;
     size_t ro[kRowsSlots];
     rows_reserve(cw, 1, nJ, 4, ro);
@@ -361,12 +331,12 @@ sp_status extract_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
     else SP_TRY(count(JSorted{pl->jsk, pl->jsp, nJ}));
   }
   SP_TRY(launch_scan(ctx, s, LoadArray<long long>{pl->vp},
-                     StoreDual<long long>{pl->vp, nullptr, ctx->dstatus}, nI, cv.at<char>(o_scan)));
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail, pl->vp + nI, 8, cudaMemcpyDeviceToHost, s));
-  SP_CUDA(cudaMemcpyAsync(pl->h_tail + 6, pl->counters + 4, 4, cudaMemcpyDeviceToHost, s));
+                     StoreCounted{pl->vp, nI, ctx->dres, RES_NNZ, pl->counters + 4, pl->counters + 0}, nI,
+                     cv.at<char>(o_scan), SP_PHASE_SCAN, true));
   SP_TRY(ctx_collect(ctx, s));
-  pl->nnz_out = pl->h_tail[0];
-  pl->n_slow = (long long)*reinterpret_cast<const unsigned*>(pl->h_tail + 6);
+  pl->nnz_out = ctx->hres[RES_NNZ];
+  pl->n_slow = ctx->hres[RES_SLOW];
+  pl->n_long = ctx->hres[RES_LONG];
   return SP_OK;
 }
 
@@ -374,7 +344,8 @@ template <class RP, class CI, class VT, class IX>
 sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s) {
   const sp_csr& A = pl->A;
   const long long nI = pl->nI, nnz_out = pl->nnz_out;
-  SP_TRY(store_rowptr(ctx, s, pl->vp, nI + 1, B->rowptr_type, B->rowptr));
+  // (general and ascending J: the fill writes B's row pointer as it reads it)
+  if (nnz_out == 0 || pl->j_shape >= 2) SP_TRY(store_rowptr(ctx, s, pl->vp, nI + 1, B->rowptr_type, B->rowptr));
   if (nnz_out == 0) return SP_OK;
   CI* oc = static_cast<CI*>(B->colidx);
   VT* ov = static_cast<VT*>(B->values);
@@ -411,15 +382,17 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     return sort_rows_in_place<CI, VT>(ctx, s, pl->vp, nI, nnz_out, kb, w, oc, ov);
   }
   const bool sorted = pl->j_shape == 1;  // ascending J: the relabelling keeps rows in order
-  rows_reserve(cv, nI, nnz_out, sizeof(VT), ro, !sorted, pl->n_slow);
-  const size_t o_tk = cv.reserve(16);
+  const bool queue = !sorted && pl->n_slow > 0;  // rows that the fill queues for a sort
+  // cleared by one memset: the sort's counters and a ticket
+  const size_t o_cnt = cv.reserve(16 * 4 + 16);
+  rows_reserve(cv, nI, nnz_out, sizeof(VT), ro, queue, pl->n_slow);
   char* base;
   SP_TRY(ctx_workspace(ctx, cv.total(), s, &base));
   cv.bind(base);
-  const RowsWs w = rows_bind(cv, nI, nnz_out, ro, !sorted, pl->n_slow);
-  unsigned* ticket = cv.at<unsigned>(o_tk);
-  SP_CUDA(cudaMemsetAsync(ticket, 0, 16, s));
-  SP_CUDA(cudaMemsetAsync(w.counters, 0, 16 * 4, s));
+  RowsWs w = rows_bind(cv, nI, nnz_out, ro, queue, pl->n_slow);
+  w.counters = cv.at<unsigned>(o_cnt);
+  unsigned* ticket = w.counters + 16;
+  if (queue || pl->n_long > 0) SP_CUDA(cudaMemsetAsync(w.counters, 0, 16 * 4 + 16, s));
   const int nsm = ctx->num_sms;
   const int kb = ceil_log2_u64(uint64_t(pl->nJ));
   const CI* ci = static_cast<const CI*>(A.colidx);
@@ -434,12 +407,15 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
       const XOne<CI, VT, Rel> src{ci, vv, rel, A.nnz};
       if (sorted)
         k_xfill<XOne<CI, VT, Rel>, true><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->kmask, pl->vp, oc, ov,
-                                                          w.lists(), lane_rows, ctx->dstatus);
+                                                          w.lists(), lane_rows, B->rowptr,
+                                                          B->rowptr_type == SP_I32, ctx->dstatus);
       else
         k_xfill<XOne<CI, VT, Rel>, false><<<g, XB, 0, s>>>(src, nI, pl->sstart, pl->slen, pl->kmask, pl->vp, oc, ov,
-                                                           w.lists(), lane_rows, ctx->dstatus);
+                                                           w.lists(), lane_rows, B->rowptr,
+                                                          B->rowptr_type == SP_I32, ctx->dstatus);
     }
     SP_CUDA(cudaGetLastError());
+    if (pl->n_long == 0) return SP_OK;
     // rows of more than SRC_LONG source entries: one CTA each, kept entries in source order
     const XLongRows<CI, VT, Rel> lr{ci, vv, rel, pl->sstart, pl->slen};
     {
@@ -454,7 +430,7 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
     SP_TRY(fill(JRank<IX>{pl->jmeta, static_cast<const IX*>(pl->jrpos), A.ncols}));
   else
     SP_TRY(fill(JSorted{pl->jsk, pl->jsp, pl->nJ}));
-  if (sorted) return SP_OK;
+  if (!queue) return SP_OK;
   // the rows the warp path did not sort (more than XFAST source entries)
   return sort_queued<CI, VT>(ctx, s, w, nnz_out, kb, oc, ov);
 }

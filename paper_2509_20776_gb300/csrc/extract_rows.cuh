@@ -423,7 +423,8 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
                                                 const long long* __restrict__ vp,
                                                 typename Src::CI* __restrict__ out_col,
                                                 typename Src::VT* __restrict__ out_val, SortLists sl, int lane_rows,
-                                                DevStatus* st) {
+                                                void* __restrict__ out_rp, int rp32, DevStatus* st) {
+  // out_rp (may be null): the output's own row pointer, 4 or 8 bytes wide
   // lane_rows: XF_LANE when every key is below kDropped (the lane path pads with it), else 0
   using CI = typename Src::CI;
   using VT = typename Src::VT;
@@ -452,7 +453,16 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
       L = rsn[i];
       mask = kmask[i];
       o = vp[i];
-      const long long k = vp[i + 1] - o;
+      const long long oe = vp[i + 1], k = oe - o;
+      if (out_rp) {
+        if (rp32) {
+          static_cast<int32_t*>(out_rp)[i] = int32_t(o);
+          if (i == nI - 1) static_cast<int32_t*>(out_rp)[nI] = int32_t(oe);
+        } else {
+          static_cast<long long*>(out_rp)[i] = o;
+          if (i == nI - 1) static_cast<long long*>(out_rp)[nI] = oe;
+        }
+      }
       nkeep = k < (1 << 30) ? int(k) : (1 << 30);  // (only rows of at most XFAST entries use it)
       h = src.handle(i);
       // a row the warp paths do not sort

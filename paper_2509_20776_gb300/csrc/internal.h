@@ -21,11 +21,16 @@ struct sp_ctx {
   char* ws = nullptr;
   size_t ws_cap = 0;
   cudaStream_t ws_stream = nullptr;
-  sp::DevStatus* dstatus = nullptr;  // device error record
+  // device error record and, behind it, the words that a call's kernels leave for the host
+  // (dres: totals, flags); a synchronising call reads both back with one copy
+  sp::DevStatus* dstatus = nullptr;
   sp::DevStatus* hstatus = nullptr;  // pinned host mirror
-  // pinned host scratch for the totals a synchronising call reads back (16 words); one
-  // buffer per context, so no call allocates page-locked memory (which would stop kernels
-  // on other streams from running concurrently with later work)
+  long long* dres = nullptr;
+  const long long* hres = nullptr;
+  long long epoch = 0;               // of flags in dres: a flag is set when it holds its call's epoch
+  // pinned host scratch (16 words); one buffer per context, so no call allocates page-locked
+  // memory (which would stop kernels on other streams from running concurrently with later
+  // work)
   long long* hbuf = nullptr;
   // a second stream of this context (highest priority) and the events that fork work onto
   // it and join it back; overlap = 0 keeps every launch on the caller's stream
@@ -56,6 +61,19 @@ struct sp_ctx {
 };
 
 namespace sp {
+
+constexpr int kResWords = 14;  // words of dres
+constexpr size_t kStatusBytes = sizeof(DevStatus) + kResWords * sizeof(long long);
+// words of dres, by what a count leaves in them
+enum ResWord : int {
+  RES_NNZ = 0,      // entries of the result
+  RES_TEMP = 1,     // assignment: entries of the rebuilt rows
+  RES_SLOW = 2,     // rows that the fill queues for a sort
+  RES_LONG = 3,     // rows listed for one CTA each
+  RES_MAXLB = 4,    // assignment: longest row of B
+  RES_FIRST = 5,    // extraction: J[0]
+  RES_FLAG = 6      // extraction, three flags: J not ascending, not consecutive, repeats
+};
 
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }

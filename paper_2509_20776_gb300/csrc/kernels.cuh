@@ -30,32 +30,6 @@ __global__ void k_inverse_map(const IX* __restrict__ idx, long long len, long lo
   }
 }
 
-// The same map with a membership bitmap beside it: a repeated index is found by the
-// bitmap's atomicOr (1 bit per value, small enough to stay in L2) and the map takes one
-// plain store per index instead of a compare-and-swap on an entry of the n-entry map.
-// The first index to set a value's bit writes its position; a later repeat only reports
-// dup_code.  inv (-1) and bits (0) are cleared before the launch; afterwards bits is J's,
-// I's or q's membership bitmap.
-template <class IX>
-__global__ void k_inverse_map_bits(const IX* __restrict__ idx, long long len, long long n,
-                                   IX* __restrict__ inv, uint32_t* __restrict__ bits, DevStatus* st,
-                                   int dup_code) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
-       k += (long long)gridDim.x * blockDim.x) {
-    const long long v = (long long)idx[k];
-    if (v < 0 || v >= n) {
-      dev_fail(st, SP_ERR_INDEX_RANGE, k);
-      continue;
-    }
-    const uint32_t m = 1u << (v & 31);
-    if (atomicOr(bits + (v >> 5), m) & m) {
-      dev_fail(st, dup_code, k);
-      continue;
-    }
-    inv[v] = IX(k);
-  }
-}
-
 // A permutation's two vectors in one pass: the inverse column map qinv[q[j]] = j with q's
 // bitmap, and p's bitmap (either vector may be null).  The bitmaps (cleared before the
 // launch) find repeats; qinv is not cleared: for a permutation every entry is written, and
@@ -87,28 +61,6 @@ __global__ void k_perm_maps(const IX* __restrict__ q, long long n, IX* __restric
   }
 }
 
-// membership bitmap (1 bit per index); repeated indices are reported as dup_code, or
-// only flagged in *dup_flag when one is given
-template <class IX>
-__global__ void k_mark_bits(const IX* __restrict__ idx, long long len, long long n,
-                            uint32_t* __restrict__ bits, DevStatus* st, int dup_code,
-                            int* dup_flag = nullptr) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
-       k += (long long)gridDim.x * blockDim.x) {
-    const long long v = (long long)idx[k];
-    if (v < 0 || v >= n) {
-      dev_fail(st, SP_ERR_INDEX_RANGE, k);
-      continue;
-    }
-    const uint32_t m = 1u << (v & 31);
-    const uint32_t old = atomicOr(bits + (v >> 5), m);
-    if (old & m) {
-      if (dup_flag) *dup_flag = 1;  // repeats are allowed here: only flagged
-      else dev_fail(st, dup_code, k);
-    }
-  }
-}
-
 template <class IX>
 __global__ void k_range_check(const IX* __restrict__ idx, long long len, long long n, DevStatus* st) {
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
@@ -118,15 +70,37 @@ __global__ void k_range_check(const IX* __restrict__ idx, long long len, long lo
   }
 }
 
-// Shape of an index vector: flags[0] = 1 unless strictly ascending, flags[1] = 1 unless
-// consecutive (idx[k+1] = idx[k] + 1 for all k); the flags are zeroed before the launch.
+// An extraction's J in one pass: its membership bitmap (cleared before the launch), its
+// first index and its shape, left in the context's result words (res): RES_FLAG + 0 holds
+// `epoch` unless J is strictly ascending, + 1 unless consecutive (J[k+1] = J[k] + 1), + 2 if
+// an index repeats.
 template <class IX>
-__global__ void k_index_shape(const IX* __restrict__ idx, long long len, int* flags) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k + 1 < len;
+__global__ void k_j_shape_bits(const IX* __restrict__ J, long long len, long long n, uint32_t* __restrict__ bits,
+                               long long* __restrict__ res, long long epoch, DevStatus* st) {
+  bool f0 = false, f1 = false, f2 = false;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < len;
        k += (long long)gridDim.x * blockDim.x) {
-    const long long a = (long long)idx[k], b = (long long)idx[k + 1];
-    if (b <= a) flags[0] = 1;
-    if (b != a + 1) flags[1] = 1;
+    const long long v = (long long)J[k];
+    if (k == 0) res[RES_FIRST] = v;
+    if (k + 1 < len) {
+      const long long w = (long long)J[k + 1];
+      f0 |= w <= v;
+      f1 |= w != v + 1;
+    }
+    if (v < 0 || v >= n) {
+      dev_fail(st, SP_ERR_INDEX_RANGE, k);
+      continue;
+    }
+    const uint32_t m = 1u << (v & 31);
+    f2 |= (atomicOr(bits + (v >> 5), m) & m) != 0u;
+  }
+  f0 = __any_sync(0xffffffffu, f0);
+  f1 = __any_sync(0xffffffffu, f1);
+  f2 = __any_sync(0xffffffffu, f2);
+  if ((threadIdx.x & 31) == 0) {
+    if (f0) res[RES_FLAG] = epoch;
+    if (f1) res[RES_FLAG + 1] = epoch;
+    if (f2) res[RES_FLAG + 2] = epoch;
   }
 }
 
@@ -173,6 +147,24 @@ __device__ __forceinline__ void push_row(long long* list, unsigned* n, long long
   if (q < cap) list[q] = r;
   else dev_fail(st, SP_ERR_INTERNAL, -12);
 }
+
+// The row pointer of a count (scan output): vp, and with its last element the totals that
+// the host reads back (res[what] = the entries; the lists' lengths when given).
+struct StoreCounted {
+  long long* vp;
+  long long n;
+  long long* res;
+  int what;
+  const unsigned* n_slow;  // may be null: RES_SLOW
+  const unsigned* n_long;  // may be null: RES_LONG
+  __device__ void operator()(long long i, long long v, long long) const {
+    vp[i] = v;
+    if (i != n) return;
+    res[what] = v;
+    if (n_slow) res[RES_SLOW] = *n_slow;
+    if (n_long) res[RES_LONG] = *n_long;
+  }
+};
 
 // Count kernels take a loader (see loaders.cuh) and count the entries its map keeps.
 // Short rows: one warp handles COUNT_RB rows per step, reading the first 32 entries of

@@ -48,17 +48,15 @@ struct sp_plan {
   uint32_t* jsk = nullptr;
   uint32_t* jsp = nullptr;
   long long n_slow = 0;
+  long long n_long = 0;    // rows of more than SRC_LONG source entries (cl_rows)
   long long max_lb = 0;  // assignment: longest row of B (the merge fill takes rows of at most 32)
   long long list_cap = 0;
   unsigned* counters = nullptr;  // [0] n_cl [3] count ticket [4] rows of more than XFAST entries
-  long long* h_tail = nullptr;   // the context's pinned scratch: totals read back by the count call
 };
 
 namespace sp {
 sp_status store_rowptr(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long n1, sp_itype t,
                        void* out);
-sp_status widen_rowptr(sp_ctx* ctx, cudaStream_t s, const void* in, sp_itype t, long long n1,
-                       long long* out);
 sp_status plan_alloc(sp_ctx* ctx, sp_plan* pl, size_t bytes, cudaStream_t s);
 sp_status plan_release(sp_ctx* ctx, sp_plan* pl);
 }  // namespace sp
