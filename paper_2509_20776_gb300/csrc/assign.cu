@@ -216,6 +216,19 @@ struct StoreRebuilt {
   }
 };
 
+// Scan output of A''s row pointer: the row pointer, the total for the host, and the row that
+// holds the first position of every chunk of the copy.
+struct StoreAssigned {
+  StoreCounted counted;
+  long long* chunk_row;
+  long long nchunks;  // its capacity
+  __device__ void operator()(long long i, long long v, long long vn) const {
+    counted(i, v, vn);
+    if (i == counted.n) return;
+    for (long long k = (v + SC_CH - 1) >> SC_CHLOG; (k << SC_CHLOG) < vn && k < nchunks; ++k) chunk_row[k] = i;
+  }
+};
+
 // The index maps of an assignment in one pass: the row map (row of A -> position in I) with
 // I's bitmap, J's bitmap (with jinv, column of A -> position in J, for the union modes), B's
 // row pointer widened to int64, and the length of B's longest row (saturated at 2^32 - 1).
@@ -267,20 +280,27 @@ __global__ void k_assign_maps(const IX* __restrict__ I, long long nI, long long 
 
 // Assembly of A' as segments (segcopy.cuh): a segment starts at row 0, at every row of I
 // and after every row of I; a run of rows outside I is contiguous in A and in A', a row
-// of I is its staged rebuilt row.  The scan over the bitmap words of I's rows numbers the
+// of I is its staged rebuilt row.  Where the merge writes the rows of I (each = false), a
+// segment starts only where rows of I and others meet: a run of rows of I is one segment.  The scan over the bitmap words of I's rows numbers the
 // segment starts (32 rows per element); its store writes each segment (first output
 // position, source position) and the count.
-__device__ __forceinline__ uint32_t seg_starts(const uint32_t* ibits, long long w, long long m) {
+__device__ __forceinline__ uint32_t seg_starts(const uint32_t* ibits, long long w, long long m, bool each) {
   const uint32_t b = ibits[w], prev = w > 0 ? ibits[w - 1] >> 31 : 1u;  // row 0 starts one
-  uint32_t s = b | (b << 1) | prev;
+  uint32_t s = each ? b | (b << 1) | prev : (b ^ ((b << 1) | prev)) | (w == 0 ? 1u : 0u);
   const long long r0 = w * 32;
   if (m - r0 < 32) s &= (1u << (m - r0)) - 1u;  // rows past the last do not start one
   return s;
 }
+__device__ __forceinline__ long long SegFinder::operator()(long long k) const {
+  const long long r = chunk_row[k], w = r >> 5;
+  const uint32_t upto = 0xFFFFFFFFu >> (31 - int(r & 31));
+  return wseg[w] + __popc(seg_starts(ibits, w, m, each) & upto) - 1;
+}
 struct SegWordCount {
   const uint32_t* ibits;
   long long m;
-  __device__ long long operator()(long long w) const { return __popc(seg_starts(ibits, w, m)); }
+  bool each;
+  __device__ long long operator()(long long w) const { return __popc(seg_starts(ibits, w, m, each)); }
 };
 template <class RP, class IX>
 struct SegWordStore {
@@ -291,7 +311,9 @@ struct SegWordStore {
                         // them in place (their segments are kSegSkip)
   const long long* vp_out;
   CopySeg* segs;
+  long long* wseg;
   long long m, nw, cap;
+  bool each;
   long long* nseg;
   DevStatus* dst;
   __device__ void operator()(long long w, long long j, long long) const {
@@ -304,7 +326,8 @@ struct SegWordStore {
       segs[j] = CopySeg{vp_out[m], 0};
       return;
     }
-    uint32_t sm = seg_starts(ibits, w, m);
+    wseg[w] = j;
+    uint32_t sm = seg_starts(ibits, w, m, each);
     const uint32_t b = ibits[w];
     while (sm) {
       const int k = __ffs(sm) - 1;
@@ -418,7 +441,11 @@ struct MergeSrc {
         bv = valB[sB + lane];
       }
     }
-    const int P = LB <= 2 ? 2 : 1 << (32 - __clz(int(LB) - 1));
+    return sort_b(int(LB), bk, bv);
+  }
+  // sorts the (key, value) of B's LB entries across the warp (padding keys for the others)
+  __device__ int sort_b(int LB, uint32_t& bk, VT& bv) const {
+    const int P = LB <= 2 ? 2 : 1 << (32 - __clz(LB - 1));
     warp_sort(bk, bv, P);
     return __popc(__ballot_sync(0xffffffffu, bk != kPadKey));
   }
@@ -432,59 +459,99 @@ __device__ __forceinline__ long long merge_out(const long long* vdst, const IX* 
   return vdst ? vdst[(long long)I[i]] : vp[i];
 }
 
-// Rows of at most SRC_LONG source entries (A's and B's together), one warp each.
+// Rows whose run of A has at most SRC_LONG entries, a warp each.  A warp takes 32 rows: lane l
+// resolves row i0 + l (runs and output place), so the index chains of 32 rows are in flight
+// together, and a row's B entries and first 32 A entries are loaded while the row before it
+// is merged (one row at a time behind its own chain of five dependent loads: 1.21 ms for 2^21
+// rows of R-MAT scale 25; this 1.05).  rpw: rows a warp takes, fewer than 32 where there are
+// not enough rows for every warp of the chip.
 template <class RP, class CI, class VT, class IX>
-__global__ void __launch_bounds__(256) k_assign_merge_warp(MergeSrc<RP, CI, VT, IX> ms, long long nI,
-                                                           const long long* __restrict__ vp,
-                                                           const long long* __restrict__ vdst, CI* __restrict__ tcol,
-                                                           VT* __restrict__ tval, DevStatus* st) {
+__global__ void __launch_bounds__(256, 4) k_assign_merge_warp(MergeSrc<RP, CI, VT, IX> ms, long long nI, int rpw,
+                                                              const long long* __restrict__ vp,
+                                                              const long long* __restrict__ vdst,
+                                                              CI* __restrict__ tcol, VT* __restrict__ tval,
+                                                              DevStatus* st) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const long long w0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long i = w0; i < nI; i += nw) {
-    long long sA, LA, sB, LB;
-    ms.rows(i, sA, LA, sB, LB);
-    if (LA > SRC_LONG) continue;  // k_assign_merge_long (the count listed it)
-    const long long o = merge_out(vdst, ms.I, vp, i), oe = o + (vp[i + 1] - vp[i]);
-    uint32_t bk;
-    VT bv;
-    const int nb = ms.load_b(sB, LB, bk, bv);
-    long long kbase = 0;
-    unsigned cntA = 0;
-    for (long long e0 = 0; e0 < LA; e0 += 32) {
-      const long long e = e0 + lane;
-      const bool valid = e < LA;
-      const long long c = valid ? (long long)ld_stream(ms.colA + sA + e) : 0;
-      const bool kept = valid && c >= 0 && c < ms.n && !ms.in_j(c);
-      VT v;
-      if (kept) v = ld_stream(ms.valA + sA + e);
-      const unsigned km = __ballot_sync(0xffffffffu, kept);
-      const uint32_t ck = valid ? uint32_t(c) : kPadKey;
-      const int nless = warp_lower_bound(bk, ck);   // B' keys below this A column
-      const int lbc = warp_lower_bound(ck, bk);     // this chunk's A columns below this B' key
-      if (kept) {
-        const long long pos = o + kbase + __popc(km & lt) + nless;
+  for (long long i0 = w0 * rpw; i0 < nI; i0 += nw * rpw) {
+    long long rA = 0, rB = 0, ro = 0;  // this lane's row: runs of A and B, output place
+    int nA = 0, nB = 0, nout = -1;     // their lengths (nout < 0: not this kernel's row)
+    if (lane < rpw && i0 + lane < nI) {
+      const long long i = i0 + lane;
+      long long LA, LB;
+      ms.rows(i, rA, LA, rB, LB);
+      if (LA <= SRC_LONG) {  // else k_assign_merge_long (the count listed it)
+        nA = int(LA);
+        nB = int(LB);        // (at most 32: the fill's choice of this path)
+        ro = merge_out(vdst, ms.I, vp, i);
+        nout = int(vp[i + 1] - vp[i]);
+      }
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, nout >= 0);
+    // the entries of a row as loaded ahead
+    CI cb = CI(0), ca = CI(0);
+    VT vb = VT(0), va = VT(0);
+    auto fetch = [&](int k) {
+      const long long sA = __shfl_sync(0xffffffffu, rA, k), sB = __shfl_sync(0xffffffffu, rB, k);
+      const int LA = __shfl_sync(0xffffffffu, nA, k), LB = __shfl_sync(0xffffffffu, nB, k);
+      cb = lane < LB ? ms.colB[sB + lane] : CI(-1);
+      vb = lane < LB ? ms.valB[sB + lane] : VT(0);
+      ca = lane < LA ? ld_stream(ms.colA + sA + lane) : CI(0);
+      va = lane < LA ? ld_stream(ms.valA + sA + lane) : VT(0);
+    };
+    int k = todo ? __ffs(todo) - 1 : 0;
+    if (todo) fetch(k);
+    while (todo) {
+      todo &= todo - 1;
+      const long long sA = __shfl_sync(0xffffffffu, rA, k), o = __shfl_sync(0xffffffffu, ro, k);
+      const int LA = __shfl_sync(0xffffffffu, nA, k), LB = __shfl_sync(0xffffffffu, nB, k);
+      const long long oe = o + __shfl_sync(0xffffffffu, nout, k);
+      uint32_t bk = kPadKey;
+      VT bv = vb;
+      if ((long long)cb >= 0 && (long long)cb < ms.nJ) bk = uint32_t((long long)ld_map(ms.J + (long long)cb));
+      const CI c0 = ca;
+      const VT v0 = va;
+      if (todo) {
+        k = __ffs(todo) - 1;
+        fetch(k);
+      }
+      const int nb = ms.sort_b(LB, bk, bv);
+      int kbase = 0;
+      unsigned cntA = 0;
+      for (int e0 = 0; e0 < LA; e0 += 32) {
+        const bool valid = e0 + lane < LA;
+        const long long c = (long long)(e0 == 0 ? c0 : valid ? ld_stream(ms.colA + sA + e0 + lane) : CI(0));
+        const VT v = e0 == 0 ? v0 : valid ? ld_stream(ms.valA + sA + e0 + lane) : VT(0);
+        const bool kept = valid && c >= 0 && c < ms.n && !ms.in_j(c);
+        const unsigned km = __ballot_sync(0xffffffffu, kept);
+        const uint32_t ck = valid ? uint32_t(c) : kPadKey;
+        const int nless = warp_lower_bound(bk, ck);   // B' keys below this A column
+        const int lbc = warp_lower_bound(ck, bk);     // this chunk's A columns below this B' key
+        if (kept) {
+          const long long pos = o + kbase + __popc(km & lt) + nless;
+          if (pos < oe) {
+            st_stream(tcol + pos, CI(c));
+            st_stream(tval + pos, v);
+          } else {
+            dev_fail(st, SP_ERR_INTERNAL, -30);
+          }
+        }
+        cntA += __popc(km & (lbc >= 32 ? 0xffffffffu : ((1u << lbc) - 1u)));
+        kbase += __popc(km);
+      }
+      if (lane < nb) {
+        const long long pos = o + lane + cntA;
         if (pos < oe) {
-          st_stream(tcol + pos, CI(c));
-          st_stream(tval + pos, v);
+          st_stream(tcol + pos, CI(bk));
+          st_stream(tval + pos, bv);
         } else {
-          dev_fail(st, SP_ERR_INTERNAL, -30);
+          dev_fail(st, SP_ERR_INTERNAL, -31);
         }
       }
-      cntA += __popc(km & (lbc >= 32 ? 0xffffffffu : ((1u << lbc) - 1u)));
-      kbase += __popc(km);
+      if (lane == 0 && o + kbase + nb != oe) dev_fail(st, SP_ERR_INTERNAL, -32);
     }
-    if (lane < nb) {
-      const long long pos = o + lane + cntA;
-      if (pos < oe) {
-        st_stream(tcol + pos, CI(bk));
-        st_stream(tval + pos, bv);
-      } else {
-        dev_fail(st, SP_ERR_INTERNAL, -31);
-      }
-    }
-    if (lane == 0 && o + kbase + nb != oe) dev_fail(st, SP_ERR_INTERNAL, -32);
   }
 }
 
@@ -623,6 +690,8 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   pl->list_cap = nI + 1;
   const size_t o_cl = cv.reserve(size_t(pl->list_cap) * 8);
   const size_t o_ji = cv.reserve(merge ? size_t(n) * sizeof(IX) : 0);
+  const long long crcap = ((A.nnz + B.nnz) >> SC_CHLOG) + 1;  // chunks of A' at most
+  const size_t o_cr = cv.reserve(size_t(crcap) * 8);
   const size_t o_r0 = cv.reserve(merge ? 0 : size_t(nI) * 8);  // REPLACE: A's run of every row of I
   const size_t o_rn = cv.reserve(merge ? 0 : size_t(nI) * 8);
   SP_TRY(plan_alloc(ctx, pl, cv.total(), s));
@@ -637,6 +706,7 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
   pl->cl_rows = cv.at<long long>(o_cl);
   pl->counters = cv.at<unsigned>(o_cn);
   pl->ibits = cv.at<uint32_t>(o_ib);
+  pl->chunk_row = cv.at<long long>(o_cr);
   int* delta = cv.at<int>(o_dl);
   pl->sstart = merge ? nullptr : cv.at<long long>(o_r0);
   pl->slen = merge ? nullptr : cv.at<long long>(o_rn);
@@ -714,8 +784,10 @@ sp_status assign_count_impl(sp_ctx* ctx, sp_plan* pl, cudaStream_t s) {
     SP_TRY(launch_scan(ctx, s, RebuiltLen{pl->vp, pl->rpB}, rebuilt, nI, cv.at<char>(o_s1), SP_PHASE_SCAN, true));
   }
   AssignLen<RP> len{static_cast<const RP*>(A.rowptr), delta, A.nnz};
-  SP_TRY(launch_scan(ctx, s, len, StoreCounted{pl->vp_out, m, ctx->dres, RES_NNZ, nullptr, nullptr}, m,
-                     cv.at<char>(o_s2), SP_PHASE_SCAN, true));
+  SP_TRY(launch_scan(ctx, s, len,
+                     StoreAssigned{StoreCounted{pl->vp_out, m, ctx->dres, RES_NNZ, nullptr, nullptr}, pl->chunk_row,
+                                   crcap},
+                     m, cv.at<char>(o_s2), SP_PHASE_SCAN, true));
   SP_TRY(ctx_collect(ctx, s));
   pl->nnz_out = ctx->hres[RES_NNZ];
   pl->nnz_temp = ctx->hres[RES_TEMP];
@@ -778,11 +850,14 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
   Carver cv;
   const size_t o_tc = cv.reserve(staged ? size_t(nt) * sizeof(CI) : 0);
   const size_t o_tv = cv.reserve(staged ? size_t(nt) * sizeof(VT) : 0);
+  // cleared by one memset: a ticket and the status words of the segments' scan
+  const long long nw = (m + 31) / 32;
   const size_t o_tk = cv.reserve(16);
+  const size_t o_sc = cv.reserve(scan_ws_bytes(nw));
+  const size_t zero_bytes = cv.total() - o_tk;
   const size_t o_sg = cv.reserve(size_t(segcap + 1) * sizeof(CopySeg));
   const size_t o_ns = cv.reserve(8);
-  const size_t o_cf = cv.reserve(size_t(nchunks) * 8);
-  const size_t o_sc = cv.reserve(scan_ws_bytes(m));
+  const size_t o_ws = cv.reserve(size_t(nw) * 8);
   size_t r1[kRowsSlots];
   rows_reserve(cv, staged ? nI : 0, staged ? nt : 0, sizeof(VT), r1);
   char* base;
@@ -791,9 +866,9 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
   CI* tcol = staged ? cv.at<CI>(o_tc) : nullptr;
   VT* tval = staged ? cv.at<VT>(o_tv) : nullptr;
   const int nsm = ctx->num_sms;
+  SP_CUDA(cudaMemsetAsync(cv.at<char>(o_tk), 0, zero_bytes, s));
   if (staged) {
     // rebuilt rows: A's surviving entries and B's relabelled ones, staged, then sorted
-    SP_CUDA(cudaMemsetAsync(cv.at<char>(o_tk), 0, 16, s));
     SP_TRY((assign_stage<RP, CI, VT, IX>(ctx, pl, tcol, tval, cv.at<unsigned>(o_tk), s)));
     const RowsWs w1 = rows_bind(cv, nI, nt, r1);
     const int kb = ceil_log2_u64(uint64_t(A.ncols));
@@ -804,23 +879,14 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
   const IX* rowmap = static_cast<const IX*>(pl->rowmap);
   CopySeg* segs = cv.at<CopySeg>(o_sg);
   long long* nseg = cv.at<long long>(o_ns);
-  long long* chunk_first = cv.at<long long>(o_cf);
-  const long long nw = (m + 31) / 32;
-  SP_TRY(launch_scan(ctx, s, SegWordCount{pl->ibits, m},
+  long long* wseg = cv.at<long long>(o_ws);
+  SP_TRY(launch_scan(ctx, s, SegWordCount{pl->ibits, m, staged},
                      SegWordStore<RP, IX>{pl->ibits, rowmap, static_cast<const RP*>(A.rowptr),
-                                          staged ? pl->vp : nullptr, pl->vp_out, segs, m, nw, segcap, nseg,
+                                          staged ? pl->vp : nullptr, pl->vp_out, segs, wseg, m, nw, segcap, staged, nseg,
                                           ctx->dstatus},
-                     nw, cv.at<char>(o_sc), SP_PHASE_PARTITION));
-  SP_CUDA(cudaMemsetAsync(chunk_first, 0xFF, size_t(nchunks) * 8, s));
-  {
-    SP_PHASE(SP_PHASE_PARTITION);
-    k_seg_chunks<<<grid_for(segcap, 256, nsm * 8), 256, 0, s>>>(segs, nseg, nchunks, chunk_first);
-  }
-  SP_CUDA(cudaGetLastError());
+                     nw, cv.at<char>(o_sc), SP_PHASE_PARTITION, true));
   using CW = std::conditional_t<sizeof(CI) == 4, uint32_t, unsigned long long>;
   using VW = std::conditional_t<sizeof(VT) == 4, uint32_t, unsigned long long>;
-  auto al = [](const void* p) { return p == nullptr || (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const int vec = al(A.colidx) && al(A.values) && al(tcol) && al(tval) && al(Ap->colidx) && al(Ap->values);
   // The copy and the merge write disjoint rows of A'.  With the context's overlap on, the
   // copy (bandwidth-bound) runs on the side stream at SC_MINB_OVERLAP CTAs per SM while
   // the merge (latency-bound) takes the rest of each SM on `s`.
@@ -833,12 +899,13 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
   cudaError_t launched;
   {
     ::sp::PhaseScope ph(ctx, cs, SP_PHASE_GATHER);
-    const long long gmax = (long long)(fork ? SC_MINB_OVERLAP : SC_MINB) * nsm;
-    const long long g = nchunks < gmax ? nchunks : gmax;
+    const long long gmax = (long long)(fork ? SC_MINB_OVERLAP : SC_MINB) * nsm, need = (nchunks + SC_BLOCK / 32 - 1) / (SC_BLOCK / 32);
+    const long long g = need < gmax ? need : gmax;
     k_seg_copy<CW, VW><<<unsigned(g), SC_BLOCK, 0, cs>>>(
-        segs, nseg, nnz_out, chunk_first, nchunks, static_cast<const CW*>(A.colidx), static_cast<const VW*>(A.values),
-        A.nnz, reinterpret_cast<const CW*>(tcol), reinterpret_cast<const VW*>(tval), staged ? nt : 0,
-        static_cast<CW*>(Ap->colidx), static_cast<VW*>(Ap->values), vec, ctx->dstatus);
+        segs, nseg, nnz_out, SegFinder{pl->chunk_row, wseg, pl->ibits, m, staged}, nchunks, reinterpret_cast<const CW*>(A.colidx),
+        reinterpret_cast<const VW*>(A.values), A.nnz, reinterpret_cast<const CW*>(tcol),
+        reinterpret_cast<const VW*>(tval), staged ? nt : 0, reinterpret_cast<CW*>(Ap->colidx),
+        reinterpret_cast<VW*>(Ap->values), ctx->dstatus);
     launched = cudaGetLastError();
   }
   if (fork) SP_CUDA(cudaEventRecord(ctx->join_ev, cs));
@@ -852,10 +919,11 @@ sp_status assign_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* Ap, cudaStream_t s)
     CI* oc = static_cast<CI*>(Ap->colidx);
     VT* ov = static_cast<VT*>(Ap->values);
     unsigned* ticket = cv.at<unsigned>(o_tk);
-    launched = cudaMemsetAsync(ticket, 0, 16, s);
-    if (launched == cudaSuccess) {
+    {
       SP_PHASE(SP_PHASE_GATHER);
-      k_assign_merge_warp<<<grid_for(nI * 32, 256, nsm * 16), 256, 0, s>>>(ms, nI, pl->vp, pl->vp_out, oc, ov,
+      const long long per = nI / (nsm * 32ll) + 1;
+      const int rpw = per < 32 ? int(per) : 32;
+      k_assign_merge_warp<<<grid_for((nI + rpw - 1) / rpw * 32, 256, nsm * 8), 256, 0, s>>>(ms, nI, rpw, pl->vp, pl->vp_out, oc, ov,
                                                                             ctx->dstatus);
       launched = cudaGetLastError();
     }
