@@ -347,10 +347,12 @@ struct SegWordStore {
 struct AssignKeep {
   const uint32_t* jbits;
   long long n;
-  __device__ __forceinline__ bool test(long long c) const {
-    return c >= 0 && c < n && !((ld_map(jbits + (c >> 5)) >> (c & 31)) & 1u);
+  template <class CI>
+  __device__ __forceinline__ bool test(CI c) const {
+    return col_inside(c, n) && !((ld_map(jbits + col_word(c)) >> (uint32_t(c) & 31u)) & 1u);
   }
-  __device__ __forceinline__ bool map(long long c, uint32_t& key) const {
+  template <class CI>
+  __device__ __forceinline__ bool map(CI c, uint32_t& key) const {
     if (!test(c)) return false;
     key = uint32_t(c);
     return true;

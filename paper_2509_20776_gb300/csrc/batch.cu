@@ -215,19 +215,21 @@ struct XBatchSrc {
   __device__ static __forceinline__ H shfl(const H& h, int k) { return H{__shfl_sync(kFull, h.k, k)}; }
   __device__ __forceinline__ const CI* cols(const H& h) const { return static_cast<const CI*>(rv[h.k].col); }
   __device__ __forceinline__ const VT* vals(const H& h) const { return static_cast<const VT*>(rv[h.k].val); }
-  __device__ __forceinline__ bool test(const H& h, long long c) const {
-    const long long n = __ldg(&rv[h.k].ncol);
-    if (c < 0 || c >= n) return false;
-    const unsigned long long* meta = rv[h.k].meta;
-    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + (c >> 5));
-    return (uint32_t(w) >> (c & 31)) & 1u;
+  // the request's rank-map slice and column count, read once per row
+  struct T {
+    const unsigned long long* meta;
+    long long n;
+  };
+  __device__ __forceinline__ T tab(const H& h) const { return T{rv[h.k].meta, __ldg(&rv[h.k].ncol)}; }
+  __device__ __forceinline__ bool test(const T& t, CI c) const {
+    if (!col_inside(c, t.n)) return false;
+    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(t.meta) + col_word(c));
+    return (uint32_t(w) >> (uint32_t(c) & 31u)) & 1u;
   }
-  __device__ __forceinline__ bool map(const H& h, long long c, uint32_t& key) const {
-    const long long n = __ldg(&rv[h.k].ncol);
-    if (c < 0 || c >= n) return false;
-    const unsigned long long* meta = rv[h.k].meta;
-    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + (c >> 5));
-    const uint32_t bits = uint32_t(w), b = 1u << (c & 31);
+  __device__ __forceinline__ bool map(const T& t, CI c, uint32_t& key) const {
+    if (!col_inside(c, t.n)) return false;
+    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(t.meta) + col_word(c));
+    const uint32_t bits = uint32_t(w), b = 1u << (uint32_t(c) & 31u);
     if (!(bits & b)) return false;
     key = ld_plain(jrp + (uint32_t(w >> 32) + __popc(bits & (b - 1u))));
     return true;

@@ -107,12 +107,26 @@ constexpr int XB = 256;       // threads per CTA of the count / fill
 constexpr unsigned kDropped = 0xFFFFFFFFu;  // padding key: never below a key
 
 // ---- identify ------------------------------------------------------------------------
+// A stored column inside [0, n): one 32-bit comparison for 4-byte columns (n <= 2^31 then).
+template <class CI>
+__device__ __forceinline__ bool col_inside(CI c, long long n) {
+  if constexpr (sizeof(CI) == 4) return uint32_t(c) < uint32_t(n);
+  else return c >= 0 && c < n;
+}
+// The bitmap word of a column (inside).
+template <class CI>
+__device__ __forceinline__ size_t col_word(CI c) {
+  if constexpr (sizeof(CI) == 4) return uint32_t(c) >> 5;
+  else return size_t(c) >> 5;
+}
+
 // Membership only (the count): the bitmap of J.
 struct JBits {
   const uint32_t* bits;
   long long n;
-  __device__ __forceinline__ bool test(long long c) const {
-    return c >= 0 && c < n && ((ld_map(bits + (c >> 5)) >> (c & 31)) & 1u);
+  template <class CI>
+  __device__ __forceinline__ bool test(CI c) const {
+    return col_inside(c, n) && ((ld_map(bits + col_word(c)) >> (uint32_t(c) & 31u)) & 1u);
   }
 };
 
@@ -122,15 +136,17 @@ struct JRank {
   const unsigned long long* meta;
   const IX* jpos;
   long long n;
-  __device__ __forceinline__ bool test(long long c) const {
-    if (c < 0 || c >= n) return false;
-    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + (c >> 5));
-    return (uint32_t(w) >> (c & 31)) & 1u;
+  template <class CI>
+  __device__ __forceinline__ bool test(CI c) const {
+    if (!col_inside(c, n)) return false;
+    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + col_word(c));
+    return (uint32_t(w) >> (uint32_t(c) & 31u)) & 1u;
   }
-  __device__ __forceinline__ bool map(long long c, uint32_t& key) const {
-    if (c < 0 || c >= n) return false;
-    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + (c >> 5));
-    const uint32_t bits = uint32_t(w), b = 1u << (c & 31);
+  template <class CI>
+  __device__ __forceinline__ bool map(CI c, uint32_t& key) const {
+    if (!col_inside(c, n)) return false;
+    const unsigned long long w = (unsigned long long)ld_map(reinterpret_cast<const long long*>(meta) + col_word(c));
+    const uint32_t bits = uint32_t(w), b = 1u << (uint32_t(c) & 31u);
     if (!(bits & b)) return false;
     const uint32_t r = uint32_t(w >> 32) + __popc(bits & (b - 1u));
     key = uint32_t((long long)ld_plain(jpos + r));  // |J| words: larger than L2 at scale
@@ -208,7 +224,8 @@ __global__ void k_jsorted_init(const IX* __restrict__ J, long long nJ, uint32_t*
 //   H handle(long long i) const;             the handle of listed row i (lane-per-row)
 //   static H shfl(const H& h, int lane);     another lane's handle
 //   const CI* cols(const H&); const VT* vals(const H&);
-//   bool test(const H&, long long c);  bool map(const H&, long long c, uint32_t& key);
+//   T tab(const H&);                         what the row's columns are tested and relabelled with
+//   bool test(const T&, CI c);  bool map(const T&, CI c, uint32_t& key);
 //   long long nnz(const H&);                 entries of the row's matrix
 //   kLongCta: rows of more than SRC_LONG entries go to the CTA-per-row kernels
 // One matrix and one identify for every row:
@@ -227,8 +244,9 @@ struct XOne {
   __device__ static __forceinline__ H shfl(const H& h, int) { return h; }
   __device__ __forceinline__ const CI* cols(const H&) const { return col; }
   __device__ __forceinline__ const VT* vals(const H&) const { return val; }
-  __device__ __forceinline__ bool test(const H&, long long c) const { return rel.test(c); }
-  __device__ __forceinline__ bool map(const H&, long long c, uint32_t& key) const { return rel.map(c, key); }
+  __device__ __forceinline__ H tab(const H&) const { return H{}; }
+  __device__ __forceinline__ bool test(const H&, CI c) const { return rel.test(c); }
+  __device__ __forceinline__ bool map(const H&, CI c, uint32_t& key) const { return rel.map(c, key); }
 };
 
 // Row resolvers of the count: listed row i -> (source start, length).
@@ -302,8 +320,9 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
     if (L > 0 && L <= XL) {
       CI cc[XL];
       load_row<XL>(src.cols(h) + s, int(L), s >= 3 && s + L + 3 <= src.nnz(h), cc);
+      const auto tb = src.tab(h);
 #pragma unroll
-      for (int e = 0; e < XL; ++e) mask |= (e < L && src.test(h, (long long)cc[e])) ? 1u << e : 0u;
+      for (int e = 0; e < XL; ++e) mask |= (e < L && src.test(tb, cc[e])) ? 1u << e : 0u;
       mine = __popc(mask);
     }
     // rows of at most 32 entries: the warp, one entry per lane, XC_ROWS1 rows at a time; then
@@ -328,8 +347,8 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
       bool k0[R1];
 #pragma unroll
       for (int u = 0; u < R1; ++u) {
-        const H hu = Src::shfl(h, ln[u]);
-        k0[u] = lane < LL[u] && src.test(hu, (long long)c0[u]);
+        const auto tb = src.tab(Src::shfl(h, ln[u]));
+        k0[u] = lane < LL[u] && src.test(tb, c0[u]);
       }
 #pragma unroll
       for (int u = 0; u < R1; ++u) {
@@ -365,9 +384,9 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
       bool k0[R], k1[R];
 #pragma unroll
       for (int u = 0; u < R; ++u) {
-        const H hu = hof(u);
-        k0[u] = lane < LL[u] && src.test(hu, (long long)c0[u]);
-        k1[u] = lane + 32 < LL[u] && src.test(hu, (long long)c1[u]);
+        const auto tb = src.tab(hof(u));
+        k0[u] = lane < LL[u] && src.test(tb, c0[u]);
+        k1[u] = lane + 32 < LL[u] && src.test(tb, c1[u]);
       }
 #pragma unroll
       for (int u = 0; u < R; ++u) {
@@ -375,6 +394,7 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
         // rows of more than XFAST entries: the rest in batches of LOAD_U x 32
         const H hu = hof(u);
         const CI* cp = src.cols(hu);
+        const auto tb = src.tab(hu);
         // (single matrix: LL is the length itself; batched rows re-read a capped length)
         using LT = std::conditional_t<Src::kLongCta, int, long long>;
         LT Lu = LT(LL[u]);
@@ -391,7 +411,7 @@ __global__ void __launch_bounds__(XB, 4) k_xcount(Src src, Res res, long long nI
 #pragma unroll
           for (int v = 0; v < LOAD_U; ++v) {
             const LT e = e0 + v * 32 + lane;
-            c += __popc(__ballot_sync(kFull, e < Lu && src.test(hu, (long long)cc[v])));
+            c += __popc(__ballot_sync(kFull, e < Lu && src.test(tb, cc[v])));
           }
         }
         if (g + u < nr && lane == ln[u]) mine = c;
@@ -480,12 +500,13 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
       load_row<XF_LANE>(src.cols(h) + s, int(L), s >= 3 && s + L + 3 <= src.nnz(h), cc);
       const VT* vq = src.vals(h) + s;
       uint32_t kk[XF_LANE], id[XF_LANE];
+      const auto tb = src.tab(h);
 #pragma unroll
       for (int e = 0; e < XF_LANE; ++e) {
         kk[e] = kDropped;
         id[e] = e;
         uint32_t key;
-        if (((mask >> e) & 1u) && src.map(h, (long long)cc[e], key)) kk[e] = key;
+        if (((mask >> e) & 1u) && src.map(tb, cc[e], key)) kk[e] = key;
       }
       sort8(kk, id);
 #pragma unroll
@@ -516,14 +537,16 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
         const long long ss = __shfl_sync(kFull, s, ln[u]) + lane;
         const H hu = Src::shfl(h, ln[u]);
         const bool kept = (mk[u] >> lane) & 1u;
-        c[u] = kept ? ld_stream(src.cols(hu) + ss) : CI(0);
-        v[u] = kept ? ld_stream(src.vals(hu) + ss) : VT(0);
+        const CI* cp = src.cols(hu) + ss;
+        const VT* vq = src.vals(hu) + ss;
+        c[u] = kept ? ld_stream(cp) : CI(0);
+        v[u] = kept ? ld_stream(vq) : VT(0);
       }
 #pragma unroll
       for (int u = 0; u < R1; ++u) {
         key[u] = kDropped;
-        const H hu = Src::shfl(h, ln[u]);
-        if ((mk[u] >> lane) & 1u) src.map(hu, (long long)c[u], key[u]);
+        const auto tb = src.tab(Src::shfl(h, ln[u]));
+        if ((mk[u] >> lane) & 1u) src.map(tb, c[u], key[u]);
       }
       if constexpr (!kSorted) {
         __syncwarp();  // the previous group's ranks have been read
@@ -589,8 +612,9 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
       bool p0[R], p1[R];
 #pragma unroll
       for (int u = 0; u < R; ++u) {
-        p0[u] = lane < LL[u] && src.map(hh[u], (long long)c0[u], k0[u]);
-        p1[u] = lane + 32 < LL[u] && src.map(hh[u], (long long)c1[u], k1[u]);
+        const auto tb = src.tab(hh[u]);
+        p0[u] = lane < LL[u] && src.map(tb, c0[u], k0[u]);
+        p1[u] = lane + 32 < LL[u] && src.map(tb, c1[u], k1[u]);
       }
 #pragma unroll
       for (int u = 0; u < R; ++u) {
@@ -660,6 +684,7 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
       const H hk = Src::shfl(h, k);
       const CI* cp = src.cols(hk);
       const VT* vq = src.vals(hk);
+      const auto tb = src.tab(hk);
       long long ok = __shfl_sync(kFull, o, k);
       const long long ek = vp[i0 + k + 1];
       for (long long e0 = 0; e0 < Lk; e0 += 32 * LOAD_U) {
@@ -676,7 +701,7 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
 #pragma unroll
         for (int v = 0; v < LOAD_U; ++v) {
           const long long e = e0 + v * 32 + lane;
-          pp[v] = e < Lk && src.map(hk, (long long)cc[v], kk[v]);
+          pp[v] = e < Lk && src.map(tb, cc[v], kk[v]);
         }
 #pragma unroll
         for (int v = 0; v < LOAD_U; ++v) {
