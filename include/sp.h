@@ -137,12 +137,13 @@ SP_API int sp_last_cuda_error(const char** where);
  *                          (SP_ERR_NOT_CANONICAL); default 0. */
 /* Kernel shapes (the autotuner's knobs; every value gives the same output, bit for bit):
  *   SP_OPT_TILE_SHAPE      row sort of short rows: 0 = tiles of 1024 entries holding rows
- *                          of at most 512, 128 threads, 9 CTAs per SM (default);
+ *                          of at most 512, 256 threads, 5 CTAs per SM (default);
  *                          1 = tiles of 2048 entries holding rows of at most 1024,
  *                          256 threads, 4 CTAs per SM;
- *   SP_OPT_HEAVY           a bucket of the row sort with more keys than this is written
- *                          in bucket order and sorted by a later pass: 128 (default) to
- *                          4096;
+ *   SP_OPT_HEAVY           a bucket of the row sort with more keys than this is sorted
+ *                          over its own key range: bucketed again in place by a row that
+ *                          is sorted alone, queued as such a run by a tile: 128 (default)
+ *                          to 4096;
  *   SP_OPT_COUNT_ROWS      rows a warp takes per step in the kept-entry count of
  *                          assignment: 1 to 4 (default 4);
  *   SP_OPT_FILL_ROWS       the same for its compacting fill: 1 or 2 (default 2);

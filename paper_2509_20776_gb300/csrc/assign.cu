@@ -7,11 +7,11 @@
 //     relabelled through J; both parts have distinct columns, so sorting their union
 //     gives the merged canonical row.
 // Identify: rowmap (row -> position in I, -1 elsewhere) and a bitmap of J; counting:
-// per row of I, len_A - |A[I[i],:] ∩ J| + len_B(i); two exclusive scans give the row
-// pointer of the rebuilt rows and of A'.  Fill: the rebuilt rows are gathered into a
-// staging buffer (kept entries of both parts, relabelled) and sorted there in place;
-// one load-balanced gather then assembles A' from A's untouched rows and the staged
-// rows.
+// per row of I, len_A - |A[I[i],:] ∩ J| + len_B(i); exclusive scans give the row pointer
+// of A' (and of the staged rows).  Fill: under REPLACE with short rows of B the rebuilt rows
+// are merged in order straight into A' beside the copy of A's untouched rows; otherwise they
+// are gathered into a staging buffer (both parts, relabelled), sorted there in place, and the
+// segment copy assembles A' from A's untouched rows and the staged rows.
 #include "dispatch.h"
 #include "extract_rows.cuh"
 #include "kernels.cuh"

@@ -9,9 +9,8 @@
 //   per request: inverse column map qinv_k (validates q_k) and a bitmap of p_k
 //   (validates p_k) -> every output row's source (request k and start s packed as
 //   k * 2^40 + s) and length -> exclusive scan of the lengths (the row pointer) -> the
-//   two-phase path of the single permutation over the whole batch: partition of the
-//   output rows, load-balanced chunk gather with the relabelling through each row's
-//   request, in-place row sort.
+//   single permutation's row sort over the whole batch, which reads every row at its
+//   request's matrix and relabels through its request's map.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -139,7 +138,7 @@ __global__ void k_pbatch_rowinfo(const PermReq* __restrict__ reqs, const sp_csr*
   }
 }
 
-// Phase-1 gather (rowsort.cuh) of the batch: output row r reads its request's matrix at
+// Row source (rowsort.cuh) of the batch: output row r reads its request's matrix at
 // the packed source position; every column is relabelled through the request's qinv
 // (identity without one).  Under a column map a column outside [0, ncols) becomes the
 // key 0xFFFFFFFF, which the sort reports as SP_ERR_INDEX_RANGE.

@@ -33,7 +33,7 @@ struct PermLen {
   }
 };
 
-// Phase-1 gather of the permutation: output row r is source row p[r] (its start was
+// Row source of the permutation (rowsort.cuh): output row r is source row p[r] (its start was
 // recorded by the length scan), every column relabelled through qinv (identity when
 // there is no column permutation).  A column outside [0, n) becomes the key
 // 0xFFFFFFFF, which the sort reports as SP_ERR_INDEX_RANGE.

@@ -4,11 +4,11 @@
 //     of consecutive rows, k_seg_sort<SsTile / SsTileL>: the tile reads its rows' source
 //     entries itself (column, relabel lookup, value), sorts them in shared memory and
 //     writes them once.
-//   * Rows of TMAX < L <= SS_RUN_MAX entries go alone, k_seg_sort<SsRun> (of at most
-//     SS_SMALL_RUN entries: k_seg_sort<SsRunS>), read and written the same way.
-//   * Longer rows are gathered in chunks to their place in the output (k_gather_long), cut
-//     by key range (k_split: a coarse, then a fine split) into runs of at most SS_RUN_MAX
-//     entries, and the runs sorted by k_seg_sort<SsRun / SsRunS>.
+//   * Rows of TMAX < L <= SS_RUN_MAX entries go alone, read and written the same way:
+//     k_seg_sort<SsRunS / SsRunM / SsRun> by their length.
+//   * Longer rows are cut by key range, chunk by chunk, into runs of at most SS_RUN_MAX
+//     entries (k_long_hist, k_long_scatter and, where a key range can overflow a run,
+//     k_split_fine), and the runs sorted by the same kernels.
 // Rows that lie in the output already (a sort alone) take the same kernels with the output
 // as their source; a gather without a sort is k_gather_chunks.  One pass over the row
 // pointer (RowsPartition) finds the tiles' first rows and lists the rows that fit none.
@@ -39,7 +39,8 @@ struct SsCfg {
   static_assert(B % 32 == 0 && B * MINB <= 2048, "whole warps, resident CTAs");
   static_assert(CAP <= 4096 && ROWS < 65536 / 2, "packed positions and counts");
 };
-// Shapes by measurement (R-MAT scale 25, 1.05 G entries, whole permutation; start 21.0 ms):
+// Shapes by measurement (R-MAT scale 25, 1.05 G entries, whole permutation with the long
+// rows' split of one CTA per row; gather and sort apart: 21.0 ms):
 // few entries per thread and many threads -- 256 x 4 at 5 CTAs per SM 17.6 ms, 6 CTAs 18.4,
 // 4 CTAs 18.4, 128 x 8 at 8 CTAs 24.0, 64 x 16 31 (longer unrolled code, and the lookups of a
 // thread in flight at once evict one another's lines from the L1 that shared memory leaves).
@@ -899,9 +900,9 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 }
 
 // Work items: tiles [0, ntiles) of the partition, or the runs of one slice of the run
-// lists: whole rows at their source, rows in the output arrays, and k_split's runs in the
-// output or in the temporary arrays.  Every
-// item's entries are loaded before any of them is written, so a run is sorted in place.
+// lists: whole rows at their source, rows in the output arrays, and the split's runs in the
+// output or in the temporary arrays.  Every item's entries are loaded before any of them is
+// written, so a run is sorted in place.
 //
 // The bucket sort: an entry's bucket counter (shared memory) returns its arrival number,
 // one block scan turns the counters into bucket starts, the entry's key is put at start +
@@ -922,7 +923,8 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // pass over the entries instead of two), an entry stays with its thread from load to
 // staging, and buckets hold one key on average.  Uniform rows of 32 over 2^25 columns: 25.8
 // -> 16.4 ms per permutation, of which the lookups alone take 12.9 in a plain gather; rows
-// of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms.
+// of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms (17.2 with the
+// long rows split chunk by chunk and the partition part of the scan).
 template <class Cfg, class Gs>
 __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
     k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nnz, const long long* __restrict__ tile_first,
@@ -1318,8 +1320,8 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
 }
 
 // Runs of at most SS_WARP_RUN entries (the first slice of the run lists: rows in the output
-// arrays, k_split's groups in either buffer), a warp each: every lane keeps four entries and counts the run's smaller keys,
-// four at a time from shared memory (broadcast).
+// arrays, the split's groups in either buffer), a warp each: every lane keeps four entries
+// and counts the run's smaller keys, four at a time from shared memory (broadcast).
 constexpr int WR_BLOCK = 256, WR_MINB = 4;
 template <class CI, class VT>
 __global__ void __launch_bounds__(WR_BLOCK, WR_MINB)
@@ -1530,8 +1532,8 @@ sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz,
     SP_CUDA(cudaGetLastError());
     return SP_OK;
   };
-  // few runs in all: one launch whose CTAs take any of them (three launches, two of them
-  // empty or short, cost 6 us more than the small runs gain from small CTAs)
+  // few runs in all: one launch whose CTAs take any of them (an empty launch costs 2 to 3 us;
+  // the other two cost more than few small runs gain from small CTAs)
   if (nnz > SS_SMALL_RUN && nnz <= SS_ONE_LAUNCH) return run(SsRun{}, -1);
   SP_TRY(run(SsRunS{}, 1));
   if (nnz > SS_SMALL_RUN) SP_TRY(run(SsRunM{}, 2));
