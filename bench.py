@@ -36,14 +36,11 @@ UNIT = "output nnz/s"
 WORKLOAD = ("R-MAT scale {scale} (a,b,c,d)=(0.57,0.19,0.19,0.05), edge factor 16, symmetrised; "
             "P A P^T random p + P A P^T degree-descending p + P A Q^T random p,q")
 
-# DRAM bytes (read + write) per output entry of one k_gather_chunks launch on the
-# first P A P^T (random p), from a one-kernel ncu capture of only
-# dram__bytes_read.sum + dram__bytes_write.sum on the rows-limited instance of the same
-# workload (bench.py --rows-limit 2097152: 2^21 random rows, all 2^25 columns, so the
-# relabel map keeps its full-size L2 pressure); scaled to a full launch by the entries
-# it moves (profiles/gather_dram_rmat25_rows2m.md).  Only valid for the kernel
-# as captured: retake the capture when it changes.
-GATHER_DRAM_BYTES_PER_ENTRY = 25.07  # 1 655 663 104 B over 66 045 976 entries
+# DRAM bytes (read + write) per output entry of one launch of a gather that moves every
+# entry, from a capture; None: the permutation's sorts read their source rows themselves,
+# and no capture of them at the workload's size is kept.
+GATHER_DRAM_BYTES_PER_ENTRY = None
+
 
 _T0 = time.time()
 
@@ -205,7 +202,7 @@ def row_classes(rowptr):
     return out
 
 
-def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup_peak, concurrent=()):
+def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup_peak, concurrent=(), fused=False):
     """Roofline of the phase that takes the most device time: its algorithmic bytes per
     launch over its average CUDA-event duration (int32 columns, fp32 values).  The gather
     moves 16 B per entry (read and write column + value, the scope's per-entry bytes) plus
@@ -213,9 +210,11 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
     counted separately (frac_incl_lookup) and against the measured random-lookup rate.
     Phases in `concurrent` run on a second stream beside another phase: their event times
     include the time they share the SMs, so they are reported but never taken as the
-    dominant kernel."""
+    dominant kernel.  With `fused` the sorts read their source rows themselves: the phase
+    "gather" is then the long rows' histogram pass alone, and the lookups of a phase are
+    those of the rows it reads.  Otherwise the gather moves every entry first."""
     e_tile, r_tile = classes["tile"]
-    e_long, _ = classes["long"]
+    e_long, r_long = classes["long"]
     e_huge, _ = classes["huge"]
     nnz = e_tile + e_long + e_huge
     per_op = {
@@ -232,6 +231,18 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
         "map": 12 * n,
         "partition": 8 * m,
     }
+    lookups = {"gather": nnz}
+    if fused:
+        per_op |= {
+            # the long rows' keys: read, relabelled, written
+            "gather": 8 * e_huge,
+            # source col + val read, sorted col + val written; row pointer pair, source start
+            "tile": 16 * e_tile + 24 * m,
+            "long": 16 * (e_long + e_huge) + 24 * r_long,
+            # the long rows' keys and values read and put in key-range order
+            "huge": 16 * e_huge,
+        }
+        lookups = {"gather": e_huge, "tile": e_tile, "long": e_long}
     launches_total = ops_per_step * steps
     best = None
     for ph, (ms, cnt) in stats.items():
@@ -241,7 +252,9 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
             best = (ph, ms, cnt)
     ph, ms, cnt = best
     kernel = {"gather": "k_gather_chunks", "tile": "k_seg_sort<SsTile>", "long": "k_seg_sort<SsRun>",
-              "huge": "k_split", "scan": "k_scan", "map": "k_inverse_map", "partition": "k_scan"}[ph]
+              "huge": "k_long_scatter", "scan": "k_scan", "map": "k_perm_maps", "partition": "k_partition"}[ph]
+    if fused and ph == "gather":
+        kernel = "k_long_hist"
     byts = per_op[ph] * launches_total
     sec = ms * 1e-3
     achieved = byts / sec / 1e9
@@ -253,13 +266,13 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
            "phase_ms": {k: round(v[0], 3) for k, v in stats.items() if v[1]}}
     if concurrent:
         out["phase_ms_concurrent"] = sorted(concurrent)
-    if ph == "gather":
-        with_lookup = (per_op[ph] + 4 * nnz) * launches_total / sec / 1e9
+    if ph in lookups:
+        with_lookup = (per_op[ph] + 4 * lookups[ph]) * launches_total / sec / 1e9
         out["frac_incl_lookup"] = round(with_lookup / peak_gbs, 4)
-        if GATHER_DRAM_BYTES_PER_ENTRY is not None:
+        if GATHER_DRAM_BYTES_PER_ENTRY is not None and not fused:
             out["traffic"] = int(GATHER_DRAM_BYTES_PER_ENTRY * nnz)
         if lookup_peak:
-            rate = nnz * launches_total / sec
+            rate = lookups[ph] * launches_total / sec
             out["lookup_roofline"] = {"achieved": round(rate / 1e9, 2), "peak": lookup_peak["g_per_s"],
                                       "unit": "G lookups/s", "frac": round(rate / 1e9 / lookup_peak["g_per_s"], 4),
                                       "table_bytes": lookup_peak["table_bytes"], "probe": lookup_peak["probe"]}
@@ -269,8 +282,8 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
 def lookup_probe(table_elems, cols, device):
     """Measured rate of the relabel lookups alone: PyTorch's gather of an int32 map of
     `table_elems` entries at the workload's own column indices `cols` (the same lookups,
-    in the same order, that the gather makes; the index stream is read and the result
-    written as well), best of 3 after a warm-up.  The gather cannot relabel faster than
+    in the same order, that the permutation makes; the index stream is read and the result
+    written as well), best of 3 after a warm-up.  A permutation cannot relabel faster than
     this, so its lookup rate over this one is its fraction of the lookup ceiling."""
     import torch
     t = torch.arange(table_elems, dtype=torch.int32, device=device)
@@ -467,7 +480,7 @@ def run_ours(args, ws, rank, local):
     value = out_per_step * args.steps * ws / (ms * 1e-3)
     lk = lookup_probe(A.ncols, A.colidx, dev)
     roof = roofline_permute(stats_timed, classes, m, A.ncols, len(ops), args.steps, hbm, lk,
-                            concurrent=("huge",) if args.overlap else ())
+                            concurrent=("gather", "huge") if args.overlap else (), fused=True)
     # whole op: read and write col + val per entry, p and rowptr pair per row, q and qinv
     alg_bytes_op = 16 * nnz + 28 * m + 12 * A.ncols
     op_frac = alg_bytes_op * len(ops) * args.steps / (ms * 1e-3) / 1e9 / hbm
