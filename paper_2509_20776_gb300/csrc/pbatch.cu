@@ -37,6 +37,7 @@ struct PermView {
   unsigned long long val;   // const VT*
   unsigned long long qinv;  // const IX*: the request's inverse column map (0: identity)
   long long ncol;
+  long long nnz;
 };
 
 constexpr int kReqShift = 40;  // source position = request * 2^40 + entry of its matrix
@@ -149,9 +150,11 @@ struct PermBatchGs {
   const PermView* pv;
   const long long* rsrc;
   __device__ const long long* srcs() const { return rsrc; }
-  __device__ GsView<CI, VT> view(long long src, long long) const {
+  // (the length comes from the row pointer, which a scan's timeout leaves inconsistent)
+  __device__ GsView<CI, VT> view(long long src, long long L) const {
     const PermView* v = pv + (src >> kReqShift);
     const long long e = src & kEntryMask;
+    if (e + L > __ldg(&v->nnz)) return {};
     return {reinterpret_cast<const CI*>(__ldg(&v->col)) + e, reinterpret_cast<const VT*>(__ldg(&v->val)) + e,
             unsigned(src >> kReqShift)};
   }
@@ -358,7 +361,7 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
       const PermReq& r = b->hreq[size_t(k)];
       const sp_csr& a = mats[r.mat];
       b->hview[size_t(k)] = PermView{(unsigned long long)a.colidx, (unsigned long long)a.values,
-                                     r.q ? (unsigned long long)(qbase + size_t(r.qoff) * is) : 0ull, a.ncols};
+                                     r.q ? (unsigned long long)(qbase + size_t(r.qoff) * is) : 0ull, a.ncols, a.nnz};
     }
   }
   sp_status st = upload(cv.at<char>(b->o_req), b->hreq.data(), size_t(nreq) * sizeof(PermReq), s);

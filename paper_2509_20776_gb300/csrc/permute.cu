@@ -45,9 +45,12 @@ struct PermGs {
   const VT* v_;
   const IX* qinv;           // old column -> new column (null: identity)
   const long long* sstart;  // source start of output row r
-  long long n;
+  long long n, nnz;
   __device__ const long long* srcs() const { return sstart; }
-  __device__ GsView<CI, VT> view(long long src, long long) const { return {c_ + src, v_ + src, 0u}; }
+  // (the length comes from the row pointer, which a scan's timeout leaves inconsistent)
+  __device__ GsView<CI, VT> view(long long src, long long L) const {
+    return src + L <= nnz ? GsView<CI, VT>{c_ + src, v_ + src, 0u} : GsView<CI, VT>{};
+  }
   __device__ uint32_t map(unsigned, uint32_t c) const {  // (a sort follows only a column permutation: n > 0)
     return c > uint32_t(n - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
   }
@@ -114,7 +117,7 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   VT* out_val = static_cast<VT*>(B->values);
   // gather and relabel; with a column permutation also sort every row
   const PermGs<CI, VT, IX> g{static_cast<const CI*>(A->colidx), static_cast<const VT*>(A->values), qinv,
-                             sstart, n};
+                             sstart, n, nnz};
   if (!sort) return gather_rows(ctx, s, vp, m, nnz, w, g, out_col, out_val);
   return sort_rows_from(ctx, s, vp, m, nnz, ceil_log2_u64(uint64_t(n)), w, g, out_col, out_val);
 }

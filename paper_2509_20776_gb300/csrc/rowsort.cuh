@@ -138,8 +138,11 @@ constexpr int GC_H = 4;                        // gather: positions a thread loa
 // [t * 2^wlog, (t + 1) * 2^wlog): a closed form of the row pointer, so no scan of weights is
 // needed and the number of tiles is known on the host (a window inside a longer row is an
 // empty tile).  Gather chunk k starts at the row holding output position k * GC_CH.
-// The row pointer is clamped to nnz (lengths that do not add up to it were reported), so
-// no tile, run or chunk reaches past the output arrays.
+// The row pointer is clamped to [0, nnz], so no run or chunk reaches outside the output
+// arrays.  It need not ascend: a scan that gave up waiting (SP_ERR_TIMEOUT) takes the prefix it
+// missed as 0, so the pointer drops, or jumps, where one of the scan's own tiles ends, and some
+// of tile_first stays unwritten; a caller's own row pointer may hold anything.  So k_seg_sort
+// checks the tiles and their rows itself before it reads or writes by them.
 struct RowsPartition {
   long long nrows, nnz;
   long long ntiles;         // tile_first holds ntiles + 1 entries
@@ -152,8 +155,9 @@ struct RowsPartition {
   DevStatus* st;
   // row r at output positions [o0, o1)
   __device__ void operator()(long long r, long long o0, long long o1) const {
-    o0 = o0 < nnz ? o0 : nnz;
-    o1 = o1 < nnz ? o1 : nnz;
+    if (o0 < 0 || o1 < o0) dev_fail(st, SP_ERR_NOT_CANONICAL, r);
+    o0 = o0 < 0 ? 0 : o0 < nnz ? o0 : nnz;
+    o1 = o1 < 0 ? 0 : o1 < nnz ? o1 : nnz;
     const long long L = o1 - o0;
     if (tile_first) {
       constexpr int W = SsTile::W;
@@ -266,14 +270,15 @@ __device__ void smem_incl_max_w(uint32_t* a, int n, uint32_t* tmp) {
 //     using CI, VT;                            // column / value words
 //     const long long* srcs() const;           // source start of every output row (packed
 //                                              // with whatever view() needs)
-//     GsView<CI, VT> view(long long src, long long L) const;  // the row's first entry
+//     GsView<CI, VT> view(long long src, long long L) const;  // the row's first entry (no
+//                                              // L entries from src on in the arrays: null)
 //     uint32_t map(unsigned mid, uint32_t c) const;  // new column (0xFFFFFFFF: c lies
 //                                              // outside the matrix)
 //     CI map_ci(unsigned mid, CI c) const;     // the same in the column's own width
 //   };
 template <class CI, class VT>
 struct GsView {
-  const CI* c;   // null: the row's source is inconsistent (a library bug)
+  const CI* c;   // null: the row's source is inconsistent (a row pointer after a timeout, a library bug)
   const VT* v;
   unsigned mid;  // which relabelling
 };
@@ -927,8 +932,8 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // long rows split chunk by chunk and the partition part of the scan).
 template <class Cfg, class Gs>
 __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
-    k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nnz, const long long* __restrict__ tile_first,
-               long long ntiles,
+    k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nrows, long long nnz,
+               const long long* __restrict__ tile_first, long long ntiles,
                RunLists rl, int slice, const uint32_t* __restrict__ tkey_g,
                const typename Gs::VT* __restrict__ tval_g, typename Gs::CI* __restrict__ out_col,
                typename Gs::VT* __restrict__ out_val, int key_bits, int heavy, DevStatus* st) {
@@ -985,7 +990,8 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
   long long lf0 = 0;
   int ln = 0, lbase = 0;  // (ntiles < 2^31: checked by the launch)
   unsigned lmask = 0;
-  // tiles: the next tile's first row and number of rows in (pf0, pfn), or false
+  // tiles: the next tile's first row and number of rows in (pf0, pfn), or false.  A range that
+  // is no tile of the partition (see there) is passed over.
   auto next_tile = [&]() -> bool {
     while (lmask == 0) {
       if (lbase >= nitems) return false;
@@ -993,7 +999,9 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       ln = 0;
       if (i >= 0 && i < nitems) {
         lf0 = tile_first[i];
-        ln = int(tile_first[i + 1] - lf0);
+        const long long lf1 = tile_first[i + 1];
+        if (lf0 >= 0 && lf0 <= lf1 && lf1 <= nrows && lf1 - lf0 <= ROWS) ln = int(lf1 - lf0);
+        else dev_fail(st, SP_ERR_INTERNAL, -17);
       }
       lmask = __ballot_sync(0xffffffffu, ln > 0);
       lbase = lbase > 0x7fffffff - 32 * int(gridDim.x) ? 0x7fffffff : lbase + 32 * int(gridDim.x);
@@ -1007,10 +1015,9 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
   // tiles: start copying the row pointers of the tile in (pf0, pfn)
   auto prefetch_rows = [&](bool any) {
     if (any) {
-      const int n = pfn < ROWS ? pfn : ROWS;
-      for (int x = t; x <= n; x += B) {
+      for (int x = t; x <= pfn; x += B) {
         cp_async8(pre_o + x, vp + pf0 + x);
-        if (x < n) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
+        if (x < pfn) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
       }
     }
     cp_async_commit();
@@ -1043,10 +1050,6 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
     };
     if constexpr (Cfg::kTiles) {
       nrow = pfn;
-      if (nrow > ROWS) {  // cannot happen: see RowsPartition
-        if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -17);
-        nrow = ROWS;
-      }
       cp_async_wait_all();  // this tile's row pointers
       __syncthreads();      // and the previous round's last reads of the tables
       ss_clear<B, ITEMS>(cnt);
@@ -1054,28 +1057,40 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       base = pre_o[0];
       uint32_t L[RPT], off[RPT], mine = 0;
       long long src[RPT];
+      // A tile whose rows do not ascend from `base`, each starting in its window, is left out
+      // (see RowsPartition): in any other the rows' places are apart, and their lengths add up
+      // to less than WIN + TMAX.
+      bool bad = base < 0;
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
         const int r = ra + t * RPT + k;
         L[k] = off[k] = 0;
         if (r < nrow) {
-          const long long o0 = pre_o[r], l = pre_o[r + 1] - o0;
-          off[k] = uint32_t(o0 - base);  // < WIN
+          const long long o0 = pre_o[r], l = pre_o[r + 1] - o0, d = o0 - base;
+          off[k] = uint32_t(d);
           src[k] = pre_s[r];
           if (l > 0 && l <= Cfg::TMAX && o0 + l <= nnz) L[k] = uint32_t(l);
+          bad |= l < 0 || (L[k] && (unsigned long long)d >= (unsigned long long)Cfg::WIN);
         }
         mine += L[k] ? ((L[k] << 16) | 1u) : 0u;
       }
       // packed start (high half) and rank among the item's rows (low half)
       const uint32_t inc = warp_incl_sum(mine);
-      if (lane == 31) tmp32[wid] = inc;
+      const bool wbad = __any_sync(0xffffffffu, bad);
+      if (lane == 31) tmp32[wid] = wbad ? 0xFFFFFFFFu : inc;
       __syncthreads();
       uint32_t pre = inc - mine, tot = 0;
+      bad = false;
 #pragma unroll
       for (int k = 0; k < B / 32; ++k) {
         const uint32_t x = tmp32[k];
+        bad |= x == 0xFFFFFFFFu;
         pre += k < wid ? x : 0u;
         tot += x;
+      }
+      if (bad) {
+        if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -19);
+        tot = 0;
       }
       E = int(tot >> 16);
       rnext = nrow;
@@ -1526,7 +1541,7 @@ sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz,
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_LONG);
     const long long cap = (long long)Cfg::MINB * ctx->num_sms, n = slice >= 0 ? w.run_cap[slice] : w.runs_total();
-    k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, nullptr, 0, w.runs(), slice, w.tkey,
+    k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, 0, nullptr, 0, w.runs(), slice, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
@@ -1601,7 +1616,7 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_TILE);
     const long long cap = (long long)Cfg::MINB * nsm, g = ntiles < cap ? ntiles : cap;
-    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
+    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nrows, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());

@@ -1,0 +1,153 @@
+"""A row pointer that does not ascend: a scan that gives up waiting (SP_ERR_TIMEOUT) leaves one
+behind for the kernels launched after it, and a caller's own may hold anything.  Each call
+reports its error, writes nothing outside its output arrays, and leaves the context usable."""
+import ctypes
+from contextlib import contextmanager
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import assert_same, from_oracle
+
+pytestmark = pytest.mark.gpu
+
+N = 1 << 20
+PAD = 1 << 16
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2509_20776_gb300 import Context, build
+    build.build()
+    c = Context(0)
+    yield c
+    c.close()
+
+
+@contextmanager
+def held(ctx):
+    """Tile 1 of every scan never publishes: the row pointer drops to 0 where tile 2 begins
+    (row 2048 of a scan of at most 2^17 rows)."""
+    from paper_2509_20776_gb300 import SP_OPT_SCAN_HOLD_TILE, SP_OPT_SPIN_LIMIT
+    ctx.set_option(SP_OPT_SPIN_LIMIT, 2000)
+    ctx.set_option(SP_OPT_SCAN_HOLD_TILE, 1)
+    try:
+        yield
+    finally:
+        ctx.set_option(SP_OPT_SCAN_HOLD_TILE, -1)
+        ctx.set_option(SP_OPT_SPIN_LIMIT, -1)
+
+
+def matrix(lens, seed, n=N):
+    g = np.random.default_rng(seed)
+    lens = np.asarray(lens)
+    col = np.concatenate([np.sort(g.choice(n, int(x), replace=False)) for x in lens])
+    return oracle.CSR.of(len(lens), n, np.concatenate([[0], np.cumsum(lens)]), col, g.random(len(col)).astype(np.float32))
+
+
+class Padded:
+    """Output arrays with PAD words before and after that nothing may write."""
+
+    def __init__(self, nrows, ncols, nnz, vt=torch.float32):
+        from paper_2509_20776_gb300 import CSR
+        self.col = torch.full((nnz + 2 * PAD,), 7, dtype=torch.int32, device="cuda")
+        self.val = torch.full((nnz + 2 * PAD,), 7.0, dtype=vt, device="cuda")
+        self.out = CSR(nrows, ncols, torch.empty(nrows + 1, dtype=torch.int64, device="cuda"),
+                       self.col[PAD:PAD + nnz], self.val[PAD:PAD + nnz])
+
+    def check(self):
+        for a in (self.col, self.val):
+            assert bool((a[:PAD] == 7).all()) and bool((a[-PAD:] == 7).all())
+
+
+KINDS = {  # row lengths of a matrix of 6000 rows
+    "sparse": lambda g: g.integers(0, 4, 6000),       # the drop lies inside a window
+    "tiles": lambda g: g.integers(0, 513, 6000),
+    "runs": lambda g: np.where(g.random(6000) < 0.1, g.integers(513, 2500, 6000), g.integers(0, 30, 6000)),
+}
+
+
+def expect(ctx, name, call):
+    from paper_2509_20776_gb300 import SpError
+    with pytest.raises(SpError) as e:
+        call()
+        ctx.sync()
+    assert e.value.name == name
+
+
+def idx(n, seed):
+    return torch.from_numpy(np.random.default_rng(seed).permutation(n).astype(np.int32)).cuda()
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("tile_shape", [0, 1])
+def test_permute(ctx, kind, tile_shape):
+    O = matrix(KINDS[kind](np.random.default_rng(1)), 2)
+    A, p, q = from_oracle(O), idx(6000, 3), idx(N, 4)
+    P = Padded(6000, N, A.nnz)
+    ctx.set_shapes(tile_shape=tile_shape)
+    try:
+        with held(ctx):
+            expect(ctx, "SP_ERR_TIMEOUT", lambda: ctx.sp_permute(A, p, q, out=P.out))
+        P.check()
+        assert_same(ctx.sp_permute(A, p, q), oracle.permute(O, p.cpu().numpy(), q.cpu().numpy()), kind)
+    finally:
+        ctx.set_shapes(tile_shape=-1)
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+def test_permute_batch(ctx, kind):
+    mats = [from_oracle(matrix(KINDS[kind](np.random.default_rng(s))[:2500], s)) for s in (5, 6, 7)]
+    reqs = [(k, idx(2500, 10 + k), idx(N, 20 + k)) for k in range(3)]
+    bt = ctx.permute_batch(mats, reqs)
+    try:
+        P = Padded(7500, N, sum(m.nnz for m in mats))
+        with held(ctx):
+            expect(ctx, "SP_ERR_TIMEOUT", lambda: bt.fill(P.out))
+        P.check()
+    finally:
+        bt.close()
+
+
+def assign_plan(ctx, A, I, J, B):
+    plan, nnz = ctypes.c_void_p(), ctypes.c_int64()
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    ctx._check(ctx.lib.sp_assign_count(ctx.handle, ctypes.byref(A.desc()), ctypes.c_void_p(I.data_ptr()), I.numel(),
+                                       ctypes.c_void_p(J.data_ptr()), J.numel(), 0, ctypes.byref(B.desc()), 0,
+                                       ctypes.byref(plan), ctypes.byref(nnz), st), "sp_assign_count")
+    return plan, nnz.value, st
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+def test_assign_permute(ctx, kind):
+    A = from_oracle(matrix(KINDS[kind](np.random.default_rng(8)), 9))
+    I, J = idx(6000, 30)[:900].contiguous(), idx(N, 31)[:3000].contiguous()
+    B = from_oracle(matrix(np.random.default_rng(10).integers(0, 9, 900), 11, 3000))
+    p, q = idx(6000, 32), idx(N, 33)
+    plan, nnz, st = assign_plan(ctx, A, I, J, B)
+    try:
+        P = Padded(6000, N, nnz)
+        d = P.out.desc()
+        with held(ctx):
+            expect(ctx, "SP_ERR_TIMEOUT", lambda: ctx._check(ctx.lib.sp_assign_permute_fill(
+                ctx.handle, plan, ctypes.c_void_p(p.data_ptr()), ctypes.c_void_p(q.data_ptr()), ctypes.byref(d), st), ""))
+        P.check()
+    finally:
+        ctx.lib.sp_plan_destroy(ctx.handle, plan)
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("fault", ["drop"])
+def test_sort_rows_of_a_bad_row_pointer(ctx, kind, fault):
+    O = matrix(KINDS[kind](np.random.default_rng(12)), 13)
+    rp = O.rowptr.copy()
+    rp[3000:] -= rp[3000]
+    P = Padded(len(rp) - 1, N, len(O.colidx))
+    P.out.rowptr = torch.from_numpy(rp).cuda()
+    P.out.colidx.copy_(torch.from_numpy(O.colidx.astype(np.int32)))
+    expect(ctx, "SP_ERR_NOT_CANONICAL", lambda: ctx.sp_sort_rows(P.out))
+    P.check()
