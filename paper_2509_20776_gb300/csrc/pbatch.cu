@@ -32,12 +32,15 @@ struct PermReq {  // a request with its offsets in the batch's rows, map words a
 };
 
 // what an output row needs from its request (read through the read-only cache)
-struct PermView {
+struct alignas(16) PermView {
   unsigned long long col;   // const CI*
   unsigned long long val;   // const VT*
   unsigned long long qinv;  // const IX*: the request's inverse column map (0: identity)
-  long long ncol;
-  long long nnz;
+  unsigned long long ncol;
+  unsigned long long nnz, pad;
+  // a pair of its words at once
+  __device__ __forceinline__ ulonglong2 arrays() const { return __ldg(reinterpret_cast<const ulonglong2*>(&col)); }
+  __device__ __forceinline__ ulonglong2 map() const { return __ldg(reinterpret_cast<const ulonglong2*>(&qinv)); }
 };
 
 constexpr int kReqShift = 40;  // source position = request * 2^40 + entry of its matrix
@@ -154,23 +157,21 @@ struct PermBatchGs {
   __device__ GsView<CI, VT> view(long long src, long long L) const {
     const PermView* v = pv + (src >> kReqShift);
     const long long e = src & kEntryMask;
-    if (e + L > __ldg(&v->nnz)) return {};
-    return {reinterpret_cast<const CI*>(__ldg(&v->col)) + e, reinterpret_cast<const VT*>(__ldg(&v->val)) + e,
-            unsigned(src >> kReqShift)};
+    const ulonglong2 a = v->arrays();
+    if ((unsigned long long)(e + L) > __ldg(&v->nnz)) return {};
+    return {reinterpret_cast<const CI*>(a.x) + e, reinterpret_cast<const VT*>(a.y) + e, unsigned(src >> kReqShift)};
   }
   __device__ uint32_t map(unsigned mid, uint32_t c) const {
-    const PermView* v = pv + mid;
-    const IX* qinv = reinterpret_cast<const IX*>(__ldg(&v->qinv));
-    if (!qinv) return c;
-    return c > uint32_t(__ldg(&v->ncol) - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
+    const ulonglong2 m = pv[mid].map();
+    if (!m.x) return c;
+    return c > uint32_t(m.y - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(reinterpret_cast<const IX*>(m.x) + c));
   }
   __device__ CI map_ci(unsigned mid, CI c) const {
-    const PermView* v = pv + mid;
-    const IX* qinv = reinterpret_cast<const IX*>(__ldg(&v->qinv));
-    if (!qinv) return c;
+    const ulonglong2 m = pv[mid].map();
+    if (!m.x) return c;
     const long long cl = (long long)c;
-    if (cl < 0 || cl >= __ldg(&v->ncol)) return CI(-1);
-    return CI(ld_map(qinv + cl));
+    if (cl < 0 || cl >= (long long)m.y) return CI(-1);
+    return CI(ld_map(reinterpret_cast<const IX*>(m.x) + cl));
   }
 };
 
@@ -361,7 +362,8 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
       const PermReq& r = b->hreq[size_t(k)];
       const sp_csr& a = mats[r.mat];
       b->hview[size_t(k)] = PermView{(unsigned long long)a.colidx, (unsigned long long)a.values,
-                                     r.q ? (unsigned long long)(qbase + size_t(r.qoff) * is) : 0ull, a.ncols, a.nnz};
+                                     r.q ? (unsigned long long)(qbase + size_t(r.qoff) * is) : 0ull,
+                                     (unsigned long long)a.ncols, (unsigned long long)a.nnz, 0ull};
     }
   }
   sp_status st = upload(cv.at<char>(b->o_req), b->hreq.data(), size_t(nreq) * sizeof(PermReq), s);

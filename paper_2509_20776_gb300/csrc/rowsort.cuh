@@ -1057,38 +1057,38 @@ __global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
       base = pre_o[0];
       uint32_t L[RPT], off[RPT], mine = 0;
       long long src[RPT];
-      // A tile whose rows do not ascend from `base`, each starting in its window, is left out
-      // (see RowsPartition): in any other the rows' places are apart, and their lengths add up
-      // to less than WIN + TMAX.
-      bool bad = base < 0;
+      // A tile whose rows do not ascend from `base`, all starting in its window, is left out (see
+      // RowsPartition): in any other the rows' places are apart, and the lengths kept add up to
+      // less than WIN + TMAX.  What is wrong is counted from bit 8 on of a warp's sum, above the
+      // number of its rows (at most 64).
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
         const int r = ra + t * RPT + k;
         L[k] = off[k] = 0;
         if (r < nrow) {
-          const long long o0 = pre_o[r], l = pre_o[r + 1] - o0, d = o0 - base;
-          off[k] = uint32_t(d);
+          const long long o0 = pre_o[r], l = pre_o[r + 1] - o0;
+          off[k] = uint32_t(o0 - base);
           src[k] = pre_s[r];
           if (l > 0 && l <= Cfg::TMAX && o0 + l <= nnz) L[k] = uint32_t(l);
-          bad |= l < 0 || (L[k] && (unsigned long long)d >= (unsigned long long)Cfg::WIN);
+          mine += uint32_t((unsigned long long)l >> 63) << 8;
         }
         mine += L[k] ? ((L[k] << 16) | 1u) : 0u;
       }
+      if (t == 0 && (base < 0 || pre_o[nrow - 1] - base >= Cfg::WIN)) mine += 1u << 8;
       // packed start (high half) and rank among the item's rows (low half)
+      static_assert(RPT <= 2, "row and fault counts of a warp in bits 0 to 6 and 8 to 14");
       const uint32_t inc = warp_incl_sum(mine);
-      const bool wbad = __any_sync(0xffffffffu, bad);
-      if (lane == 31) tmp32[wid] = wbad ? 0xFFFFFFFFu : inc;
+      if (lane == 31) tmp32[wid] = inc;
       __syncthreads();
-      uint32_t pre = inc - mine, tot = 0;
-      bad = false;
+      uint32_t pre = inc - mine, tot = 0, any = 0;
 #pragma unroll
       for (int k = 0; k < B / 32; ++k) {
         const uint32_t x = tmp32[k];
-        bad |= x == 0xFFFFFFFFu;
+        any |= x;
         pre += k < wid ? x : 0u;
         tot += x;
       }
-      if (bad) {
+      if (any & (0xFFu << 8)) {
         if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -19);
         tot = 0;
       }
