@@ -463,6 +463,9 @@ __device__ __forceinline__ uint32_t ss_bucket(uint32_t key, float scale, uint32_
 //                  consecutive small buckets whose starts fall in one GROUP_CAP window are
 //                  one run; a bucket of more than GROUP_CAP entries is a run of its own,
 //                  or (more than SS_RUN_MAX entries) goes to the fine split.
+//                  A row whose counts do not add up to its length is reported and left out:
+//                  its entries were outside the matrix, or another row lies on it (a row
+//                  pointer that does not ascend), so its groups could reach past its end.
 //   k_long_scatter moves a chunk's entries to their groups in the temporary arrays: staged
 //                  in shared memory by group, then each group's share written as one piece
 //                  at a place taken from the group's cursor.
@@ -551,6 +554,7 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
   __shared__ uint32_t hist[NB], prv[NB], nxb[NB];
   __shared__ uint32_t tmp32[B / 32 + 1];
   __shared__ int s_last;
+  __shared__ unsigned long long s_total;
   const int t = threadIdx.x;
   const uint32_t kmax = key_bits >= 32 ? 0xFFFFFFFFu : (1u << key_bits) - 1u;
   const int nbl = key_bits < SL_NBL ? key_bits : SL_NBL, sh = key_bits - nbl, nb = 1 << nbl;
@@ -563,6 +567,7 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
     const int len = L - e0 < SL_CH ? int(L - e0) : SL_CH;
     const unsigned nc = unsigned((L + SL_CH - 1) / SL_CH);
     for (int x = t; x < NB; x += B) hist[x] = 0;
+    if (t == 0) s_total = 0;
     __syncthreads();
     const bool here = in_place<Gs>::value || hp->buf != BUF_SRC;
     GsView<CI, typename Gs::VT> gv{out_col + off, nullptr, 0u};
@@ -613,6 +618,7 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
     // the row's last chunk: add up the counts and form the groups
     __threadfence();
     if (__ldcg(&hp->bad)) continue;  // uniform: written before the last arrival
+    unsigned long long mine = 0;
     for (int w = t; w < NB / 2; w += B) {
       uint32_t lo = 0, hi = 0;
 #pragma unroll 4
@@ -623,8 +629,20 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
       }
       hist[2 * w] = lo;
       hist[2 * w + 1] = hi;
+      mine += (unsigned long long)lo + hi;
     }
+    mine = warp_sum(mine);
+    if ((t & 31) == 0) atomicAdd(&s_total, mine);
     __syncthreads();
+    const bool whole = s_total == (unsigned long long)L;
+    __syncthreads();  // s_total is cleared for the next chunk
+    if (!whole) {
+      if (t == 0) {
+        dev_fail(st, SP_ERR_INTERNAL, -5);
+        hp->bad = 1;
+      }
+      continue;
+    }
     smem_excl_sum_w<B>(hist, NB, tmp32);
     uint32_t* const cur = cursor + off / SL_GSLOT;
     split_groups<B, NB>(hist, prv, nxb, tmp32, nb, uint32_t(L), [&](int, bool big, uint32_t s, uint32_t e) {
@@ -675,6 +693,11 @@ __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
   __shared__ uint32_t tmp32[B / 32 + 1];
   const int t = threadIdx.x;
   const int sh = key_bits - (key_bits < SL_NBL ? key_bits : SL_NBL);
+  // (clamped: a key may have changed since its chunk was counted, where rows lie on each other)
+  auto group = [&](uint32_t key) -> uint32_t {
+    const uint32_t x = key >> sh, g = gm[x < NB ? x : NB - 1];
+    return g < NB ? g : NB - 1;
+  };
   long long n = *sl.lchunk_n;
   if (n > sl.lchunk_cap) n = sl.lchunk_cap;
   for (long long k = blockIdx.x; k < n; k += gridDim.x) {
@@ -706,7 +729,7 @@ __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
     for (int u = 0; u < U; ++u) {
       pk[u] = 0xFFFFFFFFu;
       if (t + u * B >= len) continue;
-      const uint32_t g = gm[key[u] >> sh];
+      const uint32_t g = group(key[u]);
       pk[u] = (g << 16) | atomicAdd(&lh[g], 1u);
     }
     __syncthreads();
@@ -722,7 +745,7 @@ __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
     }
     __syncthreads();
     for (int i = t; i < len; i += B) {
-      const uint32_t kk = sk[i], g = gm[kk >> sh];
+      const uint32_t kk = sk[i], g = group(kk);
       const uint32_t q = gb[g] + (uint32_t(i) - lh[g]);
       if (q >= uint32_t(he.len)) continue;
       st_stream(tkey + he.off + q, kk);

@@ -68,6 +68,7 @@ KINDS = {  # row lengths of a matrix of 6000 rows
     "sparse": lambda g: g.integers(0, 4, 6000),       # the drop lies inside a window
     "tiles": lambda g: g.integers(0, 513, 6000),
     "runs": lambda g: np.where(g.random(6000) < 0.1, g.integers(513, 2500, 6000), g.integers(0, 30, 6000)),
+    "long": lambda g: np.where(g.random(6000) < 0.03, g.integers(4097, 20000, 6000), g.integers(0, 9, 6000)),
 }
 
 
@@ -80,15 +81,16 @@ def expect(ctx, name, call):
 
 
 def idx(n, seed):
-    return torch.from_numpy(np.random.default_rng(seed).permutation(n).astype(np.int32)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randperm(n, generator=g, device="cuda").to(torch.int32)
 
 
 @pytest.mark.parametrize("kind", sorted(KINDS))
-@pytest.mark.parametrize("tile_shape", [0, 1])
-def test_permute(ctx, kind, tile_shape):
-    O = matrix(KINDS[kind](np.random.default_rng(1)), 2)
-    A, p, q = from_oracle(O), idx(6000, 3), idx(N, 4)
-    P = Padded(6000, N, A.nnz)
+@pytest.mark.parametrize("tile_shape,n", [(0, N), (1, N), (0, 1 << 24)])  # (keys of 24 bits: the fine split follows)
+def test_permute(ctx, kind, tile_shape, n):
+    O = matrix(KINDS[kind](np.random.default_rng(1)), 2, n)
+    A, p, q = from_oracle(O), idx(6000, 3), idx(n, 4)
+    P = Padded(6000, n, A.nnz)
     ctx.set_shapes(tile_shape=tile_shape)
     try:
         with held(ctx):
@@ -141,11 +143,14 @@ def test_assign_permute(ctx, kind):
 
 
 @pytest.mark.parametrize("kind", sorted(KINDS))
-@pytest.mark.parametrize("fault", ["drop"])
+@pytest.mark.parametrize("fault", ["drop", "negative"])
 def test_sort_rows_of_a_bad_row_pointer(ctx, kind, fault):
     O = matrix(KINDS[kind](np.random.default_rng(12)), 13)
     rp = O.rowptr.copy()
-    rp[3000:] -= rp[3000]
+    if fault == "drop":
+        rp[3000:] -= rp[3000]
+    else:
+        rp[100] = -(1 << 40)
     P = Padded(len(rp) - 1, N, len(O.colidx))
     P.out.rowptr = torch.from_numpy(rp).cuda()
     P.out.colidx.copy_(torch.from_numpy(O.colidx.astype(np.int32)))
