@@ -101,7 +101,10 @@ constexpr int SL_CH = 4096;
 
 // What a pass over the output rows queues for the sort: rows of at most SS_RUN_MAX entries
 // as runs, longer ones for the key-range split, chunk by chunk.  The capacities bound what
-// nnz entries can hold (huge_cap rows longer than SS_RUN_MAX, lchunk_cap chunks of them).
+// nnz entries can hold (huge_cap rows longer than SS_RUN_MAX, lchunk_cap chunks of them).  Rows
+// that lie on one another (a row pointer that does not ascend) can hold more: such a row is
+// reported, and the chunks it has already taken from the list are marked as nobody's.
+constexpr unsigned SL_NONE = 0xFFFFFFFFu;
 struct SortLists {
   RunLists runs;
   HugeEntry* huge;
@@ -119,12 +122,10 @@ __device__ __forceinline__ void queue_row(const SortLists& sl, long long off, lo
   }
   const unsigned h = atomicAdd(sl.huge_n, 1u), nc = unsigned((L + SL_CH - 1) / SL_CH);
   const unsigned c = atomicAdd(sl.lchunk_n, nc);
-  if (h >= sl.huge_cap || (long long)c + nc > sl.lchunk_cap) {
-    dev_fail(st, SP_ERR_INTERNAL, err);
-    return;
-  }
-  sl.huge[h] = HugeEntry{off, L, row, buf, 0u, 0, 0};
-  for (unsigned k = 0; k < nc; ++k) sl.lchunk[c + k] = LongChunk{h, k};
+  const bool fits = h < sl.huge_cap && (long long)c + nc <= sl.lchunk_cap;
+  if (fits) sl.huge[h] = HugeEntry{off, L, row, buf, 0u, 0, 0};
+  else dev_fail(st, SP_ERR_INTERNAL, err);
+  for (long long k = 0; k < nc && c + k < sl.lchunk_cap; ++k) sl.lchunk[c + k] = LongChunk{fits ? h : SL_NONE, unsigned(k)};
 }
 
 constexpr int GC_BLOCK = 256;                  // gather: threads per CTA
@@ -562,6 +563,7 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
   if (n > sl.lchunk_cap) n = sl.lchunk_cap;
   for (long long k = blockIdx.x; k < n; k += gridDim.x) {
     const LongChunk lc = sl.lchunk[k];
+    if (lc.huge == SL_NONE) continue;
     HugeEntry* const hp = sl.huge + lc.huge;
     const long long off = hp->off, L = hp->len, e0 = (long long)lc.chunk * SL_CH;
     const int len = L - e0 < SL_CH ? int(L - e0) : SL_CH;
@@ -702,6 +704,7 @@ __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
   if (n > sl.lchunk_cap) n = sl.lchunk_cap;
   for (long long k = blockIdx.x; k < n; k += gridDim.x) {
     const LongChunk lc = sl.lchunk[k];
+    if (lc.huge == SL_NONE) continue;
     const HugeEntry he = sl.huge[lc.huge];
     if (he.bad) continue;
     const long long e0 = (long long)lc.chunk * SL_CH;

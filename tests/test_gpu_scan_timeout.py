@@ -143,14 +143,18 @@ def test_assign_permute(ctx, kind):
 
 
 @pytest.mark.parametrize("kind", sorted(KINDS))
-@pytest.mark.parametrize("fault", ["drop", "negative"])
+@pytest.mark.parametrize("fault", ["drop", "negative", "past", "comb"])
 def test_sort_rows_of_a_bad_row_pointer(ctx, kind, fault):
     O = matrix(KINDS[kind](np.random.default_rng(12)), 13)
     rp = O.rowptr.copy()
     if fault == "drop":
         rp[3000:] -= rp[3000]
-    else:
+    elif fault == "negative":
         rp[100] = -(1 << 40)
+    elif fault == "past":
+        rp[2000] = rp[-1] + 12345
+    else:  # every second row lies on all the later ones: more long rows than the entries can hold
+        rp[1::2] = rp[-1]
     P = Padded(len(rp) - 1, N, len(O.colidx))
     P.out.rowptr = torch.from_numpy(rp).cuda()
     P.out.colidx.copy_(torch.from_numpy(O.colidx.astype(np.int32)))
