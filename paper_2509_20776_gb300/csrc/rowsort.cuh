@@ -310,7 +310,9 @@ template <class Gs>
 struct in_place<Gs, std::void_t<decltype(Gs::kInPlace)>> : std::bool_constant<Gs::kInPlace> {};
 
 // ---- gather without a sort ----------------------------------------------------------------
-// Chunk k is GC_CH consecutive output positions, starting inside row chunk_first[k].
+// Chunk k is GC_CH consecutive output positions, starting inside row chunk_first[k].  After a
+// scan's timeout (see RowsPartition) chunk_first can hold anything, so it is bounded here, and a
+// chunk ends where a batch of rows ends before it.
 template <class Gs>
 __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, const long long* __restrict__ vp,
                                                             long long nrows, long long total,
@@ -342,15 +344,19 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
   };
   // persistent: chunks blockIdx.x, + gridDim.x, ...; a batch is B consecutive rows.  The
   // next batch's row setup is loaded while this batch's entries are in flight.
+  auto first_row = [&](long long k) -> long long {
+    const long long r = chunk_first[k];
+    return r >= 0 && r < nrows ? r : nrows;
+  };
   long long c = blockIdx.x;
   if (c >= nchunks) return;
-  long long rb = chunk_first[c];
+  long long rb = first_row(c);
   long long o0, o1, so;
   setup(rb + t, o0, o1, so);
   for (;;) {
     const long long c0 = c * (long long)GC_CH, c1 = c0 + GC_CH < total ? c0 + GC_CH : total;
     const long long cn = c + gridDim.x;
-    const long long rb_next_chunk = cn < nchunks ? chunk_first[cn] : 0;
+    const long long rb_next_chunk = cn < nchunks ? first_row(cn) : 0;
     bool active = rb + t < nrows && o1 > o0 && o1 > c0 && o0 < c1;
     if (active) {
       r_v[t] = gs.view(so, o1 - o0);
@@ -374,7 +380,7 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
       smem_incl_max_w<B>(owner, GC_CH, tmp32);
     }
     // the chunk ends with this batch once its last row reaches the end of the chunk
-    const bool last_batch = rb + B - 1 >= nrows - 1 || s_last >= c1;
+    const bool last_batch = rb + B - 1 >= nrows - 1 || s_last >= c1 || s_last <= c0;
     const bool more = !last_batch || cn < nchunks;
     const long long rb_next = last_batch ? rb_next_chunk : rb + B;
     long long n0 = 0, n1 = 0, ns = 0;

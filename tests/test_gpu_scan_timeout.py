@@ -87,24 +87,26 @@ def idx(n, seed):
 
 @pytest.mark.parametrize("kind", sorted(KINDS))
 @pytest.mark.parametrize("tile_shape,n", [(0, N), (1, N), (0, 1 << 24)])  # (keys of 24 bits: the fine split follows)
-def test_permute(ctx, kind, tile_shape, n):
+@pytest.mark.parametrize("columns", [True, False])  # (rows alone: gathered without a sort)
+def test_permute(ctx, kind, tile_shape, n, columns):
     O = matrix(KINDS[kind](np.random.default_rng(1)), 2, n)
-    A, p, q = from_oracle(O), idx(6000, 3), idx(n, 4)
+    A, p, q = from_oracle(O), idx(6000, 3), idx(n, 4) if columns else None
     P = Padded(6000, n, A.nnz)
     ctx.set_shapes(tile_shape=tile_shape)
     try:
         with held(ctx):
             expect(ctx, "SP_ERR_TIMEOUT", lambda: ctx.sp_permute(A, p, q, out=P.out))
         P.check()
-        assert_same(ctx.sp_permute(A, p, q), oracle.permute(O, p.cpu().numpy(), q.cpu().numpy()), kind)
+        assert_same(ctx.sp_permute(A, p, q), oracle.permute(O, p.cpu().numpy(), q.cpu().numpy() if columns else None), kind)
     finally:
         ctx.set_shapes(tile_shape=-1)
 
 
 @pytest.mark.parametrize("kind", sorted(KINDS))
-def test_permute_batch(ctx, kind):
+@pytest.mark.parametrize("columns", [True, False])
+def test_permute_batch(ctx, kind, columns):
     mats = [from_oracle(matrix(KINDS[kind](np.random.default_rng(s))[:2500], s)) for s in (5, 6, 7)]
-    reqs = [(k, idx(2500, 10 + k), idx(N, 20 + k)) for k in range(3)]
+    reqs = [(k, idx(2500, 10 + k), idx(N, 20 + k) if columns else None) for k in range(3)]
     bt = ctx.permute_batch(mats, reqs)
     try:
         P = Padded(7500, N, sum(m.nnz for m in mats))
