@@ -52,6 +52,11 @@ struct SegFinder {
   __device__ long long operator()(long long k) const;
 };
 
+// The segments are numbered by a scan; one that gave up waiting (SP_ERR_TIMEOUT) leaves a list
+// whose starts do not ascend and whose closing entry another segment may have taken.  Every step
+// below moves on in the chunk or in the list, or gives the chunk up, so the copy ends and stays in
+// its chunk whatever the list holds.
+//
 // CI / VT: column / value words (uint32 or unsigned long long views of the arrays).
 template <class CI, class VT>
 __global__ void __launch_bounds__(SC_BLOCK, SC_MINB)
@@ -74,6 +79,10 @@ __global__ void __launch_bounds__(SC_BLOCK, SC_MINB)
       continue;
     }
     while (pos < c1) {
+      if (j0 >= nseg) {  // cannot happen for a consistent segment list
+        if (lane == 0) dev_fail(st, SP_ERR_INTERNAL, -35);
+        break;
+      }
       // segments j0 + lane (the list is closed by the total at nseg)
       const long long j = j0 + lane;
       const long long dst = segs[j < nseg ? j : nseg].dst, src = j < nseg ? segs[j].src : kSegSkip;
@@ -136,6 +145,11 @@ __global__ void __launch_bounds__(SC_BLOCK, SC_MINB)
         const long long d0 = __shfl_sync(0xffffffffu, dst, cur), d1 = __shfl_sync(0xffffffffu, dst, cur + 1);
         const long long s = __shfl_sync(0xffffffffu, src, cur);
         const long long end = d1 < c1 ? d1 : c1;
+        if (d0 > pos || end <= pos) {  // cannot happen for a consistent segment list
+          if (lane == 0) dev_fail(st, SP_ERR_INTERNAL, -31);
+          pos = c1;
+          break;
+        }
         if (s != kSegSkip) {
           const long long from = (s & ~kSegB) + (pos - d0);
           const bool second = (s & kSegB) != 0;

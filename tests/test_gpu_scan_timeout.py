@@ -117,11 +117,11 @@ def test_permute_batch(ctx, kind, columns):
         bt.close()
 
 
-def assign_plan(ctx, A, I, J, B):
+def assign_plan(ctx, A, I, J, B, mode=0):
     plan, nnz = ctypes.c_void_p(), ctypes.c_int64()
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     ctx._check(ctx.lib.sp_assign_count(ctx.handle, ctypes.byref(A.desc()), ctypes.c_void_p(I.data_ptr()), I.numel(),
-                                       ctypes.c_void_p(J.data_ptr()), J.numel(), 0, ctypes.byref(B.desc()), 0,
+                                       ctypes.c_void_p(J.data_ptr()), J.numel(), 0, ctypes.byref(B.desc()), mode,
                                        ctypes.byref(plan), ctypes.byref(nnz), st), "sp_assign_count")
     return plan, nnz.value, st
 
@@ -162,3 +162,28 @@ def test_sort_rows_of_a_bad_row_pointer(ctx, kind, fault):
     P.out.colidx.copy_(torch.from_numpy(O.colidx.astype(np.int32)))
     expect(ctx, "SP_ERR_NOT_CANONICAL", lambda: ctx.sp_sort_rows(P.out))
     P.check()
+
+
+@pytest.mark.parametrize("mode", [0, 1])  # REPLACE: merged beside the copy; SELECT2ND: staged
+@pytest.mark.parametrize("runs", [1, 5])  # of rows of I: segments of one row, of some rows
+def test_assign(ctx, mode, runs):
+    """The segments' scan takes 32 rows a value, tiles of 1024: the timeout needs 2^16 rows."""
+    m = 200_000
+    g = np.random.default_rng(14)
+    O = matrix(g.integers(0, 5, m), 15, 5000)
+    A = from_oracle(O)
+    r = np.arange(m)
+    rows = r[(r // runs) % 2 == 0].astype(np.int32)
+    I, J = torch.from_numpy(rows).cuda(), idx(5000, 34)[:300].contiguous()
+    Bo = matrix(g.integers(0, 4, len(rows)), 16, 300)
+    B = from_oracle(Bo)
+    plan, nnz, st = assign_plan(ctx, A, I, J, B, mode)
+    try:
+        P = Padded(m, 5000, nnz)
+        d = P.out.desc()
+        with held(ctx):
+            expect(ctx, "SP_ERR_TIMEOUT", lambda: ctx._check(ctx.lib.sp_assign_fill(ctx.handle, plan, ctypes.byref(d), st), ""))
+        P.check()
+    finally:
+        ctx.lib.sp_plan_destroy(ctx.handle, plan)
+    assert_same(ctx.sp_assign(A, I, J, B, mode=mode), oracle.assign(O, rows, J.cpu().numpy(), Bo, mode), f"{mode} {runs}")
