@@ -482,6 +482,8 @@ __device__ __forceinline__ uint32_t ss_bucket(uint32_t key, float scale, uint32_
 //                  spans at most 2^9 < SS_RUN_MAX keys: with keys unique within a row it
 //                  holds fewer than SS_RUN_MAX entries and no third split is needed; with
 //                  key_bits <= 22 no coarse bucket can be oversized and it is not launched.
+//                  (Only keys that repeat within a row, which no canonical matrix has, make a
+//                  bucket larger: SP_ERR_INTERNAL, from k_long_hist where no fine split follows.)
 // The runs are then sorted by k_seg_sort.
 constexpr int SL_NBL = 10, SL_NB = 1 << SL_NBL;
 constexpr int SL_HB = 256, SL_HMINB = 5;  // k_long_hist
@@ -492,6 +494,8 @@ constexpr int SF_NBL = 13, SF_B = 512, SF_MINB = 2, SF_U = 4;  // k_split_fine
 constexpr int SS_RUN_LOG = 12;             // SS_RUN_MAX = 2^SS_RUN_LOG
 static_assert((1 << SS_RUN_LOG) == SS_RUN_MAX, "run capacity is a power of two");
 static_assert(32 - SL_NBL - SF_NBL <= SS_RUN_LOG, "fine-split buckets fit a run");
+// whether a coarse bucket can hold more than SS_RUN_MAX distinct keys
+__host__ __device__ constexpr bool fine_split_follows(int key_bits) { return key_bits > SL_NBL + SS_RUN_LOG; }
 constexpr int GROUP_CAP = SS_SMALL_RUN;    // small buckets grouped up to this start window: runs of at most SS_MID_RUN
 // A row's groups: at most one per GROUP_CAP window of starts, one per bucket of more than
 // GROUP_CAP entries and one after each such bucket: 3 L / GROUP_CAP + 1 < L / SL_GSLOT - 1
@@ -656,6 +660,8 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
     split_groups<B, NB>(hist, prv, nxb, tmp32, nb, uint32_t(L), [&](int, bool big, uint32_t s, uint32_t e) {
       if (e - s <= uint32_t(SS_RUN_MAX)) {
         queue_run(sl.runs, FinalEntry{off + s, int(e - s), BUF_TEMP, 0}, st, -6);
+      } else if (!fine_split_follows(key_bits)) {  // repeated keys
+        dev_fail(st, SP_ERR_INTERNAL, -7);
       } else {
         const unsigned q = atomicAdd(nxt_n, 1u);  // the fine split finds its key range itself
         if (q < nxt_cap) nxt[q] = HugeEntry{off + s, (long long)(e - s), 0, BUF_TEMP, 0u, 0, 0};
@@ -1549,7 +1555,7 @@ sp_status split_long(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits,
                                                                        w.gmap, w.cursor, key_bits);
   }
   SP_CUDA(cudaGetLastError());
-  if (key_bits <= SL_NBL + SS_RUN_LOG) return SP_OK;  // a bucket spans at most SS_RUN_MAX keys
+  if (!fine_split_follows(key_bits)) return SP_OK;
   constexpr size_t fsm = split_fine_smem();
   SP_CUDA(set_smem(k_split_fine<CI, VT>, fsm));
   {
