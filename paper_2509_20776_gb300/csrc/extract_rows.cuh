@@ -578,6 +578,7 @@ __global__ void __launch_bounds__(XB, XF_MINB) k_xfill(Src src, long long nI, co
         }
       }
     }
+    __syncwarp();  // the last group's ranks have been read: the rows below write the same buffer
     // rows of 33 to XFAST entries: the warp, XF_ROWS rows at a time
     for (int g = nr1; g < nr; g += R) {
       long long ss[R];
