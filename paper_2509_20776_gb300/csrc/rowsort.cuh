@@ -506,6 +506,16 @@ static_assert(GROUP_CAP == 4 * SL_GSLOT && SS_RUN_MAX > 3 * GROUP_CAP, "cursor s
 // which nothing else uses before the scatter: ceil(L / SL_CH) * SL_NB / 2 <= L words.
 static_assert(SL_CH / (SL_NB / 2) >= 2, "chunk histograms fit the temporary keys");
 
+// The group of bucket 32 w + lane of a long row, minus none before the first: starts = lane's
+// word of the bitmap of the buckets that start a group, before = the starts in earlier words (a
+// warp holds the bitmap, one word per lane).  All lanes call it.
+static_assert(SL_NB == 32 * 32, "a warp holds a row's bitmap");
+__device__ __forceinline__ uint32_t group_of_bucket(uint32_t starts, uint32_t before, int w) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t b = __shfl_sync(0xffffffffu, starts, w), p = __shfl_sync(0xffffffffu, before, w);
+  return p + __popc(b & (0xFFFFFFFFu >> (31 - lane))) - 1u;
+}
+
 // Groups of a split: hist (exclusive starts of nb buckets, SIZE of them scanned, the rest
 // empty; total L) -> a bucket is big, or the head of a group.  All threads of the CTA call
 // it; prv and nxb hold SIZE words.  Afterwards emit(x, big, start, end) is called for every
@@ -558,7 +568,7 @@ __device__ void split_groups(const uint32_t* hist, uint32_t* prv, uint32_t* nxb,
 template <class Gs>
 __global__ void __launch_bounds__(SL_HB, SL_HMINB)
     k_long_hist(Gs gs, SortLists sl, uint32_t* __restrict__ tkey, typename Gs::CI* __restrict__ out_col,
-                uint16_t* __restrict__ gmap, uint32_t* __restrict__ cursor, HugeEntry* __restrict__ nxt,
+                uint32_t* __restrict__ gstart, uint32_t* __restrict__ cursor, HugeEntry* __restrict__ nxt,
                 unsigned* nxt_n, long long nxt_cap, int key_bits, DevStatus* st) {
   using CI = typename Gs::CI;
   constexpr int B = SL_HB, NB = SL_NB, ITEMS = SL_CH / B, H = 4;
@@ -669,19 +679,18 @@ __global__ void __launch_bounds__(SL_HB, SL_HMINB)
       }
     });
     __syncthreads();  // prv has been read
-    // number the groups: group of bucket x = starts at or before x, minus 1
+    // the buckets that start a group, for the scatter, and every group's cursor
+    uint32_t* const gs_bits = gstart + (long long)lc.huge * (NB / 32);
     for (int x = t; x < NB; x += B) {
       const uint32_t a = nxb[NB - 1 - x], b = x + 1 < NB ? nxb[NB - 1 - (x + 1)] : 0u;
-      prv[x] = a != b ? 1u : 0u;  // the suffix minimum changes exactly at a start
+      const uint32_t bits = __ballot_sync(0xffffffffu, a != b);  // the suffix minimum changes exactly at a start
+      if ((x & 31) == 0) prv[x >> 5] = gs_bits[x >> 5] = bits;
     }
     __syncthreads();
-    smem_excl_sum_w<B>(prv, NB, tmp32);
+    const uint32_t starts = prv[t & 31], count = __popc(starts), before = warp_incl_sum(count) - count;
     for (int x = t; x < NB; x += B) {
-      const uint32_t a = nxb[NB - 1 - x], b = x + 1 < NB ? nxb[NB - 1 - (x + 1)] : 0u;
-      const bool start = a != b;
-      const uint32_t g = prv[x] - (start ? 0u : 1u);
-      gmap[(long long)lc.huge * NB + x] = uint16_t(g);
-      if (start) cur[g] = hist[x];
+      const uint32_t g = group_of_bucket(starts, before, x >> 5);
+      if ((prv[x >> 5] >> (x & 31)) & 1u) cur[g] = hist[x];
     }
     __syncthreads();
   }
@@ -695,7 +704,7 @@ template <class Gs>
 __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
     k_long_scatter(Gs gs, SortLists sl, uint32_t* __restrict__ tkey, typename Gs::VT* __restrict__ tval,
                    const typename Gs::CI* __restrict__ out_col, const typename Gs::VT* __restrict__ out_val,
-                   const uint16_t* __restrict__ gmap, uint32_t* __restrict__ cursor, int key_bits) {
+                   const uint32_t* __restrict__ gstart, uint32_t* __restrict__ cursor, int key_bits) {
   using VT = typename Gs::VT;
   constexpr int B = SL_SB, NB = SL_NB, U = SL_CH / B;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -723,9 +732,11 @@ __global__ void __launch_bounds__(SL_SB, sl_sminb<typename Gs::VT>())
     const int len = he.len - e0 < SL_CH ? int(he.len - e0) : SL_CH;
     const VT* vp = out_val + he.off;
     if (!in_place<Gs>::value && he.buf == BUF_SRC) vp = gs.view(gs.srcs()[he.row], he.len).v;
+    const uint32_t starts = gstart[(long long)lc.huge * (NB / 32) + (t & 31)], count = __popc(starts),
+                   before = warp_incl_sum(count) - count;
     for (int x = t; x < NB; x += B) {
       lh[x] = 0;
-      gm[x] = gmap[(long long)lc.huge * NB + x];
+      gm[x] = uint16_t(group_of_bucket(starts, before, x >> 5));
     }
     uint32_t key[U], pk[U];  // group << 16 | rank in the group's share of the chunk
     VT val[U];
@@ -1451,7 +1462,7 @@ struct RowsWs {
   HugeEntry* huge = nullptr;
   HugeEntry* nxt = nullptr;      // oversized buckets (fine split); as many as long rows
   LongChunk* lchunk = nullptr;
-  uint16_t* gmap = nullptr;      // long rows: group of each bucket
+  uint32_t* gstart = nullptr;    // long rows: the buckets that start a group, one bit each
   uint32_t* cursor = nullptr;    // long rows: next free place of each group
   uint32_t* tkey = nullptr;
   void* tval = nullptr;
@@ -1473,12 +1484,12 @@ inline RowsWs rows_caps(long long nrows, long long nnz, bool sort, long long ext
   w.ntiles_cap = (nnz + SsTile::W * nrows) / SsTile::WIN + 1;
   // the split's groups (at most 3 L / GROUP_CAP + 1 of a row, and as many of the fine
   // split's buckets), the rows sorted alone, the tiles' heavy buckets (more than SS_HEAVY
-  // entries each)
+  // entries each); the runs lie apart, so a slice for longer ones is bounded by their length
   const long long groups = nnz > SS_RUN_MAX ? 2 * (3 * (nnz / GROUP_CAP) + nnz / SS_RUN_MAX + 16) : 0;
   w.run_cap[0] = extra_runs > 0 ? groups + extra_runs : 0;
   w.run_cap[1] = groups + nnz / SS_HEAVY + 1;
-  w.run_cap[2] = groups + nnz / SS_SMALL_RUN + 1;
-  w.run_cap[3] = groups + nnz / SS_MID_RUN + 1;
+  w.run_cap[2] = nnz / (SS_SMALL_RUN + 1) + 1;
+  w.run_cap[3] = nnz / (SS_MID_RUN + 1) + 1;
   if (nnz > SS_RUN_MAX) {
     w.huge_cap = nnz / SS_RUN_MAX + 1;
     w.lchunk_cap = nnz / SL_CH + w.huge_cap;
@@ -1500,7 +1511,7 @@ inline void rows_reserve(Carver& cv, long long nrows, long long nnz, size_t vbyt
   off[6] = cv.reserve(need_temp ? size_t(nnz) * 4 : 0);
   off[7] = cv.reserve(need_temp ? size_t(nnz) * vbytes : 0);
   off[8] = cv.reserve(size_t(w.lchunk_cap) * sizeof(LongChunk));
-  off[9] = cv.reserve(size_t(w.huge_cap) * SL_NB * 2);
+  off[9] = cv.reserve(size_t(w.huge_cap) * (SL_NB / 8));
   off[10] = cv.reserve(size_t(w.cur_cap) * 4);
 }
 
@@ -1516,7 +1527,7 @@ inline RowsWs rows_bind(const Carver& cv, long long nrows, long long nnz, const 
   w.tkey = cv.at<uint32_t>(off[6]);
   w.tval = cv.at<void>(off[7]);
   w.lchunk = cv.at<LongChunk>(off[8]);
-  w.gmap = cv.at<uint16_t>(off[9]);
+  w.gstart = cv.at<uint32_t>(off[9]);
   w.cursor = cv.at<uint32_t>(off[10]);
   return w;
 }
@@ -1543,7 +1554,7 @@ sp_status split_long(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits,
   auto grid = [&](long long minb, long long cap) { return unsigned(cap < minb * nsm ? cap : minb * nsm); };
   {
     ::sp::PhaseScope ph(ctx, s, in_place<Gs>::value ? SP_PHASE_HUGE : SP_PHASE_GATHER);
-    k_long_hist<Gs><<<grid(SL_HMINB, w.lchunk_cap), SL_HB, 0, s>>>(gs, sl, w.tkey, out_col, w.gmap, w.cursor, w.nxt,
+    k_long_hist<Gs><<<grid(SL_HMINB, w.lchunk_cap), SL_HB, 0, s>>>(gs, sl, w.tkey, out_col, w.gstart, w.cursor, w.nxt,
                                                                   w.counters + 5, w.huge_cap, key_bits, ctx->dstatus);
   }
   SP_CUDA(cudaGetLastError());
@@ -1552,7 +1563,7 @@ sp_status split_long(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, int key_bits,
   {
     SP_PHASE(SP_PHASE_HUGE);
     k_long_scatter<Gs><<<grid(sl_sminb<VT>(), w.lchunk_cap), SL_SB, ssm, s>>>(gs, sl, w.tkey, tval, out_col, out_val,
-                                                                       w.gmap, w.cursor, key_bits);
+                                                                       w.gstart, w.cursor, key_bits);
   }
   SP_CUDA(cudaGetLastError());
   if (!fine_split_follows(key_bits)) return SP_OK;
