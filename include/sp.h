@@ -139,7 +139,7 @@ SP_API int sp_last_cuda_error(const char** where);
  *   SP_OPT_TILE_SHAPE      row sort of short rows: 0 = tiles of 1024 entries holding rows
  *                          of at most 512, 256 threads, 5 CTAs per SM (default);
  *                          1 = tiles of 2048 entries holding rows of at most 1024,
- *                          256 threads, 4 CTAs per SM;
+ *                          256 threads, 4 CTAs per SM (3 with 8-byte values);
  *   SP_OPT_HEAVY           a bucket of the row sort with more keys than this is sorted
  *                          over its own key range: bucketed again in place by a row that
  *                          is sorted alone, queued as such a run by a tile: 128 (default)

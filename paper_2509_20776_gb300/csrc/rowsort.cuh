@@ -45,7 +45,7 @@ struct SsCfg {
 // 4 CTAs 18.4, 128 x 8 at 8 CTAs 24.0, 64 x 16 31 (longer unrolled code, and the lookups of a
 // thread in flight at once evict one another's lines from the L1 that shared memory leaves).
 using SsTile = SsCfg<256, 4, 5, true>;   // tiles of rows of at most 512 entries
-using SsTileL = SsCfg<256, 8, 4, true>;  // tile shape 1: rows of at most 1024 entries
+using SsTileL = SsCfg<256, 8, 4, true>;  // tile shape 1: rows of at most 1024 entries (8-byte values: 3 CTAs)
 using SsRun = SsCfg<512, 8, 2>;          // single runs of at most 4096 entries
 using SsRunM = SsCfg<256, 8, 4>;         // of at most 2048
 using SsRunS = SsCfg<256, 4, 5>;         // of at most 1024
@@ -888,6 +888,16 @@ __host__ __device__ constexpr size_t ss_smem_bytes() {
          (Cfg::kTiles ? size_t(Cfg::ROWS) * 32 + size_t(Cfg::WORDS) * 8 : 0);
 }
 
+// Resident CTAs per SM: MINB, or as many as their shared memory leaves room for (228 KB per SM,
+// 1 KB of it per CTA for the system; the arrays above and the kernel's own).  Tile shape 1 with
+// 8-byte values holds 3, not 4.
+template <class Cfg, class VT>
+constexpr int ss_minb() {
+  const size_t per = ss_smem_bytes<Cfg, VT>() + (Cfg::kTiles ? size_t(Cfg::ROWS + 1) * 16 : 0) + 256 + 1024;
+  const int fit = int(228 * 1024 / per);
+  return fit < Cfg::MINB ? fit : Cfg::MINB;
+}
+
 struct SsRow {     // a tile's row (one 16-byte word)
   uint32_t rdel;   // output offset from base - packed start
   uint32_t ps_L;   // packed start | length << 16
@@ -980,7 +990,7 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms (17.2 with the
 // long rows split chunk by chunk and the partition part of the scan).
 template <class Cfg, class Gs>
-__global__ void __launch_bounds__(Cfg::B, Cfg::MINB)
+__global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
     k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nrows, long long nnz,
                const long long* __restrict__ tile_first, long long ntiles,
                RunLists rl, int slice, const uint32_t* __restrict__ tkey_g,
@@ -1589,7 +1599,7 @@ sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz,
     constexpr size_t sm = ss_smem_bytes<Cfg, VT>();
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_LONG);
-    const long long cap = (long long)Cfg::MINB * ctx->num_sms, n = slice >= 0 ? w.run_cap[slice] : w.runs_total();
+    const long long cap = (long long)ss_minb<Cfg, VT>() * ctx->num_sms, n = slice >= 0 ? w.run_cap[slice] : w.runs_total();
     k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, 0, nullptr, 0, w.runs(), slice, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
@@ -1664,7 +1674,7 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
     constexpr size_t sm = ss_smem_bytes<Cfg, VT>();
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_TILE);
-    const long long cap = (long long)Cfg::MINB * nsm, g = ntiles < cap ? ntiles : cap;
+    const long long cap = (long long)ss_minb<Cfg, VT>() * nsm, g = ntiles < cap ? ntiles : cap;
     k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nrows, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
