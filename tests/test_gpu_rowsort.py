@@ -110,3 +110,41 @@ def test_repeated_row_in_p_stays_inside(ctx):
         ctx.sp_permute(A, p, q, out=out)
     assert e.value.name == "SP_ERR_NOT_PERMUTATION"
     assert bool((col[A.nnz:] == 7).all()) and bool((val[A.nnz:] == 7.0).all())
+
+
+LARGE = EDGES * 5  # more entries than one launch for all runs takes: each run by the kernel of its length
+
+
+@pytest.mark.parametrize("vt", [np.float32, np.float64])
+@pytest.mark.parametrize("skew", [False, True])  # (the identity keeps the columns crowded: heavy buckets)
+@pytest.mark.parametrize("tile_shape", [0, 1])
+def test_permute_runs_by_length(ctx, tile_shape, skew, vt):
+    assert sum(LARGE) > 1 << 17
+    A = matrix(LARGE, skew, vt, 8)
+    g = np.random.default_rng(9)
+    p = g.permutation(A.nrows).astype(np.int32)
+    q = (np.arange(N) if skew else g.permutation(N)).astype(np.int32)
+    ctx.set_shapes(tile_shape=tile_shape)
+    try:
+        B = ctx.sp_permute(from_oracle(A), torch.from_numpy(p).cuda(), torch.from_numpy(q).cuda())
+    finally:
+        ctx.set_shapes(tile_shape=-1)
+    assert_same(B, oracle.permute(A, p, q), f"{tile_shape} {skew}")
+
+
+@pytest.mark.parametrize("vt", [np.float32, np.float64])
+@pytest.mark.parametrize("skew", [False, True])
+@pytest.mark.parametrize("tile_shape", [0, 1])
+def test_sort_runs_in_place_by_length(ctx, tile_shape, skew, vt):
+    A = matrix(LARGE, skew, vt, 10)
+    g = np.random.default_rng(11)
+    M = from_oracle(A)
+    order = np.concatenate([b + g.permutation(e - b) for b, e in zip(A.rowptr[:-1], A.rowptr[1:])])
+    order = torch.from_numpy(order).cuda()
+    M.colidx, M.values = M.colidx[order].contiguous(), M.values[order].contiguous()
+    ctx.set_shapes(tile_shape=tile_shape)
+    try:
+        ctx.sp_sort_rows(M)
+    finally:
+        ctx.set_shapes(tile_shape=-1)
+    assert_same(M, A, f"{tile_shape} {skew}")
