@@ -454,13 +454,6 @@ struct MergeSrc {
   __device__ bool in_j(long long c) const { return (ld_map(jbits + (c >> 5)) >> (c & 31)) & 1u; }
 };
 
-// First output position of rebuilt row i: in A' itself (vdst = A''s row pointer, row I[i])
-// or in the staging buffer (vdst null, row pointer vp of the rebuilt rows).
-template <class IX>
-__device__ __forceinline__ long long merge_out(const long long* vdst, const IX* I, const long long* vp, long long i) {
-  return vdst ? vdst[(long long)I[i]] : vp[i];
-}
-
 // Rows whose run of A has at most SRC_LONG entries, a warp each.  A warp takes 32 rows: lane l
 // resolves row i0 + l (runs and output place), so the index chains of 32 rows are in flight
 // together, and a row's B entries and first 32 A entries are loaded while the row before it
@@ -487,7 +480,7 @@ __global__ void __launch_bounds__(256, 4) k_assign_merge_warp(MergeSrc<RP, CI, V
       if (LA <= SRC_LONG) {  // else k_assign_merge_long (the count listed it)
         nA = int(LA);
         nB = int(LB);        // (at most 32: the fill's choice of this path)
-        ro = merge_out(vdst, ms.I, vp, i);
+        ro = vdst[(long long)ms.I[i]];
         nout = int(vp[i + 1] - vp[i]);
       }
     }
@@ -590,7 +583,7 @@ __global__ void __launch_bounds__(1024) k_assign_merge_long(MergeSrc<RP, CI, VT,
     const long long i = cl_rows[item];
     long long sA, LA, sB, LB;
     ms.rows(i, sA, LA, sB, LB);
-    const long long o = merge_out(vdst, ms.I, vp, i), oe = o + (vp[i + 1] - vp[i]);
+    const long long o = vdst[(long long)ms.I[i]], oe = o + (vp[i + 1] - vp[i]);
     uint32_t bk;
     VT bv;
     const int nb = ms.load_b(sB, LB, bk, bv);

@@ -31,8 +31,6 @@ __host__ __device__ __forceinline__ int ceil_log2_u64(uint64_t x) {
 #endif
 }
 
-__device__ __forceinline__ int ceil_log2_u32(uint32_t x) { return x <= 1 ? 0 : 32 - __clz(x - 1); }
-
 // ---- cache-hinted loads ------------------------------------------------------
 // Streaming data (column indices and values read once) is loaded with an L1
 // no-allocate hint so that the L1/L2 capacity stays with the index maps, which are
@@ -99,18 +97,6 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
   const unsigned d = unsigned(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
-// 16-byte and single-word global -> shared copies (16-byte: both addresses 16-byte aligned)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const unsigned d = unsigned(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-}
-template <int BYTES>
-__device__ __forceinline__ void cp_async_word(void* dst, const void* src) {
-  static_assert(BYTES == 4 || BYTES == 8, "4- or 8-byte words");
-  const unsigned d = unsigned(__cvta_generic_to_shared(dst));
-  if constexpr (BYTES == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -174,112 +160,6 @@ __device__ __forceinline__ T block_excl_sum(T v, T* tmp, T* total) {
   *total = tmp[NW];
   __syncthreads();
   return res;
-}
-
-template <int BLOCK, class T>
-__device__ __forceinline__ T block_incl_max(T v, T* tmp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int NW = BLOCK / 32;
-  T inc = warp_incl_max(v);
-  if (lane == 31) tmp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    T w = lane < NW ? tmp[lane] : T(0);
-    T wi = warp_incl_max(w);
-    // exclusive max of warp totals
-    T ex = __shfl_up_sync(0xffffffffu, wi, 1);
-    if (lane == 0) ex = T(0);
-    if (lane < NW) tmp[lane] = ex;
-  }
-  __syncthreads();
-  T pre = tmp[warp];
-  T res = pre > inc ? pre : inc;
-  __syncthreads();
-  return res;
-}
-
-// In-place exclusive sum over a shared array a[0..n), n <= BLOCK*ITEMS.  Each thread
-// owns ITEMS consecutive entries.  Returns the total.
-template <int BLOCK, int ITEMS>
-__device__ __forceinline__ uint32_t smem_excl_sum(uint32_t* a, int n, uint32_t* tmp) {
-  const int t = threadIdx.x;
-  uint32_t v[ITEMS];
-  uint32_t s = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    int x = t * ITEMS + j;
-    v[j] = x < n ? a[x] : 0u;
-    s += v[j];
-  }
-  uint32_t total;
-  uint32_t run = block_excl_sum<BLOCK>(s, tmp, &total);
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    int x = t * ITEMS + j;
-    if (x < n) a[x] = run;
-    run += v[j];
-  }
-  __syncthreads();
-  return total;
-}
-
-// In-place inclusive max over a shared array a[0..n), n <= BLOCK*ITEMS.
-template <int BLOCK, int ITEMS>
-__device__ __forceinline__ void smem_incl_max(uint32_t* a, int n, uint32_t* tmp) {
-  const int t = threadIdx.x;
-  uint32_t v[ITEMS];
-  uint32_t m = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    int x = t * ITEMS + j;
-    v[j] = x < n ? a[x] : 0u;
-    m = v[j] > m ? v[j] : m;
-  }
-  // exclusive max of thread maxima
-  uint32_t incl = block_incl_max<BLOCK>(m, tmp);
-  uint32_t prev = __shfl_up_sync(0xffffffffu, incl, 1);
-  // the exclusive value of lane 0 of each warp comes from the previous warp's total;
-  // recompute it through shared memory
-  __shared__ uint32_t warp_last[BLOCK / 32];
-  if ((t & 31) == 31) warp_last[t >> 5] = incl;
-  __syncthreads();
-  if ((t & 31) == 0) prev = (t >> 5) ? warp_last[(t >> 5) - 1] : 0u;
-  uint32_t run = prev;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    int x = t * ITEMS + j;
-    run = v[j] > run ? v[j] : run;
-    if (x < n) a[x] = run;
-  }
-  __syncthreads();
-}
-
-// In-place inclusive max over a shared array of 16-bit values a[0..n), n <= BLOCK*ITEMS.
-template <int BLOCK, int ITEMS>
-__device__ __forceinline__ void smem_incl_max16(uint16_t* a, int n, uint32_t* tmp) {
-  const int t = threadIdx.x;
-  uint32_t v[ITEMS];
-  uint32_t m = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const int x = t * ITEMS + j;
-    v[j] = x < n ? a[x] : 0u;
-    m = v[j] > m ? v[j] : m;
-  }
-  const uint32_t incl = block_incl_max<BLOCK>(m, tmp);
-  uint32_t prev = __shfl_up_sync(0xffffffffu, incl, 1);
-  __shared__ uint32_t warp_last16[BLOCK / 32];
-  if ((t & 31) == 31) warp_last16[t >> 5] = incl;
-  __syncthreads();
-  if ((t & 31) == 0) prev = (t >> 5) ? warp_last16[(t >> 5) - 1] : 0u;
-  uint32_t run = prev;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    const int x = t * ITEMS + j;
-    run = v[j] > run ? v[j] : run;
-    if (x < n) a[x] = uint16_t(run);
-  }
-  __syncthreads();
 }
 
 }  // namespace sp

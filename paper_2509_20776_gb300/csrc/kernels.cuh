@@ -137,8 +137,6 @@ struct CountLists {
   long long* cl_rows;  // source-long rows waiting for k_count_long
   unsigned* n_cl;
   long long cl_cap;
-  long long* rs0 = nullptr;  // when given: source start and length of every listed row
-  long long* rsn = nullptr;  //   (single-run loaders), for a fill that reads them back
 };
 
 __device__ __forceinline__ void push_row(long long* list, unsigned* n, long long cap, long long r,
@@ -191,10 +189,6 @@ __global__ void k_count_warp(Ct ct, long long nlisted, long long* __restrict__ c
       const long long i = i0 + u;
       const bool mine = u < rb && i < nlisted;
       rs[u] = mine ? ct.row(i) : RowSrc{0, 0, 0, 0};
-      if (cl.rs0 && lane == 0 && mine) {
-        cl.rs0[i] = rs[u].s0;
-        cl.rsn[i] = rs[u].n0;
-      }
       Ls[u] = rs[u].n0 + rs[u].n1;
       lng[u] = row_is_long<Ct>(rs[u]);
       bt.valid[u] = !lng[u] && lane < Ls[u];

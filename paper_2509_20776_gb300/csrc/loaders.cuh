@@ -100,16 +100,6 @@ struct Batch {
 
 constexpr int LOAD_U = 4;  // entries per thread per batch
 
-// A loader whose rows come from arrays recorded by the count pass (source start and
-// length of every listed row: one contiguous read instead of the index -> row pointer
-// chain), with every survival test and relabel of the underlying single-run loader.
-template <class Ld>
-struct RecordedRows : Ld {
-  const long long* rs0;
-  const long long* rsn;
-  __device__ __forceinline__ RowSrc row(long long i) const { return RowSrc{rs0[i], 0, rsn[i], 0}; }
-};
-
 // A loader view for counting passes: membership only (no key, no value loads).
 template <class Ld>
 struct CountOnly {

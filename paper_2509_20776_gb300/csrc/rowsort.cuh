@@ -50,7 +50,6 @@ using SsRun = SsCfg<512, 8, 2>;          // single runs of at most 4096 entries
 using SsRunM = SsCfg<256, 8, 4>;         // of at most 2048
 using SsRunS = SsCfg<256, 4, 5>;         // of at most 1024
 constexpr int SS_SMALL_RUN = SsRunS::CAP, SS_MID_RUN = SsRunM::CAP;
-constexpr int SS_TILE_MAX = SsTile::TMAX;  // longest row a tile accepts (the smaller tile shape)
 constexpr int SS_RUN_MAX = 4096;           // longest row sorted alone
 constexpr long long SS_ONE_LAUNCH = 1 << 17;  // sorts of at most this many entries take one launch for all runs
 static_assert(SsRun::CAP == SS_RUN_MAX, "run capacity");
