@@ -45,7 +45,7 @@ constexpr int xc_lane() { return sizeof(CI) == 4 ? 16 : 8; }  // rows a lane cou
 // Rows of at most 32 entries whose kept entries a filling warp loads together.  Measured at 4
 // CTAs per SM (Erdos-Renyi 2^25 x 32, half of rows and columns / 3000 batched requests):
 // 3 rows 4.77 / 2.42 ms per fill, 4 rows 4.68 / 2.64, 2 rows 5.43 / 2.38; 5 CTAs with 4 or 2
-// rows 5.33 and 5.78, 3 CTAs 6.24 (the start's fill, which tested every entry: 5.65 / 2.75).
+// rows 5.33 and 5.78, 3 CTAs 6.24 (a fill that tests every entry again, without masks: 5.65 / 2.75).
 template <class VT>
 constexpr int xf_rows1() { return sizeof(VT) == 4 ? 3 : 2; }
 constexpr int XF_MINB = 4;

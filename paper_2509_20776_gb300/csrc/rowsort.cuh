@@ -439,19 +439,18 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
 }
 
 // ---- approximate square-root bucketing of the row sort -----------------------------------
-// Bucket of key k in a row of L entries: nb = 2^(ceil(log2 L) - 1) buckets spaced evenly
-// in an approximate square root of k over the row's key range [0, kmax].  The root is
-// the exponent-halving bit trick on the float of k (exact at even powers of two, up to
-// 6% high in between): monotone in k (every step is), so buckets stay in key order; the
-// scale nb / root(kmax) maps [0, kmax] onto the nb buckets.  The square root keeps
-// buckets balanced both for uniformly relabelled columns and for labels crowded at the
-// low end (degree-descending orderings).
+// Bucket of key k in a row of L entries: L buckets spaced evenly in an approximate square
+// root of k over the row's key range [0, kmax].  The root is the exponent-halving bit trick
+// on the float of k (exact at even powers of two, up to 6% high in between): monotone in k
+// (every step is), so buckets stay in key order; the scale L / root(kmax) maps [0, kmax]
+// onto the L buckets.  The square root keeps buckets balanced both for uniformly relabelled
+// columns and for labels crowded at the low end (degree-descending orderings).
 __device__ __forceinline__ float ss_root(uint32_t k) {
   return __uint_as_float((__float_as_uint(__uint2float_rn(k)) >> 1) + 0x1FC00000u);
 }
-// 1 / root(kmax): the scale of a range [0, kmax] is nb * ss_inv_root(kmax)
+// 1 / root(kmax): the scale of a range [0, kmax] over L buckets is L * ss_inv_root(kmax)
 __device__ __forceinline__ float ss_inv_root(uint32_t kmax) { return kmax ? 1.0f / ss_root(kmax) : 0.0f; }
-// bucket of `key` given the row's scale and last bucket nb - 1
+// bucket of `key` given the row's scale and last bucket L - 1
 __device__ __forceinline__ uint32_t ss_bucket(uint32_t key, float scale, uint32_t last) {
   const uint32_t b = __float2uint_rz(ss_root(key) * scale);
   return b < last ? b : last;
@@ -970,8 +969,8 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // The bucket sort: an entry's bucket counter (shared memory) returns its arrival number,
 // one block scan turns the counters into bucket starts, the entry's key is put at start +
 // arrival, and its owner (the thread that loaded it, which keeps key and bucket in
-// registers) ranks it among its bucket's keys, two on average.  Keys then go to their
-// sorted position with the index of their value, and both are written coalesced.
+// registers) ranks it among its bucket's keys, one on average.  Keys and
+// values then go to their sorted position in shared memory and are written coalesced.
 // A bucket of more than `heavy` keys (skewed keys): a tile writes it in bucket order and
 // queues it as a run; a run buckets it again over its own key range, in the counters of
 // its own positions, for up to SS_LEVELS levels (the last ranks whatever is left).
@@ -980,14 +979,16 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // own position, which no bucket uses, so it passes through the sort in place and every pass
 // runs without a bounds check; only loads and stores look at the length.
 //
-// What bounds it: shared-memory wavefronts and issue slots (a profile of a tile sort of
-// 512-entry rows: 80 % of the LSU data pipe, 53 % of issue, 15 % of DRAM), and for a matrix
-// whose column map exceeds L2 the random lookups.  So the gather is part of the sort (one
+// What bounds it: shared-memory wavefronts and issue slots (profiles of a tile sort: rows of
+// 512 entries 80 % of the LSU data pipe, 53 % of issue, 22 % of the DRAM copy rate; 2 M random
+// rows of R-MAT scale 25, where the lookups miss L2, 58, 52 and 27 %), and for a matrix whose
+// column map exceeds L2 the random lookups.  So the gather is part of the sort (one
 // pass over the entries instead of two), an entry stays with its thread from load to
 // staging, and buckets hold one key on average.  Uniform rows of 32 over 2^25 columns: 25.8
 // -> 16.4 ms per permutation, of which the lookups alone take 12.9 in a plain gather; rows
 // of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms (17.2 with the
-// long rows split chunk by chunk and the partition part of the scan).
+// long rows split chunk by chunk and the partition part of the scan, 17.4 since tiles and
+// rows are checked against a row pointer that does not ascend).
 template <class Cfg, class Gs>
 __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
     k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nrows, long long nnz,

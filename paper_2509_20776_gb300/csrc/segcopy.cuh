@@ -8,7 +8,7 @@
 // A warp takes SC_CH output positions at a time; its lanes hold the next 32 segments.  Inside
 // a segment it moves sc_u() x 32 entries per step, all loads before any store: source and
 // destination differ in alignment by an arbitrary number of entries, so words of one entry
-// with eight of each array in flight per lane keep more bytes on the way than 16-byte words
+// with sc_u() of each array in flight per lane keep more bytes on the way than 16-byte words
 // realigned in registers, one group per thread behind a search for its segment.
 //
 // Where the held segments are short (less than 16 sc_u() entries each: rows of I side by side),
@@ -37,7 +37,7 @@ template <class CI, class VT>
 constexpr int sc_u() { return sizeof(CI) + sizeof(VT) == 8 ? 4 : 2; }  // entries of each array in flight per lane
 // Persistent grid, CTAs per SM: alone, and while the merge shares the SMs.  R-MAT scale 25,
 // 789 M entries, whole assignment: 4 entries at 8 / 3 CTAs 4.62 ms, 8 at 5 / 3 4.69, 8 at 5 / 2
-// 4.84, 6 at 6 / 2 5.12 (the start's copy by aligned 16-byte words: 5.28).
+// 4.84, 6 at 6 / 2 5.12 (16-byte words realigned in registers: 5.28).
 constexpr int SC_MINB = 8, SC_MINB_OVERLAP = 3;
 
 // Which segment holds the first position of every chunk: the chunk's row (recorded by the
