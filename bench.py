@@ -36,11 +36,14 @@ UNIT = "output nnz/s"
 WORKLOAD = ("R-MAT scale {scale} (a,b,c,d)=(0.57,0.19,0.19,0.05), edge factor 16, symmetrised; "
             "P A P^T random p + P A P^T degree-descending p + P A Q^T random p,q")
 
-# DRAM bytes (read + write) per output entry of one launch of a gather that moves every
-# entry, from a capture; None: the permutation's sorts read their source rows themselves,
-# and no capture of them at the workload's size is kept.
+# DRAM bytes (read + write) per entry that the sorts of a permutation handle, by phase: all
+# launches of a phase over the entries it sorts, averaged over the three permutations of the
+# headline workload (profiles/permute_dram_rmat25.md).  Only valid for that matrix and the
+# kernels as captured: retake the capture when they change.
+SORT_DRAM_ROWS = 1 << 25
+SORT_DRAM_BYTES_PER_ENTRY = {"tile": 30.50, "long": 18.68}
+# the same of a gather that moves every entry (no permutation of the workload runs one)
 GATHER_DRAM_BYTES_PER_ENTRY = None
-
 
 _T0 = time.time()
 
@@ -271,6 +274,9 @@ def roofline_permute(stats, classes, m, n, ops_per_step, steps, peak_gbs, lookup
         out["frac_incl_lookup"] = round(with_lookup / peak_gbs, 4)
         if GATHER_DRAM_BYTES_PER_ENTRY is not None and not fused:
             out["traffic"] = int(GATHER_DRAM_BYTES_PER_ENTRY * nnz)
+        if fused and m == SORT_DRAM_ROWS and ph in SORT_DRAM_BYTES_PER_ENTRY:
+            entries = {"tile": e_tile, "long": e_long + e_huge}[ph]
+            out["traffic"] = int(SORT_DRAM_BYTES_PER_ENTRY[ph] * entries)
         if lookup_peak:
             rate = lookups[ph] * launches_total / sec
             out["lookup_roofline"] = {"achieved": round(rate / 1e9, 2), "peak": lookup_peak["g_per_s"],

@@ -76,3 +76,28 @@ def test_latency_stats():
     assert abs(s["p50_ms"] - 50.5) < 1e-6 and abs(s["mean_ms"] - 50.5) < 1e-6
     assert 99.0 <= s["p99_ms"] <= 100.0
     assert abs(s["span_s"] - (0.99 + 0.1)) < 1e-9
+
+
+def test_roofline_of_the_fused_sorts():
+    """The sorts read their source rows themselves: "gather" is the long rows' histogram pass,
+    and each phase's lookups and traffic are those of the rows it reads."""
+    classes = {"tile": (400, 10), "long": (300, 2), "huge": (200, 1)}
+    lk = {"g_per_s": 100.0, "table_bytes": 400, "probe": "x"}
+
+    def roof(m, **ms):
+        return bench.roofline_permute({k: (v, 6) for k, v in ms.items()}, classes, m, 50, 3, 2, 1000.0, lk,
+                                      concurrent=("gather", "huge"), fused=True)
+
+    r = roof(100, tile=3.0, long=2.0, gather=9.0, huge=8.0)
+    assert r["phase"] == "tile" and r["kernel"] == "k_seg_sort<SsTile>"
+    assert r["alg_bytes_per_launch"] == 16 * 400 + 24 * 100
+    assert r["lookup_roofline"]["achieved"] == round(400 * 6 / 3e-3 / 1e9, 2)
+    assert r["traffic"] is None  # not the captured matrix
+    m = bench.SORT_DRAM_ROWS
+    r = roof(m, tile=3.0, long=2.0)
+    assert r["traffic"] == int(bench.SORT_DRAM_BYTES_PER_ENTRY["tile"] * 400)
+    r = roof(m, tile=1.0, long=2.0)
+    assert r["phase"] == "long" and r["alg_bytes_per_launch"] == 16 * 500 + 24 * 2
+    assert r["traffic"] == int(bench.SORT_DRAM_BYTES_PER_ENTRY["long"] * 500)
+    r = bench.roofline_permute({"gather": (1.0, 6)}, classes, 100, 50, 3, 2, 1000.0, lk, fused=True)
+    assert r["kernel"] == "k_long_hist" and r["alg_bytes_per_launch"] == 8 * 200
