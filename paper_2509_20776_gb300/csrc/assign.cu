@@ -1035,12 +1035,13 @@ sp_status assign_permute_impl(sp_ctx* ctx, sp_plan* pl, const IX* p, const IX* q
   RowsWs w = rows_bind(cv, m, nnz_out, ro);
   w.counters = cv.at<unsigned>(o_cnt);
   const RowsPartition part = sort_partition(ctx, w, m, nnz_out, BUF_SRC);
+  unsigned* const bad = w.counters + RUNS_BAD;
   if (out64) {
     SP_TRY(launch_scan(ctx, s, len, StorePartition<long long>{vp, nullptr, part, ctx->dstatus}, m, cv.at<char>(o_scan),
-                       SP_PHASE_SCAN, true));
+                       SP_PHASE_SCAN, true, bad));
   } else {
     SP_TRY(launch_scan(ctx, s, len, StorePartition<int32_t>{vp, static_cast<int32_t*>(out->rowptr), part, ctx->dstatus},
-                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
+                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true, bad));
   }
   if (nnz_out == 0) return SP_OK;
   const FusedGs<CI, VT, IX> g{static_cast<const CI*>(A.colidx), static_cast<const VT*>(A.values), tcol, tval,

@@ -361,7 +361,7 @@ sp_status extract_fill_impl(sp_ctx* ctx, sp_plan* pl, sp_csr* B, cudaStream_t s)
                                    pl->sstart, pl->j0};
     const RowsWs w = rows_bind(cv, nI, nnz_out, ro, false);
     SP_TRY(launch_partition(ctx, s, gather_partition(ctx, w, nI, nnz_out), pl->vp));
-    return gather_rows(ctx, s, pl->vp, nI, nnz_out, w, g, oc, ov);
+    return gather_rows(ctx, s, pl->vp, nI, nnz_out, w, nullptr, g, oc, ov);
   }
   if (pl->j_shape == 3) {
     // repeated J: every kept entry once per position of its column, then the row sort

@@ -37,7 +37,6 @@ struct alignas(16) PermView {
   unsigned long long val;   // const VT*
   unsigned long long qinv;  // const IX*: the request's inverse column map (0: identity)
   unsigned long long ncol;
-  unsigned long long nnz, pad;
   // a pair of its words at once
   __device__ __forceinline__ ulonglong2 arrays() const { return __ldg(reinterpret_cast<const ulonglong2*>(&col)); }
   __device__ __forceinline__ ulonglong2 map() const { return __ldg(reinterpret_cast<const ulonglong2*>(&qinv)); }
@@ -153,12 +152,10 @@ struct PermBatchGs {
   const PermView* pv;
   const long long* rsrc;
   __device__ const long long* srcs() const { return rsrc; }
-  // (the length comes from the row pointer, which a scan's timeout leaves inconsistent)
-  __device__ GsView<CI, VT> view(long long src, long long L) const {
+  __device__ GsView<CI, VT> view(long long src, long long) const {
     const PermView* v = pv + (src >> kReqShift);
     const long long e = src & kEntryMask;
     const ulonglong2 a = v->arrays();
-    if ((unsigned long long)(e + L) > __ldg(&v->nnz)) return {};
     return {reinterpret_cast<const CI*>(a.x) + e, reinterpret_cast<const VT*>(a.y) + e, unsigned(src >> kReqShift)};
   }
   __device__ uint32_t map(unsigned mid, uint32_t c) const {
@@ -250,14 +247,15 @@ sp_status pbatch_fill_impl(sp_ctx* ctx, sp_pbatch* b, sp_csr* out, cudaStream_t 
   w.counters = cv.at<unsigned>(b->o_cnt);
   const RowsPartition part = sort ? sort_partition(ctx, w, rows, nnz, BUF_SRC) : gather_partition(ctx, w, rows, nnz);
   // row pointer of the batch: scan of the row lengths, mirrored into the output's type
+  unsigned* const bad = w.counters + RUNS_BAD;
   if (out->rowptr_type == SP_I64) {
     SP_TRY(launch_scan(ctx, s, LoadArray<long long>{rsn},
                        StoreCapped<long long>{vp, static_cast<long long*>(out->rowptr), rows, nnz, part, ctx->dstatus},
-                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true));
+                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true, bad));
   } else {
     SP_TRY(launch_scan(ctx, s, LoadArray<long long>{rsn},
                        StoreCapped<int32_t>{vp, static_cast<int32_t*>(out->rowptr), rows, nnz, part, ctx->dstatus},
-                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true));
+                       rows, cv.at<char>(b->o_scan), SP_PHASE_SCAN, true, bad));
   }
   if (nnz == 0 || rows == 0) return SP_OK;
   CI* oc = static_cast<CI*>(out->colidx);
@@ -265,7 +263,7 @@ sp_status pbatch_fill_impl(sp_ctx* ctx, sp_pbatch* b, sp_csr* out, cudaStream_t 
   // gather + relabel over the whole batch; with any column map also the row sort
   const int kb = ceil_log2_u64(uint64_t(b->max_cols > 1 ? b->max_cols : 1));
   const PermBatchGs<CI, VT, IX> g{views, rsrc};
-  if (!sort) return gather_rows(ctx, s, vp, rows, nnz, w, g, oc, ov);
+  if (!sort) return gather_rows(ctx, s, vp, rows, nnz, w, bad, g, oc, ov);
   return sort_rows_from(ctx, s, vp, rows, nnz, kb, w, g, oc, ov);
 }
 
@@ -363,7 +361,7 @@ extern "C" sp_status sp_permute_batch_plan(sp_ctx* ctx, const sp_csr* mats, int6
       const sp_csr& a = mats[r.mat];
       b->hview[size_t(k)] = PermView{(unsigned long long)a.colidx, (unsigned long long)a.values,
                                      r.q ? (unsigned long long)(qbase + size_t(r.qoff) * is) : 0ull,
-                                     (unsigned long long)a.ncols, (unsigned long long)a.nnz, 0ull};
+                                     (unsigned long long)a.ncols};
     }
   }
   sp_status st = upload(cv.at<char>(b->o_req), b->hreq.data(), size_t(nreq) * sizeof(PermReq), s);

@@ -45,12 +45,9 @@ struct PermGs {
   const VT* v_;
   const IX* qinv;           // old column -> new column (null: identity)
   const long long* sstart;  // source start of output row r
-  long long n, nnz;
+  long long n;
   __device__ const long long* srcs() const { return sstart; }
-  // (the length comes from the row pointer, which a scan's timeout leaves inconsistent)
-  __device__ GsView<CI, VT> view(long long src, long long L) const {
-    return src + L <= nnz ? GsView<CI, VT>{c_ + src, v_ + src, 0u} : GsView<CI, VT>{};
-  }
+  __device__ GsView<CI, VT> view(long long src, long long) const { return {c_ + src, v_ + src, 0u}; }
   __device__ uint32_t map(unsigned, uint32_t c) const {  // (a sort follows only a column permutation: n > 0)
     return c > uint32_t(n - 1) ? 0xFFFFFFFFu : uint32_t(ld_map(qinv + c));
   }
@@ -105,20 +102,21 @@ sp_status permute_impl(sp_ctx* ctx, const sp_csr* A, const IX* p, const IX* q, s
   long long* sstart = cv.at<long long>(o_ss);
   PermLen<RP, IX> len{static_cast<const RP*>(A->rowptr), p, m, nnz, sstart};
   RowsPartition part = sort ? sort_partition(ctx, w, m, nnz, BUF_SRC) : gather_partition(ctx, w, m, nnz);
+  unsigned* const bad = w.counters + RUNS_BAD;
   if (out64) {
     SP_TRY(launch_scan(ctx, s, len, StorePartition<long long>{vp, nullptr, part, ctx->dstatus}, m,
-                       cv.at<char>(o_scan), SP_PHASE_SCAN, true));
+                       cv.at<char>(o_scan), SP_PHASE_SCAN, true, bad));
   } else {
     SP_TRY(launch_scan(ctx, s, len, StorePartition<int32_t>{vp, static_cast<int32_t*>(B->rowptr), part, ctx->dstatus},
-                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true));
+                       m, cv.at<char>(o_scan), SP_PHASE_SCAN, true, bad));
   }
   if (nnz == 0 || m == 0) return SP_OK;
   CI* out_col = static_cast<CI*>(B->colidx);
   VT* out_val = static_cast<VT*>(B->values);
   // gather and relabel; with a column permutation also sort every row
   const PermGs<CI, VT, IX> g{static_cast<const CI*>(A->colidx), static_cast<const VT*>(A->values), qinv,
-                             sstart, n, nnz};
-  if (!sort) return gather_rows(ctx, s, vp, m, nnz, w, g, out_col, out_val);
+                             sstart, n};
+  if (!sort) return gather_rows(ctx, s, vp, m, nnz, w, bad, g, out_col, out_val);
   return sort_rows_from(ctx, s, vp, m, nnz, ceil_log2_u64(uint64_t(n)), w, g, out_col, out_val);
 }
 

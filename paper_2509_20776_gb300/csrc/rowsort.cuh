@@ -70,9 +70,10 @@ struct FinalEntry {  // a run of at most SS_RUN_MAX entries left to sort
 // them on), of at most SS_SMALL_RUN, SS_MID_RUN, SS_RUN_MAX entries a CTA of SsRunS,
 // SsRunM, SsRun -- each with its own count and bound.
 constexpr int SS_WARP_RUN = 128;
+constexpr int RUNS_BAD = 8;    // of the counters: the row pointer does not ascend (RowsPartition)
 struct RunLists {
   FinalEntry* list;
-  unsigned* n;               // 4 counts
+  unsigned* n;               // 4 counts (the first of the counters)
   long long c0, c1, c2, c3;  // capacity of each slice
   __device__ __forceinline__ FinalEntry* slice(int k) const { return list + (k > 0 ? c0 : 0) + (k > 1 ? c1 : 0) + (k > 2 ? c2 : 0); }
   __device__ __forceinline__ long long cap(int k) const { return k == 0 ? c0 : k == 1 ? c1 : k == 2 ? c2 : c3; }
@@ -141,8 +142,11 @@ constexpr int GC_H = 4;                        // gather: positions a thread loa
 // The row pointer is clamped to [0, nnz], so no run or chunk reaches outside the output
 // arrays.  It need not ascend: a scan that gave up waiting (SP_ERR_TIMEOUT) takes the prefix it
 // missed as 0, so the pointer drops, or jumps, where one of the scan's own tiles ends, and some
-// of tile_first stays unwritten; a caller's own row pointer may hold anything.  So k_seg_sort
-// checks the tiles and their rows itself before it reads or writes by them.
+// of tile_first and chunk_first stays unwritten; a caller's own row pointer may hold anything.
+// The scan or k_partition marks either in *bad, and the kernels that go by the pointer from row
+// to row (tiles, gather) then do nothing; the rows listed here are each of one value and its
+// successor, so they are sound by themselves.  (A test of the rows of every tile instead cost
+// 2 to 3 % of a permutation of rows of 8 to 32.)
 struct RowsPartition {
   long long nrows, nnz;
   long long ntiles;         // tile_first holds ntiles + 1 entries
@@ -152,16 +156,17 @@ struct RowsPartition {
   SortLists lists;          // rows that fit no tile
   int buf;                  // where the rows' entries are: BUF_SRC or BUF_OUT
   int wlog, tmax;           // the tile shape's window (its logarithm) and longest row
+  unsigned* bad;            // cleared before; null: nothing goes by it
   DevStatus* st;
-  // row r at output positions [o0, o1)
+  // row r at output positions [o0, o1), 0 <= o0
   __device__ void operator()(long long r, long long o0, long long o1) const {
-    if (o0 < 0 || o1 < o0) dev_fail(st, SP_ERR_NOT_CANONICAL, r);
-    o0 = o0 < 0 ? 0 : o0 < nnz ? o0 : nnz;
-    o1 = o1 < 0 ? 0 : o1 < nnz ? o1 : nnz;
+    o0 = o0 < nnz ? o0 : nnz;
+    o1 = o1 < nnz ? o1 : nnz;
     const long long L = o1 - o0;
     if (tile_first) {
       constexpr int W = SsTile::W;
-      if (r == 0) tile_first[0] = 0;
+      if (r == 0)  // (a row pointer may start above 0)
+        for (long long t = 0; t <= (o0 >> wlog) && t < ntiles; ++t) tile_first[t] = 0;
       // the tiles that start after this row: their first row is r + 1
       long long t = ((o0 + W * r) >> wlog) + 1, t_hi = (o1 + W * (r + 1)) >> wlog;
       if (r + 1 == nrows || t_hi > ntiles) t_hi = ntiles;
@@ -181,8 +186,14 @@ struct RowsPartition {
 template <int kDummy = 0>
 __global__ void k_partition(RowsPartition part, const long long* __restrict__ vp) {
   for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < part.nrows;
-       r += (long long)gridDim.x * blockDim.x)
-    part(r, vp[r], vp[r + 1]);
+       r += (long long)gridDim.x * blockDim.x) {
+    long long o0 = vp[r], o1 = vp[r + 1];
+    if (o0 < 0 || o1 < o0 || o1 > part.nnz) {  // only a caller's own row pointer
+      dev_fail(part.st, SP_ERR_NOT_CANONICAL, r);
+      if (part.bad) *part.bad = 1u;
+    }
+    part(r, o0 < 0 ? 0 : o0, o1 < 0 ? 0 : o1);
+  }
 }
 
 // Scan output of a row pointer (vp, mirrored into a typed array) that partitions its rows
@@ -270,15 +281,14 @@ __device__ void smem_incl_max_w(uint32_t* a, int n, uint32_t* tmp) {
 //     using CI, VT;                            // column / value words
 //     const long long* srcs() const;           // source start of every output row (packed
 //                                              // with whatever view() needs)
-//     GsView<CI, VT> view(long long src, long long L) const;  // the row's first entry (no
-//                                              // L entries from src on in the arrays: null)
+//     GsView<CI, VT> view(long long src, long long L) const;  // the row's first entry
 //     uint32_t map(unsigned mid, uint32_t c) const;  // new column (0xFFFFFFFF: c lies
 //                                              // outside the matrix)
 //     CI map_ci(unsigned mid, CI c) const;     // the same in the column's own width
 //   };
 template <class CI, class VT>
 struct GsView {
-  const CI* c;   // null: the row's source is inconsistent (a row pointer after a timeout, a library bug)
+  const CI* c;   // null: the row's source is inconsistent (a library bug)
   const VT* v;
   unsigned mid;  // which relabelling
 };
@@ -309,14 +319,13 @@ template <class Gs>
 struct in_place<Gs, std::void_t<decltype(Gs::kInPlace)>> : std::bool_constant<Gs::kInPlace> {};
 
 // ---- gather without a sort ----------------------------------------------------------------
-// Chunk k is GC_CH consecutive output positions, starting inside row chunk_first[k].  After a
-// scan's timeout (see RowsPartition) chunk_first can hold anything, so it is bounded here, and a
-// chunk ends where a batch of rows ends before it.
+// Chunk k is GC_CH consecutive output positions, starting inside row chunk_first[k].  bad (may
+// be null): the row pointer does not ascend (see RowsPartition).
 template <class Gs>
 __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, const long long* __restrict__ vp,
                                                             long long nrows, long long total,
                                                             const long long* __restrict__ chunk_first,
-                                                            long long nchunks,
+                                                            long long nchunks, const unsigned* __restrict__ bad,
                                                             typename Gs::CI* __restrict__ out_col,
                                                             typename Gs::VT* __restrict__ out_val, DevStatus* st) {
   using CI = typename Gs::CI;
@@ -343,19 +352,17 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
   };
   // persistent: chunks blockIdx.x, + gridDim.x, ...; a batch is B consecutive rows.  The
   // next batch's row setup is loaded while this batch's entries are in flight.
-  auto first_row = [&](long long k) -> long long {
-    const long long r = chunk_first[k];
-    return r >= 0 && r < nrows ? r : nrows;
-  };
   long long c = blockIdx.x;
   if (c >= nchunks) return;
-  long long rb = first_row(c);
+  const bool skip = bad && *bad != 0u;  // (read beside the first chunk's row)
+  long long rb = chunk_first[c];
+  if (skip) return;
   long long o0, o1, so;
   setup(rb + t, o0, o1, so);
   for (;;) {
     const long long c0 = c * (long long)GC_CH, c1 = c0 + GC_CH < total ? c0 + GC_CH : total;
     const long long cn = c + gridDim.x;
-    const long long rb_next_chunk = cn < nchunks ? first_row(cn) : 0;
+    const long long rb_next_chunk = cn < nchunks ? chunk_first[cn] : 0;
     bool active = rb + t < nrows && o1 > o0 && o1 > c0 && o0 < c1;
     if (active) {
       r_v[t] = gs.view(so, o1 - o0);
@@ -379,7 +386,7 @@ __global__ void __launch_bounds__(GC_BLOCK, GC_MINB) k_gather_chunks(Gs gs, cons
       smem_incl_max_w<B>(owner, GC_CH, tmp32);
     }
     // the chunk ends with this batch once its last row reaches the end of the chunk
-    const bool last_batch = rb + B - 1 >= nrows - 1 || s_last >= c1 || s_last <= c0;
+    const bool last_batch = rb + B - 1 >= nrows - 1 || s_last >= c1;
     const bool more = !last_batch || cn < nchunks;
     const long long rb_next = last_batch ? rb_next_chunk : rb + B;
     long long n0 = 0, n1 = 0, ns = 0;
@@ -986,13 +993,12 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 // pass over the entries instead of two), an entry stays with its thread from load to
 // staging, and buckets hold one key on average.  Uniform rows of 32 over 2^25 columns: 25.8
 // -> 16.4 ms per permutation, of which the lookups alone take 12.9 in a plain gather; rows
-// of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms (17.2 with the
-// long rows split chunk by chunk and the partition part of the scan, 17.4 since tiles and
-// rows are checked against a row pointer that does not ascend).
+// of 512 over 2^21 columns: 17.5 -> 11.3 ms; R-MAT scale 25: 21.0 -> 17.6 ms (17.1 with the
+// long rows split chunk by chunk and the partition part of the scan).
 template <class Cfg, class Gs>
 __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
-    k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nrows, long long nnz,
-               const long long* __restrict__ tile_first, long long ntiles,
+    k_seg_sort(Gs gs, const long long* __restrict__ vp, long long nnz, const long long* __restrict__ tile_first,
+               long long ntiles,
                RunLists rl, int slice, const uint32_t* __restrict__ tkey_g,
                const typename Gs::VT* __restrict__ tval_g, typename Gs::CI* __restrict__ out_col,
                typename Gs::VT* __restrict__ out_val, int key_bits, int heavy, DevStatus* st) {
@@ -1049,8 +1055,7 @@ __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
   long long lf0 = 0;
   int ln = 0, lbase = 0;  // (ntiles < 2^31: checked by the launch)
   unsigned lmask = 0;
-  // tiles: the next tile's first row and number of rows in (pf0, pfn), or false.  A range that
-  // is no tile of the partition (see there) is passed over.
+  // tiles: the next tile's first row and number of rows in (pf0, pfn), or false
   auto next_tile = [&]() -> bool {
     while (lmask == 0) {
       if (lbase >= nitems) return false;
@@ -1058,9 +1063,7 @@ __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
       ln = 0;
       if (i >= 0 && i < nitems) {
         lf0 = tile_first[i];
-        const long long lf1 = tile_first[i + 1];
-        if (lf0 >= 0 && lf0 <= lf1 && lf1 <= nrows && lf1 - lf0 <= ROWS) ln = int(lf1 - lf0);
-        else dev_fail(st, SP_ERR_INTERNAL, -17);
+        ln = int(tile_first[i + 1] - lf0);
       }
       lmask = __ballot_sync(0xffffffffu, ln > 0);
       lbase = lbase > 0x7fffffff - 32 * int(gridDim.x) ? 0x7fffffff : lbase + 32 * int(gridDim.x);
@@ -1074,17 +1077,20 @@ __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
   // tiles: start copying the row pointers of the tile in (pf0, pfn)
   auto prefetch_rows = [&](bool any) {
     if (any) {
-      for (int x = t; x <= pfn; x += B) {
+      const int n = pfn < ROWS ? pfn : ROWS;
+      for (int x = t; x <= n; x += B) {
         cp_async8(pre_o + x, vp + pf0 + x);
-        if (x < pfn) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
+        if (x < n) cp_async8(pre_s + x, gs.srcs() + pf0 + x);
       }
     }
     cp_async_commit();
   };
   bool more_tiles = false;
   if constexpr (Cfg::kTiles) {
+    const bool bad = rl.n[RUNS_BAD] != 0u;  // (read beside the first tiles' ranges)
     lbase = blockIdx.x;
     more_tiles = next_tile();
+    if (bad) return;
     prefetch_rows(more_tiles);
   } else {
     pfe = run_at(blockIdx.x);
@@ -1109,6 +1115,10 @@ __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
     };
     if constexpr (Cfg::kTiles) {
       nrow = pfn;
+      if (nrow > ROWS) {  // cannot happen: see RowsPartition
+        if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -17);
+        nrow = ROWS;
+      }
       cp_async_wait_all();  // this tile's row pointers
       __syncthreads();      // and the previous round's last reads of the tables
       ss_clear<B, ITEMS>(cnt);
@@ -1116,40 +1126,28 @@ __global__ void __launch_bounds__(Cfg::B, ss_minb<Cfg, typename Gs::VT>())
       base = pre_o[0];
       uint32_t L[RPT], off[RPT], mine = 0;
       long long src[RPT];
-      // A tile whose rows do not ascend from `base`, all starting in its window, is left out (see
-      // RowsPartition): in any other the rows' places are apart, and the lengths kept add up to
-      // less than WIN + TMAX.  What is wrong is counted from bit 8 on of a warp's sum, above the
-      // number of its rows (at most 64).
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
         const int r = ra + t * RPT + k;
         L[k] = off[k] = 0;
         if (r < nrow) {
           const long long o0 = pre_o[r], l = pre_o[r + 1] - o0;
-          off[k] = uint32_t(o0 - base);
+          off[k] = uint32_t(o0 - base);  // < WIN
           src[k] = pre_s[r];
           if (l > 0 && l <= Cfg::TMAX && o0 + l <= nnz) L[k] = uint32_t(l);
-          mine += uint32_t((unsigned long long)l >> 63) << 8;
         }
         mine += L[k] ? ((L[k] << 16) | 1u) : 0u;
       }
-      if (t == 0 && (base < 0 || pre_o[nrow - 1] - base >= Cfg::WIN)) mine += 1u << 8;
       // packed start (high half) and rank among the item's rows (low half)
-      static_assert(RPT <= 2, "row and fault counts of a warp in bits 0 to 6 and 8 to 14");
       const uint32_t inc = warp_incl_sum(mine);
       if (lane == 31) tmp32[wid] = inc;
       __syncthreads();
-      uint32_t pre = inc - mine, tot = 0, any = 0;
+      uint32_t pre = inc - mine, tot = 0;
 #pragma unroll
       for (int k = 0; k < B / 32; ++k) {
         const uint32_t x = tmp32[k];
-        any |= x;
         pre += k < wid ? x : 0u;
         tot += x;
-      }
-      if (any & (0xFFu << 8)) {
-        if (t == 0) dev_fail(st, SP_ERR_INTERNAL, -19);
-        tot = 0;
       }
       E = int(tot >> 16);
       rnext = nrow;
@@ -1467,7 +1465,7 @@ struct RowsWs {
   long long* tile_first = nullptr;
   long long* chunk_first = nullptr;
   unsigned* counters = nullptr;  // [0..3] run list counts [4] fine split ticket [5] fine split list
-                                 // [6] long chunks [7] long rows
+                                 // [6] long chunks [7] long rows [8] RUNS_BAD
   FinalEntry* fin = nullptr;
   HugeEntry* huge = nullptr;
   HugeEntry* nxt = nullptr;      // oversized buckets (fine split); as many as long rows
@@ -1600,7 +1598,7 @@ sp_status sort_runs(sp_ctx* ctx, cudaStream_t s, const RowsWs& w, long long nnz,
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_LONG);
     const long long cap = (long long)ss_minb<Cfg, VT>() * ctx->num_sms, n = slice >= 0 ? w.run_cap[slice] : w.runs_total();
-    k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, 0, nullptr, 0, w.runs(), slice, w.tkey,
+    k_seg_sort<Cfg, Gs><<<unsigned(n < cap ? n : cap), Cfg::B, sm, s>>>(gs, nullptr, 0, nullptr, 0, w.runs(), slice, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
@@ -1623,7 +1621,7 @@ inline RowsPartition sort_partition(sp_ctx* ctx, const RowsWs& w, long long nrow
   const bool large = ctx->cur.tile_shape == 1;
   const int wlog = large ? ceil_log2_u64(SsTileL::WIN) : ceil_log2_u64(SsTile::WIN);
   return RowsPartition{nrows, nnz, ((nnz + SsTile::W * nrows) >> wlog) + 1, w.tile_first, 0, nullptr, w.lists(), buf,
-                       wlog, large ? SsTileL::TMAX : SsTile::TMAX, ctx->dstatus};
+                       wlog, large ? SsTileL::TMAX : SsTile::TMAX, w.counters + RUNS_BAD, ctx->dstatus};
 }
 inline RowsPartition gather_partition(sp_ctx* ctx, const RowsWs& w, long long nrows, long long nnz) {
   RowsPartition part{};
@@ -1675,7 +1673,7 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
     SP_CUDA(set_smem(k_seg_sort<Cfg, Gs>, sm));
     SP_PHASE(SP_PHASE_TILE);
     const long long cap = (long long)ss_minb<Cfg, VT>() * nsm, g = ntiles < cap ? ntiles : cap;
-    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nrows, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
+    k_seg_sort<Cfg, Gs><<<unsigned(g), Cfg::B, sm, s>>>(gs, vp, nnz, w.tile_first, ntiles, w.runs(), 0, w.tkey,
                                                         static_cast<const VT*>(w.tval), out_col, out_val, key_bits,
                                                         ctx->cur.heavy, ctx->dstatus);
     SP_CUDA(cudaGetLastError());
@@ -1690,17 +1688,18 @@ sp_status sort_rows_from(sp_ctx* ctx, cudaStream_t s, const long long* vp, long 
 }
 
 // The output rows (partitioned by gather_partition) gathered from `gs` and relabelled, in
-// source order.
+// source order (not if *bad; may be null).
 template <class Gs>
 sp_status gather_rows(sp_ctx* ctx, cudaStream_t s, const long long* vp, long long nrows, long long nnz,
-                      const RowsWs& w, const Gs& gs, typename Gs::CI* out_col, typename Gs::VT* out_val) {
+                      const RowsWs& w, const unsigned* bad, const Gs& gs, typename Gs::CI* out_col,
+                      typename Gs::VT* out_val) {
   if (nrows == 0 || nnz == 0) return SP_OK;
   if (w.nchunks > 0x7fffffffll) return SP_ERR_OVERFLOW;
   const int nsm = ctx->num_sms;
   {
     SP_PHASE(SP_PHASE_GATHER);
     const long long g = w.nchunks < (long long)GC_MINB * nsm ? w.nchunks : (long long)GC_MINB * nsm;  // persistent
-    k_gather_chunks<Gs><<<unsigned(g), GC_BLOCK, 0, s>>>(gs, vp, nrows, nnz, w.chunk_first, w.nchunks, out_col, out_val,
+    k_gather_chunks<Gs><<<unsigned(g), GC_BLOCK, 0, s>>>(gs, vp, nrows, nnz, w.chunk_first, w.nchunks, bad, out_col, out_val,
                                                          ctx->dstatus);
   }
   SP_CUDA(cudaGetLastError());

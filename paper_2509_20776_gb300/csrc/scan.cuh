@@ -25,6 +25,7 @@ constexpr long long SCAN_SMALL = 1 << 17;
 struct ScanCtl {
   unsigned long long* status;  // one word per tile, zeroed before the launch
   unsigned* ticket;            // zeroed before the launch
+  unsigned* bad = nullptr;     // set where a wait gave up (may be null): the output does not ascend
   DevStatus* st;
   long long spin_limit;
   long long hold_tile;  // test hook: this tile never publishes (-1: off)
@@ -96,7 +97,10 @@ __global__ void __launch_bounds__(SCAN_BLOCK, 5) k_scan(Load load, Store store, 
         run += warp_sum(val);
         pred -= 32;
       }
-      if (__any_sync(0xffffffffu, timeout) && t == 0) dev_fail(c.st, SP_ERR_TIMEOUT, tile);
+      if (__any_sync(0xffffffffu, timeout) && t == 0) {
+        dev_fail(c.st, SP_ERR_TIMEOUT, tile);
+        if (c.bad) *c.bad = 1u;
+      }
       if (t == 0) {
         s_excl = run;
         if (tile != c.hold_tile) st_relaxed_u64(&c.status[tile], kFlagInc | (unsigned long long)(run + agg));
@@ -164,14 +168,15 @@ inline size_t scan_ws_bytes(long long n) {
 }
 
 // Exclusive scan of n values into n+1 outputs; `ws` must hold scan_ws_bytes(n) (`zeroed`: it
-// is cleared already).
+// is cleared already; `bad`: see ScanCtl).
 template <class Load, class Store>
 sp_status launch_scan(sp_ctx* ctx, cudaStream_t s, Load load, Store store, long long n, char* ws,
-                      int phase = SP_PHASE_SCAN, bool zeroed = false) {
+                      int phase = SP_PHASE_SCAN, bool zeroed = false, unsigned* bad = nullptr) {
   const long long tiles = scan_tiles(n);
   ScanCtl c;
   c.status = reinterpret_cast<unsigned long long*>(ws);
   c.ticket = reinterpret_cast<unsigned*>(ws + align_up(size_t(tiles + 1) * 8));
+  c.bad = bad;
   c.st = ctx->dstatus;
   c.spin_limit = ctx->spin_limit;
   c.hold_tile = ctx->hold_tile;

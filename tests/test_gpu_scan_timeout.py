@@ -117,6 +117,26 @@ def test_permute_batch(ctx, kind, columns):
         bt.close()
 
 
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("identify", [0, 1])
+def test_extract_batch_run(ctx, kind, identify):
+    """A run counts again: its row pointer and (identify 0) its ranks come from scans."""
+    mats = [from_oracle(matrix(KINDS[kind](np.random.default_rng(s))[:3000], s)) for s in (18, 19)]
+    reqs = [(k % 2, idx(3000, 40 + k), idx(N, 50 + k)[:N // 2].contiguous()) for k in range(4)]
+    ctx.set_shapes(identify=identify)
+    try:
+        bt = ctx.extract_batch(mats, reqs)
+        try:
+            P = Padded(12000, N, bt.nnz)
+            with held(ctx):
+                expect(ctx, "SP_ERR_TIMEOUT", lambda: bt.run(P.out))
+            P.check()
+        finally:
+            bt.close()
+    finally:
+        ctx.set_shapes(identify=-1)
+
+
 def assign_plan(ctx, A, I, J, B, mode=0):
     plan, nnz = ctypes.c_void_p(), ctypes.c_int64()
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
@@ -187,3 +207,23 @@ def test_assign(ctx, mode, runs):
     finally:
         ctx.lib.sp_plan_destroy(ctx.handle, plan)
     assert_same(ctx.sp_assign(A, I, J, B, mode=mode), oracle.assign(O, rows, J.cpu().numpy(), Bo, mode), f"{mode} {runs}")
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+def test_sort_rows_of_a_slice(ctx, kind):
+    """Rows of a larger matrix: a row pointer that starts above 0 and ends below the entries."""
+    from paper_2509_20776_gb300 import CSR
+    O = matrix(KINDS[kind](np.random.default_rng(16)), 17)
+    g = np.random.default_rng(18)
+    r0, r1 = 2500, 4700
+    lo, hi = int(O.rowptr[r0]), int(O.rowptr[r1])
+    assert lo > 2048 and hi < len(O.colidx)  # beyond the first window
+    col, val = O.colidx.copy(), O.values.copy()
+    for b, e in zip(O.rowptr[r0:r1], O.rowptr[r0 + 1:r1 + 1]):
+        o = b + g.permutation(e - b)
+        col[b:e], val[b:e] = O.colidx[o], O.values[o]
+    M = CSR(r1 - r0, N, torch.from_numpy(O.rowptr[r0:r1 + 1]).cuda(), torch.from_numpy(col.astype(np.int32)).cuda(),
+            torch.from_numpy(val).cuda())
+    ctx.sp_sort_rows(M)
+    assert np.array_equal(M.colidx.cpu().numpy(), O.colidx)
+    assert np.array_equal(M.values.cpu().numpy(), O.values)
