@@ -456,8 +456,11 @@ SP_API sp_status sp_kept_counts(sp_ctx* ctx, const sp_csr* A, const void* I, int
 
 /* Sort every row of M by column, in place, moving values with their columns (the
  * Build step's sort, Sec. 3.1 Step 3).  Column indices must be distinct within each
- * row and in [0, M->ncols).  Errors: SP_ERR_INVALID_ARG, SP_ERR_OVERFLOW (ncols too
- * large for the 32-bit sort keys). */
+ * row and in [0, M->ncols).  The rows may be a part of the arrays: the row pointer may
+ * start above 0 and end below M->nnz.  Errors: SP_ERR_INVALID_ARG, SP_ERR_OVERFLOW (ncols
+ * too large for the 32-bit sort keys); found on the device: SP_ERR_NOT_CANONICAL (the row
+ * pointer decreases or leaves [0, M->nnz]; detail: a row), SP_ERR_INDEX_RANGE (a column),
+ * SP_ERR_INTERNAL (columns repeated thousands of times within a row). */
 SP_API sp_status sp_sort_rows(sp_ctx* ctx, sp_csr* M, sp_stream_t stream);
 
 /* Check that A is canonical CSR.  Synchronises; returns SP_ERR_NOT_CANONICAL (detail:
