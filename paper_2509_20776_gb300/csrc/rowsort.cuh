@@ -988,7 +988,7 @@ __device__ __forceinline__ uint32_t ss_rank(const uint32_t* sk, uint32_t s, uint
 //
 // What bounds it: shared-memory wavefronts and issue slots (profiles of a tile sort: rows of
 // 512 entries 80 % of the LSU data pipe, 53 % of issue, 22 % of the DRAM copy rate; 2 M random
-// rows of R-MAT scale 25, where the lookups miss L2, 58, 52 and 27 %), and for a matrix whose
+// rows of R-MAT scale 25, where the lookups miss L2, 60, 55 and 28 %), and for a matrix whose
 // column map exceeds L2 the random lookups.  So the gather is part of the sort (one
 // pass over the entries instead of two), an entry stays with its thread from load to
 // staging, and buckets hold one key on average.  Uniform rows of 32 over 2^25 columns: 25.8
